@@ -4,7 +4,10 @@ The functions carry the C names (sd_plan_create, sd_plan_create_ex, sd_spmm,
 sd_spmm_host, sd_plan_destroy, sd_plan_get_info, sd_plan_get_bsr,
 sd_plan_get_tiles, sd_last_error); `Plan` is a small convenience wrapper over
 them.  torch is used for device memory and streams only.  There is no
-fallback: if the shared library is missing, loading raises.
+fallback: if the shared library is missing, loading raises.  sd_spmm and
+sd_plan_update_values, the two calls of an inner loop, go through the extension
+module _pycall (csrc/sd_pycall.c) instead of ctypes, which costs more host time
+than a small product takes on the GPU.
 """
 from __future__ import annotations
 
@@ -67,6 +70,7 @@ class sd_features_t(C.Structure):
 
 
 _lib = None
+_call = None   # the _pycall module, bound to the library's addresses at the first call
 
 
 def load():
@@ -121,6 +125,23 @@ def load():
     lib.sd_version.restype = C.c_char_p
     _lib = lib
     return lib
+
+
+def _bind():
+    """Bind the _pycall module to libsd.so and to torch's current stream (torch's CUDA state is initialised here)."""
+    global _call
+    lib = load()
+    import torch
+    try:
+        from . import _pycall
+    except ImportError as e:
+        raise RuntimeError("the _pycall extension is missing or does not fit this Python: run "
+                           "`python -m paper_2608_05033_b200.build`") from e
+    torch.cuda.current_stream()
+    _pycall.bind(C.cast(lib.sd_spmm, C.c_void_p).value, C.cast(lib.sd_plan_update_values, C.c_void_p).value,
+                 torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream)
+    _call = _pycall
+    return _pycall
 
 
 class SdError(RuntimeError):
@@ -181,7 +202,7 @@ def sd_plan_create_ex(rowptr, colind, vals, M: int, K: int, N: int, dtype: int =
 
 
 def sd_spmm(plan, B, ldb: int, Cmat, ldc: int, alpha: float, beta: float, stream=None):
-    rc = load().sd_spmm(plan, _ptr(B), ldb, _ptr(Cmat), ldc, alpha, beta, _stream_handle(stream))
+    rc = (_call or _bind()).spmm(plan, B, ldb, Cmat, ldc, alpha, beta, stream)
     if rc != SD_OK:
         _raise(rc)
 
@@ -193,7 +214,7 @@ def sd_spmm_host_async(plan, B_host, ldb: int, C_host, ldc: int, alpha: float, b
 
 
 def sd_plan_update_values(plan, vals, stream=None):
-    rc = load().sd_plan_update_values(plan, _ptr(vals), _stream_handle(stream))
+    rc = (_call or _bind()).update_values(plan, vals, stream)
     if rc != SD_OK:
         _raise(rc)
 
@@ -341,7 +362,9 @@ class Plan:
                                         test_wait_expiry=test_wait_expiry, heavy_len=heavy_len)
 
     def spmm(self, B, Cmat, alpha: float = 1.0, beta: float = 0.0, stream=None):
-        sd_spmm(self.handle, B, B.stride(0), Cmat, Cmat.stride(0), alpha, beta, stream)
+        rc = (_call or _bind()).spmm_tensors(self.handle, B, Cmat, alpha, beta, stream)
+        if rc != SD_OK:
+            _raise(rc)
         return Cmat
 
     def spmm_host(self, B_host, C_host, alpha: float = 1.0, beta: float = 0.0):

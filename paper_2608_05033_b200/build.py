@@ -3,8 +3,9 @@
     python -m paper_2608_05033_b200.build [--force] [--verbose]
 
 Every .cu under csrc/ is compiled to an object in build/ (in parallel) and the
-objects are linked into paper_2608_05033_b200/libsd.so.  Nothing is compiled
-for any other architecture and there is no fallback.
+objects are linked into paper_2608_05033_b200/libsd.so; csrc/sd_pycall.c becomes
+the extension module _pycall (CPython entry points of the calls inside a loop).
+Nothing is compiled for any other architecture and there is no fallback.
 """
 from __future__ import annotations
 
@@ -13,12 +14,14 @@ import glob
 import os
 import subprocess
 import sys
+import sysconfig
 
 PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(ROOT, "build", "obj")
 LIB = os.path.join(PKG, "libsd.so")
+PYCALL = os.path.join(PKG, "_pycall.so")
 
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -57,6 +60,12 @@ def build(force: bool = False, verbose: bool = False) -> str:
                                                       "-Xcompiler", "-fPIC"]
         subprocess.check_call(cmd)
         os.replace(tmp, LIB)
+    src = os.path.join(CSRC, "sd_pycall.c")
+    if force or not os.path.exists(PYCALL) or os.path.getmtime(PYCALL) < os.path.getmtime(src):
+        tmp = PYCALL + ".tmp.%d" % os.getpid()
+        subprocess.check_call([os.environ.get("CC", "gcc"), "-O2", "-Wall", "-shared", "-fPIC", "-fvisibility=hidden",
+                               "-I", sysconfig.get_path("include"), src, "-o", tmp])
+        os.replace(tmp, PYCALL)
     return LIB
 
 
