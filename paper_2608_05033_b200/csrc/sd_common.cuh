@@ -207,6 +207,30 @@ inline int occupancy_cached(std::atomic<int> (&cache)[kMaxDevices], Kernel kerne
     return v;
 }
 
+// ---- overlapped launches ---------------------------------------------------------------------
+// Kernels of this library that follow one another in a stream overlap their ends: a kernel launched with
+// launch_overlapped starts once every CTA of the kernel before it has begun and called overlap_next(), and may
+// read what never changes during the life of a plan (row pointers, columns, plan tables).  Before it touches
+// anything that earlier work in the stream may write (values, B, C, scratch) every thread calls overlap_wait(), which
+// returns when the earlier kernels have completed and their writes are visible.  Each kernel waits, so completion
+// is transitive.  A small kernel (2,048 rows, 32 columns) repeats every 6.1 us without this.
+__device__ __forceinline__ void overlap_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void overlap_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... Params, typename... Args>
+inline cudaError_t launch_overlapped(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+}
+
 inline int ceil_div(int64_t a, int64_t b) { return static_cast<int>((a + b - 1) / b); }
 
 }  // namespace sd

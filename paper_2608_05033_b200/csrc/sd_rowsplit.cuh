@@ -29,6 +29,11 @@ rowsplit_kernel(const SpmmArgs a) {
         p0 = __ldg(a.ptr + row);
         len = __ldg(a.ptr + row + 1) - p0;
     }
+    // the first (column, value) pairs' columns do not depend on earlier work in the stream
+    int firstc = 0;
+    if (lg < len) firstc = __ldg(a.colind + p0 + lg);
+    overlap_next();
+    overlap_wait();
     // trip counts are made warp-uniform so that the shuffles below are always converged
     const int maxlen = (LPR == 32) ? len : __reduce_max_sync(FULL, len);
 
@@ -83,7 +88,7 @@ rowsplit_kernel(const SpmmArgs a) {
         int myc = 0;
         float myv = 0.f;
         if (base + lg < len) {
-            myc = __ldg(a.colind + p0 + base + lg);
+            myc = base == 0 ? firstc : __ldg(a.colind + p0 + base + lg);
             myv = to_float(vals[p0 + base + lg]);
         }
         const int cnt = min(LPR, maxlen - base);
@@ -139,9 +144,8 @@ cudaError_t launch_rowsplit_one(const SpmmArgs &a, cudaStream_t st) {
     const int rows_per_cta = kRowsplitThreads / LPR;
     dim3 grid(static_cast<unsigned>((a.S + rows_per_cta - 1) / rows_per_cta),
               static_cast<unsigned>((a.N + LPR * NV * VW - 1) / (LPR * NV * VW)));
-    if (a.max_len > 0 && a.max_len <= 32 * LPR) rowsplit_kernel<T, VW, LPR, NV, false><<<grid, kRowsplitThreads, 0, st>>>(a);
-    else rowsplit_kernel<T, VW, LPR, NV, true><<<grid, kRowsplitThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    if (a.max_len > 0 && a.max_len <= 32 * LPR) return launch_overlapped(rowsplit_kernel<T, VW, LPR, NV, false>, grid, kRowsplitThreads, 0, st, a);
+    return launch_overlapped(rowsplit_kernel<T, VW, LPR, NV, true>, grid, kRowsplitThreads, 0, st, a);
 }
 
 // Lane geometry for a dense width: VW elements per 16-byte load when `vec`, LPR lanes per

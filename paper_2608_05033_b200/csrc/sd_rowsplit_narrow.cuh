@@ -28,6 +28,8 @@ rowsplit_narrow_kernel(const SpmmArgs a) {
         p0 = __ldg(a.ptr + row);
         p1 = __ldg(a.ptr + row + 1);
     }
+    overlap_next();
+    overlap_wait();
     float acc[N], tot[LONG ? N : 1];
 #pragma unroll
     for (int e = 0; e < N; ++e) {
@@ -137,6 +139,8 @@ rowsplit_ksplit_kernel(const SpmmArgs a) {
         p0 = __ldg(a.ptr + row);
         p1 = __ldg(a.ptr + row + 1);
     }
+    overlap_next();
+    overlap_wait();
     float acc[VW], tot[LONG ? VW : 1];
 #pragma unroll
     for (int e = 0; e < VW; ++e) {
@@ -211,9 +215,8 @@ cudaError_t launch_ksplit_g(const SpmmArgs &a, cudaStream_t st) {
         const int rows_per_cta = kNarrowThreads / (LPR * G);
         const unsigned grid = static_cast<unsigned>((a.S + rows_per_cta - 1) / rows_per_cta);
         const bool is_long = !(a.max_len > 0 && a.max_len <= static_cast<int64_t>(kNarrowFold) * G);
-        if (is_long) rowsplit_ksplit_kernel<T, VW, LPR, G, true><<<grid, kNarrowThreads, 0, st>>>(a);
-        else rowsplit_ksplit_kernel<T, VW, LPR, G, false><<<grid, kNarrowThreads, 0, st>>>(a);
-        return cudaGetLastError();
+        if (is_long) return launch_overlapped(rowsplit_ksplit_kernel<T, VW, LPR, G, true>, grid, kNarrowThreads, 0, st, a);
+        return launch_overlapped(rowsplit_ksplit_kernel<T, VW, LPR, G, false>, grid, kNarrowThreads, 0, st, a);
     }
 }
 
@@ -253,14 +256,12 @@ cudaError_t launch_narrow_g(const SpmmArgs &a, bool vec, cudaStream_t st) {
     constexpr bool CAN_VEC = sizeof(T) == 4 && N == 4;
     if constexpr (CAN_VEC) {
         if (vec) {
-            if (is_long) rowsplit_narrow_kernel<T, N, G, true, true><<<grid, kNarrowThreads, 0, st>>>(a);
-            else rowsplit_narrow_kernel<T, N, G, true, false><<<grid, kNarrowThreads, 0, st>>>(a);
-            return cudaGetLastError();
+            if (is_long) return launch_overlapped(rowsplit_narrow_kernel<T, N, G, true, true>, grid, kNarrowThreads, 0, st, a);
+            return launch_overlapped(rowsplit_narrow_kernel<T, N, G, true, false>, grid, kNarrowThreads, 0, st, a);
         }
     }
-    if (is_long) rowsplit_narrow_kernel<T, N, G, false, true><<<grid, kNarrowThreads, 0, st>>>(a);
-    else rowsplit_narrow_kernel<T, N, G, false, false><<<grid, kNarrowThreads, 0, st>>>(a);
-    return cudaGetLastError();
+    if (is_long) return launch_overlapped(rowsplit_narrow_kernel<T, N, G, false, true>, grid, kNarrowThreads, 0, st, a);
+    return launch_overlapped(rowsplit_narrow_kernel<T, N, G, false, false>, grid, kNarrowThreads, 0, st, a);
 }
 
 template <typename T, int N>
