@@ -10,6 +10,7 @@
 #include <cub/cub.cuh>
 
 #include "sd_common.cuh"
+#include "sd_hybrid.cuh"
 #include "sd_launch.cuh"
 
 // =====================================================================================
@@ -464,7 +465,9 @@ struct sd_plan {
     int64_t h_ng = 0;
     int32_t *h_light = nullptr;      // [M - h_nl] light rows, longest first, ascending inside a length
     int64_t h_nm = 0;                // the first h_nm of them have at least kHybridMedium nonzeros: one lane group per row
+    int64_t h_nw = 0;                // the first h_nw of those at least kHybridWide: a warp per row
     int4 *h_desc = nullptr;          // [M - h_nl] per light row, in list order: {row, first nonzero, its column, length} (rebuilt at load)
+    int4 *h_items = nullptr;         // [h_nc] chunks in the order of h_order: {chunk, first nonzero, 0, length} (rebuilt at load)
     int64_t h_nl = 0, h_nc = 0;
     int32_t h_T = 0;
 
@@ -611,6 +614,7 @@ constexpr int kHybridHeavy = 256;   // hybrid family: rows of at least this many
 constexpr int kHybridMedium = 4;    // light rows of at least this many nonzeros take one lane group each, a step of nonzeros
                                     // at a time; shorter ones run several rows per lane group, a nonzero at a time
                                     // (2 / 3 / 4 / 8 / 16 / 32 measured on six workloads: 4 is best or level on five)
+constexpr int kHybridWide = 32;     // light rows of at least this many nonzeros take a whole warp each, like a chunk
 constexpr int kHybridHeavyMax = 256;   // upper limit: a light row is one running sum
 
 // Re-buckets the nonzeros by column window and builds the (row, window) segment list, ordered by
@@ -998,10 +1002,27 @@ hybrid_desc_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict
     desc[i] = make_int4(r, p0, len > 0 ? colind[p0] : 0, len);
 }
 
-static sd_status_t build_light_desc(sd_plan *p, cudaStream_t st) {
+__global__ void __launch_bounds__(256)
+hybrid_items_kernel(const int2 *__restrict__ ranges, const int32_t *__restrict__ order, int64_t n, int4 *__restrict__ items) {
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int2 r = ranges[order[i]];
+    items[i] = make_int4(order[i], r.x, 0, r.y - r.x);
+}
+
+// What sd_spmm reads in place of the introspectable lists: one descriptor per chunk and per light row.
+static sd_status_t build_hybrid_desc(sd_plan *p, cudaStream_t st) {
     const int64_t n = p->M - p->h_nl;
-    if (n <= 0) return SD_OK;
     sd_status_t s;
+    if (p->h_nc > 0) {
+        if ((s = dev_alloc(p, reinterpret_cast<void **>(&p->h_items), sizeof(int4) * p->h_nc, "chunk descriptors"))) return s;
+        hybrid_items_kernel<<<ceil_div(p->h_nc, 256), 256, 0, st>>>(p->h_ranges, p->h_order, p->h_nc, p->h_items);
+        SD_CUDA_TRY(cudaGetLastError());
+    }
+    if (n <= 0) {
+        SD_CUDA_TRY(cudaStreamSynchronize(st));
+        return SD_OK;
+    }
     if ((s = dev_alloc(p, reinterpret_cast<void **>(&p->h_desc), sizeof(int4) * n, "light row descriptors"))) return s;
     hybrid_desc_kernel<<<ceil_div(n, 256), 256, 0, st>>>(p->rowptr, p->colind, p->h_light, n, p->h_desc);
     SD_CUDA_TRY(cudaGetLastError());
@@ -1028,7 +1049,7 @@ static sd_status_t build_hybrid(sd_plan *p, int W, int32_t T, cudaStream_t st) {
     p->h_T = T;
     TempBuf sel, nsel, tmp, start, by_row, by_win, row_off, win_off;
     if ((s = sel.get(sizeof(int32_t) * p->M, "heavy rows"))) return s;
-    if ((s = nsel.get(sizeof(int64_t), "heavy row count"))) return s;
+    if ((s = nsel.get(2 * sizeof(int64_t), "heavy row count"))) return s;
     size_t tb = 0;
     cub::CountingInputIterator<int32_t> ids(0);
     HeavyRow pred{p->rowptr, T};
@@ -1124,18 +1145,21 @@ static sd_status_t build_hybrid(sd_plan *p, int W, int32_t T, cudaStream_t st) {
         if ((s = dev_alloc(p, reinterpret_cast<void **>(&p->h_light), sizeof(int32_t) * (p->M - nl), "light rows"))) return s;
         SD_CUDA_TRY(cudaMemcpyAsync(p->h_light, static_cast<int32_t *>(id_out.p) + nl, sizeof(int32_t) * (p->M - nl),
                                     cudaMemcpyDeviceToDevice, st));
-        // sorted keys: 0 for the heavy rows, then T - length ascending; lengths of at least kHybridMedium have keys up to T - kHybridMedium
-        int64_t upto = nl;
-        if (T > kHybridMedium) {
-            count_not_above_kernel<<<1, 1, 0, st>>>(static_cast<int32_t *>(key_out.p), p->M, T - kHybridMedium,
-                                                    static_cast<int64_t *>(nsel.p));
-            SD_CUDA_TRY(cudaGetLastError());
-            SD_CUDA_TRY(cudaMemcpyAsync(&upto, nsel.p, sizeof upto, cudaMemcpyDeviceToHost, st));
-        }
+        // sorted keys: 0 for the heavy rows, then T - length ascending; lengths of at least L have keys up to T - L
+        int64_t upto[2] = {nl, nl};
+        const int limits[2] = {kHybridMedium, kHybridWide};
+        for (int k = 0; k < 2; ++k)
+            if (T > limits[k]) {
+                count_not_above_kernel<<<1, 1, 0, st>>>(static_cast<int32_t *>(key_out.p), p->M, T - limits[k],
+                                                        static_cast<int64_t *>(nsel.p) + k);
+                SD_CUDA_TRY(cudaGetLastError());
+                SD_CUDA_TRY(cudaMemcpyAsync(&upto[k], static_cast<int64_t *>(nsel.p) + k, sizeof upto[k], cudaMemcpyDeviceToHost, st));
+            }
         SD_CUDA_TRY(cudaStreamSynchronize(st));
-        p->h_nm = upto - nl;
-        if ((s = build_light_desc(p, st))) return s;
+        p->h_nm = upto[0] - nl;
+        p->h_nw = upto[1] - nl;
     }
+    if ((s = build_hybrid_desc(p, st))) return s;
     p->num_chunks = p->h_nc;
     p->info.num_segments = p->h_nc;
     p->info.num_tiles = p->h_nl;
@@ -1365,6 +1389,7 @@ static void free_plan(sd_plan *p) {
     cudaFree(p->h_order);
     cudaFree(p->h_light);
     cudaFree(p->h_desc);
+    cudaFree(p->h_items);
     cudaFree(p->h_giant);
     cudaFree(p->coo_row);
     cudaFree(p->coo_c1_row);
@@ -1436,7 +1461,7 @@ static sd_status_t pattern_hash(const int32_t *rowptr, const int32_t *colind, in
 }
 
 constexpr uint64_t kBlobMagic = 0x31304E414C504453ull;   // "SDPLAN01"
-constexpr uint32_t kBlobVersion = 2;
+constexpr uint32_t kBlobVersion = 3;
 constexpr int kBlobArrays = 19;
 
 struct BlobHeader {
@@ -1451,7 +1476,7 @@ struct BlobHeader {
     sd_plan_info_t info;
     int64_t num_segments, num_chunks, ntiles, nnzb;
     int32_t bsr_nparts, has_coo;
-    int64_t h_nl, h_nc, h_ng, h_nm;
+    int64_t h_nl, h_nc, h_ng, h_nm, h_nw;
     int32_t h_T, reserved;
     uint64_t array_bytes[kBlobArrays];   // payload sizes, in the order of blob_arrays(); each padded to 16 bytes in the blob
 };
@@ -1961,23 +1986,30 @@ sd_status_t sd_spmm(const sd_plan_t *plan, const void *B, int64_t ldb, float *C,
         return SD_OK;
     }
     case SD_HYBRID: {
-        // one launch for the chunks of the heavy rows, the rows of medium length and the short rows; then the chunk sums
-        SpmmArgs ca = a, ma = a, la = a;
-        ca.ranges = plan->h_ranges;
-        ca.order = plan->h_order;
-        ca.S = plan->h_nc;
-        ca.C = plan->chunk_out;
-        ca.ldc = N;
-        ca.alpha = 1.f;
-        ca.beta = 0.f;
-        ma.desc = plan->h_desc;
-        ma.S = plan->h_nm;
-        la.desc = plan->h_desc + plan->h_nm;
-        la.S = M - plan->h_nl - plan->h_nm;
-        SD_CUDA_TRY(run_hybrid_fused(ca, ma, la, plan->dtype, vec, st));
+        // one launch for the chunks of the heavy rows and all light rows; then the chunk sums
+        const int vw = piece_width(plan->dtype, N, B, ldb, C, ldc);
+        HybridArgs h;
+        h.colind = plan->colind;
+        h.vals = plan->vals;
+        h.B = B;
+        h.C = C;
+        h.scratch = plan->chunk_out;
+        h.items = plan->h_items;
+        h.desc = plan->h_desc;
+        h.ldc = ldc;
+        h.ldb_bytes = a.ldb_bytes;
+        h.N = static_cast<int32_t>(N);
+        h.chunks = static_cast<int32_t>(plan->h_nc);
+        h.wide = static_cast<int32_t>(plan->h_nw);
+        h.medium = static_cast<int32_t>(plan->h_nm - plan->h_nw);
+        h.light = static_cast<int32_t>(M - plan->h_nl - plan->h_nm);
+        h.gc = h.gm = 0;
+        h.alpha = alpha;
+        h.beta = beta;
+        SD_CUDA_TRY(plan->dtype == SD_F32 ? run_hybrid_f32(h, vw, st) : run_hybrid_bf16(h, vw, st));
         if (plan->h_nl > 0) {
             SD_CUDA_TRY(run_chunk_reduce(plan->chunk_out, plan->h_chunk_ptr, plan->h_rows, 0, plan->h_nl, C, ldc,
-                                         static_cast<int32_t>(N), alpha, beta, st, plan->h_ng > 0 ? kGiantChunks : 0));
+                                         static_cast<int32_t>(N), alpha, beta, st, plan->h_ng > 0 ? kGiantChunks : 0, true));
             if (plan->h_ng > 0)
                 SD_CUDA_TRY(run_chunk_reduce_wide(plan->chunk_out, plan->h_chunk_ptr, plan->h_rows, plan->h_giant,
                                                   plan->h_ng, C, ldc, static_cast<int32_t>(N), alpha, beta, st));
@@ -2150,7 +2182,7 @@ sd_status_t sd_plan_save(const sd_plan_t *plan, void *buf, size_t cap, size_t *b
     h.nnzb = p->nnzb;
     h.bsr_nparts = p->bsr_nparts;
     h.has_coo = p->coo_row ? 1 : 0;
-    h.h_nl = p->h_nl; h.h_nc = p->h_nc; h.h_ng = p->h_ng; h.h_nm = p->h_nm; h.h_T = p->h_T;
+    h.h_nl = p->h_nl; h.h_nc = p->h_nc; h.h_ng = p->h_ng; h.h_nm = p->h_nm; h.h_nw = p->h_nw; h.h_T = p->h_T;
     for (int i = 0; i < kBlobArrays; ++i) h.array_bytes[i] = arr[i].bytes;
     unsigned char *out = static_cast<unsigned char *>(buf);
     memset(out, 0, need);
@@ -2244,7 +2276,7 @@ sd_status_t sd_plan_load(const void *blob, size_t bytes, const int32_t *rowptr, 
     p->ntiles = h.ntiles;
     p->nnzb = h.nnzb;
     p->bsr_nparts = h.bsr_nparts;
-    p->h_nl = h.h_nl; p->h_nc = h.h_nc; p->h_ng = h.h_ng; p->h_nm = h.h_nm; p->h_T = h.h_T;
+    p->h_nl = h.h_nl; p->h_nc = h.h_nc; p->h_ng = h.h_ng; p->h_nm = h.h_nm; p->h_nw = h.h_nw; p->h_T = h.h_T;
     const unsigned char *in = static_cast<const unsigned char *>(blob);
     size_t off = pad16(sizeof(BlobHeader));
     p->wins.resize(h.nwins);
@@ -2300,7 +2332,7 @@ sd_status_t sd_plan_load(const void *blob, size_t bytes, const int32_t *rowptr, 
         if (p->h_nl > 0 &&
             (s = dev_alloc(p, reinterpret_cast<void **>(&p->chunk_out), sizeof(float) * p->h_nc * p->N, "chunk sums")))
             return fail(s);
-        if ((s = build_light_desc(p, nullptr))) return fail(s);
+        if ((s = build_hybrid_desc(p, nullptr))) return fail(s);
     } else if (p->info.family == SD_BSR_TC) {
         if ((s = dev_alloc(p, &p->bval, es * 256 * p->nnzb, "bval"))) return fail(s);
         if ((s = dev_alloc(p, &p->bval_mma, (p->dtype == SD_BF16 ? 512 : 2048) * static_cast<size_t>(p->nnzb), "bval (tensor-core image)"))) return fail(s);

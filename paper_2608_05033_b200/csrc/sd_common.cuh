@@ -112,6 +112,14 @@ __device__ __forceinline__ void store_cols(float *c, const float (&acc)[VW], flo
         if (accumulate) r += *c;
         else if (beta != 0.f) r += beta * *c;
         *c = r;
+    } else if constexpr (VW == 2) {
+        float2 r = make_float2(alpha * acc[0], alpha * acc[1]);
+        if (accumulate || beta != 0.f) {
+            const float2 o = *reinterpret_cast<const float2 *>(c);
+            const float b = accumulate ? 1.f : beta;
+            r.x += b * o.x; r.y += b * o.y;
+        }
+        __stcs(reinterpret_cast<float2 *>(c), r);
     } else {
 #pragma unroll
         for (int q = 0; q < VW / 4; ++q) {
@@ -154,11 +162,7 @@ struct SpmmArgs {
     float alpha, beta;
     int64_t max_len;        // longest row / segment if known (0: unknown); lets the row-split kernel drop its second accumulator
     int64_t mean_len;       // mean row length rounded up if known (0: unknown): lanes per row of the narrow row-split kernel
-    // hybrid family (light rows row-wise, heavy rows as chunks):
     bool load_only = false;          // host side only: the launcher loads the kernel instance it would launch and returns
-    const int4 *desc = nullptr;      // light-rows kernel: {row, first nonzero, its column, length} of every row it takes
-    const int2 *ranges = nullptr;    // chunk kernel: nonzero range [x, y) of every chunk (in the caller's CSR arrays) ...
-    const int32_t *order = nullptr;  // ... and the order in which the chunks are taken (column-window-major); work item i is chunk order[i]
 };
 
 // A/B measurement switches (none is needed in normal use).  The environment is read once, at the

@@ -22,7 +22,11 @@ struct MergeArgs {
 
 // Family (a).  `vec`: B, C, ldb, ldc and N allow 16-byte accesses.
 cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st);
-cudaError_t run_hybrid_fused(const SpmmArgs &ca, const SpmmArgs &ma, const SpmmArgs &la, int dtype, bool vec, cudaStream_t st);
+
+// Hybrid family in one launch: items (chunks of the heavy rows, long light rows), medium rows, short rows.
+struct HybridArgs;
+cudaError_t run_hybrid_f32(const HybridArgs &a, int vw, cudaStream_t st);
+cudaError_t run_hybrid_bf16(const HybridArgs &a, int vw, cudaStream_t st);
 
 // One lane group per segment (a.seg_row: output rows), or per chunk of a long segment
 // (`scratch`: chunk c writes its plain sum to row c of a.C).
@@ -35,7 +39,7 @@ cudaError_t run_single(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st);
 // seg_chunk[s+1]-1 of chunk_out ([chunks][N]); their sum, taken in order, updates C[seg_row[s]].
 cudaError_t run_chunk_reduce(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row, int64_t seg_begin,
                              int64_t seg_end, float *C, int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st,
-                             int32_t skip_above = 0);
+                             int32_t skip_above = 0, bool overlap = false);
 constexpr int kGiantChunks = 64;   // segments of more chunks than this are summed by a whole CTA
 cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row,
                                   const int32_t *list, int64_t count, float *C, int64_t ldc, int32_t N, float alpha,

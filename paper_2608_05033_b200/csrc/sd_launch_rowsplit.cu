@@ -1,6 +1,5 @@
 #include "sd_launch.cuh"
 #include "sd_rowsplit.cuh"
-#include "sd_light.cuh"
 #include "sd_rowsplit_narrow.cuh"
 #include "sd_segment.cuh"
 
@@ -25,12 +24,6 @@ cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st
     return launch_rowsplit<__nv_bfloat16>(a, vec, st);
 }
 
-// Hybrid family in one launch: chunks of the heavy rows (ca), rows of medium length (ma), short rows (la).
-cudaError_t run_hybrid_fused(const SpmmArgs &ca, const SpmmArgs &ma, const SpmmArgs &la, int dtype, bool vec, cudaStream_t st) {
-    if (dtype == SD_F32) return launch_hybrid<float>(ca, ma, la, vec, st);
-    return launch_hybrid<__nv_bfloat16>(ca, ma, la, vec, st);
-}
-
 cudaError_t run_segments(const SpmmArgs &a, int dtype, bool vec, bool scratch, cudaStream_t st) {
     if (dtype == SD_F32) return launch_seg<float>(a, vec, scratch ? 1 : 0, st);
     return launch_seg<__nv_bfloat16>(a, vec, scratch ? 1 : 0, st);
@@ -41,29 +34,26 @@ cudaError_t run_single(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st) 
     return launch_single<__nv_bfloat16>(a, vec, st);
 }
 
+// `overlap`: the kernel may be placed while the one before it in the stream drains (a plan whose kernels all run on the
+// caller's stream; not behind the events of the side-stream schedules).
 cudaError_t run_chunk_reduce(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row, int64_t seg_begin,
                              int64_t seg_end, float *C, int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st,
-                             int32_t skip_above) {
-    const int64_t n = seg_end - seg_begin;
-    if (N % 4 == 0)   // scratch rows are then 16-byte aligned
-        chunk_reduce_kernel<4><<<static_cast<unsigned>((n + 7) / 8), 256, 0, st>>>(chunk_out, seg_chunk, seg_row, seg_begin,
-                                                                                 seg_end, C, ldc, N, alpha, beta, skip_above);
-    else
-        chunk_reduce_kernel<1><<<static_cast<unsigned>((n + 7) / 8), 256, 0, st>>>(chunk_out, seg_chunk, seg_row, seg_begin,
-                                                                                 seg_end, C, ldc, N, alpha, beta, skip_above);
+                             int32_t skip_above, bool overlap) {
+    const unsigned grid = static_cast<unsigned>((seg_end - seg_begin + 7) / 8);
+    auto kernel = N % 4 == 0 ? chunk_reduce_kernel<4> : chunk_reduce_kernel<1>;   // 4: scratch rows are then 16-byte aligned
+    if (overlap)
+        return launch_overlapped(kernel, grid, 256, 0, st, chunk_out, seg_chunk, seg_row, seg_begin, seg_end, C, ldc, N,
+                                 alpha, beta, skip_above);
+    kernel<<<grid, 256, 0, st>>>(chunk_out, seg_chunk, seg_row, seg_begin, seg_end, C, ldc, N, alpha, beta, skip_above);
     return cudaGetLastError();
 }
 
 cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row,
                                   const int32_t *list, int64_t count, float *C, int64_t ldc, int32_t N, float alpha,
                                   float beta, cudaStream_t st) {
-    if (N % 4 == 0)
-        chunk_reduce_wide_kernel<4><<<static_cast<unsigned>(count), 256, 0, st>>>(chunk_out, seg_chunk, seg_row, list, C, ldc,
-                                                                                 N, alpha, beta);
-    else
-        chunk_reduce_wide_kernel<1><<<static_cast<unsigned>(count), 256, 0, st>>>(chunk_out, seg_chunk, seg_row, list, C, ldc,
-                                                                                 N, alpha, beta);
-    return cudaGetLastError();
+    auto kernel = N % 4 == 0 ? chunk_reduce_wide_kernel<4> : chunk_reduce_wide_kernel<1>;
+    return launch_overlapped(kernel, static_cast<unsigned>(count), 256, 0, st, chunk_out, seg_chunk, seg_row, list, C, ldc, N,
+                             alpha, beta);
 }
 
 // Loads every kernel instance that the multi-stream schedules of a plan of this value type and dense width can launch

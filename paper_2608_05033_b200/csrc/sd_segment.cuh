@@ -17,13 +17,10 @@ constexpr int kSegThreads = 256;
 
 // MODE 1 (SCRATCH): the segments are chunks; chunk c writes its plain sum to row c of a.C (the scratch
 // matrix).  MODE 0: a.seg_row gives the output row and whether an earlier window wrote it.
-// MODE 2: the segments are whole rows of the caller's CSR arrays named by the descriptors a.desc (hybrid
-// family, rows of medium length); walked like chunks, written like segments.
 // Up to four lanes per row: six CTAs per SM (40 registers) measure 6 % faster; wider groups lose with that cap.
-// seg_body is the kernel's body for CTA number `bx` of `nbx` (a kernel of its own, or one role of the fused kernel
-// of the hybrid family).
 template <typename T, int VW, int LPR, int NV, int MODE>
-__device__ __forceinline__ void seg_body(const SpmmArgs &a, const unsigned bx, const unsigned nbx) {
+__global__ void __launch_bounds__(kSegThreads, (LPR <= 4 && NV * VW < 8) ? 6 : 1)
+seg_kernel(const SpmmArgs a) {
     constexpr bool SCRATCH = MODE == 1;   // output: scratch rows
     constexpr bool STREAM = MODE != 0;    // walk: whole steps untested, next step's pairs requested ahead
     const int lane = threadIdx.x & 31;
@@ -41,28 +38,11 @@ __device__ __forceinline__ void seg_body(const SpmmArgs &a, const unsigned bx, c
     constexpr int QW = (NV * VW >= 8) ? 2 : (STREAM ? 8 : 4);
     constexpr int QU = LPR < QW ? LPR : QW;
 
-    const int64_t gstride = static_cast<int64_t>(nbx) * (kSegThreads / LPR);
-    for (int64_t s = (static_cast<int64_t>(bx) * kSegThreads + threadIdx.x) / LPR; s < a.S; s += gstride) {
-        int p0, p1;
-        int64_t out_row = s;   // SCRATCH: scratch row of this chunk
-        if (SCRATCH && a.ranges) {
-            // hybrid family: work item s is chunk order[s], a sub-range of one long row inside one column window
-            out_row = a.order ? __ldg(a.order + s) : s;
-            const int2 pr = __ldg(a.ranges + out_row);
-            p0 = pr.x;
-            p1 = pr.y;
-        } else if (MODE == 2) {
-            const int4 d = __ldg(a.desc + s);   // {row, first nonzero, its column, length}
-            out_row = d.x;
-            p0 = d.y;
-            p1 = d.y + d.w;
-        } else {
-            p0 = __ldg(a.ptr + s);
-            p1 = __ldg(a.ptr + s + 1);
-        }
+    const int64_t gstride = static_cast<int64_t>(gridDim.x) * (kSegThreads / LPR);
+    for (int64_t s = (static_cast<int64_t>(blockIdx.x) * kSegThreads + threadIdx.x) / LPR; s < a.S; s += gstride) {
+        const int p0 = __ldg(a.ptr + s), p1 = __ldg(a.ptr + s + 1);
         int32_t r = 0;
         if (MODE == 0) r = __ldg(a.seg_row + s);
-        if (MODE == 2) r = static_cast<int32_t>(out_row);
         float acc[NV][VW];
 #pragma unroll
         for (int v = 0; v < NV; ++v)
@@ -177,7 +157,7 @@ __device__ __forceinline__ void seg_body(const SpmmArgs &a, const unsigned bx, c
             }
         }
         if (SCRATCH) {
-            float *crow = a.C + out_row * a.ldc + cbase;
+            float *crow = a.C + s * a.ldc + cbase;
 #pragma unroll
             for (int v = 0; v < NV; ++v)
                 if (colok[v]) store_cols<VW>(crow + (v * LPR + lg) * VW, acc[v], 1.f, 0.f, 0);
@@ -188,12 +168,6 @@ __device__ __forceinline__ void seg_body(const SpmmArgs &a, const unsigned bx, c
                 if (colok[v]) store_cols<VW>(crow + (v * LPR + lg) * VW, acc[v], a.alpha, a.beta, r < 0 ? 1 : 0);
         }
     }
-}
-
-template <typename T, int VW, int LPR, int NV, int MODE>
-__global__ void __launch_bounds__(kSegThreads, (LPR <= 4 && NV * VW < 8) ? 6 : 1)
-seg_kernel(const SpmmArgs a) {
-    seg_body<T, VW, LPR, NV, MODE>(a, blockIdx.x, gridDim.x);
 }
 
 constexpr int kSingleBatch = 4;   // segments per lane group: their loads are all in flight together
@@ -256,14 +230,19 @@ __global__ void __launch_bounds__(256)
 chunk_reduce_kernel(const float *__restrict__ chunk_out, const int32_t *__restrict__ seg_chunk,
                     const int32_t *__restrict__ seg_row, int64_t seg_begin, int64_t seg_end, float *__restrict__ C,
                     int64_t ldc, int32_t N, float alpha, float beta, int32_t skip_above) {
+    overlap_next();
     const int lane = threadIdx.x & 31;
     const int64_t s = seg_begin + static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
-    if (s >= seg_end) return;
+    if (s >= seg_end) {
+        overlap_wait();
+        return;
+    }
     const int units = (N + CW - 1) / CW;
     int lpc = 1;                       // lanes per chain: a power of two covering min(units, 32)
     while (lpc < 32 && lpc < units) lpc <<= 1;
     const int nchain = 32 / lpc, chain = lane / lpc, cl = lane % lpc;
     const int32_t c0 = __ldg(seg_chunk + s), c1 = __ldg(seg_chunk + s + 1);
+    overlap_wait();
     if (skip_above > 0 && c1 - c0 > skip_above) return;   // left to chunk_reduce_wide_kernel
     const int32_t r = __ldg(seg_row + s);
     const bool accumulate = r < 0;
@@ -309,6 +288,7 @@ chunk_reduce_wide_kernel(const float *__restrict__ chunk_out, const int32_t *__r
                          const int32_t *__restrict__ seg_row, const int32_t *__restrict__ list, float *__restrict__ C,
                          int64_t ldc, int32_t N, float alpha, float beta) {
     __shared__ float part[8][32 * CW];
+    overlap_next();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t s = __ldg(list + blockIdx.x);
     const int units = (N + CW - 1) / CW;
@@ -317,6 +297,7 @@ chunk_reduce_wide_kernel(const float *__restrict__ chunk_out, const int32_t *__r
     const int nchain = 32 / lpc, chain = lane / lpc, cl = lane % lpc;
     const int32_t c0 = __ldg(seg_chunk + s), c1 = __ldg(seg_chunk + s + 1);
     const int32_t r = __ldg(seg_row + s);
+    overlap_wait();
     const bool accumulate = r < 0;
     float *crow = C + static_cast<int64_t>(r & 0x7FFFFFFF) * ldc;
     for (int ub = 0; ub < units; ub += lpc) {
@@ -364,22 +345,19 @@ cudaError_t launch_seg_one(const SpmmArgs &a, int mode, cudaStream_t st) {
     if (a.load_only) {
         cudaFuncAttributes at;
         return mode == 1 ? cudaFuncGetAttributes(&at, seg_kernel<T, VW, LPR, NV, 1>)
-             : mode == 2 ? cudaFuncGetAttributes(&at, seg_kernel<T, VW, LPR, NV, 2>)
                          : cudaFuncGetAttributes(&at, seg_kernel<T, VW, LPR, NV, 0>);
     }
     const int per_cta = kSegThreads / LPR;
     const int64_t need = (a.S + per_cta - 1) / per_cta;
     // persistent grid: exactly the CTAs that are resident together (the registers of an instance decide how
     // many of the eight 256-thread CTAs an SM takes); a larger grid would run a thin second wave
-    static std::atomic<int> occ_scratch[kMaxDevices], occ_plain[kMaxDevices], occ_rows[kMaxDevices];
+    static std::atomic<int> occ_scratch[kMaxDevices], occ_plain[kMaxDevices];
     const int occ = mode == 1 ? occupancy_cached(occ_scratch, seg_kernel<T, VW, LPR, NV, 1>, kSegThreads)
-                  : mode == 2 ? occupancy_cached(occ_rows, seg_kernel<T, VW, LPR, NV, 2>, kSegThreads)
                               : occupancy_cached(occ_plain, seg_kernel<T, VW, LPR, NV, 0>, kSegThreads);
     const int64_t cap = static_cast<int64_t>(sm_count_cached()) * occ;
     dim3 grid(static_cast<unsigned>(need < cap ? need : cap),
               static_cast<unsigned>((a.N + LPR * NV * VW - 1) / (LPR * NV * VW)));
     if (mode == 1) seg_kernel<T, VW, LPR, NV, 1><<<grid, kSegThreads, 0, st>>>(a);
-    else if (mode == 2) seg_kernel<T, VW, LPR, NV, 2><<<grid, kSegThreads, 0, st>>>(a);
     else seg_kernel<T, VW, LPR, NV, 0><<<grid, kSegThreads, 0, st>>>(a);
     return cudaGetLastError();
 }
