@@ -618,31 +618,4 @@ bsr_tc_kernel(const __grid_constant__ CUtensorMap tmapB, const TcArgs a) {
     }
 }
 
-// Permutes row-major 16x16 bf16 blocks into the K-major, unswizzled operand image:
-// 8x8 core matrices of 128 contiguous bytes, ordered [k group][row group].
-static __global__ void bsr_mma_image_bf16_kernel(const uint16_t *__restrict__ bval, uint16_t *__restrict__ img,
-                                                 int64_t nnzb) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= nnzb * 256) return;
-    const int64_t b = i >> 8;
-    const int r = (i >> 4) & 15, c = i & 15;
-    const int off = (((c >> 3) * 2 + (r >> 3)) * 8 + (r & 7)) * 8 + (c & 7);
-    img[b * 256 + off] = bval[i];
-}
-
-// fp32 blocks: hi / lo split and the K-major image: per k step (8 block columns) 1 KB holding the
-// hi block (rows 0..15) over the lo block (rows 16..31) as core matrices of 8 rows x 4 floats, ordered
-// [k half][row group: hi 0..7, hi 8..15, lo 0..7, lo 8..15].
-static __global__ void bsr_mma_image_tf32_kernel(const float *__restrict__ bval, float *__restrict__ img, int64_t nnzb) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (i >= nnzb * 256) return;
-    const int64_t b = i >> 8;
-    const int r = (i >> 4) & 15, c = i & 15;
-    const int off = (c >> 3) * 256 + ((c & 7) >> 2) * 128 + (r >> 3) * 32 + (r & 7) * 4 + (c & 3);
-    const float x = bval[i];
-    const float h = __uint_as_float(__float_as_uint(x) & 0xFFFFE000u);
-    img[b * 512 + off] = h;
-    img[b * 512 + off + 64] = x - h;
-}
-
 }  // namespace sd

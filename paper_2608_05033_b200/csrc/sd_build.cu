@@ -1,0 +1,553 @@
+// Representation builders of plan creation.
+#include <algorithm>
+
+#include <cub/cub.cuh>
+
+#include "sd_plan.cuh"
+
+namespace sd {
+
+// =====================================================================================
+// memory
+// =====================================================================================
+static std::mutex g_pool_mutex;
+static std::atomic<cudaMemPool_t> g_pools[kMaxDevices];
+
+cudaError_t pool_alloc(void **out, size_t bytes, cudaStream_t st) {
+    *out = nullptr;
+    if (bytes == 0) bytes = 16;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    if (dev >= kMaxDevices) return cudaMallocAsync(out, bytes, st);
+    cudaMemPool_t pool = g_pools[dev].load(std::memory_order_acquire);
+    if (!pool) {
+        std::lock_guard<std::mutex> lock(g_pool_mutex);
+        pool = g_pools[dev].load(std::memory_order_acquire);
+        if (!pool) {
+            cudaMemPoolProps props{};
+            props.allocType = cudaMemAllocationTypePinned;
+            props.location.type = cudaMemLocationTypeDevice;
+            props.location.id = dev;
+            uint64_t keep = kPoolKeep;
+            if ((e = cudaMemPoolCreate(&pool, &props)) != cudaSuccess) return e;
+            if ((e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep)) != cudaSuccess) return e;
+            g_pools[dev].store(pool, std::memory_order_release);
+        }
+    }
+    return cudaMallocFromPoolAsync(out, bytes, pool, st);
+}
+
+sd_status_t dev_alloc_bytes(sd_plan *p, void **out, size_t bytes, const char *what, cudaStream_t st) {
+    if (bytes == 0) bytes = 16;
+    const cudaError_t e = pool_alloc(out, bytes, st);
+    if (e != cudaSuccess) {
+        cudaGetLastError();
+        *out = nullptr;
+        set_error(SD_ERR_ALLOC, "allocating %zu bytes for %s failed: %s", bytes, what, cudaGetErrorString(e));
+        return SD_ERR_ALLOC;
+    }
+    if (p) {
+        p->owned += static_cast<int64_t>(bytes);
+        p->allocs.push_back(*out);
+    }
+    return SD_OK;
+}
+
+static std::mutex g_block_mutex;
+static std::vector<void *> g_blocks;
+constexpr size_t kHostBlocks = 8;
+
+HostBlock::HostBlock() {
+    {
+        std::lock_guard<std::mutex> lock(g_block_mutex);
+        if (!g_blocks.empty()) {
+            p = g_blocks.back();
+            g_blocks.pop_back();
+        }
+    }
+    if (!p && cudaHostAlloc(&p, kBytes, cudaHostAllocPortable) != cudaSuccess) {
+        cudaGetLastError();
+        p = nullptr;
+    }
+}
+
+HostBlock::~HostBlock() {
+    if (!p) return;
+    {
+        std::lock_guard<std::mutex> lock(g_block_mutex);
+        if (g_blocks.size() < kHostBlocks) {
+            g_blocks.push_back(p);
+            return;
+        }
+    }
+    cudaFreeHost(p);
+}
+
+// =====================================================================================
+// schedule of the merge and hybrid families
+// =====================================================================================
+// Rows by length: a stable counting sort on the key 0 (heavy) or T - length, one pass over the row pointers to count and one
+// to place.  The row-length histogram of the scan gives every key's first position, so the only scan left is over the
+// tiles of one key.
+constexpr int kSortTile = 2048, kSortWarps = 8, kSortBins = kHybridHeavyMax + 1;
+
+__device__ __forceinline__ int sort_key(int len, int T) { return len >= T ? 0 : T - len; }
+
+// Keys of a warp's 256 rows (8 per lane), counted into its bins.
+__device__ __forceinline__ void count_keys(const int32_t *__restrict__ rowptr, int64_t M, int64_t base, int T, int (&key)[8], int *bins) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int64_t r = base + i * 32 + lane;
+        key[i] = r < M ? sort_key(__ldg(rowptr + r + 1) - __ldg(rowptr + r), T) : -1;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const unsigned same = __match_any_sync(0xffffffffu, key[i]);
+        if (key[i] >= 0 && lane == __ffs(same) - 1) bins[key[i]] += __popc(same);
+        __syncwarp();
+    }
+}
+
+__global__ void __launch_bounds__(32 * kSortWarps)
+sort_count_kernel(const int32_t *__restrict__ rowptr, int64_t M, int T, int32_t ntiles, int32_t *__restrict__ hist) {
+    __shared__ int bins[kSortWarps][kSortBins];
+    for (int i = threadIdx.x; i < kSortWarps * kSortBins; i += blockDim.x) (&bins[0][0])[i] = 0;
+    __syncthreads();
+    int key[8];
+    count_keys(rowptr, M, static_cast<int64_t>(blockIdx.x) * kSortTile + (threadIdx.x >> 5) * 256, T, key, bins[threadIdx.x >> 5]);
+    __syncthreads();
+    for (int k = threadIdx.x; k <= T; k += blockDim.x) {
+        int n = 0;
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) n += bins[w][k];
+        hist[static_cast<int64_t>(k) * ntiles + blockIdx.x] = n;
+    }
+}
+
+struct SortBases {
+    int32_t first[kSortBins];
+};
+
+// One warp per key: counts become first positions.
+__global__ void __launch_bounds__(256)
+sort_prefix_kernel(const SortBases b, int T, int32_t ntiles, int32_t *__restrict__ hist) {
+    const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    if (k > T) return;
+    int run = b.first[k];
+    for (int t0 = 0; t0 < ntiles; t0 += 32) {
+        int32_t *h = hist + static_cast<int64_t>(k) * ntiles + t0 + lane;
+        const int n = t0 + lane < ntiles ? *h : 0;
+        int x = n;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int y = __shfl_up_sync(0xffffffffu, x, d);
+            if (lane >= d) x += y;
+        }
+        if (t0 + lane < ntiles) *h = run + x - n;
+        run += __shfl_sync(0xffffffffu, x, 31);
+    }
+}
+
+// Places the rows; a light row's descriptor holds everything its first gather needs, in one 16-byte load.
+__global__ void __launch_bounds__(32 * kSortWarps)
+sort_place_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, int64_t M, int T, int32_t ntiles,
+                  const int32_t *__restrict__ hist, int32_t nl, int32_t *__restrict__ rows, int4 *__restrict__ desc) {
+    __shared__ int bins[kSortWarps][kSortBins];
+    for (int i = threadIdx.x; i < kSortWarps * kSortBins; i += blockDim.x) (&bins[0][0])[i] = 0;
+    __syncthreads();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t base = static_cast<int64_t>(blockIdx.x) * kSortTile + warp * 256;
+    int key[8];
+    count_keys(rowptr, M, base, T, key, bins[warp]);
+    __syncthreads();
+    for (int k = threadIdx.x; k <= T; k += blockDim.x) {   // counts of the warps become their first positions
+        int at = hist[static_cast<int64_t>(k) * ntiles + blockIdx.x];
+#pragma unroll
+        for (int w = 0; w < kSortWarps; ++w) {
+            const int n = bins[w][k];
+            bins[w][k] = at;
+            at += n;
+        }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const unsigned same = __match_any_sync(0xffffffffu, key[i]);
+        int at = 0;
+        if (key[i] >= 0) at = bins[warp][key[i]] + __popc(same & ((1u << lane) - 1u));
+        __syncwarp();
+        if (key[i] >= 0 && lane == __ffs(same) - 1) bins[warp][key[i]] += __popc(same);
+        __syncwarp();
+        if (key[i] < 0) continue;
+        const int64_t r = base + i * 32 + lane;
+        rows[at] = static_cast<int32_t>(r);
+        if (at >= nl) {
+            const int32_t p0 = __ldg(rowptr + r), len = __ldg(rowptr + r + 1) - p0;
+            desc[at - nl] = make_int4(static_cast<int32_t>(r), p0, len > 0 ? __ldg(colind + p0) : 0, len);
+        }
+    }
+}
+
+// Chunk pointers of the heavy rows and the list of the rows of very many chunks: one CTA walks the rows (a few thousand).
+// row_off: chunks before every (row, window) pair; null with one window, where a row's length says how many it has.
+__global__ void __launch_bounds__(1024)
+chunk_ptr_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ row_off, int32_t W,
+                 int64_t nl, int32_t *__restrict__ chunk_ptr, int32_t *__restrict__ giant, int32_t *__restrict__ ngiant) {
+    using Scan = cub::BlockScan<int, 1024>;
+    __shared__ typename Scan::TempStorage tmp;
+    int c = 0, g = 0;   // chunks and listed rows before this step, the same in all threads
+    for (int64_t i0 = 0; i0 < nl; i0 += 1024) {
+        const int64_t i = i0 + threadIdx.x;
+        int n = 0;
+        if (i < nl) {
+            if (row_off) {
+                n = row_off[(i + 1) * W] - row_off[i * W];
+            } else {
+                const int32_t r = rows[i];
+                n = (__ldg(rowptr + r + 1) - __ldg(rowptr + r) + kChunkNnz - 1) / kChunkNnz;
+            }
+        }
+        int before, total, listed, all;
+        Scan(tmp).ExclusiveSum(n, before, total);
+        __syncthreads();
+        Scan(tmp).ExclusiveSum(n > kGiantChunks ? 1 : 0, listed, all);
+        __syncthreads();
+        if (i < nl) {
+            chunk_ptr[i] = c + before;
+            if (n > kGiantChunks) giant[g + listed] = static_cast<int32_t>(i);
+        }
+        c += total;
+        g += all;
+    }
+    if (threadIdx.x == 0) {
+        chunk_ptr[nl] = c;
+        *ngiant = g;
+    }
+}
+
+// One window: the chunks in row order.  A warp per heavy row.
+__global__ void __launch_bounds__(256)
+items_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ chunk_ptr, int64_t nl,
+             int4 *__restrict__ items) {
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < nl; i += warps) {
+        const int32_t r = rows[i], p0 = __ldg(rowptr + r), p1 = __ldg(rowptr + r + 1), c0 = chunk_ptr[i], c1 = chunk_ptr[i + 1];
+        for (int32_t c = c0 + lane; c < c1; c += 32) {
+            const int32_t x = p0 + (c - c0) * kChunkNnz;
+            items[c] = make_int4(c, x, 0, min(kChunkNnz, p1 - x));
+        }
+    }
+}
+
+__device__ __forceinline__ int32_t first_not_below(const int32_t *__restrict__ colind, int32_t lo, int32_t hi, int64_t col) {
+    while (lo < hi) {
+        const int32_t mid = lo + ((hi - lo) >> 1);
+        if (colind[mid] < col) lo = mid + 1;
+        else hi = mid;
+    }
+    return lo;
+}
+
+// Column windows, one thread per (heavy row i, window w): the nonzeros of the row whose columns fall in the window are a
+// contiguous range (columns ascend); counts its chunks into a row-major and a window-major table.
+__global__ void __launch_bounds__(256)
+window_count_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, const int32_t *__restrict__ rows,
+                    int64_t nl, int32_t W, int64_t wcols, int32_t *__restrict__ start, int32_t *__restrict__ by_row,
+                    int32_t *__restrict__ by_win) {
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t > nl * W) return;
+    if (t == nl * W) {
+        by_row[t] = 0;
+        by_win[t] = 0;
+        return;
+    }
+    const int64_t i = t / W;
+    const int32_t w = static_cast<int32_t>(t % W);
+    const int32_t r = rows[i], p0 = rowptr[r], p1 = rowptr[r + 1];
+    const int32_t lo = w == 0 ? p0 : first_not_below(colind, p0, p1, w * wcols);
+    const int32_t hi = w == W - 1 ? p1 : first_not_below(colind, lo, p1, (w + 1) * wcols);
+    const int32_t n = (hi - lo + kChunkNnz - 1) / kChunkNnz;
+    start[2 * t] = lo;
+    start[2 * t + 1] = hi;
+    by_row[t] = n;
+    by_win[static_cast<int64_t>(w) * nl + i] = n;
+}
+
+__global__ void __launch_bounds__(256)
+window_items_kernel(const int32_t *__restrict__ start, const int32_t *__restrict__ row_off, const int32_t *__restrict__ win_off,
+                    int64_t nl, int32_t W, int4 *__restrict__ items) {
+    const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (t >= nl * W) return;
+    const int64_t i = t / W;
+    const int32_t w = static_cast<int32_t>(t % W);
+    const int32_t c = row_off[t], o = win_off[static_cast<int64_t>(w) * nl + i];
+    const int32_t lo = start[2 * t], hi = start[2 * t + 1];
+    for (int32_t j = 0, x = lo; x < hi; ++j, x += kChunkNnz) items[o + j] = make_int4(c + j, x, 0, min(kChunkNnz, hi - x));
+}
+
+sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cudaStream_t st) {
+    sd_status_t s;
+    if (W < 1) W = 1;
+    T = std::min<int32_t>(std::max<int32_t>(T, 2), kHybridHeavyMax);
+    p->h_T = T;
+    p->h_counts.chunks_long = h.chunks_long;
+    p->h_counts.giants = h.giants;
+    std::copy(h.len_hist, h.len_hist + 256, p->h_counts.len_hist);
+    int64_t nl = static_cast<int64_t>(h.long_rows), nc = static_cast<int64_t>(h.chunks_long);
+    for (int l = T; l < 256; ++l) {
+        nl += static_cast<int64_t>(h.len_hist[l]);
+        nc += static_cast<int64_t>(h.len_hist[l]) * ((l + kChunkNnz - 1) / kChunkNnz);
+    }
+    SortBases bases;
+    bases.first[0] = 0;
+    int64_t at = nl;
+    p->h_nm = p->h_nw = 0;
+    for (int l = T - 1; l >= 0; --l) {
+        bases.first[T - l] = static_cast<int32_t>(at);
+        at += static_cast<int64_t>(h.len_hist[l]);
+        if (l >= kHybridMedium) p->h_nm = at - nl;
+        if (l >= kHybridWide) p->h_nw = at - nl;
+    }
+    p->h_nl = nl;
+    const int32_t ntiles = static_cast<int32_t>((p->M + kSortTile - 1) / kSortTile);
+    TempBuf hist(st), ngiant(st), start(st), by_row(st), by_win(st), row_off(st), win_off(st), tmp(st);
+    if ((s = hist.get(sizeof(int32_t) * (T + 1) * static_cast<size_t>(ntiles), "length counts"))) return s;
+    if ((s = dev_alloc(p, &p->h_rows, p->M, "rows by length", st))) return s;
+    if ((s = dev_alloc(p, &p->h_desc, p->M - nl, "light row descriptors", st))) return s;
+    sort_count_kernel<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->M, T, ntiles, hist.as<int32_t>());
+    SD_CUDA_TRY(cudaGetLastError());
+    sort_prefix_kernel<<<(T + 8) / 8, 256, 0, st>>>(bases, T, ntiles, hist.as<int32_t>());
+    SD_CUDA_TRY(cudaGetLastError());
+    sort_place_kernel<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->colind, p->M, T, ntiles, hist.as<int32_t>(),
+                                                         static_cast<int32_t>(nl), p->h_rows, p->h_desc);
+    SD_CUDA_TRY(cudaGetLastError());
+    p->h_nc = p->h_ng = 0;
+    p->info.launches = 1;
+    if (nl > 0) {
+        int64_t ng = static_cast<int64_t>(h.giants);
+        if ((s = dev_alloc(p, &p->h_chunk_ptr, nl + 1, "chunk pointers", st))) return s;
+        if ((s = dev_alloc(p, &p->h_giant, W == 1 ? ng : nl, "rows of many chunks", st))) return s;
+        if ((s = ngiant.get(sizeof(int32_t), "count"))) return s;
+        if (W == 1) {
+            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, nullptr, 1, nl, p->h_chunk_ptr, p->h_giant, ngiant.as<int32_t>());
+            SD_CUDA_TRY(cudaGetLastError());
+            if ((s = dev_alloc(p, &p->h_items, nc, "chunk descriptors", st))) return s;
+            items_kernel<<<ceil_div(std::min<int64_t>(nl, 148 * 64), 8), 256, 0, st>>>(p->rowptr, p->h_rows, p->h_chunk_ptr, nl, p->h_items);
+            SD_CUDA_TRY(cudaGetLastError());
+        } else {
+            const int64_t cells = nl * W;
+            if (cells + 1 > INT32_MAX) {
+                set_error(SD_ERR_UNSUPPORTED, "too many (heavy row, window) pairs");
+                return SD_ERR_UNSUPPORTED;
+            }
+            if ((s = start.get(sizeof(int32_t) * 2 * cells, "window ranges"))) return s;
+            if ((s = by_row.get(sizeof(int32_t) * (cells + 1), "chunk counts"))) return s;
+            if ((s = by_win.get(sizeof(int32_t) * (cells + 1), "chunk counts"))) return s;
+            if ((s = row_off.get(sizeof(int32_t) * (cells + 1), "chunk offsets"))) return s;
+            if ((s = win_off.get(sizeof(int32_t) * (cells + 1), "chunk offsets"))) return s;
+            window_count_kernel<<<ceil_div(cells + 1, 256), 256, 0, st>>>(p->rowptr, p->colind, p->h_rows, nl, W, (p->K + W - 1) / W,
+                                                                         start.as<int32_t>(), by_row.as<int32_t>(), by_win.as<int32_t>());
+            SD_CUDA_TRY(cudaGetLastError());
+            size_t tb = 0;
+            const int n = static_cast<int>(cells + 1);
+            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, by_row.as<int32_t>(), row_off.as<int32_t>(), n, st));
+            if ((s = tmp.get(tb, "scan scratch"))) return s;
+            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, by_row.as<int32_t>(), row_off.as<int32_t>(), n, st));
+            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, by_win.as<int32_t>(), win_off.as<int32_t>(), n, st));
+            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, row_off.as<int32_t>(), W, nl, p->h_chunk_ptr, p->h_giant, ngiant.as<int32_t>());
+            SD_CUDA_TRY(cudaGetLastError());
+            int32_t got[2] = {0, 0};
+            SD_CUDA_TRY(cudaMemcpyAsync(&got[0], p->h_chunk_ptr + nl, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            SD_CUDA_TRY(cudaMemcpyAsync(&got[1], ngiant.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            SD_CUDA_TRY(cudaStreamSynchronize(st));
+            nc = got[0];
+            ng = got[1];
+            if ((s = dev_alloc(p, &p->h_items, nc, "chunk descriptors", st))) return s;
+            window_items_kernel<<<ceil_div(cells, 256), 256, 0, st>>>(start.as<int32_t>(), row_off.as<int32_t>(), win_off.as<int32_t>(), nl,
+                                                                     W, p->h_items);
+            SD_CUDA_TRY(cudaGetLastError());
+        }
+        p->h_nc = nc;
+        p->h_ng = ng;
+        if ((s = dev_alloc(p, &p->chunk_out, static_cast<size_t>(nc) * p->N, "chunk sums", st))) return s;
+        p->info.launches = 2 + (ng > 0 ? 1 : 0);   // the fused kernel, the chunk sums, the chunk sums of very long rows
+    }
+    return SD_OK;
+}
+
+// =====================================================================================
+// narrow dense operands
+// =====================================================================================
+sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
+    sd_status_t s;
+    const int cchunk = coo_chunk(static_cast<int>(p->N));
+    const int64_t chunks1 = (p->nnz + cchunk - 1) / cchunk, count2 = 2 * chunks1;
+    const int64_t chunks2 = (count2 + kCooCarryChunk - 1) / kCooCarryChunk, count3 = 2 * chunks2;
+    if ((s = dev_alloc(p, &p->coo_row, p->nnz, "row index per nonzero", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_c1_row, count2, "carry rows", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_c1_val, count2 * p->N, "carry sums", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_c2_row, count3, "carry rows (level 2)", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_c2_val, count3 * p->N, "carry sums (level 2)", st))) return s;
+    SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, p->coo_row, st));
+    p->info.launches = 2 + (count2 > kCooDirectFinal);
+    return SD_OK;
+}
+
+// =====================================================================================
+// 16x16 blocks
+// =====================================================================================
+// The occupied block columns of a block-row, ascending, from a bitmap in shared memory (a range of kMapBits block columns
+// at a time).  Without `bcol` they are only counted.
+constexpr int kMapWords = 4096, kMapBits = 32 * kMapWords, kMapThreads = 128;
+
+__global__ void __launch_bounds__(kMapThreads)
+block_cols_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, int64_t M, int64_t Kb, int32_t Mb,
+                  const int32_t *__restrict__ browptr, int32_t *__restrict__ counts, int32_t *__restrict__ bcol) {
+    using Scan = cub::BlockScan<int, kMapThreads>;
+    __shared__ typename Scan::TempStorage tmp;
+    __shared__ unsigned map[kMapWords];
+    const int64_t I = blockIdx.x;
+    const int64_t b = __ldg(rowptr + I * 16), e = __ldg(rowptr + min((I + 1) * 16, M));
+    int found = 0;   // in earlier ranges
+    for (int64_t j0 = 0; j0 < Kb; j0 += kMapBits) {
+        const int words = static_cast<int>(min(static_cast<int64_t>(kMapWords), (Kb - j0 + 31) / 32));
+        for (int i = threadIdx.x; i < words; i += kMapThreads) map[i] = 0;
+        __syncthreads();
+        for (int64_t p = b + threadIdx.x; p < e; p += kMapThreads) {
+            const int64_t j = (__ldg(colind + p) >> 4) - j0;
+            if (j >= 0 && j < static_cast<int64_t>(words) * 32) atomicOr(&map[j >> 5], 1u << (j & 31));
+        }
+        __syncthreads();
+        for (int i0 = 0; i0 < words; i0 += kMapThreads) {
+            unsigned m = i0 + threadIdx.x < words ? map[i0 + threadIdx.x] : 0u;
+            int before, total;
+            Scan(tmp).ExclusiveSum(__popc(m), before, total);
+            if (bcol) {
+                int32_t *out = bcol + browptr[I] + found + before;
+                for (; m; m &= m - 1) *out++ = static_cast<int32_t>(j0 + (i0 + threadIdx.x) * 32 + __ffs(m) - 1);
+            }
+            found += total;
+            __syncthreads();
+        }
+    }
+    if (counts && threadIdx.x == 0) {
+        counts[I] = found;
+        if (I == Mb - 1) counts[Mb] = 0;
+    }
+}
+
+// Values of a block-row's blocks: the row-major 16x16 blocks (absent entries +0) and, beside them, the tensor-core operand
+// images, in one pass over the block-row's nonzeros: batches of kValBlocks blocks are composed in shared memory and leave as
+// whole 16-byte vectors, and nothing is cleared in global memory first.  (Three passes before: clear, scatter with a search
+// per nonzero in global memory, permute; 32 us for 4.2 M bf16 values.)
+constexpr int kValBlocks = 16, kValThreads = 256;
+
+template <typename T>
+__global__ void __launch_bounds__(kValThreads)
+block_values_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, const T *__restrict__ vals, int64_t M,
+                    const int32_t *__restrict__ browptr, const int32_t *__restrict__ bcol, T *__restrict__ bval, T *__restrict__ img) {
+    constexpr int V = 16 / sizeof(T);   // elements per vector
+    __shared__ __align__(16) T blk[kValBlocks * 256];
+    __shared__ int cols[kValBlocks], bound[17];
+    const int64_t I = blockIdx.x;
+    const int b0 = __ldg(browptr + I), b1 = __ldg(browptr + I + 1);
+    if (threadIdx.x < 17) bound[threadIdx.x] = __ldg(rowptr + min(I * 16 + threadIdx.x, M));
+    const int4 zero = make_int4(0, 0, 0, 0);
+    for (int s = b0; s < b1; s += kValBlocks) {
+        const int n = min(kValBlocks, b1 - s);
+        __syncthreads();
+        if (threadIdx.x < n) cols[threadIdx.x] = __ldg(bcol + s + threadIdx.x);
+        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) reinterpret_cast<int4 *>(blk)[i] = zero;
+        __syncthreads();
+        const int first = cols[0], last = cols[n - 1];
+        int r = 0;
+        for (int64_t p = static_cast<int64_t>(bound[0]) + threadIdx.x; p < bound[16]; p += kValThreads) {
+            while (p >= bound[r + 1]) ++r;
+            const int c = __ldg(colind + p), j = c >> 4;
+            if (j < first || j > last) continue;
+            int lo = 0, hi = n - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (cols[mid] < j) lo = mid + 1;
+                else hi = mid;
+            }
+            blk[lo * 256 + r * 16 + (c & 15)] = vals[p];
+        }
+        __syncthreads();
+        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) {
+            const int4 v = reinterpret_cast<const int4 *>(blk)[i];
+            const int64_t k = s + i / (256 / V);
+            const int x = i % (256 / V) * V, row = x >> 4, col = x & 15;   // first element of the vector
+            reinterpret_cast<int4 *>(bval)[static_cast<int64_t>(s) * (256 / V) + i] = v;
+            if constexpr (sizeof(T) == 2) {
+                // 8x8 core matrices of 128 contiguous bytes, [k group][row group]: a row of a core is one vector
+                reinterpret_cast<int4 *>(img)[k * 32 + ((col >> 3) * 2 + (row >> 3)) * 8 + (row & 7)] = v;
+            } else {
+                // per k step (8 block columns) the hi block over the lo block, core matrices of 8 rows x 4 floats, ordered
+                // [k half][row group: hi 0..7, hi 8..15, lo 0..7, lo 8..15]
+                const float4 f = make_float4(__int_as_float(v.x), __int_as_float(v.y), __int_as_float(v.z), __int_as_float(v.w));
+                float4 h;
+                h.x = __uint_as_float(__float_as_uint(f.x) & 0xFFFFE000u);
+                h.y = __uint_as_float(__float_as_uint(f.y) & 0xFFFFE000u);
+                h.z = __uint_as_float(__float_as_uint(f.z) & 0xFFFFE000u);
+                h.w = __uint_as_float(__float_as_uint(f.w) & 0xFFFFE000u);
+                float4 *out = reinterpret_cast<float4 *>(img) + k * 128 + (col >> 3) * 64 + ((col & 7) >> 2) * 32 + (row >> 3) * 8 + (row & 7);
+                out[0] = h;
+                out[16] = make_float4(f.x - h.x, f.y - h.y, f.z - h.z, f.w - h.w);
+            }
+        }
+    }
+}
+
+cudaError_t fill_bsr(const sd_plan *p, cudaStream_t st) {
+    const unsigned Mb = static_cast<unsigned>((p->M + 15) / 16);
+    if (Mb == 0 || p->nnzb == 0) return cudaSuccess;
+    if (p->dtype == SD_F32)
+        block_values_kernel<float><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, static_cast<const float *>(p->vals), p->M, p->browptr,
+                                                              p->bcol, static_cast<float *>(p->bval), static_cast<float *>(p->bval_mma));
+    else
+        block_values_kernel<uint16_t><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, static_cast<const uint16_t *>(p->vals), p->M, p->browptr,
+                                                                 p->bcol, static_cast<uint16_t *>(p->bval), static_cast<uint16_t *>(p->bval_mma));
+    return cudaGetLastError();
+}
+
+sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st) {
+    const int32_t Mb = static_cast<int32_t>((p->M + 15) / 16);
+    const int64_t Kb = (p->K + 15) / 16;
+    p->nnzb = nnzb;
+    sd_status_t s;
+    TempBuf counts(st), tmp(st);
+    if ((s = dev_alloc(p, &p->browptr, static_cast<size_t>(Mb) + 1, "browptr", st))) return s;
+    if ((s = dev_alloc(p, &p->bcol, nnzb, "bcol", st))) return s;
+    if ((s = dev_alloc_bytes(p, &p->bval, (p->dtype == SD_F32 ? 4 : 2) * 256 * static_cast<size_t>(nnzb), "bval", st))) return s;
+    // tensor-core operand images: bf16 512 bytes per block, fp32 a hi and a lo image of 1 KB each
+    if ((s = dev_alloc_bytes(p, &p->bval_mma, (p->dtype == SD_BF16 ? 512 : 2048) * static_cast<size_t>(nnzb), "bval (tensor-core image)", st))) return s;
+    if ((s = dev_alloc(p, &p->dev_error, 1, "error word", st))) return s;
+    SD_CUDA_TRY(cudaMemsetAsync(p->dev_error, 0, sizeof(int32_t), st));
+    if (Mb > 0) {
+        if ((s = counts.get(sizeof(int32_t) * (static_cast<size_t>(Mb) + 1), "block counts"))) return s;
+        block_cols_kernel<<<Mb, kMapThreads, 0, st>>>(p->rowptr, p->colind, p->M, Kb, Mb, nullptr, counts.as<int32_t>(), nullptr);
+        SD_CUDA_TRY(cudaGetLastError());
+        size_t tb = 0;
+        SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, counts.as<int32_t>(), p->browptr, Mb + 1, st));
+        if ((s = tmp.get(tb, "scan scratch"))) return s;
+        SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, counts.as<int32_t>(), p->browptr, Mb + 1, st));
+        block_cols_kernel<<<Mb, kMapThreads, 0, st>>>(p->rowptr, p->colind, p->M, Kb, Mb, p->browptr, nullptr, p->bcol);
+        SD_CUDA_TRY(cudaGetLastError());
+    } else {
+        SD_CUDA_TRY(cudaMemsetAsync(p->browptr, 0, sizeof(int32_t), st));
+    }
+    SD_CUDA_TRY(fill_bsr(p, st));
+    // one persistent CTA per SM, each with a contiguous range of block-rows of about equal cost
+    p->bsr_nparts = static_cast<int32_t>(Mb < p->info.sm_count ? Mb : p->info.sm_count);
+    if (p->bsr_nparts > 0) {
+        if ((s = dev_alloc(p, &p->bsr_part, static_cast<size_t>(p->bsr_nparts) + 1, "block-row partition", st))) return s;
+        SD_CUDA_TRY(build_bsr_partition(p->browptr, Mb, p->bsr_nparts, p->bsr_part, st));
+    }
+    return SD_OK;
+}
+
+}  // namespace sd

@@ -1,0 +1,122 @@
+// Sums of the chunks of the heavy rows (merge and hybrid families).
+#pragma once
+
+#include "sd_common.cuh"
+
+namespace sd {
+
+// One warp per heavy row: chain q of the warp adds every nchain-th chunk row, the chains
+// are then added in a fixed order (no atomics: repeated runs give identical bits).  CW columns
+// per lane (4 when N is a multiple of 4: 16-byte loads of the scratch rows).
+template <int CW>
+__global__ void __launch_bounds__(256)
+chunk_reduce_kernel(const float *__restrict__ chunk_out, const int32_t *__restrict__ chunk_ptr,
+                    const int32_t *__restrict__ rows, int64_t count, float *__restrict__ C,
+                    int64_t ldc, int32_t N, float alpha, float beta, int32_t skip_above) {
+    overlap_next();
+    const int lane = threadIdx.x & 31;
+    const int64_t s = static_cast<int64_t>(blockIdx.x) * 8 + (threadIdx.x >> 5);
+    if (s >= count) {
+        overlap_wait();
+        return;
+    }
+    const int units = (N + CW - 1) / CW;
+    int lpc = 1;                       // lanes per chain: a power of two covering min(units, 32)
+    while (lpc < 32 && lpc < units) lpc <<= 1;
+    const int nchain = 32 / lpc, chain = lane / lpc, cl = lane % lpc;
+    const int32_t c0 = __ldg(chunk_ptr + s), c1 = __ldg(chunk_ptr + s + 1);
+    overlap_wait();
+    if (skip_above > 0 && c1 - c0 > skip_above) return;   // left to chunk_reduce_wide_kernel
+    const int32_t r = __ldg(rows + s);
+    float *crow = C + static_cast<int64_t>(r) * ldc;
+    for (int ub = 0; ub < units; ub += lpc) {
+        const int col = (ub + cl) * CW;
+        float sum[CW];
+#pragma unroll
+        for (int e = 0; e < CW; ++e) sum[e] = 0.f;
+        if (col < N) {
+#pragma unroll 4
+            for (int32_t c = c0 + chain; c < c1; c += nchain) {
+                const float *p = chunk_out + static_cast<int64_t>(c) * N + col;
+                if constexpr (CW == 4) {
+                    const float4 t = *reinterpret_cast<const float4 *>(p);
+                    sum[0] += t.x; sum[1] += t.y; sum[2] += t.z; sum[3] += t.w;
+                } else {
+                    sum[0] += *p;
+                }
+            }
+        }
+        for (int off = lpc; off < 32; off <<= 1)
+#pragma unroll
+            for (int e = 0; e < CW; ++e) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], off);
+        if (chain == 0 && col < N) {
+#pragma unroll
+            for (int e = 0; e < CW; ++e) {
+                float v = alpha * sum[e];
+                if (beta != 0.f) v = fmaf(beta, crow[col + e], v);
+                crow[col + e] = v;
+            }
+        }
+    }
+}
+
+// Segments of very many chunks (list[]: their positions in chunk_ptr / rows): one CTA each.  Warp w adds the chunks
+// c0 + w, c0 + w + 8, ... with the same chains as above; the eight warp sums meet in shared memory and warp 0 adds them
+// in warp order: a fixed order again.
+template <int CW>
+__global__ void __launch_bounds__(256)
+chunk_reduce_wide_kernel(const float *__restrict__ chunk_out, const int32_t *__restrict__ chunk_ptr,
+                         const int32_t *__restrict__ rows, const int32_t *__restrict__ list, float *__restrict__ C,
+                         int64_t ldc, int32_t N, float alpha, float beta) {
+    __shared__ float part[8][32 * CW];
+    overlap_next();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t s = __ldg(list + blockIdx.x);
+    const int units = (N + CW - 1) / CW;
+    int lpc = 1;
+    while (lpc < 32 && lpc < units) lpc <<= 1;
+    const int nchain = 32 / lpc, chain = lane / lpc, cl = lane % lpc;
+    const int32_t c0 = __ldg(chunk_ptr + s), c1 = __ldg(chunk_ptr + s + 1);
+    const int32_t r = __ldg(rows + s);
+    overlap_wait();
+    float *crow = C + static_cast<int64_t>(r) * ldc;
+    for (int ub = 0; ub < units; ub += lpc) {
+        const int col = (ub + cl) * CW;
+        float sum[CW];
+#pragma unroll
+        for (int e = 0; e < CW; ++e) sum[e] = 0.f;
+        if (col < N) {
+#pragma unroll 4
+            for (int32_t c = c0 + warp * nchain + chain; c < c1; c += 8 * nchain) {
+                const float *p = chunk_out + static_cast<int64_t>(c) * N + col;
+                if constexpr (CW == 4) {
+                    const float4 t = *reinterpret_cast<const float4 *>(p);
+                    sum[0] += t.x; sum[1] += t.y; sum[2] += t.z; sum[3] += t.w;
+                } else {
+                    sum[0] += *p;
+                }
+            }
+        }
+        for (int off = lpc; off < 32; off <<= 1)
+#pragma unroll
+            for (int e = 0; e < CW; ++e) sum[e] += __shfl_xor_sync(0xffffffffu, sum[e], off);
+        if (chain == 0)
+#pragma unroll
+            for (int e = 0; e < CW; ++e) part[warp][cl * CW + e] = sum[e];
+        __syncthreads();
+        if (warp == 0 && chain == 0 && col < N) {
+#pragma unroll
+            for (int e = 0; e < CW; ++e) {
+                float t = part[0][cl * CW + e];
+#pragma unroll
+                for (int w = 1; w < 8; ++w) t += part[w][cl * CW + e];
+                float v = alpha * t;
+                if (beta != 0.f) v = fmaf(beta, crow[col + e], v);
+                crow[col + e] = v;
+            }
+        }
+        __syncthreads();
+    }
+}
+
+}  // namespace sd

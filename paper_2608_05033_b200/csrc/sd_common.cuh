@@ -162,15 +162,12 @@ struct SpmmArgs {
     float alpha, beta;
     int64_t max_len;        // longest row / segment if known (0: unknown); lets the row-split kernel drop its second accumulator
     int64_t mean_len;       // mean row length rounded up if known (0: unknown): lanes per row of the narrow row-split kernel
-    bool load_only = false;          // host side only: the launcher loads the kernel instance it would launch and returns
 };
 
 // A/B measurement switches (none is needed in normal use).  The environment is read once, at the
 // first use in the process (thread-safe), never on the sd_spmm path.
 struct Switches {
     bool no_coo;           // SD_NO_COO: generic merge kernel at one to four columns
-    bool no_side_streams;  // SD_NO_SIDE_STREAMS: the classes of a window on one stream
-    bool no_chunk_ahead;   // SD_NO_CHUNK_AHEAD: chunk kernels in window order
     bool bsr_simt;         // SD_BSR_SIMT: SIMT block kernel instead of the tensor-core one
     bool no_narrow;        // SD_NO_NARROW: wide row-split kernel at one to four columns
     int geom_nv;           // SD_GEOM_NV: 1 forces one vector per lane

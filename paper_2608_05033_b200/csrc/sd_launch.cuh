@@ -28,25 +28,15 @@ struct HybridArgs;
 cudaError_t run_hybrid_f32(const HybridArgs &a, int vw, cudaStream_t st);
 cudaError_t run_hybrid_bf16(const HybridArgs &a, int vw, cudaStream_t st);
 
-// One lane group per segment (a.seg_row: output rows), or per chunk of a long segment
-// (`scratch`: chunk c writes its plain sum to row c of a.C).
-cudaError_t run_segments(const SpmmArgs &a, int dtype, bool vec, bool scratch, cudaStream_t st);
-
-// One-nonzero segments: segment s is nonzero s of a.colind / a.vals, a.seg_row[s] its output row.
-cudaError_t run_single(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st);
-
-// Long segments of a window-major plan: segment s owns the scratch rows seg_chunk[s] ..
-// seg_chunk[s+1]-1 of chunk_out ([chunks][N]); their sum, taken in order, updates C[seg_row[s]].
-cudaError_t run_chunk_reduce(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row, int64_t seg_begin,
-                             int64_t seg_end, float *C, int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st,
-                             int32_t skip_above = 0, bool overlap = false);
-constexpr int kGiantChunks = 64;   // segments of more chunks than this are summed by a whole CTA
-cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *seg_chunk, const int32_t *seg_row,
-                                  const int32_t *list, int64_t count, float *C, int64_t ldc, int32_t N, float alpha,
-                                  float beta, cudaStream_t st);
+// Heavy rows: row rows[i] owns the scratch rows chunk_ptr[i] .. chunk_ptr[i+1]-1 of chunk_out ([chunks][N]); their sum, taken in
+// order, is its product.  skip_above > 0: rows of more chunks are left to run_chunk_reduce_wide (list: their positions).
+cudaError_t run_chunk_reduce(const float *chunk_out, const int32_t *chunk_ptr, const int32_t *rows, int64_t nl, float *C,
+                             int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st, int32_t skip_above);
+constexpr int kGiantChunks = 64;   // rows of more chunks than this are summed by a whole CTA
+cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *chunk_ptr, const int32_t *rows, const int32_t *list,
+                                  int64_t count, float *C, int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st);
 
 // C = beta * C.
-cudaError_t preload_stream_kernels(int dtype, int32_t N);
 cudaError_t run_scale_c(float *C, int64_t ldc, int64_t M, int32_t N, float beta, cudaStream_t st);
 
 // Family (b): tile kernel, then the carry-out fix-up for the listed tiles (short chains one per
@@ -120,6 +110,5 @@ sd_status_t compute_feature_counts(const int32_t *rowptr, const int32_t *colind,
                                    cudaStream_t st, FeatureCounts *out);
 
 cudaError_t build_bsr_partition(const int32_t *browptr, int32_t Mb, int32_t nparts, int32_t *part, cudaStream_t st);
-cudaError_t build_bsr_mma_image(const void *bval, void *img, int64_t nnzb, int dtype, cudaStream_t st);
 
 }  // namespace sd

@@ -13,18 +13,6 @@ cudaError_t run_bsr_simt(const BsrArgs &a, int dtype, bool vec, cudaStream_t st)
     return launch_bsr_simt<__nv_bfloat16>(a, vec, st);
 }
 
-cudaError_t build_bsr_mma_image(const void *bval, void *img, int64_t nnzb, int dtype, cudaStream_t st) {
-    if (nnzb == 0) return cudaSuccess;
-    const int64_t n = nnzb * 256;
-    const unsigned blocks = static_cast<unsigned>((n + 255) / 256);
-    if (dtype == SD_BF16)
-        bsr_mma_image_bf16_kernel<<<blocks, 256, 0, st>>>(static_cast<const uint16_t *>(bval), static_cast<uint16_t *>(img),
-                                                          nnzb);
-    else
-        bsr_mma_image_tf32_kernel<<<blocks, 256, 0, st>>>(static_cast<const float *>(bval), static_cast<float *>(img), nnzb);
-    return cudaGetLastError();
-}
-
 // Block-row ranges of about equal cost for the CTAs of the tensor-core kernel: a block-row costs
 // 8 units per block plus 2 for its accumulator hand-over, so the running cost up to block-row I is
 // F(I) = 8*browptr[I] + 2*I; part[c] is the first I with F(I) >= c*F(Mb)/nparts.
