@@ -348,7 +348,7 @@ static sd_status_t pattern_hash(const int32_t *rowptr, const int32_t *colind, in
 }
 
 constexpr uint64_t kBlobMagic = 0x31304E414C504453ull;   // "SDPLAN01"
-constexpr uint32_t kBlobVersion = 4;
+constexpr uint32_t kBlobVersion = 5;
 
 // What a plan was made for and what was decided; the representation is built again from the caller's arrays when the blob is
 // loaded (no scan, no decision), which takes less time than copying it from the host.
@@ -363,7 +363,7 @@ struct BlobHeader {
     int64_t l2_bytes;
     sd_plan_info_t info;
     int32_t h_T, reserved;
-    unsigned long long chunks_long, giants, len_hist[256];   // the scan's counts that the schedule is built from
+    unsigned long long chunks_long, chunks_long2, chunks_long4, giants, len_hist[256];   // the scan's counts that the schedule is built from
 };
 
 }  // namespace sd
@@ -572,13 +572,18 @@ sd_status_t sd_plan_get_hybrid(const sd_plan_t *plan, int32_t *heavy_rows, int32
         else chunk_ptr[0] = 0;
     }
     if ((ranges || order) && nc > 0) {   // the descriptors sd_spmm reads, taken apart
-        std::vector<int4> items(nc);
-        SD_CUDA_TRY(cudaMemcpy(items.data(), plan->h_items, sizeof(int4) * nc, cudaMemcpyDeviceToHost));
-        for (int64_t i = 0; i < nc; ++i) {
-            if (order) order[i] = items[i].x;
-            if (ranges) {
-                ranges[2 * items[i].x] = items[i].y;
-                ranges[2 * items[i].x + 1] = items[i].y + items[i].w;
+        const int64_t ni = plan->h_ni;
+        std::vector<int4> items(ni);
+        SD_CUDA_TRY(cudaMemcpy(items.data(), plan->h_items, sizeof(int4) * ni, cudaMemcpyDeviceToHost));
+        int64_t at = 0;
+        for (int64_t i = 0; i < ni; ++i) {
+            int32_t c = items[i].z;
+            for (int32_t x = items[i].y, e = x + items[i].w; x < e; x += kChunkNnz, ++c) {
+                if (order) order[at++] = c;
+                if (ranges) {
+                    ranges[2 * c] = x;
+                    ranges[2 * c + 1] = std::min(x + kChunkNnz, e);
+                }
             }
         }
     }
@@ -709,7 +714,7 @@ sd_status_t sd_spmm(const sd_plan_t *plan, const void *B, int64_t ldb, float *C,
         h.ldc = ldc;
         h.ldb_bytes = a.ldb_bytes;
         h.N = static_cast<int32_t>(N);
-        h.chunks = static_cast<int32_t>(plan->h_nc);
+        h.chunks = static_cast<int32_t>(plan->h_ni);
         h.wide = static_cast<int32_t>(plan->h_nw);
         h.medium = static_cast<int32_t>(plan->h_nm - plan->h_nw);
         h.light = static_cast<int32_t>(M - plan->h_nl - plan->h_nm);
@@ -718,10 +723,10 @@ sd_status_t sd_spmm(const sd_plan_t *plan, const void *B, int64_t ldb, float *C,
         h.beta = beta;
         SD_CUDA_TRY(plan->dtype == SD_F32 ? run_hybrid_f32(h, vw, st) : run_hybrid_bf16(h, vw, st));
         if (plan->h_nl > 0) {
-            SD_CUDA_TRY(run_chunk_reduce(plan->chunk_out, plan->h_chunk_ptr, plan->h_rows, plan->h_nl, C, ldc,
+            SD_CUDA_TRY(run_chunk_reduce(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_nl, C, ldc,
                                          static_cast<int32_t>(N), alpha, beta, st, plan->h_ng > 0 ? kGiantChunks : 0));
             if (plan->h_ng > 0)
-                SD_CUDA_TRY(run_chunk_reduce_wide(plan->chunk_out, plan->h_chunk_ptr, plan->h_rows, plan->h_giant,
+                SD_CUDA_TRY(run_chunk_reduce_wide(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_giant,
                                                   plan->h_ng, C, ldc, static_cast<int32_t>(N), alpha, beta, st));
         }
         return SD_OK;
@@ -854,6 +859,8 @@ sd_status_t sd_plan_save(const sd_plan_t *plan, void *buf, size_t cap, size_t *b
     h.has_coo = plan->coo_row ? 1 : 0;
     h.h_T = plan->h_T;
     h.chunks_long = plan->h_counts.chunks_long;
+    h.chunks_long2 = plan->h_counts.chunks_long2;
+    h.chunks_long4 = plan->h_counts.chunks_long4;
     h.giants = plan->h_counts.giants;
     memcpy(h.len_hist, plan->h_counts.len_hist, sizeof h.len_hist);
     memcpy(buf, &h, sizeof h);
@@ -927,6 +934,8 @@ sd_status_t sd_plan_load(const void *blob, size_t bytes, const int32_t *rowptr, 
         ScanAccum counts{};
         counts.long_rows = static_cast<unsigned long long>(h.info.long_rows);
         counts.chunks_long = h.chunks_long;
+        counts.chunks_long2 = h.chunks_long2;
+        counts.chunks_long4 = h.chunks_long4;
         counts.giants = h.giants;
         memcpy(counts.len_hist, h.len_hist, sizeof h.len_hist);
         if ((s = build_schedule(p, h.info.windows, h.h_T, counts, nullptr))) return fail(s);

@@ -190,54 +190,63 @@ sort_place_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
     }
 }
 
-// Chunk pointers of the heavy rows and the list of the rows of very many chunks: one CTA walks the rows (a few thousand).
-// row_off: chunks before every (row, window) pair; null with one window, where a row's length says how many it has.
+// Chunk and item pointers of the heavy rows and the list of the rows of very many items: one CTA walks the rows (a few
+// thousand).  chunk_off / item_off: counts before every (row, window) pair; null with one window, where a row's length says
+// how many it has.
 __global__ void __launch_bounds__(1024)
-chunk_ptr_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ row_off, int32_t W,
-                 int64_t nl, int32_t *__restrict__ chunk_ptr, int32_t *__restrict__ giant, int32_t *__restrict__ ngiant) {
+chunk_ptr_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ chunk_off,
+                 const int32_t *__restrict__ item_off, int32_t W, int32_t F, int64_t nl, int32_t *__restrict__ chunk_ptr,
+                 int32_t *__restrict__ item_ptr, int32_t *__restrict__ giant, int32_t *__restrict__ ngiant) {
     using Scan = cub::BlockScan<int, 1024>;
     __shared__ typename Scan::TempStorage tmp;
-    int c = 0, g = 0;   // chunks and listed rows before this step, the same in all threads
+    int c = 0, m = 0, g = 0;   // chunks, items and listed rows before this step, the same in all threads
     for (int64_t i0 = 0; i0 < nl; i0 += 1024) {
         const int64_t i = i0 + threadIdx.x;
-        int n = 0;
+        int n = 0, k = 0;
         if (i < nl) {
-            if (row_off) {
-                n = row_off[(i + 1) * W] - row_off[i * W];
+            if (chunk_off) {
+                n = chunk_off[(i + 1) * W] - chunk_off[i * W];
+                k = item_off[(i + 1) * W] - item_off[i * W];
             } else {
                 const int32_t r = rows[i];
                 n = (__ldg(rowptr + r + 1) - __ldg(rowptr + r) + kChunkNnz - 1) / kChunkNnz;
+                k = (n + F - 1) / F;
             }
         }
-        int before, total, listed, all;
+        int before, total, ibefore, itotal, listed, all;
         Scan(tmp).ExclusiveSum(n, before, total);
         __syncthreads();
-        Scan(tmp).ExclusiveSum(n > kGiantChunks ? 1 : 0, listed, all);
+        Scan(tmp).ExclusiveSum(k, ibefore, itotal);
+        __syncthreads();
+        Scan(tmp).ExclusiveSum(k > kGiantChunks ? 1 : 0, listed, all);
         __syncthreads();
         if (i < nl) {
             chunk_ptr[i] = c + before;
-            if (n > kGiantChunks) giant[g + listed] = static_cast<int32_t>(i);
+            item_ptr[i] = m + ibefore;
+            if (k > kGiantChunks) giant[g + listed] = static_cast<int32_t>(i);
         }
         c += total;
+        m += itotal;
         g += all;
     }
     if (threadIdx.x == 0) {
         chunk_ptr[nl] = c;
+        item_ptr[nl] = m;
         *ngiant = g;
     }
 }
 
-// One window: the chunks in row order.  A warp per heavy row.
+// One window: the items in row order.  A warp per heavy row.
 __global__ void __launch_bounds__(256)
-items_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ chunk_ptr, int64_t nl,
-             int4 *__restrict__ items) {
+items_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ rows, const int32_t *__restrict__ chunk_ptr,
+             const int32_t *__restrict__ item_ptr, int32_t F, int64_t nl, int4 *__restrict__ items) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
     for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < nl; i += warps) {
-        const int32_t r = rows[i], p0 = __ldg(rowptr + r), p1 = __ldg(rowptr + r + 1), c0 = chunk_ptr[i], c1 = chunk_ptr[i + 1];
-        for (int32_t c = c0 + lane; c < c1; c += 32) {
-            const int32_t x = p0 + (c - c0) * kChunkNnz;
-            items[c] = make_int4(c, x, 0, min(kChunkNnz, p1 - x));
+        const int32_t r = rows[i], p0 = __ldg(rowptr + r), p1 = __ldg(rowptr + r + 1), c0 = chunk_ptr[i], m0 = item_ptr[i], m1 = item_ptr[i + 1];
+        for (int32_t m = m0 + lane; m < m1; m += 32) {
+            const int32_t x = p0 + (m - m0) * F * kChunkNnz;
+            items[m] = make_int4(m1 - m0 == 1 ? r | static_cast<int32_t>(0x80000000u) : m, x, c0 + (m - m0) * F, min(F * kChunkNnz, p1 - x));
         }
     }
 }
@@ -255,13 +264,14 @@ __device__ __forceinline__ int32_t first_not_below(const int32_t *__restrict__ c
 // contiguous range (columns ascend); counts its chunks into a row-major and a window-major table.
 __global__ void __launch_bounds__(256)
 window_count_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, const int32_t *__restrict__ rows,
-                    int64_t nl, int32_t W, int64_t wcols, int32_t *__restrict__ start, int32_t *__restrict__ by_row,
-                    int32_t *__restrict__ by_win) {
+                    int64_t nl, int32_t W, int32_t F, int64_t wcols, int32_t *__restrict__ start, int32_t *__restrict__ chunks,
+                    int32_t *__restrict__ items, int32_t *__restrict__ items_by_window) {
     const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (t > nl * W) return;
     if (t == nl * W) {
-        by_row[t] = 0;
-        by_win[t] = 0;
+        chunks[t] = 0;
+        items[t] = 0;
+        items_by_window[t] = 0;
         return;
     }
     const int64_t i = t / W;
@@ -269,23 +279,34 @@ window_count_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restric
     const int32_t r = rows[i], p0 = rowptr[r], p1 = rowptr[r + 1];
     const int32_t lo = w == 0 ? p0 : first_not_below(colind, p0, p1, w * wcols);
     const int32_t hi = w == W - 1 ? p1 : first_not_below(colind, lo, p1, (w + 1) * wcols);
-    const int32_t n = (hi - lo + kChunkNnz - 1) / kChunkNnz;
+    const int32_t n = (hi - lo + kChunkNnz - 1) / kChunkNnz, k = (n + F - 1) / F;
     start[2 * t] = lo;
     start[2 * t + 1] = hi;
-    by_row[t] = n;
-    by_win[static_cast<int64_t>(w) * nl + i] = n;
+    chunks[t] = n;
+    items[t] = k;
+    items_by_window[static_cast<int64_t>(w) * nl + i] = k;
 }
 
 __global__ void __launch_bounds__(256)
-window_items_kernel(const int32_t *__restrict__ start, const int32_t *__restrict__ row_off, const int32_t *__restrict__ win_off,
-                    int64_t nl, int32_t W, int4 *__restrict__ items) {
+window_items_kernel(const int32_t *__restrict__ rows, const int32_t *__restrict__ start, const int32_t *__restrict__ chunk_off,
+                    const int32_t *__restrict__ item_off, const int32_t *__restrict__ win_off, int64_t nl, int32_t W, int32_t F,
+                    int4 *__restrict__ items) {
     const int64_t t = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (t >= nl * W) return;
     const int64_t i = t / W;
     const int32_t w = static_cast<int32_t>(t % W);
-    const int32_t c = row_off[t], o = win_off[static_cast<int64_t>(w) * nl + i];
-    const int32_t lo = start[2 * t], hi = start[2 * t + 1];
-    for (int32_t j = 0, x = lo; x < hi; ++j, x += kChunkNnz) items[o + j] = make_int4(c + j, x, 0, min(kChunkNnz, hi - x));
+    const bool alone = item_off[(i + 1) * W] - item_off[i * W] == 1;
+    int32_t c = chunk_off[t], m = item_off[t], o = win_off[static_cast<int64_t>(w) * nl + i];
+    const int32_t hi = start[2 * t + 1], step = F * kChunkNnz;
+    for (int32_t x = start[2 * t]; x < hi; x += step, c += F, ++m, ++o)
+        items[o] = make_int4(alone ? rows[i] | static_cast<int32_t>(0x80000000u) : m, x, c, min(step, hi - x));
+}
+
+// Chunks per item: one while there are few of them (the chain of dependent gathers counts), up to four when they fill the
+// GPU several times over (fewer scratch rows to write and add up again: 80 MB each way at 128 columns on R-MAT scale 20).
+static int32_t chunks_per_item(int64_t chunks, int sms) {
+    const int64_t groups = static_cast<int64_t>(sms) * 4 * 16;   // half-warp groups resident together
+    return chunks >= 4 * groups ? 4 : (chunks >= 2 * groups ? 2 : 1);
 }
 
 sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cudaStream_t st) {
@@ -294,12 +315,18 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
     T = std::min<int32_t>(std::max<int32_t>(T, 2), kHybridHeavyMax);
     p->h_T = T;
     p->h_counts.chunks_long = h.chunks_long;
+    p->h_counts.chunks_long2 = h.chunks_long2;
+    p->h_counts.chunks_long4 = h.chunks_long4;
     p->h_counts.giants = h.giants;
     std::copy(h.len_hist, h.len_hist + 256, p->h_counts.len_hist);
+    const int32_t F = p->h_F = W == 1 ? chunks_per_item(static_cast<int64_t>(h.chunks_long), p->info.sm_count) : 1;   // with windows, items that outlast their window cost more (1,122 against 918 us on the rank-size matrix)
     int64_t nl = static_cast<int64_t>(h.long_rows), nc = static_cast<int64_t>(h.chunks_long);
+    int64_t ni = static_cast<int64_t>(F == 4 ? h.chunks_long4 : (F == 2 ? h.chunks_long2 : h.chunks_long));
     for (int l = T; l < 256; ++l) {
-        nl += static_cast<int64_t>(h.len_hist[l]);
-        nc += static_cast<int64_t>(h.len_hist[l]) * ((l + kChunkNnz - 1) / kChunkNnz);
+        const int64_t rows = static_cast<int64_t>(h.len_hist[l]), chunks = (l + kChunkNnz - 1) / kChunkNnz;
+        nl += rows;
+        nc += rows * chunks;
+        ni += rows * ((chunks + F - 1) / F);
     }
     SortBases bases;
     bases.first[0] = 0;
@@ -313,7 +340,7 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
     }
     p->h_nl = nl;
     const int32_t ntiles = static_cast<int32_t>((p->M + kSortTile - 1) / kSortTile);
-    TempBuf hist(st), ngiant(st), start(st), by_row(st), by_win(st), row_off(st), win_off(st), tmp(st);
+    TempBuf hist(st), ngiant(st), start(st), counts(st), offs(st), tmp(st);
     if ((s = hist.get(sizeof(int32_t) * (T + 1) * static_cast<size_t>(ntiles), "length counts"))) return s;
     if ((s = dev_alloc(p, &p->h_rows, p->M, "rows by length", st))) return s;
     if ((s = dev_alloc(p, &p->h_desc, p->M - nl, "light row descriptors", st))) return s;
@@ -324,55 +351,62 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
     sort_place_kernel<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->colind, p->M, T, ntiles, hist.as<int32_t>(),
                                                          static_cast<int32_t>(nl), p->h_rows, p->h_desc);
     SD_CUDA_TRY(cudaGetLastError());
-    p->h_nc = p->h_ng = 0;
+    p->h_nc = p->h_ni = p->h_ng = 0;
     p->info.launches = 1;
     if (nl > 0) {
         int64_t ng = static_cast<int64_t>(h.giants);
         if ((s = dev_alloc(p, &p->h_chunk_ptr, nl + 1, "chunk pointers", st))) return s;
         if ((s = dev_alloc(p, &p->h_giant, W == 1 ? ng : nl, "rows of many chunks", st))) return s;
         if ((s = ngiant.get(sizeof(int32_t), "count"))) return s;
+        if ((s = dev_alloc(p, &p->h_item_ptr, nl + 1, "item pointers", st))) return s;
         if (W == 1) {
-            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, nullptr, 1, nl, p->h_chunk_ptr, p->h_giant, ngiant.as<int32_t>());
+            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, nullptr, nullptr, 1, F, nl, p->h_chunk_ptr, p->h_item_ptr, p->h_giant, ngiant.as<int32_t>());
             SD_CUDA_TRY(cudaGetLastError());
-            if ((s = dev_alloc(p, &p->h_items, nc, "chunk descriptors", st))) return s;
-            items_kernel<<<ceil_div(std::min<int64_t>(nl, 148 * 64), 8), 256, 0, st>>>(p->rowptr, p->h_rows, p->h_chunk_ptr, nl, p->h_items);
+            if (F > 1 && ng > 0) {   // the scan counted the rows of many chunks, this one those of many items
+                int32_t got = 0;
+                SD_CUDA_TRY(cudaMemcpyAsync(&got, ngiant.p, sizeof got, cudaMemcpyDeviceToHost, st));
+                SD_CUDA_TRY(cudaStreamSynchronize(st));
+                ng = got;
+            }
+            if ((s = dev_alloc(p, &p->h_items, ni, "chunk descriptors", st))) return s;
+            items_kernel<<<ceil_div(std::min<int64_t>(nl, 148 * 64), 8), 256, 0, st>>>(p->rowptr, p->h_rows, p->h_chunk_ptr, p->h_item_ptr, F, nl, p->h_items);
             SD_CUDA_TRY(cudaGetLastError());
         } else {
-            const int64_t cells = nl * W;
-            if (cells + 1 > INT32_MAX) {
+            const int64_t cells = nl * W, n = cells + 1;
+            if (n > INT32_MAX) {
                 set_error(SD_ERR_UNSUPPORTED, "too many (heavy row, window) pairs");
                 return SD_ERR_UNSUPPORTED;
             }
             if ((s = start.get(sizeof(int32_t) * 2 * cells, "window ranges"))) return s;
-            if ((s = by_row.get(sizeof(int32_t) * (cells + 1), "chunk counts"))) return s;
-            if ((s = by_win.get(sizeof(int32_t) * (cells + 1), "chunk counts"))) return s;
-            if ((s = row_off.get(sizeof(int32_t) * (cells + 1), "chunk offsets"))) return s;
-            if ((s = win_off.get(sizeof(int32_t) * (cells + 1), "chunk offsets"))) return s;
-            window_count_kernel<<<ceil_div(cells + 1, 256), 256, 0, st>>>(p->rowptr, p->colind, p->h_rows, nl, W, (p->K + W - 1) / W,
-                                                                         start.as<int32_t>(), by_row.as<int32_t>(), by_win.as<int32_t>());
+            if ((s = counts.get(sizeof(int32_t) * 3 * n, "chunk counts"))) return s;
+            if ((s = offs.get(sizeof(int32_t) * 3 * n, "chunk offsets"))) return s;
+            int32_t *cnt = counts.as<int32_t>(), *off = offs.as<int32_t>();   // chunks by row, items by row, items by window
+            window_count_kernel<<<ceil_div(n, 256), 256, 0, st>>>(p->rowptr, p->colind, p->h_rows, nl, W, F, (p->K + W - 1) / W,
+                                                                 start.as<int32_t>(), cnt, cnt + n, cnt + 2 * n);
             SD_CUDA_TRY(cudaGetLastError());
             size_t tb = 0;
-            const int n = static_cast<int>(cells + 1);
-            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, by_row.as<int32_t>(), row_off.as<int32_t>(), n, st));
+            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, cnt, off, static_cast<int>(n), st));
             if ((s = tmp.get(tb, "scan scratch"))) return s;
-            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, by_row.as<int32_t>(), row_off.as<int32_t>(), n, st));
-            SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, by_win.as<int32_t>(), win_off.as<int32_t>(), n, st));
-            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, row_off.as<int32_t>(), W, nl, p->h_chunk_ptr, p->h_giant, ngiant.as<int32_t>());
+            for (int k = 0; k < 3; ++k)
+                SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(tmp.p, tb, cnt + k * n, off + k * n, static_cast<int>(n), st));
+            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, off, off + n, W, F, nl, p->h_chunk_ptr, p->h_item_ptr, p->h_giant, ngiant.as<int32_t>());
             SD_CUDA_TRY(cudaGetLastError());
-            int32_t got[2] = {0, 0};
+            int32_t got[3] = {0, 0, 0};
             SD_CUDA_TRY(cudaMemcpyAsync(&got[0], p->h_chunk_ptr + nl, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             SD_CUDA_TRY(cudaMemcpyAsync(&got[1], ngiant.p, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
+            SD_CUDA_TRY(cudaMemcpyAsync(&got[2], p->h_item_ptr + nl, sizeof(int32_t), cudaMemcpyDeviceToHost, st));
             SD_CUDA_TRY(cudaStreamSynchronize(st));
             nc = got[0];
             ng = got[1];
-            if ((s = dev_alloc(p, &p->h_items, nc, "chunk descriptors", st))) return s;
-            window_items_kernel<<<ceil_div(cells, 256), 256, 0, st>>>(start.as<int32_t>(), row_off.as<int32_t>(), win_off.as<int32_t>(), nl,
-                                                                     W, p->h_items);
+            ni = got[2];
+            if ((s = dev_alloc(p, &p->h_items, ni, "chunk descriptors", st))) return s;
+            window_items_kernel<<<ceil_div(cells, 256), 256, 0, st>>>(p->h_rows, start.as<int32_t>(), off, off + n, off + 2 * n, nl, W, F, p->h_items);
             SD_CUDA_TRY(cudaGetLastError());
         }
         p->h_nc = nc;
+        p->h_ni = ni;
         p->h_ng = ng;
-        if ((s = dev_alloc(p, &p->chunk_out, static_cast<size_t>(nc) * p->N, "chunk sums", st))) return s;
+        if ((s = dev_alloc(p, &p->chunk_out, static_cast<size_t>(ni) * p->N, "chunk sums", st))) return s;
         p->info.launches = 2 + (ng > 0 ? 1 : 0);   // the fused kernel, the chunk sums, the chunk sums of very long rows
     }
     return SD_OK;

@@ -26,7 +26,7 @@ chunk_reduce_kernel(const float *__restrict__ chunk_out, const int32_t *__restri
     const int nchain = 32 / lpc, chain = lane / lpc, cl = lane % lpc;
     const int32_t c0 = __ldg(chunk_ptr + s), c1 = __ldg(chunk_ptr + s + 1);
     overlap_wait();
-    if (skip_above > 0 && c1 - c0 > skip_above) return;   // left to chunk_reduce_wide_kernel
+    if (c1 - c0 == 1 || (skip_above > 0 && c1 - c0 > skip_above)) return;   // written already; left to chunk_reduce_wide_kernel
     const int32_t r = __ldg(rows + s);
     float *crow = C + static_cast<int64_t>(r) * ldc;
     for (int ub = 0; ub < units; ub += lpc) {

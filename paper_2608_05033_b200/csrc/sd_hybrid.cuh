@@ -28,7 +28,7 @@ struct HybridArgs {
     const void *B;
     float *C;
     float *scratch;          // [chunks][N]
-    const int4 *items;       // chunks in the order they are taken: {scratch row, first nonzero, unused, length}
+    const int4 *items;       // chunks in the order they are taken, up to four at once: {scratch row, or row | bit 31; first nonzero; chunk; length}
     const int4 *desc;        // light rows, longest first: {row, first nonzero, its column, length}
     int64_t ldc;
     uint32_t ldb_bytes;
@@ -167,8 +167,8 @@ __device__ __forceinline__ void items_body(const HybridArgs &a, unsigned bx) {
         clear_acc(acc);
         group_sum<T, VW, LPR, NV, LANES>(a, lc, d.y, d.y + d.w, mask, acc);
         if (lg < LPR) {
-            if (chunk) lc.store(a.scratch + static_cast<int64_t>(d.x) * a.N, acc, 1.f, 0.f);
-            else lc.store(a.C + d.x * a.ldc, acc, a.alpha, a.beta);
+            if (chunk && d.x >= 0) lc.store(a.scratch + static_cast<int64_t>(d.x) * a.N, acc, 1.f, 0.f);
+            else lc.store(a.C + (d.x & 0x7FFFFFFF) * a.ldc, acc, a.alpha, a.beta);   // a light row, or a heavy row of one item
         }
     }
 }
@@ -290,10 +290,11 @@ cudaError_t launch_hybrid_one(const HybridArgs &a, cudaStream_t st) {
     }
 }
 
-// Lanes across the columns for rows of `units` loads per row of B.  Full 16-byte loads: the next power of two, two
-// loads per lane beyond 32.  Narrower loads (odd widths, unaligned operands): two to four per lane, so that the work per
-// nonzero on A is spread over more columns and few lane slots are idle (R-MAT scale 17: 41 columns as 16 lanes x 3 61 us,
-// as one warp x 4 101; 25 columns as 16 x 2 46 us, as 32 x 1 56); wider rows run as slabs of about equal width.
+// Lanes across the columns for rows of `units` loads per row of B.  Full 16-byte loads: the next power of two up to 16, two
+// loads per lane beyond (128 fp32 columns on R-MAT scale 20 as 16 x 2: 1,212 us, as 32 x 1: 1,268).  Narrower loads (odd
+// widths, unaligned operands): two to four per lane, so that the work per nonzero on A is spread over more columns and few
+// lane slots are idle (R-MAT scale 17: 41 columns as 16 lanes x 3 61 us, as one warp x 4 101; 25 columns as 16 x 2 46 us,
+// as 32 x 1 56); wider rows run as slabs of about equal width.
 template <typename T, int VW>
 cudaError_t launch_hybrid(const HybridArgs &a, cudaStream_t st) {
     constexpr bool FULL = VW * sizeof(T) == 16;
@@ -307,7 +308,7 @@ cudaError_t launch_hybrid(const HybridArgs &a, cudaStream_t st) {
     if (units <= 8) return launch_hybrid_one<T, VW, 8, 1>(a, st);
     if constexpr (FULL) {
         if (units <= 16) return launch_hybrid_one<T, VW, 16, 1>(a, st);
-        if (units <= 32) return launch_hybrid_one<T, VW, 32, 1>(a, st);
+        if (units <= 32) return launch_hybrid_one<T, VW, 16, 2>(a, st);
         return launch_hybrid_one<T, VW, 32, 2>(a, st);
     } else {
         if (units <= 16) return launch_hybrid_one<T, VW, 8, 2>(a, st);

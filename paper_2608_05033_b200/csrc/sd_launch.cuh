@@ -29,10 +29,10 @@ cudaError_t run_hybrid_f32(const HybridArgs &a, int vw, cudaStream_t st);
 cudaError_t run_hybrid_bf16(const HybridArgs &a, int vw, cudaStream_t st);
 
 // Heavy rows: row rows[i] owns the scratch rows chunk_ptr[i] .. chunk_ptr[i+1]-1 of chunk_out ([chunks][N]); their sum, taken in
-// order, is its product.  skip_above > 0: rows of more chunks are left to run_chunk_reduce_wide (list: their positions).
+// order, is its product (a row of one chunk has been written already).  skip_above > 0: rows of more chunks are left to run_chunk_reduce_wide (list: their positions).
 cudaError_t run_chunk_reduce(const float *chunk_out, const int32_t *chunk_ptr, const int32_t *rows, int64_t nl, float *C,
                              int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st, int32_t skip_above);
-constexpr int kGiantChunks = 64;   // rows of more chunks than this are summed by a whole CTA
+constexpr int kGiantChunks = 64;   // rows of more scratch rows than this are summed by a whole CTA
 cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *chunk_ptr, const int32_t *rows, const int32_t *list,
                                   int64_t count, float *C, int64_t ldc, int32_t N, float alpha, float beta, cudaStream_t st);
 

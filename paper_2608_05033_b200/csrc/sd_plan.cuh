@@ -19,14 +19,17 @@ struct sd_plan {
     // column window, the rest row-wise from a list sorted by falling length
     int32_t *h_rows = nullptr;       // [M] the heavy rows, ascending, then the light rows, longest first, ascending inside a length
     int32_t *h_chunk_ptr = nullptr;  // [h_nl + 1] first chunk of every heavy row (chunks are numbered row by row)
-    int4 *h_items = nullptr;         // [h_nc] the chunks in the order they are taken: {chunk, first nonzero, 0, length}
+    int32_t *h_item_ptr = nullptr;   // [h_nl + 1] first scratch row of every heavy row
+    int4 *h_items = nullptr;         // [h_ni] the chunks in the order they are taken, h_F consecutive ones of a row and window
+                                     // together: {scratch row, or row | bit 31 for a row of one item; first nonzero; first chunk; length}
     int32_t *h_giant = nullptr;      // [h_ng] positions in h_rows of the rows of more than kGiantChunks chunks (a CTA sums each)
     int4 *h_desc = nullptr;          // [M - h_nl] per light row, in list order: {row, first nonzero, its column, length}
-    float *chunk_out = nullptr;      // [h_nc][N] partial sums of the chunks
-    int64_t h_nl = 0, h_nc = 0, h_ng = 0;
+    float *chunk_out = nullptr;      // [h_ni][N] partial sums of the items
+    int64_t h_nl = 0, h_nc = 0, h_ni = 0, h_ng = 0;
+    int32_t h_F = 1;                 // chunks per item
     int64_t h_nm = 0;                // the first h_nm light rows have at least kHybridMedium nonzeros
     int64_t h_nw = 0;                // the first h_nw of those at least kHybridWide
-    struct { unsigned long long chunks_long = 0, giants = 0, len_hist[256] = {}; } h_counts;   // of the scan, for sd_plan_save
+    struct { unsigned long long chunks_long = 0, chunks_long2 = 0, chunks_long4 = 0, giants = 0, len_hist[256] = {}; } h_counts;   // of the scan, for sd_plan_save
     int32_t h_T = 0;                 // 0: no schedule (nothing to multiply, or another executor)
 
     // narrow dense operands (N <= kCooMaxN) of the merge family
@@ -104,7 +107,8 @@ struct ScanAccum {
     unsigned long long blk_hist[9];
     unsigned long long nnz_dense_blocks, nnzb;
     unsigned long long bad_csr;           // validation: number of offending rows / entries
-    unsigned long long chunks_long;       // chunks of the rows of at least 256 nonzeros
+    unsigned long long chunks_long;       // chunks of the rows of at least 256 nonzeros ...
+    unsigned long long chunks_long2, chunks_long4;   // ... and items of two and of four chunks each (the last of a row may be shorter)
     unsigned long long giants;            // rows of more than kGiantChunks chunks
     unsigned long long len_hist[256];     // rows of exactly 0 .. 255 nonzeros
     long long nnz;                        // rowptr[M]

@@ -22,11 +22,11 @@ __device__ __forceinline__ int hist_bin(long long v) { return v <= 0 ? 0 : 64 - 
 
 // Counters of one CTA in shared memory, added to the global ones when it ends.
 struct ScanShared {
-    unsigned long long sum[12];
+    unsigned long long sum[16];
     unsigned long long mx[2];     // longest row, largest span
     unsigned int row_hist[32], blk_hist[16], len_hist[256];
 };
-enum { S_R2, S_EMPTY, S_SPAN, S_GAP, S_DIAG, S_UNSORTED, S_LONG, S_NNZ_LONG, S_CHUNKS, S_GIANTS, S_DENSE, S_BLOCKS };
+enum { S_R2, S_EMPTY, S_SPAN, S_GAP, S_DIAG, S_UNSORTED, S_LONG, S_NNZ_LONG, S_CHUNKS, S_GIANTS, S_DENSE, S_BLOCKS, S_CHUNKS2, S_CHUNKS4, S_COUNT };
 
 __device__ void scan_clear(ScanShared &s) {
     for (int i = threadIdx.x; i < static_cast<int>(sizeof(ScanShared) / 4); i += blockDim.x) reinterpret_cast<unsigned int *>(&s)[i] = 0;
@@ -35,13 +35,13 @@ __device__ void scan_clear(ScanShared &s) {
 
 __device__ void scan_flush(ScanShared &s, ScanAccum *out) {
     __syncthreads();
-    unsigned long long *const sums[12] = {&out->sum_r2, &out->empty_rows, &out->sum_span, &out->sum_gap, &out->diag,
+    unsigned long long *const sums[S_COUNT] = {&out->sum_r2, &out->empty_rows, &out->sum_span, &out->sum_gap, &out->diag,
                                           &out->unsorted_rows, &out->long_rows, &out->nnz_long_rows, &out->chunks_long,
-                                          &out->giants, &out->nnz_dense_blocks, &out->nnzb};
+                                          &out->giants, &out->nnz_dense_blocks, &out->nnzb, &out->chunks_long2, &out->chunks_long4};
     const int t = threadIdx.x;
-    if (t < 12 && s.sum[t]) atomicAdd(sums[t], s.sum[t]);
-    if (t == 12 && s.mx[0]) atomicMax(&out->max_r, s.mx[0]);
-    if (t == 13 && s.mx[1]) atomicMax(&out->max_span, s.mx[1]);
+    if (t < S_COUNT && s.sum[t]) atomicAdd(sums[t], s.sum[t]);
+    if (t == 16 && s.mx[0]) atomicMax(&out->max_r, s.mx[0]);
+    if (t == 17 && s.mx[1]) atomicMax(&out->max_span, s.mx[1]);
     if (t >= 32 && t < 64 && s.row_hist[t - 32]) atomicAdd(&out->row_hist[t - 32], static_cast<unsigned long long>(s.row_hist[t - 32]));
     if (t >= 64 && t < 73 && s.blk_hist[t - 64]) atomicAdd(&out->blk_hist[t - 64], static_cast<unsigned long long>(s.blk_hist[t - 64]));
     for (int i = t; i < 256; i += blockDim.x)
@@ -53,6 +53,8 @@ __device__ __forceinline__ void count_long_row(ScanShared &s, long long r) {
     atomicAdd(&s.sum[S_LONG], 1ull);
     atomicAdd(&s.sum[S_NNZ_LONG], static_cast<unsigned long long>(r));
     atomicAdd(&s.sum[S_CHUNKS], chunks);
+    atomicAdd(&s.sum[S_CHUNKS2], (chunks + 1) / 2);
+    atomicAdd(&s.sum[S_CHUNKS4], (chunks + 3) / 4);
     if (chunks > kGiantChunks) atomicAdd(&s.sum[S_GIANTS], 1ull);
 }
 
