@@ -299,6 +299,10 @@ static void free_plan(sd_plan *p) {
     if (!p->allocs.empty()) cudaDeviceSynchronize();
     for (void *a : p->allocs) cudaFreeAsync(a, nullptr);
     if (p->host_stream) cudaStreamDestroy(p->host_stream);
+    if (p->host_in) cudaStreamDestroy(p->host_in);
+    if (p->host_out) cudaStreamDestroy(p->host_out);
+    for (cudaEvent_t e : p->host_ev)
+        if (e) cudaEventDestroy(e);
     if (switched) cudaSetDevice(prev);
     delete p;
 }
@@ -365,6 +369,172 @@ struct BlobHeader {
     int32_t h_T, reserved;
     unsigned long long chunks_long, chunks_long2, chunks_long4, giants, len_hist[256];   // the scan's counts that the schedule is built from
 };
+
+// The product on N columns of B and C: all of the plan's, or a slice of them.
+static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, int64_t ldb, float *C, int64_t ldc, float alpha,
+                               float beta, cudaStream_t st) {
+    const int64_t M = plan->M;
+    if (M == 0 || N == 0) return SD_OK;
+    if (!C || ldc < N) {
+        set_error(SD_ERR_INVALID_ARG, "C is null or ldc < N");
+        return SD_ERR_INVALID_ARG;
+    }
+    if (alpha == 0.f || plan->nnz == 0) {
+        SD_CUDA_TRY(run_scale_c(C, ldc, M, static_cast<int32_t>(N), beta, st));
+        return SD_OK;
+    }
+    if (!B || ldb < N) {
+        set_error(SD_ERR_INVALID_ARG, "B is null or ldb < N");
+        return SD_ERR_INVALID_ARG;
+    }
+    if (ldb * (plan->dtype == SD_F32 ? 4 : 2) > static_cast<int64_t>(UINT32_MAX)) {
+        set_error(SD_ERR_UNSUPPORTED, "row pitch of B must be below 4 GiB");
+        return SD_ERR_UNSUPPORTED;
+    }
+    const int vw = plan->dtype == SD_F32 ? 4 : 8;
+    const bool vec = aligned16(B) && aligned16(C) && N % vw == 0 && ldb % vw == 0 && ldc % 4 == 0;
+
+    SpmmArgs a;
+    a.ptr = plan->rowptr;
+    a.colind = plan->colind;
+    a.vals = plan->vals;
+    a.seg_row = nullptr;
+    a.B = B;
+    a.C = C;
+    a.ldb = ldb;
+    a.ldc = ldc;
+    a.ldb_bytes = static_cast<uint32_t>(ldb * (plan->dtype == SD_F32 ? 4 : 2));
+    a.S = M;
+    a.max_len = plan->info.max_r;
+    a.mean_len = M > 0 ? (plan->nnz + M - 1) / M : 0;
+    a.N = static_cast<int32_t>(N);
+    a.alpha = alpha;
+    a.beta = beta;
+
+    switch (plan->info.family) {
+    case SD_ROWSPLIT:
+        SD_CUDA_TRY(run_rowsplit(a, plan->dtype, vec, st));
+        return SD_OK;
+    case SD_MERGE: {
+        if (plan->coo_row) {   // narrow dense operand: one writer per row
+            a.colind = plan->colind;
+            a.vals = plan->vals;
+            CooPlan cp;
+            cp.row = plan->coo_row;
+            cp.rowptr = plan->rowptr;
+            cp.M = plan->info.empty_rows > 0 ? M : 0;   // no search for rows without nonzeros when the scan found none
+            cp.nnz = plan->nnz;
+            cp.c1_row = plan->coo_c1_row;
+            cp.c1_val = plan->coo_c1_val;
+            cp.c2_row = plan->coo_c2_row;
+            cp.c2_val = plan->coo_c2_val;
+            const bool bvec = aligned16(B) && (ldb * (plan->dtype == SD_F32 ? 4 : 2)) % 16 == 0;
+            SD_CUDA_TRY(run_coo(cp, a, plan->dtype, bvec, plan->info.sm_count, st));
+            return SD_OK;
+        }
+        [[fallthrough]];   // wider ones run the hybrid schedule
+    }
+    case SD_HYBRID: {
+        // one launch for the chunks of the heavy rows and all light rows; then the chunk sums
+        const int vw = piece_width(plan->dtype, N, B, ldb, C, ldc);
+        HybridArgs h;
+        h.colind = plan->colind;
+        h.vals = plan->vals;
+        h.B = B;
+        h.C = C;
+        h.scratch = plan->chunk_out;
+        h.items = plan->h_items;
+        h.desc = plan->h_desc;
+        h.ldc = ldc;
+        h.ldb_bytes = a.ldb_bytes;
+        h.N = static_cast<int32_t>(N);
+        h.chunks = static_cast<int32_t>(plan->h_ni);
+        h.wide = static_cast<int32_t>(plan->h_nw);
+        h.medium = static_cast<int32_t>(plan->h_nm - plan->h_nw);
+        h.light = static_cast<int32_t>(M - plan->h_nl - plan->h_nm);
+        h.gc = h.gm = 0;
+        h.alpha = alpha;
+        h.beta = beta;
+        SD_CUDA_TRY(plan->dtype == SD_F32 ? run_hybrid_f32(h, vw, st) : run_hybrid_bf16(h, vw, st));
+        if (plan->h_nl > 0) {
+            SD_CUDA_TRY(run_chunk_reduce(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_nl, C, ldc,
+                                         static_cast<int32_t>(N), alpha, beta, st, plan->h_ng > 0 ? kGiantChunks : 0));
+            if (plan->h_ng > 0)
+                SD_CUDA_TRY(run_chunk_reduce_wide(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_giant,
+                                                  plan->h_ng, C, ldc, static_cast<int32_t>(N), alpha, beta, st));
+        }
+        return SD_OK;
+    }
+    case SD_BSR_TC: {
+        BsrArgs b;
+        b.browptr = plan->browptr;
+        b.bcol = plan->bcol;
+        b.bval = plan->bval;
+        b.bval_mma = plan->bval_mma;
+        b.part = plan->bsr_part;
+        b.nparts = plan->bsr_nparts;
+        b.B = B;
+        b.C = C;
+        b.ldb = ldb;
+        b.ldc = ldc;
+        b.M = M;
+        b.K = plan->K;
+        b.Mb = static_cast<int32_t>((M + 15) / 16);
+        b.N = static_cast<int32_t>(N);
+        b.alpha = alpha;
+        b.beta = beta;
+        b.map_cache = &plan->tc_map;
+        b.test_wait_expiry = plan->test_wait_expiry;
+        const bool vec4 = aligned16(B) && aligned16(C) && N % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
+                          (plan->dtype == SD_F32 || (reinterpret_cast<uintptr_t>(B) & 7u) == 0);
+        if (bsr_tc_usable(b, plan->dtype) && !switches().bsr_simt)
+            SD_CUDA_TRY(run_bsr_tc(b, plan->dtype, plan->dev_error, plan->info.sm_count, st));
+        else
+            SD_CUDA_TRY(run_bsr_simt(b, plan->dtype, vec4, st));
+        return SD_OK;
+    }
+    default:
+        set_error(SD_ERR_INTERNAL, "plan has no family");
+        return SD_ERR_INTERNAL;
+    }
+}
+
+// ---- host operands ---------------------------------------------------------------------------------
+// A rows x width rectangle between the host and a device matrix of the same shape.  Whole contiguous rectangles go as one
+// run of bytes: the two-dimensional copy of the same bytes from a host pitch below 256 took up to 30 times as long.
+static cudaError_t copy_rect(void *dst, int64_t dpitch, const void *src, int64_t spitch, int64_t width, int64_t rows, cudaMemcpyKind kind, cudaStream_t st) {
+    if (dpitch == width && spitch == width) return cudaMemcpyAsync(dst, src, static_cast<size_t>(width) * rows, kind, st);
+    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, kind, st);
+}
+
+// Column slices of a product with host operands: while one slice is multiplied, the next one's columns of B travel in and the
+// previous one's columns of C out (the bus carries both directions at once: strided copies of 256-byte pieces 99 GB/s together,
+// of 128-byte pieces 72, one direction alone 55).  Slice boundaries in columns: whole 256-byte pieces of a row of B, of a
+// 256-byte row two halves; at most eight slices.  One slice, no overlap: rows of B not of whole 128-byte pieces or below two of
+// them, or little data.
+constexpr int kHostSlices = 8;
+static int host_slices(const sd_plan *p, int64_t ldb, int64_t ldc, int64_t (&at)[kHostSlices + 1]) {
+    const int64_t es = p->dtype == SD_F32 ? 4 : 2, row = p->N * es;
+    at[0] = 0;
+    at[1] = p->N;
+    if (row % 128 != 0 || row < 256 || (ldb * es) % 128 != 0 || (ldc * 4) % 128 != 0 || p->K * row < (int64_t{1} << 20) ||
+        p->M * p->N * 4 < (int64_t{1} << 20))
+        return 1;
+    int64_t piece = row < 512 ? 128 : 256;
+    while (row / piece > kHostSlices) piece *= 2;
+    const int n = static_cast<int>(row / piece);
+    for (int i = 1; i < n; ++i) at[i] = i * piece / es;
+    at[n] = p->N;
+    return n;
+}
+
+static sd_status_t host_streams(sd_plan *p) {
+    if (p->host_in) return SD_OK;
+    SD_CUDA_TRY(cudaStreamCreateWithFlags(&p->host_out, cudaStreamNonBlocking));
+    for (cudaEvent_t &e : p->host_ev) SD_CUDA_TRY(cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
+    SD_CUDA_TRY(cudaStreamCreateWithFlags(&p->host_in, cudaStreamNonBlocking));
+    return SD_OK;
+}
 
 }  // namespace sd
 
@@ -638,131 +808,7 @@ sd_status_t sd_spmm(const sd_plan_t *plan, const void *B, int64_t ldb, float *C,
         set_error(SD_ERR_INVALID_ARG, "plan is null");
         return SD_ERR_INVALID_ARG;
     }
-    const int64_t M = plan->M, N = plan->N;
-    if (M == 0 || N == 0) return SD_OK;
-    if (!C || ldc < N) {
-        set_error(SD_ERR_INVALID_ARG, "C is null or ldc < N");
-        return SD_ERR_INVALID_ARG;
-    }
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if (alpha == 0.f || plan->nnz == 0) {
-        SD_CUDA_TRY(run_scale_c(C, ldc, M, static_cast<int32_t>(N), beta, st));
-        return SD_OK;
-    }
-    if (!B || ldb < N) {
-        set_error(SD_ERR_INVALID_ARG, "B is null or ldb < N");
-        return SD_ERR_INVALID_ARG;
-    }
-    if (ldb * (plan->dtype == SD_F32 ? 4 : 2) > static_cast<int64_t>(UINT32_MAX)) {
-        set_error(SD_ERR_UNSUPPORTED, "row pitch of B must be below 4 GiB");
-        return SD_ERR_UNSUPPORTED;
-    }
-    const int vw = plan->dtype == SD_F32 ? 4 : 8;
-    const bool vec = aligned16(B) && aligned16(C) && N % vw == 0 && ldb % vw == 0 && ldc % 4 == 0;
-
-    SpmmArgs a;
-    a.ptr = plan->rowptr;
-    a.colind = plan->colind;
-    a.vals = plan->vals;
-    a.seg_row = nullptr;
-    a.B = B;
-    a.C = C;
-    a.ldb = ldb;
-    a.ldc = ldc;
-    a.ldb_bytes = static_cast<uint32_t>(ldb * (plan->dtype == SD_F32 ? 4 : 2));
-    a.S = M;
-    a.max_len = plan->info.max_r;
-    a.mean_len = M > 0 ? (plan->nnz + M - 1) / M : 0;
-    a.N = static_cast<int32_t>(N);
-    a.alpha = alpha;
-    a.beta = beta;
-
-    switch (plan->info.family) {
-    case SD_ROWSPLIT:
-        SD_CUDA_TRY(run_rowsplit(a, plan->dtype, vec, st));
-        return SD_OK;
-    case SD_MERGE: {
-        if (plan->coo_row) {   // narrow dense operand: one writer per row
-            a.colind = plan->colind;
-            a.vals = plan->vals;
-            CooPlan cp;
-            cp.row = plan->coo_row;
-            cp.rowptr = plan->rowptr;
-            cp.M = plan->info.empty_rows > 0 ? M : 0;   // no search for rows without nonzeros when the scan found none
-            cp.nnz = plan->nnz;
-            cp.c1_row = plan->coo_c1_row;
-            cp.c1_val = plan->coo_c1_val;
-            cp.c2_row = plan->coo_c2_row;
-            cp.c2_val = plan->coo_c2_val;
-            const bool bvec = aligned16(B) && (ldb * (plan->dtype == SD_F32 ? 4 : 2)) % 16 == 0;
-            SD_CUDA_TRY(run_coo(cp, a, plan->dtype, bvec, plan->info.sm_count, st));
-            return SD_OK;
-        }
-        [[fallthrough]];   // wider ones run the hybrid schedule
-    }
-    case SD_HYBRID: {
-        // one launch for the chunks of the heavy rows and all light rows; then the chunk sums
-        const int vw = piece_width(plan->dtype, N, B, ldb, C, ldc);
-        HybridArgs h;
-        h.colind = plan->colind;
-        h.vals = plan->vals;
-        h.B = B;
-        h.C = C;
-        h.scratch = plan->chunk_out;
-        h.items = plan->h_items;
-        h.desc = plan->h_desc;
-        h.ldc = ldc;
-        h.ldb_bytes = a.ldb_bytes;
-        h.N = static_cast<int32_t>(N);
-        h.chunks = static_cast<int32_t>(plan->h_ni);
-        h.wide = static_cast<int32_t>(plan->h_nw);
-        h.medium = static_cast<int32_t>(plan->h_nm - plan->h_nw);
-        h.light = static_cast<int32_t>(M - plan->h_nl - plan->h_nm);
-        h.gc = h.gm = 0;
-        h.alpha = alpha;
-        h.beta = beta;
-        SD_CUDA_TRY(plan->dtype == SD_F32 ? run_hybrid_f32(h, vw, st) : run_hybrid_bf16(h, vw, st));
-        if (plan->h_nl > 0) {
-            SD_CUDA_TRY(run_chunk_reduce(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_nl, C, ldc,
-                                         static_cast<int32_t>(N), alpha, beta, st, plan->h_ng > 0 ? kGiantChunks : 0));
-            if (plan->h_ng > 0)
-                SD_CUDA_TRY(run_chunk_reduce_wide(plan->chunk_out, plan->h_item_ptr, plan->h_rows, plan->h_giant,
-                                                  plan->h_ng, C, ldc, static_cast<int32_t>(N), alpha, beta, st));
-        }
-        return SD_OK;
-    }
-    case SD_BSR_TC: {
-        BsrArgs b;
-        b.browptr = plan->browptr;
-        b.bcol = plan->bcol;
-        b.bval = plan->bval;
-        b.bval_mma = plan->bval_mma;
-        b.part = plan->bsr_part;
-        b.nparts = plan->bsr_nparts;
-        b.B = B;
-        b.C = C;
-        b.ldb = ldb;
-        b.ldc = ldc;
-        b.M = M;
-        b.K = plan->K;
-        b.Mb = static_cast<int32_t>((M + 15) / 16);
-        b.N = static_cast<int32_t>(N);
-        b.alpha = alpha;
-        b.beta = beta;
-        b.map_cache = &plan->tc_map;
-        b.test_wait_expiry = plan->test_wait_expiry;
-        const bool vec4 = aligned16(B) && aligned16(C) && N % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
-                          (plan->dtype == SD_F32 || (reinterpret_cast<uintptr_t>(B) & 7u) == 0);
-        if (bsr_tc_usable(b, plan->dtype) && !switches().bsr_simt)
-            SD_CUDA_TRY(run_bsr_tc(b, plan->dtype, plan->dev_error, plan->info.sm_count, st));
-        else
-            SD_CUDA_TRY(run_bsr_simt(b, plan->dtype, vec4, st));
-        return SD_OK;
-    }
-    default:
-        set_error(SD_ERR_INTERNAL, "plan has no family");
-        return SD_ERR_INTERNAL;
-    }
+    return run_product(plan, plan->N, B, ldb, C, ldc, alpha, beta, static_cast<cudaStream_t>(stream));
 }
 
 sd_status_t sd_plan_update_values(sd_plan_t *plan, const void *vals, void *stream) {
@@ -799,11 +845,37 @@ sd_status_t sd_spmm_host_async(sd_plan_t *plan, const void *B_host, int64_t ldb,
     if (!plan->stage_C && (s = dev_alloc(plan, &plan->stage_C, static_cast<size_t>(M) * N, "C staging", plan->host_stream)))
         return s;
     cudaStream_t st = plan->host_stream;
-    SD_CUDA_TRY(cudaMemcpy2DAsync(plan->stage_B, es * N, B_host, es * ldb, es * N, K, cudaMemcpyHostToDevice, st));
-    if (beta != 0.f)
-        SD_CUDA_TRY(cudaMemcpy2DAsync(plan->stage_C, 4 * N, C_host, 4 * ldc, 4 * N, M, cudaMemcpyHostToDevice, st));
-    if ((s = sd_spmm(plan, plan->stage_B, N, plan->stage_C, N, alpha, beta, st))) return s;
-    SD_CUDA_TRY(cudaMemcpy2DAsync(C_host, 4 * ldc, plan->stage_C, 4 * N, 4 * N, M, cudaMemcpyDeviceToHost, st));
+    int64_t at[kHostSlices + 1];
+    const int n = host_slices(plan, ldb, ldc, at);
+    const char *bh = static_cast<const char *>(B_host);
+    char *bd = static_cast<char *>(plan->stage_B);
+    if (n == 1) {
+        SD_CUDA_TRY(copy_rect(bd, es * N, bh, es * ldb, es * N, K, cudaMemcpyHostToDevice, st));
+        if (beta != 0.f) SD_CUDA_TRY(copy_rect(plan->stage_C, 4 * N, C_host, 4 * ldc, 4 * N, M, cudaMemcpyHostToDevice, st));
+        if ((s = run_product(plan, N, bd, N, plan->stage_C, N, alpha, beta, st))) return s;
+        SD_CUDA_TRY(copy_rect(C_host, 4 * ldc, plan->stage_C, 4 * N, 4 * N, M, cudaMemcpyDeviceToHost, st));
+        return SD_OK;
+    }
+    if ((s = host_streams(plan))) return s;
+    // forked from the plan's stream and joined back into it: the staging buffers belong to one call at a time
+    cudaEvent_t ev = plan->host_ev[0], out_ev = plan->host_ev[1];
+    SD_CUDA_TRY(cudaEventRecord(ev, st));
+    SD_CUDA_TRY(cudaStreamWaitEvent(plan->host_in, ev, 0));
+    SD_CUDA_TRY(cudaStreamWaitEvent(plan->host_out, ev, 0));
+    for (int i = 0; i < n; ++i) {
+        const int64_t c = at[i], w = at[i + 1] - c;
+        SD_CUDA_TRY(cudaMemcpy2DAsync(bd + es * c, es * N, bh + es * c, es * ldb, es * w, K, cudaMemcpyHostToDevice, plan->host_in));
+        if (beta != 0.f)
+            SD_CUDA_TRY(cudaMemcpy2DAsync(plan->stage_C + c, 4 * N, C_host + c, 4 * ldc, 4 * w, M, cudaMemcpyHostToDevice, plan->host_in));
+        SD_CUDA_TRY(cudaEventRecord(ev, plan->host_in));
+        SD_CUDA_TRY(cudaStreamWaitEvent(st, ev, 0));
+        if ((s = run_product(plan, w, bd + es * c, N, plan->stage_C + c, N, alpha, beta, st))) return s;
+        SD_CUDA_TRY(cudaEventRecord(out_ev, st));
+        SD_CUDA_TRY(cudaStreamWaitEvent(plan->host_out, out_ev, 0));
+        SD_CUDA_TRY(cudaMemcpy2DAsync(C_host + c, 4 * ldc, plan->stage_C + c, 4 * N, 4 * w, M, cudaMemcpyDeviceToHost, plan->host_out));
+    }
+    SD_CUDA_TRY(cudaEventRecord(out_ev, plan->host_out));
+    SD_CUDA_TRY(cudaStreamWaitEvent(st, out_ev, 0));
     return SD_OK;
 }
 

@@ -53,6 +53,8 @@ struct sd_plan {
     void *stage_B = nullptr;
     float *stage_C = nullptr;
     cudaStream_t host_stream = nullptr;
+    cudaStream_t host_in = nullptr, host_out = nullptr;   // column slices: copies in and out, beside the products on host_stream
+    cudaEvent_t host_ev[2] = {nullptr, nullptr};
 
     std::vector<void *> allocs;   // every device allocation of the plan
     int64_t owned = 0;            // their bytes

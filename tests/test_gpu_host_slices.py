@@ -1,0 +1,36 @@
+"""Products with host operands large enough to travel in column slices, and just below: rows of B of 256 bytes (two slices of
+128), of whole and of odd numbers of 256-byte pieces, more than eight pieces, padded rows, both value types, beta != 0."""
+import numpy as np
+import pytest
+
+import oracle
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+
+
+@pytest.mark.parametrize("N,dtype,pad,beta", [(64, W.SD_F32, 0, 0.0), (96, W.SD_F32, 0, 0.5), (128, W.SD_F32, 64, -1.0), (160, W.SD_F32, 0, 0.0),
+                                              (640, W.SD_F32, 0, 0.0), (65, W.SD_F32, 0, 0.5), (128, W.SD_BF16, 0, 0.0), (320, W.SD_BF16, 0, 0.5)])
+def test_host_operands_in_column_slices(N, dtype, pad, beta):
+    import paper_2608_05033_b200 as sd
+    from util import DeviceWorkload
+    rng = np.random.default_rng(N)
+    M, K = 4200, 4300
+    w = W.random_csr(M, K, N, np.r_[3000, rng.integers(0, 12, M - 1)], seed=N, dtype=dtype, alpha=0.75, beta=beta)
+    for family in (sd.SD_AUTO, sd.SD_ROWSPLIT):
+        plan = DeviceWorkload(w).plan(family=family)
+        Bh = np.zeros((K, N + pad), w.B.dtype)
+        Bh[:, :N] = w.B
+        Ch = np.full((M, N + pad), -7.25, np.float32)
+        if w.C0 is not None:
+            Ch[:, :N] = w.C0
+        B = torch.from_numpy(Bh.view(np.int16) if Bh.dtype == np.uint16 else Bh).pin_memory()
+        C = torch.from_numpy(Ch).pin_memory()
+        plan.spmm_host(B, C, w.alpha, w.beta)
+        got = C.numpy()
+        r = oracle.check(w.rowptr, w.colind, w.vals, w.B, N, np.ascontiguousarray(got[:, :N]), w.C0, w.alpha, w.beta)
+        assert r["ok"], r
+        assert np.all(got[:, N:] == np.float32(-7.25))
+        plan.close()
