@@ -413,7 +413,7 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
 
     switch (plan->info.family) {
     case SD_ROWSPLIT:
-        SD_CUDA_TRY(run_rowsplit(a, plan->dtype, vec, st));
+        SD_CUDA_TRY(run_rowsplit(a, plan->dtype, piece_width(plan->dtype, N, B, ldb, C, ldc), st));
         return SD_OK;
     case SD_MERGE: {
         if (plan->coo_row) {   // narrow dense operand: one writer per row

@@ -1,0 +1,125 @@
+// Sums of the nonzeros of a row (or of a part of one) by a group of lanes: some of them stand across the columns of B and C,
+// the others share the nonzeros.  Used by the hybrid schedule and by the row-group kernel.
+#pragma once
+
+#include <type_traits>
+
+#include "sd_common.cuh"
+#include "sd_piece.cuh"
+
+namespace sd {
+
+// Per-lane view of B and C for one column slab.
+template <typename T, int VW, int LPR, int NV>
+struct LaneCols {
+    const T *B;
+    int cbase;
+    bool ok[NV];
+    __device__ __forceinline__ LaneCols(const void *b, int32_t N, int lg) {
+        const int slab = blockIdx.y * (LPR * NV * VW);
+        cbase = slab + lg * VW;
+        B = static_cast<const T *>(b) + cbase;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) ok[v] = cbase + v * LPR * VW < N;
+    }
+    // gathers of one row of B; `use` = false gathers nothing (row 0 of B may hold non-finite values)
+    __device__ __forceinline__ void gather(int col, uint32_t ldb_bytes, bool use, Piece<T, VW> (&b)[NV]) const {
+        const T *row = b_row(B, col, ldb_bytes);
+#pragma unroll
+        for (int v = 0; v < NV; ++v) {
+            if (use && ok[v]) b[v].ld(row + v * LPR * VW);
+            else b[v].zero();
+        }
+    }
+    __device__ __forceinline__ void fma(float w, const Piece<T, VW> (&b)[NV], float (&acc)[NV][VW]) const {
+#pragma unroll
+        for (int v = 0; v < NV; ++v) b[v].fma(w, acc[v]);
+    }
+    __device__ __forceinline__ void store(float *crow, const float (&acc)[NV][VW], float alpha, float beta) const {
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+            if (ok[v]) store_cols<VW>(crow + cbase + v * LPR * VW, acc[v], alpha, beta, 0);
+    }
+};
+
+template <int NV, int VW>
+__device__ __forceinline__ void clear_acc(float (&acc)[NV][VW]) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) acc[v][e] = 0.f;
+}
+
+// Sum over the LANES / LPR lane sets of a group (a fixed order: results repeat bit for bit).
+template <int LANES, int LPR, int NV, int VW>
+__device__ __forceinline__ void sum_sets(float (&acc)[NV][VW], unsigned mask) {
+#pragma unroll
+    for (int d = LANES / 2; d >= LPR; d >>= 1)
+#pragma unroll
+        for (int v = 0; v < NV; ++v)
+#pragma unroll
+            for (int e = 0; e < VW; ++e) acc[v][e] += __shfl_xor_sync(mask, acc[v][e], d);
+}
+
+// Nonzeros [p0, p1) by a group of LANES lanes.  A step loads NB x LANES (column, value) pairs, one coalesced load of each
+// per NB, and requests the next step's before this step's gathers; set k of the group takes pairs k, k + G, ... of a load,
+// handed round by shuffle.  Q gathers of a lane are in flight together.  Whole steps run without any test; only the
+// last, partly filled one tests every pair: nothing may be gathered for a pair beyond the end (row 0 of B may hold
+// non-finite values, and 0 * Inf is NaN).
+template <typename T, int VW, int LPR, int NV, int LANES, typename Args>
+__device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, LPR, NV> &lc, int p0, int p1,
+                                          unsigned mask, float (&acc)[NV][VW]) {
+    constexpr int G = LANES / LPR;
+    constexpr int NB = LPR >= 4 ? 1 : 4 / LPR;          // loads of pairs per step: at least four gathers per lane and step
+    constexpr int PER = NB * LPR;                       // gathers of a lane per step
+    constexpr int QM = NV * VW * sizeof(T) > 16 ? 4 : 8;
+    constexpr int Q = PER < QM ? PER : QM;
+    const T *__restrict__ vals = static_cast<const T *>(a.vals);
+    const int lg = threadIdx.x % LANES, k = lg / LPR;
+    int c[NB];
+    float w[NB];
+    auto fetch = [&](int p) {
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            const bool in = p + n * LANES + lg < p1;
+            c[n] = in ? __ldg(a.colind + p + n * LANES + lg) : -1;
+            w[n] = in ? to_float(vals[p + n * LANES + lg]) : 0.f;
+        }
+    };
+    auto step = [&](int p, auto whole_tag) {
+        constexpr bool WHOLE = decltype(whole_tag)::value;
+        int cc[NB];
+        float cw[NB];
+#pragma unroll
+        for (int n = 0; n < NB; ++n) {
+            cc[n] = c[n];
+            cw[n] = w[n];
+        }
+        constexpr int QS = WHOLE || Q < 4 ? Q : 4;
+        if (WHOLE) fetch(p + NB * LANES);
+#pragma unroll 1
+        for (int i0 = 0; i0 < PER; i0 += QS) {   // one batch at a time: unrolled, the compiler starts all of them and spills
+            if (!WHOLE && p + i0 * G >= p1) break;
+            Piece<T, VW> b[QS][NV];
+#pragma unroll
+            for (int u = 0; u < QS; ++u) {
+                const int n = NB == 1 ? 0 : u / LPR, src = NB == 1 ? (i0 + u) * G + k : u % LPR * G + k;
+                const int col = LPR == 1 ? cc[n] : __shfl_sync(mask, cc[n], src, LANES);
+                lc.gather(col, a.ldb_bytes, WHOLE || col >= 0, b[u]);
+            }
+#pragma unroll
+            for (int u = 0; u < QS; ++u) {
+                const int n = NB == 1 ? 0 : u / LPR, src = NB == 1 ? (i0 + u) * G + k : u % LPR * G + k;
+                lc.fma(LPR == 1 ? cw[n] : __shfl_sync(mask, cw[n], src, LANES), b[u], acc);
+            }
+        }
+    };
+    int p = p0;
+    fetch(p);
+#pragma unroll 1
+    for (; p + NB * LANES <= p1; p += NB * LANES) step(p, std::true_type{});
+    if (p < p1) step(p, std::false_type{});
+    sum_sets<LANES, LPR, NV, VW>(acc, mask);
+}
+
+}  // namespace sd

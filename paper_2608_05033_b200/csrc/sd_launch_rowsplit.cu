@@ -1,17 +1,47 @@
 #include "sd_launch.cuh"
+#include "sd_rowgroup.cuh"
 #include "sd_rowsplit.cuh"
 #include "sd_rowsplit_narrow.cuh"
 #include "sd_chunk_sums.cuh"
 
 namespace sd {
 
-cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, bool vec, cudaStream_t st) {
+// Lane sets per row of the row-group kernel, or 0 where the kernels below are ahead.  Measured on uniform rows of 5 to 128
+// nonzeros, stencils and blocks, 5 to 128 columns, both value types:
+//   not whole 16-byte loads   always (41 columns: 1.8 to 3.9 times as fast as one scalar per lane)
+//   few rows                  four sets as soon as rows are 8 long: one set leaves the GPU idle (5,000 rows of 30 at 64 columns
+//                             17.9 -> 5.3 us, at 128 bf16 24.9 -> 6.7)
+//   narrow and short          up to eight loads per row of B and below 16 nonzeros, where a row is over before sets pay (800,000
+//                             rows of 12 at 64 bf16 columns 359 -> 227 us, at 32 fp32 columns 222 -> 192); stencil rows of fp32
+//                             values keep the plain kernel (7.9 against 9.2 us at 8 columns)
+//   8 columns                 four sets up to 64 nonzeros (rows of 30: fp32 19.7 -> 17.2, bf16 25.7 -> 15.9)
+//   long rows, wide           four sets from 64 nonzeros where the set kernel below does not reach (beyond 16 loads per row of
+//                             B, or not a power of two of them): blocks at 128 fp32 columns 180 -> 139 us
+static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
+    const int units = (a.N + vw - 1) / vw;
+    const int64_t mean = a.mean_len;
+    int lanes = 1;
+    while (lanes < 32 && lanes < units) lanes <<= 1;
+    const bool fills = a.S * lanes >= static_cast<int64_t>(sm_count_cached()) * 5 * kRowGroupThreads;
+    int sets = 0;
+    if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
+    else if (!fills && mean >= 8) sets = 4;
+    else if (a.N <= 8 && mean >= 8 && mean < 64) sets = 4;
+    else if (units <= 8 && mean < 16 && (dtype == SD_BF16 || mean > 6)) sets = 1;
+    else if (mean >= 64 && (units > 16 || (units & (units - 1)) != 0)) sets = 4;
+    return a.max_len > 0 && a.max_len <= static_cast<int64_t>(kRowGroupTerms) * sets ? sets : 0;
+}
+
+cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t st) {
+    const int vw = dtype == SD_F32 ? 4 : 8;
+    const bool vec = vw_now == vw;
     if (a.N >= 1 && a.N <= 4 && !switches().no_narrow) {   // one to four columns: lanes share a row, not its columns
         if (dtype == SD_F32) return launch_rowsplit_narrow<float>(a, vec, st);
         return launch_rowsplit_narrow<__nv_bfloat16>(a, vec, st);
     }
+    if (const int sets = rowgroup_sets(a, dtype, vw_now, vec))
+        return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, sets, st) : run_rowgroup_bf16(a, vw_now, sets, st);
     // 8 to 64 columns (fp32; 8 to 128 bf16) as whole 16-byte vectors and long rows: several lane sets per row
-    const int vw = dtype == SD_F32 ? 4 : 8;
     if (vec && a.N % vw == 0 && a.N / vw <= 16 && ((a.N / vw) & (a.N / vw - 1)) == 0) {
         const int lpr = a.N / vw;
         const int g = ksplit_group(a.mean_len, lpr);

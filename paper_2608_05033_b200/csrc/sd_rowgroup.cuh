@@ -1,0 +1,76 @@
+// Family (a), one group of LANES lanes per row in natural order: LPR lanes stand across the columns, LANES / LPR lane sets share
+// the row's nonzeros (group_sum).  It serves every width that is not a whole number of 16-byte loads (odd widths, unaligned
+// operands: two to four loads of 8, 4 or 2 bytes per lane) and rows long enough to share at the others; rows longer than
+// kRowGroupTerms terms per lane set keep the kernels with a second accumulator.
+#pragma once
+
+#include "sd_group.cuh"
+
+namespace sd {
+
+constexpr int kRowGroupThreads = 256;
+constexpr int kRowGroupTerms = 512;
+
+template <typename T, int VW, int LPR, int NV, int LANES>
+__global__ void __launch_bounds__(kRowGroupThreads, 5)
+rowgroup_kernel(const SpmmArgs a) {
+    const int lane = threadIdx.x & 31, lg = threadIdx.x % LANES;
+    const unsigned mask = LANES == 32 ? 0xffffffffu : ((1u << LANES % 32) - 1u) << (lane & ~(LANES - 1));
+    const int64_t row = (static_cast<int64_t>(blockIdx.x) * kRowGroupThreads + threadIdx.x) / LANES;
+    int p0 = 0, p1 = 0;
+    if (row < a.S) {
+        p0 = __ldg(a.ptr + row);
+        p1 = __ldg(a.ptr + row + 1);
+    }
+    overlap_next();
+    overlap_wait();
+    const LaneCols<T, VW, LPR, NV> lc(a.B, a.N, lg % LPR);
+    float acc[NV][VW];
+    clear_acc(acc);
+    group_sum<T, VW, LPR, NV, LANES>(a, lc, p0, p1, mask, acc);
+    if (row < a.S && lg < LPR) lc.store(a.C + row * a.ldc, acc, a.alpha, a.beta);
+}
+
+template <typename T, int VW, int LPR, int NV, int LANES>
+cudaError_t launch_rowgroup_lanes(const SpmmArgs &a, cudaStream_t st) {
+    constexpr int rows = kRowGroupThreads / LANES, slab = LPR * NV * VW;
+    return launch_overlapped(rowgroup_kernel<T, VW, LPR, NV, LANES>,
+                             dim3(static_cast<unsigned>((a.S + rows - 1) / rows), static_cast<unsigned>((a.N + slab - 1) / slab)),
+                             kRowGroupThreads, 0, st, a);
+}
+
+// Lane sets per row: 1 or 4 (as many as fit a warp).
+template <typename T, int VW, int LPR, int NV>
+cudaError_t launch_rowgroup_one(const SpmmArgs &a, int sets, cudaStream_t st) {
+    constexpr int MANY = LPR * 4 > 32 ? 32 : LPR * 4;
+    if (sets > 1) return launch_rowgroup_lanes<T, VW, LPR, NV, MANY>(a, st);
+    return launch_rowgroup_lanes<T, VW, LPR, NV, LPR>(a, st);
+}
+
+template <typename T, int VW>
+cudaError_t launch_rowgroup(const SpmmArgs &a, int sets, cudaStream_t st) {
+    constexpr bool FULL = VW * sizeof(T) == 16;
+    const int all = (a.N + VW - 1) / VW, widest = FULL ? 64 : 128;
+    const int slabs = (all + widest - 1) / widest, units = (all + slabs - 1) / slabs;
+    if constexpr (FULL) {
+        if (units <= 1) return launch_rowgroup_one<T, VW, 1, 1>(a, sets, st);
+        if (units <= 2) return launch_rowgroup_one<T, VW, 2, 1>(a, sets, st);
+    }
+    if (units <= 4) return launch_rowgroup_one<T, VW, 4, 1>(a, sets, st);
+    if (units <= 8) return launch_rowgroup_one<T, VW, 8, 1>(a, sets, st);
+    if constexpr (FULL) {
+        if (units <= 16) return launch_rowgroup_one<T, VW, 16, 1>(a, sets, st);
+        if (units <= 32) return launch_rowgroup_one<T, VW, 16, 2>(a, sets, st);
+        return launch_rowgroup_one<T, VW, 32, 2>(a, sets, st);
+    } else {
+        if (units <= 16) return launch_rowgroup_one<T, VW, 8, 2>(a, sets, st);
+        if (units <= 24) return launch_rowgroup_one<T, VW, 8, 3>(a, sets, st);
+        if (units <= 32) return launch_rowgroup_one<T, VW, 16, 2>(a, sets, st);
+        if (units <= 48) return launch_rowgroup_one<T, VW, 16, 3>(a, sets, st);
+        if (units <= 64) return launch_rowgroup_one<T, VW, 32, 2>(a, sets, st);
+        if (units <= 96) return launch_rowgroup_one<T, VW, 32, 3>(a, sets, st);
+        return launch_rowgroup_one<T, VW, 32, 4>(a, sets, st);
+    }
+}
+
+}  // namespace sd

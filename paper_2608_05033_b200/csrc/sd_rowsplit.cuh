@@ -29,11 +29,13 @@ rowsplit_kernel(const SpmmArgs a) {
         p0 = __ldg(a.ptr + row);
         len = __ldg(a.ptr + row + 1) - p0;
     }
-    // the first (column, value) pairs' columns do not depend on earlier work in the stream
-    int firstc = 0;
-    if (lg < len) firstc = __ldg(a.colind + p0 + lg);
+    // the columns of the first step do not depend on earlier work in the stream
+    int myc = 0;
+    if (lg < len) myc = __ldg(a.colind + p0 + lg);
     overlap_next();
     overlap_wait();
+    float myv = 0.f;
+    if (lg < len) myv = to_float(vals[p0 + lg]);
     // trip counts are made warp-uniform so that the shuffles below are always converged
     const int maxlen = (LPR == 32) ? len : __reduce_max_sync(FULL, len);
 
@@ -85,11 +87,10 @@ rowsplit_kernel(const SpmmArgs a) {
             }
         }
         // the group fetches LPR (column, value) pairs with one coalesced load each ...
-        int myc = 0;
-        float myv = 0.f;
-        if (base + lg < len) {
-            myc = base == 0 ? firstc : __ldg(a.colind + p0 + base + lg);
-            myv = to_float(vals[p0 + base + lg]);
+        if (base != 0) {
+            const bool in = base + lg < len;
+            myc = in ? __ldg(a.colind + p0 + base + lg) : 0;
+            myv = in ? to_float(vals[p0 + base + lg]) : 0.f;
         }
         const int cnt = min(LPR, maxlen - base);
         // ... and hands them round by shuffle

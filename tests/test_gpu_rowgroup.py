@@ -1,0 +1,35 @@
+"""The row-group kernel of the row-split family: one group of lanes per row, one or four lane sets, loads of 16, 8, 4 or 2
+bytes by what width and operands allow.  Rows at the edges of a batch, of a group of lanes and of the longest sum one lane
+set may take (512 terms), with empty rows between them."""
+import numpy as np
+import pytest
+
+import workloads as W
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if torch.cuda.is_available():
+    import paper_2608_05033_b200 as sd
+    from test_gpu_parity import check
+    from util import DeviceWorkload, run_spmm
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [5, 8, 12, 31, 34, 64, 97, 132, 260, 521])
+@pytest.mark.parametrize("edges", [[0, 1, 7, 8, 9, 15], [0, 1, 31, 32, 33, 512], [64, 127, 0, 513, 2047, 2048]])
+def test_row_group_lengths_widths_and_alignment(edges, N, dtype):
+    rng = np.random.default_rng(N + len(edges))
+    M, K = 203, 2100
+    lengths = rng.permutation(np.resize(edges, M))
+    w = W.random_csr(M, K, N, lengths, seed=N, dtype=dtype, alpha=-0.75, beta=0.5)
+    dw = DeviceWorkload(w)
+    plan = dw.plan(family=sd.SD_ROWSPLIT)
+    for kw in (dict(), dict(pad_b=3, pad_c=5), dict(offset=1), dict(offset=2, pad_b=2)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+        again, _ = run_spmm(plan, w, **kw)
+        assert np.array_equal(got, again)
+    got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
