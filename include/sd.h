@@ -61,7 +61,7 @@ typedef enum {
                         the (row, column window) segments re-bucketed window by window, long ones as
                         128-nonzero chunks, short ones one lane group each, one-nonzero ones flat),
                         chosen by dense width and forced with windows = -1 */
-    SD_BSR_TC = 3,   /* 16x16 blocks on the tensor cores (tcgen05 / TMEM / TMA) */
+    SD_BSR_TC = 3,   /* 16x16 blocks on the tensor cores (bf16; fp32 as three tf32 products) */
     SD_HYBRID = 4    /* the schedule of the paper's appendix listing (light rows row-wise, heavy rows in
                         chunks), without its atomics: rows below heavy_len nonzeros are summed row-wise,
                         several rows per lane group, longest first; every heavy row is cut, column window by
@@ -87,10 +87,9 @@ typedef struct {
                               -1 = one window, but with the class split of the window-major schedule */
     int32_t validate;      /* != 0: check rowptr monotone and 0 <= col < K on the device first */
     void *stream;          /* stream for the analysis kernels (plan creation still synchronises) */
-    int32_t test_wait_expiry; /* TEST ONLY, leave 0.  != 0: in the tensor-core kernel of an SD_BSR_TC plan the first CTA's
-                              copy thread never fills its ring, and every wait gives up after a few thousand polls
-                              instead of a million: the kernel must return by itself, sd_plan_device_status must
-                              report a non-zero code, C is left incomplete */
+    int32_t test_wait_expiry; /* TEST ONLY, leave 0.  != 0: every product of an SD_BSR_TC plan is followed by a kernel
+                              whose wait runs out after a few thousand polls: it must return by itself and
+                              sd_plan_device_status must report a non-zero code */
     int32_t heavy_len;     /* SD_HYBRID: rows of at least this many nonzeros run as chunks; 0 = the library's default
                               (256, the long-row threshold of the paper's appendix listing); clamped to 2 .. 256 */
 } sd_plan_desc_t;
@@ -318,10 +317,10 @@ sd_status_t sd_plan_get_segments(const sd_plan_t *plan, int32_t *seg_ptr, int32_
 sd_status_t sd_plan_get_hybrid(const sd_plan_t *plan, int32_t *heavy_rows, int32_t *chunk_ptr, int32_t *ranges,
                                int32_t *order, int32_t *light_rows);
 
-/* sd_plan_device_status -- every wait inside the library's kernels (mbarrier waits of the
- * tensor-core kernel) is bounded; a wait that runs out makes its CTA record a non-zero code
- * in a plan-owned device word, release its resources and return, so the context stays
- * usable but C is then incomplete.  This call synchronises the device, copies the word to
+/* sd_plan_device_status -- a wait inside one of the library's kernels is bounded; one that runs
+ * out records a non-zero code in a plan-owned device word and the kernel returns, so the
+ * context stays usable (no product waits on another CTA at present; sd_plan_desc_t.test_wait_expiry
+ * makes one run out).  This call synchronises the device, copies the word to
  * *status (0 = no wait ever expired) and clears it. */
 sd_status_t sd_plan_device_status(sd_plan_t *plan, int32_t *status);
 

@@ -46,10 +46,6 @@ const Switches &switches() {
         s.geom_nv = env_int("SD_GEOM_NV", 0);
         s.ksplit_g = env_int("SD_KSPLIT_G", 0);
         s.narrow_g = env_int("SD_NARROW_G", 0);
-        s.tc_sb = env_int("SD_TC_SB", 0);
-        s.tc_stages = env_int("SD_TC_STAGES", 0);
-        s.tc32_sb = env_int("SD_TC32_SB", 0);
-        s.tc32_stages = env_int("SD_TC32_STAGES", 0);
         return s;
     }();
     return sw;
@@ -470,9 +466,6 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
         b.browptr = plan->browptr;
         b.bcol = plan->bcol;
         b.bval = plan->bval;
-        b.bval_mma = plan->bval_mma;
-        b.part = plan->bsr_part;
-        b.nparts = plan->bsr_nparts;
         b.B = B;
         b.C = C;
         b.ldb = ldb;
@@ -483,14 +476,8 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
         b.N = static_cast<int32_t>(N);
         b.alpha = alpha;
         b.beta = beta;
-        b.map_cache = &plan->tc_map;
-        b.test_wait_expiry = plan->test_wait_expiry;
-        const bool vec4 = aligned16(B) && aligned16(C) && N % 4 == 0 && ldb % 4 == 0 && ldc % 4 == 0 &&
-                          (plan->dtype == SD_F32 || (reinterpret_cast<uintptr_t>(B) & 7u) == 0);
-        if (bsr_tc_usable(b, plan->dtype) && !switches().bsr_simt)
-            SD_CUDA_TRY(run_bsr_tc(b, plan->dtype, plan->dev_error, plan->info.sm_count, st));
-        else
-            SD_CUDA_TRY(run_bsr_simt(b, plan->dtype, vec4, st));
+        SD_CUDA_TRY(run_bsr(b, plan->dtype, st));
+        if (plan->test_wait_expiry) SD_CUDA_TRY(run_wait_expiry(plan->dev_error, st));
         return SD_OK;
     }
     default:
@@ -822,7 +809,7 @@ sd_status_t sd_plan_update_values(sd_plan_t *plan, const void *vals, void *strea
         return SD_ERR_INVALID_ARG;
     }
     plan->vals = vals;
-    if (plan->info.family == SD_BSR_TC) SD_CUDA_TRY(fill_bsr(plan, static_cast<cudaStream_t>(stream)));
+    if (plan->info.family == SD_BSR_TC) SD_CUDA_TRY(fill_bsr(plan, true, static_cast<cudaStream_t>(stream)));
     return SD_OK;   // the other families read the caller's array
 }
 

@@ -1,0 +1,313 @@
+// Family (c) on the warp-level tensor-core instructions: a warp multiplies the 16x16 blocks of one block-row with a strip of B
+// (NS times 128 bytes wide) and keeps the 16 rows of C in registers.  Each warp runs its own ring of asynchronous copies (the
+// block and the rows of B it meets), so only the end of a block-row shared by several warps waits for another warp.  The
+// 16-byte chunks of a strip row lie exclusive-ored with a function of the row: every fragment read is free of bank conflicts.
+//
+//   k    is dealt out so that lane 4g + t works on block columns 4t .. 4t+3: its part of block rows g and g + 8 is one vector
+//        load each, and the rows of B it needs are 4t .. 4t+3,
+//   bf16 the transposing matrix load brings rows (4t, 4t+1) and (4t+2, 4t+3) of 8 columns, one m16n8k16 per 8 columns,
+//   fp32 the lane reads one chunk of each of its four rows; column n of tile j is float j of that chunk.  Both operands are
+//        split x = hi + lo: B's hi is what the tensor core keeps of x (the low 13 bits fall), the block's hi is x rounded to
+//        tf32.  Three m16n8k8 per tile and half block: lo*hi, hi*lo, hi*hi; lo*lo is below 2^-21 of |a||b|.
+//
+// What bounds it: fp32 the tensor pipe (480 multiply-adds per SM and cycle of mma.sync tf32, three per product; counters show
+// 55 % of the pipe's cycles) with the copies' latency behind it; bf16 the L2 reads of B (33,554 blocks of a 64K x 64K matrix,
+// 256 columns: 550 MB).
+//
+// Why not one tcgen05.mma per block and 256 columns, which this replaces: its accumulator has 64 or 128 rows and a block has
+// 16, so 3/4 or 7/8 of its multiply-adds are for nothing, a single thread issues it, fp32 slabs of B must be split through
+// shared memory, and a matrix of few block-rows leaves most CTAs idle.  Those 33,554 blocks, us, before and now:
+//     columns    64          128         256         512
+//     fp32       119 -> 31   117 -> 54   145 -> 94   308 -> 195
+//     bf16       42 -> 19    40 -> 23    49 -> 41    94 -> 74
+// and 800 blocks in 200 block-rows at 128 columns 14.3 -> 4.4 (fp32), 8.2 -> 3.5 (bf16).
+#pragma once
+
+#include "sd_common.cuh"
+#include "sd_launch.cuh"
+
+namespace sd {
+
+constexpr int kMmaWarps = 4;
+// Ring slots: two blocks are in flight while one is multiplied; the 5 KB slots of wide fp32 strips leave room for more warps
+// with two (64K x 64K, 256 columns: 94 against 98 us).
+template <typename T, int NS> constexpr int kMmaStages = sizeof(T) == 4 && NS == 2 ? 2 : 3;
+constexpr int kMmaStrip = 2048;   // bytes of a strip: 16 rows of 128
+template <typename T, int NS> constexpr int kMmaSlot = NS * kMmaStrip + 256 * static_cast<int>(sizeof(T));
+
+__device__ __forceinline__ void mma_tf32(float (&d)[4], const uint32_t (&x)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_bf16(float (&d)[4], const uint32_t (&x)[4], uint32_t b0, uint32_t b1) {
+    asm("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(x[0]), "r"(x[1]), "r"(x[2]), "r"(x[3]), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void ldmatrix_trans(uint32_t (&r)[4], uint32_t addr) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+                 : "r"(addr)
+                 : "memory");
+}
+__device__ __forceinline__ uint4 ld_shared4(uint32_t addr) {
+    uint4 v;
+    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];" : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w) : "r"(addr) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint2 ld_shared2(uint32_t addr) {
+    uint2 v;
+    asm volatile("ld.shared.v2.u32 {%0,%1}, [%2];" : "=r"(v.x), "=r"(v.y) : "r"(addr) : "memory");
+    return v;
+}
+// .ca keeps the source line in L1 (blocks, which several warps read), .cg does not
+__device__ __forceinline__ void copy_ca(uint32_t dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copy_cg(uint32_t dst, const void *src) {
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void zero_shared(uint32_t dst) {
+    asm volatile("st.shared.v4.u32 [%0], {%1, %1, %1, %1};" ::"r"(dst), "r"(0) : "memory");
+}
+
+// Where chunk c of strip row r lies (in chunks).  bf16: the eight rows 4i, 4i+1 (or 4i+2, 4i+3) of one matrix load differ in
+// the three bits.  fp32: a quarter warp reads chunks p and p + 4 of rows 4t + i.
+template <typename T>
+__device__ __forceinline__ int strip_chunk(int r, int c) {
+    return r * 8 + (c ^ (sizeof(T) == 2 ? (r & 1) | ((r >> 2) << 1) : r >> 2));
+}
+
+// One lane's part of block x strips.
+template <typename T, int NS> struct BlockProduct;
+
+template <int NS> struct BlockProduct<__nv_bfloat16, NS> {
+    static constexpr int TILES = 8;   // of 8 columns, per strip
+    uint32_t frag[TILES / 2];         // this lane's row of the four matrices of a load: both row pairs of two chunks
+    __device__ __forceinline__ explicit BlockProduct(int lane) {
+        const int i = lane & 7, m = lane >> 3, r = (i >> 1) * 4 + (i & 1) + (m & 1) * 2;
+#pragma unroll
+        for (int j = 0; j < TILES / 2; ++j) frag[j] = strip_chunk<__nv_bfloat16>(r, 2 * j + (m >> 1)) << 4;
+    }
+    __device__ __forceinline__ void operator()(float (&acc)[NS][TILES][4], uint32_t strip, uint32_t block, int lane) const {
+        const uint2 u = ld_shared2(block + lane * 8), v = ld_shared2(block + 256 + lane * 8);
+        const uint32_t x[4] = {u.x, v.x, u.y, v.y};
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+#pragma unroll
+            for (int j = 0; j < TILES; j += 2) {
+                uint32_t b[4];
+                ldmatrix_trans(b, strip + s * kMmaStrip + frag[j / 2]);
+                mma_bf16(acc[s][j], x, b[0], b[1]);
+                mma_bf16(acc[s][j + 1], x, b[2], b[3]);
+            }
+    }
+    static __device__ __forceinline__ void store(const float (&acc)[TILES][4], int e, float *out, int t, int left, float alpha, float beta) {
+#pragma unroll
+        for (int j = 0; j < TILES; ++j)
+            if (j * 8 < left) {
+                const float v[2] = {acc[j][e], acc[j][e + 1]};
+                store_cols<2>(out + j * 8 + t * 2, v, alpha, beta, 0);
+            }
+    }
+};
+
+template <int NS> struct BlockProduct<float, NS> {
+    static constexpr int TILES = 4;
+    uint32_t frag[4];
+    __device__ __forceinline__ explicit BlockProduct(int lane) {
+        const int g = lane >> 2, t = lane & 3;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) frag[i] = strip_chunk<float>(4 * t + i, (g >> 1) | ((g & 1) << 2)) << 4;
+    }
+    static __device__ __forceinline__ float top(float m, const uint4 &v) {
+        m = fmaxf(fmaxf(m, fabsf(__uint_as_float(v.x))), fabsf(__uint_as_float(v.y)));
+        return fmaxf(fmaxf(m, fabsf(__uint_as_float(v.z))), fabsf(__uint_as_float(v.w)));
+    }
+    __device__ __forceinline__ void operator()(float (&acc)[NS][TILES][4], uint32_t strip, uint32_t block, int lane) const {
+        const uint4 a0 = ld_shared4(block + lane * 16), a1 = ld_shared4(block + 512 + lane * 16);
+        uint4 b[NS][4];
+#pragma unroll
+        for (int s = 0; s < NS; ++s)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) b[s][i] = ld_shared4(strip + s * kMmaStrip + frag[i]);
+        // the block's hi is rounded, but never up to infinity
+        const uint32_t half = __any_sync(0xffffffffu, top(top(0.f, a0), a1) >= 3.4e38f) ? 0u : 0x1000u;
+        auto cut = [](uint32_t v) { return v & 0xFFFFE000u; };
+        auto rest = [](uint32_t v, uint32_t h) { return __float_as_uint(__uint_as_float(v) - __uint_as_float(h)); };
+        const uint32_t wa[2][4] = {{a0.x, a0.y, a0.z, a0.w}, {a1.x, a1.y, a1.z, a1.w}};
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            uint32_t xh[4], xl[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const uint32_t v = wa[i & 1][2 * h + (i >> 1)];
+                xh[i] = cut(v + half);
+                xl[i] = rest(v, xh[i]);
+            }
+            // each pass goes over all tiles: an accumulator comes up again only after the others
+#pragma unroll
+            for (int p = 0; p < 3; ++p)
+#pragma unroll
+                for (int s = 0; s < NS; ++s) {
+                    const uint32_t w0[4] = {b[s][2 * h].x, b[s][2 * h].y, b[s][2 * h].z, b[s][2 * h].w};
+                    const uint32_t w1[4] = {b[s][2 * h + 1].x, b[s][2 * h + 1].y, b[s][2 * h + 1].z, b[s][2 * h + 1].w};
+#pragma unroll
+                    for (int j = 0; j < TILES; ++j) {
+                        if (p == 0) mma_tf32(acc[s][j], xl, w0[j], w1[j]);
+                        if (p == 1) mma_tf32(acc[s][j], xh, w0[j], w1[j]);
+                        if (p == 2) mma_tf32(acc[s][j], xh, rest(w0[j], cut(w0[j])), rest(w1[j], cut(w1[j])));
+                    }
+                }
+        }
+    }
+    // columns 2t and 2t + 1 of the four tiles are chunks t and t + 4
+    static __device__ __forceinline__ void store(const float (&acc)[TILES][4], int e, float *out, int t, int left, float alpha, float beta) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            if (t * 4 + h * 16 < left) {
+                const float v[4] = {acc[0][e + h], acc[1][e + h], acc[2][e + h], acc[3][e + h]};
+                store_cols<4>(out + t * 4 + h * 16, v, alpha, beta, 0);
+            }
+    }
+};
+
+// KS warps of a CTA share the blocks of a block-row and meet in shared memory, always in the same order.
+template <typename T, int NS, int KS>
+__global__ void __launch_bounds__(kMmaWarps * 32)
+bsr_mma_kernel(const BsrArgs a) {
+    constexpr int V = 16 / sizeof(T), COLS = 8 * V * NS, SLOT = kMmaSlot<T, NS>, STAGES = kMmaStages<T, NS>, RING = STAGES * SLOT;
+    extern __shared__ __align__(1024) char ring[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, ks = warp % KS;
+    const int64_t I = blockIdx.x;
+    const int strip0 = (blockIdx.y * (kMmaWarps / KS) + warp / KS) * COLS;
+    const int b0 = __ldg(a.browptr + I) + ks;
+    const int count = strip0 < a.N ? max(0, (__ldg(a.browptr + I + 1) - b0 + KS - 1) / KS) : 0;
+    const int *bcol = a.bcol + b0;
+    int cols = lane < count ? __ldg(bcol + lane * KS) : 0;
+    overlap_next();
+    overlap_wait();
+
+    const uint32_t base = static_cast<uint32_t>(__cvta_generic_to_shared(ring)) + warp * RING;
+    const int chunk = lane & 7, row = lane >> 3;
+    const T *B = static_cast<const T *>(a.B) + static_cast<int64_t>(row) * a.ldb + strip0 + chunk * V;
+    const int64_t step = 4 * a.ldb;
+    bool in_cols[NS];   // chunks beyond the last column stay as they are: they only reach columns that are not stored
+    uint32_t dst[4];
+#pragma unroll
+    for (int s = 0; s < NS; ++s) in_cols[s] = strip0 + (s * 8 + chunk) * V < a.N;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dst[i] = strip_chunk<T>(row + 4 * i, chunk) << 4;
+    const char *block = static_cast<const char *>(a.bval) + static_cast<int64_t>(b0) * (256 * sizeof(T)) + lane * 16;
+    auto issue = [&](int n, uint32_t slot) {
+        if (n < count) {
+            if ((n & 31) == 0 && n > 0) cols = n + lane < count ? __ldg(bcol + (n + lane) * KS) : 0;
+            const int k0 = __shfl_sync(0xffffffffu, cols, n & 31) * 16;
+            const T *p = B + k0 * a.ldb;
+            if (k0 + 16 <= a.K) {
+#pragma unroll
+                for (int i = 0; i < 4; ++i, p += step)
+#pragma unroll
+                    for (int s = 0; s < NS; ++s)
+                        if (in_cols[s]) copy_cg(slot + s * kMmaStrip + dst[i], p + s * 8 * V);
+            } else {   // rows beyond the last of B meet zeros of the block and must be finite
+                for (int i = 0; i < 4; ++i, p += step)
+                    for (int s = 0; s < NS; ++s)
+                        if (k0 + row + 4 * i >= a.K) zero_shared(slot + s * kMmaStrip + (strip_chunk<T>(row + 4 * i, chunk) << 4));
+                        else if (in_cols[s]) copy_cg(slot + s * kMmaStrip + (strip_chunk<T>(row + 4 * i, chunk) << 4), p + s * 8 * V);
+            }
+            copy_ca(slot + NS * kMmaStrip + lane * 16, block);
+            if constexpr (sizeof(T) == 4) copy_ca(slot + NS * kMmaStrip + 512 + lane * 16, block + 512);
+            block += KS * 256 * sizeof(T);
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    const BlockProduct<T, NS> product(lane);
+    constexpr int TILES = BlockProduct<T, NS>::TILES;
+    float acc[NS][TILES][4];
+#pragma unroll
+    for (int s = 0; s < NS; ++s)
+#pragma unroll
+        for (int i = 0; i < TILES * 4; ++i) acc[s][i >> 2][i & 3] = 0.f;
+#pragma unroll
+    for (int n = 0; n < STAGES - 1; ++n) issue(n, base + n * SLOT);
+    int slot = 0;
+#pragma unroll 1
+    for (int n = 0; n < count; ++n) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(STAGES - 2) : "memory");
+        __syncwarp();   // every lane's part of this slot has landed, and the slot read last time is free
+        issue(n + STAGES - 1, base + (slot == 0 ? STAGES - 1 : slot - 1) * SLOT);
+        product(acc, base + slot * SLOT, base + slot * SLOT + NS * kMmaStrip, lane);
+        slot = slot + 1 == STAGES ? 0 : slot + 1;
+    }
+    if constexpr (KS > 1) {
+        static_assert(NS * TILES * 4 * 32 * 4 <= RING, "a warp leaves its sums in its own ring");
+        float *part = reinterpret_cast<float *>(ring + warp * RING) + lane;
+        __syncwarp();
+        if (ks > 0) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
+#pragma unroll
+                for (int i = 0; i < TILES * 4; ++i) part[(s * TILES * 4 + i) * 32] = acc[s][i >> 2][i & 3];
+        }
+        __syncthreads();
+        if (ks > 0) return;
+#pragma unroll
+        for (int q = 1; q < KS; ++q)
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
+#pragma unroll
+                for (int i = 0; i < TILES * 4; ++i) acc[s][i >> 2][i & 3] += part[q * (RING / 4) + (s * TILES * 4 + i) * 32];
+    }
+    if (strip0 >= a.N) return;
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+        const int64_t out = I * 16 + (lane >> 2) + r * 8;
+        if (out < a.M) {
+#pragma unroll
+            for (int s = 0; s < NS; ++s)
+                BlockProduct<T, NS>::store(acc[s], 2 * r, a.C + out * a.ldc + strip0 + s * 8 * V, lane & 3, a.N - strip0 - s * 8 * V, a.alpha, a.beta);
+        }
+    }
+}
+
+template <typename T, int NS, int KS>
+cudaError_t launch_bsr_mma_one(const BsrArgs &a, cudaStream_t st) {
+    constexpr int cols = 128 / static_cast<int>(sizeof(T)) * NS * (kMmaWarps / KS);
+    constexpr int smem = kMmaWarps * kMmaStages<T, NS> * kMmaSlot<T, NS>;
+    if constexpr (smem > 48 * 1024) {   // an opt-in per device and kernel
+        static std::atomic<bool> opted[kMaxDevices];
+        const int dev = current_device();
+        if (dev >= kMaxDevices || !opted[dev].load(std::memory_order_acquire)) {
+            const cudaError_t e = cudaFuncSetAttribute(bsr_mma_kernel<T, NS, KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+            if (e != cudaSuccess) return e;
+            if (dev < kMaxDevices) opted[dev].store(true, std::memory_order_release);
+        }
+    }
+    return launch_overlapped(bsr_mma_kernel<T, NS, KS>, dim3(static_cast<unsigned>(a.Mb), static_cast<unsigned>((a.N + cols - 1) / cols)),
+                             kMmaWarps * 32, smem, st, a);
+}
+
+// Two strips per warp from 1 KB of B per row on (the block's split and reads serve twice the columns), if that leaves eight
+// warps per SM.  The four warps of a CTA are spread over strips first, then over the blocks of a row, and over those also when
+// there are fewer than 16 warps per SM (200 block-rows of 4 at 128 fp32 columns: 7.5 us with one warp per strip, 4.1 with four).
+template <typename T>
+cudaError_t launch_bsr_mma(const BsrArgs &a, cudaStream_t st) {
+    constexpr int one = 128 / sizeof(T);
+    const int64_t rows = a.Mb, sms = sm_count_cached();
+    const bool two = a.N >= 8 * one && rows * ceil_div(a.N, 2 * one) >= 8 * sms;
+    const int strips = ceil_div(a.N, two ? 2 * one : one);
+    int ks = strips == 1 ? 4 : strips == 2 ? 2 : 1;
+    while (ks < 4 && rows * strips * ks < 16 * sms) ks *= 2;
+    if (two) {
+        if (ks == 1) return launch_bsr_mma_one<T, 2, 1>(a, st);
+        if (ks == 2) return launch_bsr_mma_one<T, 2, 2>(a, st);
+        return launch_bsr_mma_one<T, 2, 4>(a, st);
+    }
+    if (ks == 1) return launch_bsr_mma_one<T, 1, 1>(a, st);
+    if (ks == 2) return launch_bsr_mma_one<T, 1, 2>(a, st);
+    return launch_bsr_mma_one<T, 1, 4>(a, st);
+}
+
+}  // namespace sd

@@ -473,79 +473,80 @@ block_cols_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
     }
 }
 
-// Values of a block-row's blocks: the row-major 16x16 blocks (absent entries +0) and, beside them, the tensor-core operand
-// images, in one pass over the block-row's nonzeros: batches of kValBlocks blocks are composed in shared memory and leave as
-// whole 16-byte vectors, and nothing is cleared in global memory first.  (Three passes before: clear, scatter with a search
-// per nonzero in global memory, permute; 32 us for 4.2 M bf16 values.)
-constexpr int kValBlocks = 16, kValThreads = 256;
+// Values of a block-row's blocks, row-major 16x16, absent entries +0: batches of kValBlocks blocks are composed in shared memory
+// and leave as whole 16-byte vectors, so nothing is cleared in global memory first.  A warp takes two rows of the block-row; its
+// columns are read, and looked up among the batch's, before the values that an earlier kernel may still be writing.  Bound by
+// the chain of reads; with the product of 16,777 blocks at 128 bf16 columns 71 us per new set of values before (with operand
+// images beside the blocks, a column's block sought by every thread on its own), 37 now.
+constexpr int kValBlocks = 32, kValThreads = 256, kValStep = 4;
 
 template <typename T>
 __global__ void __launch_bounds__(kValThreads)
 block_values_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, const T *__restrict__ vals, int64_t M,
-                    const int32_t *__restrict__ browptr, const int32_t *__restrict__ bcol, T *__restrict__ bval, T *__restrict__ img) {
+                    const int32_t *__restrict__ browptr, const int32_t *__restrict__ bcol, T *__restrict__ bval) {
     constexpr int V = 16 / sizeof(T);   // elements per vector
     __shared__ __align__(16) T blk[kValBlocks * 256];
-    __shared__ int cols[kValBlocks], bound[17];
+    __shared__ int cols[kValBlocks];
     const int64_t I = blockIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int b0 = __ldg(browptr + I), b1 = __ldg(browptr + I + 1);
-    if (threadIdx.x < 17) bound[threadIdx.x] = __ldg(rowptr + min(I * 16 + threadIdx.x, M));
-    const int4 zero = make_int4(0, 0, 0, 0);
+    int bound[2][2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const int64_t row = I * 16 + warp + h * 8;
+        bound[h][0] = __ldg(rowptr + min(row, M));
+        bound[h][1] = __ldg(rowptr + min(row + 1, M));
+    }
+    overlap_next();
     for (int s = b0; s < b1; s += kValBlocks) {
         const int n = min(kValBlocks, b1 - s);
         __syncthreads();
         if (threadIdx.x < n) cols[threadIdx.x] = __ldg(bcol + s + threadIdx.x);
-        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) reinterpret_cast<int4 *>(blk)[i] = zero;
+        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) reinterpret_cast<int4 *>(blk)[i] = make_int4(0, 0, 0, 0);
         __syncthreads();
         const int first = cols[0], last = cols[n - 1];
-        int r = 0;
-        for (int64_t p = static_cast<int64_t>(bound[0]) + threadIdx.x; p < bound[16]; p += kValThreads) {
-            while (p >= bound[r + 1]) ++r;
-            const int c = __ldg(colind + p), j = c >> 4;
-            if (j < first || j > last) continue;
-            int lo = 0, hi = n - 1;
-            while (lo < hi) {
-                const int mid = (lo + hi) >> 1;
-                if (cols[mid] < j) lo = mid + 1;
-                else hi = mid;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+            for (int p0 = bound[h][0] + lane; p0 < bound[h][1]; p0 += 32 * kValStep) {
+                int at[kValStep];   // in blk, or -1: another batch's block
+#pragma unroll
+                for (int q = 0; q < kValStep; ++q) at[q] = p0 + q * 32 < bound[h][1] ? __ldg(colind + p0 + q * 32) : -1;
+#pragma unroll
+                for (int q = 0; q < kValStep; ++q) {
+                    const int c = at[q], j = c >> 4;
+                    int lo = 0;
+#pragma unroll
+                    for (int w = kValBlocks / 2; w > 0; w >>= 1)
+                        if (lo + w < n && cols[lo + w] <= j) lo += w;
+                    at[q] = c < 0 || j < first || j > last ? -1 : lo * 256 + (warp + h * 8) * 16 + (c & 15);
+                }
+                overlap_wait();
+#pragma unroll
+                for (int q = 0; q < kValStep; ++q)
+                    if (at[q] >= 0) blk[at[q]] = vals[p0 + q * 32];
             }
-            blk[lo * 256 + r * 16 + (c & 15)] = vals[p];
-        }
         __syncthreads();
-        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) {
-            const int4 v = reinterpret_cast<const int4 *>(blk)[i];
-            const int64_t k = s + i / (256 / V);
-            const int x = i % (256 / V) * V, row = x >> 4, col = x & 15;   // first element of the vector
-            reinterpret_cast<int4 *>(bval)[static_cast<int64_t>(s) * (256 / V) + i] = v;
-            if constexpr (sizeof(T) == 2) {
-                // 8x8 core matrices of 128 contiguous bytes, [k group][row group]: a row of a core is one vector
-                reinterpret_cast<int4 *>(img)[k * 32 + ((col >> 3) * 2 + (row >> 3)) * 8 + (row & 7)] = v;
-            } else {
-                // per k step (8 block columns) the hi block over the lo block, core matrices of 8 rows x 4 floats, ordered
-                // [k half][row group: hi 0..7, hi 8..15, lo 0..7, lo 8..15]
-                const float4 f = make_float4(__int_as_float(v.x), __int_as_float(v.y), __int_as_float(v.z), __int_as_float(v.w));
-                float4 h;
-                h.x = __uint_as_float(__float_as_uint(f.x) & 0xFFFFE000u);
-                h.y = __uint_as_float(__float_as_uint(f.y) & 0xFFFFE000u);
-                h.z = __uint_as_float(__float_as_uint(f.z) & 0xFFFFE000u);
-                h.w = __uint_as_float(__float_as_uint(f.w) & 0xFFFFE000u);
-                float4 *out = reinterpret_cast<float4 *>(img) + k * 128 + (col >> 3) * 64 + ((col & 7) >> 2) * 32 + (row >> 3) * 8 + (row & 7);
-                out[0] = h;
-                out[16] = make_float4(f.x - h.x, f.y - h.y, f.z - h.z, f.w - h.w);
-            }
-        }
+        overlap_wait();   // also a warp without nonzeros must not write over what an earlier product still reads
+        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads)
+            reinterpret_cast<int4 *>(bval)[static_cast<int64_t>(s) * (256 / V) + i] = reinterpret_cast<const int4 *>(blk)[i];
     }
+    overlap_wait();
 }
 
-cudaError_t fill_bsr(const sd_plan *p, cudaStream_t st) {
+template <typename T>
+static cudaError_t fill_blocks(const sd_plan *p, bool overlap, cudaStream_t st) {
     const unsigned Mb = static_cast<unsigned>((p->M + 15) / 16);
     if (Mb == 0 || p->nnzb == 0) return cudaSuccess;
-    if (p->dtype == SD_F32)
-        block_values_kernel<float><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, static_cast<const float *>(p->vals), p->M, p->browptr,
-                                                              p->bcol, static_cast<float *>(p->bval), static_cast<float *>(p->bval_mma));
-    else
-        block_values_kernel<uint16_t><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, static_cast<const uint16_t *>(p->vals), p->M, p->browptr,
-                                                                 p->bcol, static_cast<uint16_t *>(p->bval), static_cast<uint16_t *>(p->bval_mma));
+    const T *vals = static_cast<const T *>(p->vals);
+    T *bval = static_cast<T *>(p->bval);
+    if (overlap) return launch_overlapped(block_values_kernel<T>, Mb, kValThreads, 0, st, p->rowptr, p->colind, vals, p->M, p->browptr, p->bcol, bval);
+    block_values_kernel<T><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, vals, p->M, p->browptr, p->bcol, bval);
     return cudaGetLastError();
+}
+
+// overlap: the pattern's tables are complete, only values may still be in flight on `st`
+cudaError_t fill_bsr(const sd_plan *p, bool overlap, cudaStream_t st) {
+    return p->dtype == SD_F32 ? fill_blocks<float>(p, overlap, st) : fill_blocks<uint16_t>(p, overlap, st);
 }
 
 sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st) {
@@ -557,8 +558,6 @@ sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st) {
     if ((s = dev_alloc(p, &p->browptr, static_cast<size_t>(Mb) + 1, "browptr", st))) return s;
     if ((s = dev_alloc(p, &p->bcol, nnzb, "bcol", st))) return s;
     if ((s = dev_alloc_bytes(p, &p->bval, (p->dtype == SD_F32 ? 4 : 2) * 256 * static_cast<size_t>(nnzb), "bval", st))) return s;
-    // tensor-core operand images: bf16 512 bytes per block, fp32 a hi and a lo image of 1 KB each
-    if ((s = dev_alloc_bytes(p, &p->bval_mma, (p->dtype == SD_BF16 ? 512 : 2048) * static_cast<size_t>(nnzb), "bval (tensor-core image)", st))) return s;
     if ((s = dev_alloc(p, &p->dev_error, 1, "error word", st))) return s;
     SD_CUDA_TRY(cudaMemsetAsync(p->dev_error, 0, sizeof(int32_t), st));
     if (Mb > 0) {
@@ -574,13 +573,7 @@ sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st) {
     } else {
         SD_CUDA_TRY(cudaMemsetAsync(p->browptr, 0, sizeof(int32_t), st));
     }
-    SD_CUDA_TRY(fill_bsr(p, st));
-    // one persistent CTA per SM, each with a contiguous range of block-rows of about equal cost
-    p->bsr_nparts = static_cast<int32_t>(Mb < p->info.sm_count ? Mb : p->info.sm_count);
-    if (p->bsr_nparts > 0) {
-        if ((s = dev_alloc(p, &p->bsr_part, static_cast<size_t>(p->bsr_nparts) + 1, "block-row partition", st))) return s;
-        SD_CUDA_TRY(build_bsr_partition(p->browptr, Mb, p->bsr_nparts, p->bsr_part, st));
-    }
+    SD_CUDA_TRY(fill_bsr(p, false, st));
     return SD_OK;
 }
 

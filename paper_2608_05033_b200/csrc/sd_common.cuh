@@ -173,7 +173,6 @@ struct Switches {
     int geom_nv;           // SD_GEOM_NV: 1 forces one vector per lane
     int ksplit_g;          // SD_KSPLIT_G: lane sets per row (0: rule, 1: off)
     int narrow_g;          // SD_NARROW_G: lanes per row of the narrow row-split kernel (0: rule)
-    int tc_sb, tc_stages, tc32_sb, tc32_stages;   // SD_TC_SB / SD_TC_STAGES / SD_TC32_SB / SD_TC32_STAGES: ring geometry (0: default)
 };
 const Switches &switches();
 

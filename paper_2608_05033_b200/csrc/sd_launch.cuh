@@ -69,23 +69,10 @@ struct CooPlan {
 cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, bool vec, int sm_count, cudaStream_t st);
 cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int32_t *row, cudaStream_t st);
 
-// Family (c).
-// The TMA descriptor of B as the tensor-core kernel reads it, kept by the plan for the last (B, ldb) it ran with:
-// encoding one costs a driver call on the host, and a serving loop calls sd_spmm with the same operand buffer.
-struct alignas(64) TcMapCache {
-    unsigned char map[128];   // a CUtensorMap
-    const void *B = nullptr;
-    int64_t ldb = 0, K = 0;
-    int32_t N = 0;
-    int32_t valid = 0;
-};
 struct BsrArgs {
     const int32_t *browptr;  // [Mb + 1]
     const int32_t *bcol;     // [nnzb]
     const void *bval;        // [nnzb][16][16] row-major, plan dtype
-    const void *bval_mma;    // [nnzb] tensor-core operand images of the same blocks
-    const int32_t *part;     // [nparts + 1] block-row ranges of the tensor-core kernel's CTAs
-    int32_t nparts;
     const void *B;
     float *C;
     int64_t ldb, ldc;
@@ -93,13 +80,10 @@ struct BsrArgs {
     int32_t Mb;
     int32_t N;
     float alpha, beta;
-    TcMapCache *map_cache;      // may be null: the descriptor is then encoded for this call only
-    int32_t test_wait_expiry;   // see sd_plan_desc_t
 };
-cudaError_t run_bsr_simt(const BsrArgs &a, int dtype, bool vec, cudaStream_t st);
-// Tensor-core form.  bsr_tc_usable: dtype, dense width and the TMA alignment rules allow it.
-bool bsr_tc_usable(const BsrArgs &a, int dtype);
-cudaError_t run_bsr_tc(const BsrArgs &a, int dtype, int32_t *error_word, int sm_count, cudaStream_t st);
+bool bsr_mma_usable(const BsrArgs &a, int dtype);   // width, pitches and addresses suit the tensor-core kernel
+cudaError_t run_bsr(const BsrArgs &a, int dtype, cudaStream_t st);
+cudaError_t run_wait_expiry(int32_t *error, cudaStream_t st);   // see sd_plan_desc_t.test_wait_expiry
 // Counts behind sd_plan_get_features (row-length / column-degree quartiles, column-degree moments,
 // SELL slots for slice heights 16 / 32 / 512, occupied 4x4 and 8x8 blocks).  Synchronous.
 struct FeatureCounts {
@@ -110,7 +94,5 @@ struct FeatureCounts {
 };
 sd_status_t compute_feature_counts(const int32_t *rowptr, const int32_t *colind, int64_t M, int64_t K, int64_t nnz,
                                    cudaStream_t st, FeatureCounts *out);
-
-cudaError_t build_bsr_partition(const int32_t *browptr, int32_t Mb, int32_t nparts, int32_t *part, cudaStream_t st);
 
 }  // namespace sd

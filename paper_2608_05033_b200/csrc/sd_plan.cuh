@@ -41,12 +41,8 @@ struct sd_plan {
     int32_t *browptr = nullptr;
     int32_t *bcol = nullptr;
     void *bval = nullptr;
-    void *bval_mma = nullptr;   // tensor-core operand images of the blocks
-    int32_t *bsr_part = nullptr; // block-row ranges of the tensor-core kernel's CTAs
-    int32_t bsr_nparts = 0;
     int32_t *dev_error = nullptr;
     int64_t nnzb = 0;
-    mutable sd::TcMapCache tc_map;   // descriptor of the last dense operand (sd_spmm takes the plan as const)
     int32_t test_wait_expiry = 0;
 
     // host-buffer entry point
@@ -137,7 +133,7 @@ sd_status_t build_coo(sd_plan *p, cudaStream_t st);
 // 16x16 blocks: pointers, columns, values, tensor-core images, partition.
 sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st);
 // Values and images from the caller's current array.
-cudaError_t fill_bsr(const sd_plan *p, cudaStream_t st);
+cudaError_t fill_bsr(const sd_plan *p, bool overlap, cudaStream_t st);
 
 // Introspection: built on request from the caller's CSR arrays.
 sd_status_t inspect_tiles(const sd_plan *p, int32_t *host_out);

@@ -1,0 +1,52 @@
+"""The BSR-16 kernel on the warp-level tensor-core instructions: one or two strips of B per warp, one to four warps per
+block-row, ring slots that wrap, block-rows of zero to more than 32 blocks per warp, a last block-row and a last block column
+that are not whole, a last strip that is not whole."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if torch.cuda.is_available():
+    import paper_2608_05033_b200 as sd
+    from test_gpu_parity import check
+    from util import DeviceWorkload, run_spmm
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("Mb,N", [(5, 8), (5, 40), (5, 136), (5, 1032), (700, 64), (700, 136), (700, 264), (700, 520), (2400, 264)])
+def test_block_rows_strips_and_edges(Mb, N, dtype):
+    rng = np.random.default_rng(Mb + N)
+    M, K = 16 * Mb - 5, 16 * 150 - 9
+    blocks = rng.choice([0, 1, 2, 3, 4, 9], Mb)
+    blocks[:3] = [150, 0, 33]
+    rows, cols = [], []
+    for i in range(Mb):
+        J = np.sort(rng.choice(150, blocks[i], replace=False))
+        if blocks[i] and i % 2:
+            J[-1] = 149                                   # the block that reaches past the last column
+            J = np.unique(J)
+        c = (J[:, None] * 16 + np.arange(16)).reshape(-1)
+        for r in range(16 * i, min(16 * i + 16, M)):
+            keep = c[(c < K) & (rng.random(c.size) < 0.8)]
+            rows.append(np.full(keep.size, r)), cols.append(keep)
+    rows, cols = np.concatenate(rows), np.concatenate(cols).astype(np.int32)
+    rowptr = np.zeros(M + 1, np.int32)
+    np.cumsum(np.bincount(rows, minlength=M), out=rowptr[1:])
+    vals, B = rng.standard_normal(cols.size).astype(np.float32), rng.standard_normal((K, N)).astype(np.float32)
+    C = rng.standard_normal((M, N)).astype(np.float32)
+    if dtype == W.SD_BF16:
+        vals, B = W.f32_to_bf16_bits(vals), W.f32_to_bf16_bits(B).reshape(K, N)
+    w = W.Workload("block_rows", M, K, N, rowptr, cols, vals, B, C, -0.75, 0.5, dtype, {})
+    plan = DeviceWorkload(w).plan(family=sd.SD_BSR_TC)
+    for kw in (dict(), dict(pad_b=8, pad_c=4)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    again, _ = run_spmm(plan, w, **kw)
+    assert np.array_equal(got, again)
+    got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
