@@ -170,9 +170,9 @@ sd_status_t sd_spmm(const sd_plan_t *plan, const void *B, int64_t ldb, float *C,
  *   vals   device [nnz], dtype of the plan, in the order of the colind array given at creation;
  *          borrowed from now on in place of the previous array (which may be freed once the
  *          work queued on `stream` has run)
- * Row-split and row-ordered merge plans only swap the pointer; window-major plans refresh
- * their re-bucketed copy, block plans refill the 16x16 blocks and the tensor-core images, both
- * with kernels on `stream`: order the call before the next sd_spmm (same stream, or an event).
+ * Most plans only swap the pointer; plans that run as 16x16 blocks (SD_BSR_TC, and automatic
+ * SD_ROWSPLIT plans of matrices made of such blocks) refill the blocks with a kernel on
+ * `stream`: order the call before the next sd_spmm (same stream, or an event).
  * The family, the windows and every structural decision stay as they are. */
 sd_status_t sd_plan_update_values(sd_plan_t *plan, const void *vals, void *stream);
 

@@ -86,6 +86,20 @@ static int decide_family(const sd_plan_info_t &s, int dtype) {
     return skew ? SD_MERGE : SD_ROWSPLIT;
 }
 
+// Row-split plans the library chose itself run as blocks wherever those are ahead on the GPU, whatever the family rule says of
+// the width.  The block kernel's time goes by blocks, the row kernels' by nonzeros; measured with forced plans (4,400 and 33,554
+// blocks thinned to fills of 1, 1/2, 1/4 and 1/6), row kernel / block kernel at the largest rho taken and at the next:
+//     fp32   8 columns  rho 2: 1.0 to 1.3   4: 0.7 to 0.9        bf16   8 columns  rho 2: 1.1 to 1.6   4: 0.7 to 1.1
+//            16         rho 2: 1.4 (3 lies between)  4: 0.9             16         rho 4: 0.9 to 1.2 (3 taken)
+//            24 to 128  rho 4: 1.2 to 1.5   6: 0.9 to 1.2               24, 32     rho 4: 1.2 to 2.1   6: 0.9 to 1.5
+//            256        rho 5: 1.4          8: 1.1                      48 to 128  rho 6: 1.3 to 2.3
+static bool decide_blocks(const sd_plan_info_t &s, int dtype) {
+    const int64_t piece = dtype == SD_BF16 ? 8 : 4;
+    if (s.N < 8 || s.N % piece != 0 || s.unsorted_rows != 0 || s.nnz == 0) return false;
+    const int64_t rho = s.N < 16 ? 2 : s.N < 24 ? 3 : dtype == SD_BF16 && s.N < 48 ? 4 : 6;
+    return 256 * s.nnzb16 <= rho * s.nnz;
+}
+
 // Number of column windows: none unless the rows are short on average (nnz < 16 M, so the
 // extra read-modify-write of C per (row, window) pair stays below the gather traffic saved),
 // the columns are sorted, and B does not fit in 60 % of L2; then the smallest power of two
@@ -272,7 +286,7 @@ static sd_status_t create_plan(const sd_plan_desc_t *d, sd_plan *p) {
         } else if ((s = build_schedule(p, W, p->nnz < kSmallPlan ? kChunkNnz + 1 : kHybridHeavy, h, st))) {
             return s;
         }
-    } else if (family == SD_BSR_TC) {
+    } else if (family == SD_BSR_TC || (family == SD_ROWSPLIT && d->family == SD_AUTO && decide_blocks(info, p->dtype))) {
         if ((s = build_bsr(p, info.nnzb16, st))) return s;
     } else if (family == SD_HYBRID && some) {
         const int W = std::max(1, d->windows == 0 ? decide_windows(info, p->dtype) : d->windows);
@@ -348,7 +362,7 @@ static sd_status_t pattern_hash(const int32_t *rowptr, const int32_t *colind, in
 }
 
 constexpr uint64_t kBlobMagic = 0x31304E414C504453ull;   // "SDPLAN01"
-constexpr uint32_t kBlobVersion = 5;
+constexpr uint32_t kBlobVersion = 6;
 
 // What a plan was made for and what was decided; the representation is built again from the caller's arrays when the blob is
 // loaded (no scan, no decision), which takes less time than copying it from the host.
@@ -359,12 +373,30 @@ struct BlobHeader {
     int64_t M, K, N, nnz;
     int32_t dtype, family;
     char device_name[128];      // the plan was tuned on this GPU model (window count, thresholds)
-    int32_t sm_count, has_coo;
+    int32_t sm_count, has_coo, has_blocks;
     int64_t l2_bytes;
     sd_plan_info_t info;
     int32_t h_T, reserved;
     unsigned long long chunks_long, chunks_long2, chunks_long4, giants, len_hist[256];   // the scan's counts that the schedule is built from
 };
+
+static BsrArgs block_args(const sd_plan *plan, const SpmmArgs &a) {
+    BsrArgs b;
+    b.browptr = plan->browptr;
+    b.bcol = plan->bcol;
+    b.bval = plan->bval;
+    b.B = a.B;
+    b.C = a.C;
+    b.ldb = a.ldb;
+    b.ldc = a.ldc;
+    b.M = plan->M;
+    b.K = plan->K;
+    b.Mb = static_cast<int32_t>((plan->M + 15) / 16);
+    b.N = a.N;
+    b.alpha = a.alpha;
+    b.beta = a.beta;
+    return b;
+}
 
 // The product on N columns of B and C: all of the plan's, or a slice of them.
 static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, int64_t ldb, float *C, int64_t ldc, float alpha,
@@ -409,6 +441,10 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
 
     switch (plan->info.family) {
     case SD_ROWSPLIT:
+        if (plan->bval && bsr_mma_usable(block_args(plan, a), plan->dtype)) {
+            SD_CUDA_TRY(run_bsr(block_args(plan, a), plan->dtype, st));
+            return SD_OK;
+        }
         SD_CUDA_TRY(run_rowsplit(a, plan->dtype, piece_width(plan->dtype, N, B, ldb, C, ldc), st));
         return SD_OK;
     case SD_MERGE: {
@@ -461,25 +497,10 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
         }
         return SD_OK;
     }
-    case SD_BSR_TC: {
-        BsrArgs b;
-        b.browptr = plan->browptr;
-        b.bcol = plan->bcol;
-        b.bval = plan->bval;
-        b.B = B;
-        b.C = C;
-        b.ldb = ldb;
-        b.ldc = ldc;
-        b.M = M;
-        b.K = plan->K;
-        b.Mb = static_cast<int32_t>((M + 15) / 16);
-        b.N = static_cast<int32_t>(N);
-        b.alpha = alpha;
-        b.beta = beta;
-        SD_CUDA_TRY(run_bsr(b, plan->dtype, st));
+    case SD_BSR_TC:
+        SD_CUDA_TRY(run_bsr(block_args(plan, a), plan->dtype, st));
         if (plan->test_wait_expiry) SD_CUDA_TRY(run_wait_expiry(plan->dev_error, st));
         return SD_OK;
-    }
     default:
         set_error(SD_ERR_INTERNAL, "plan has no family");
         return SD_ERR_INTERNAL;
@@ -809,7 +830,7 @@ sd_status_t sd_plan_update_values(sd_plan_t *plan, const void *vals, void *strea
         return SD_ERR_INVALID_ARG;
     }
     plan->vals = vals;
-    if (plan->info.family == SD_BSR_TC) SD_CUDA_TRY(fill_bsr(plan, true, static_cast<cudaStream_t>(stream)));
+    if (plan->bval) SD_CUDA_TRY(fill_bsr(plan, true, static_cast<cudaStream_t>(stream)));
     return SD_OK;   // the other families read the caller's array
 }
 
@@ -916,6 +937,7 @@ sd_status_t sd_plan_save(const sd_plan_t *plan, void *buf, size_t cap, size_t *b
     h.l2_bytes = plan->info.l2_bytes;
     h.info = plan->info;
     h.has_coo = plan->coo_row ? 1 : 0;
+    h.has_blocks = plan->browptr ? 1 : 0;
     h.h_T = plan->h_T;
     h.chunks_long = plan->h_counts.chunks_long;
     h.chunks_long2 = plan->h_counts.chunks_long2;
@@ -998,7 +1020,7 @@ sd_status_t sd_plan_load(const void *blob, size_t bytes, const int32_t *rowptr, 
         counts.giants = h.giants;
         memcpy(counts.len_hist, h.len_hist, sizeof h.len_hist);
         if ((s = build_schedule(p, h.info.windows, h.h_T, counts, nullptr))) return fail(s);
-    } else if (h.info.family == SD_BSR_TC) {
+    } else if (h.has_blocks) {
         if ((s = build_bsr(p, h.info.nnzb16, nullptr))) return fail(s);
     }
     const cudaError_t e = cudaDeviceSynchronize();

@@ -473,74 +473,78 @@ block_cols_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
     }
 }
 
-// Values of a block-row's blocks, row-major 16x16, absent entries +0: batches of kValBlocks blocks are composed in shared memory
-// and leave as whole 16-byte vectors, so nothing is cleared in global memory first.  A warp takes two rows of the block-row; its
-// columns are read, and looked up among the batch's, before the values that an earlier kernel may still be writing.  Bound by
-// the chain of reads; with the product of 16,777 blocks at 128 bf16 columns 71 us per new set of values before (with operand
-// images beside the blocks, a column's block sought by every thread on its own), 37 now.
-constexpr int kValBlocks = 32, kValThreads = 256, kValStep = 4;
+// Where the values of a block's rows come from: of each row of 16 the first of its nonzeros in the caller's order and a mask of
+// the columns that are there.  The first nonzero of a block in its row writes both (the masks are cleared before).
+static __global__ void __launch_bounds__(256)
+block_rows_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, int64_t M, const int32_t *__restrict__ browptr,
+                  const int32_t *__restrict__ bcol, int32_t *__restrict__ first, uint16_t *__restrict__ mask) {
+    const int64_t I = blockIdx.x;
+    const int b0 = __ldg(browptr + I), b1 = __ldg(browptr + I + 1);
+    for (int r = threadIdx.x >> 5; r < 16 && I * 16 + r < M; r += 8) {
+        const int p1 = __ldg(rowptr + I * 16 + r + 1), p0 = __ldg(rowptr + I * 16 + r);
+        for (int p = p0 + (threadIdx.x & 31); p < p1; p += 32) {
+            const int j = __ldg(colind + p) >> 4;
+            if (p > p0 && __ldg(colind + p - 1) >> 4 == j) continue;
+            int lo = b0, hi = b1 - 1;
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if (__ldg(bcol + mid) < j) lo = mid + 1;
+                else hi = mid;
+            }
+            uint32_t m = 0;
+            for (int q = p; q < p1; ++q) {
+                const int c = __ldg(colind + q);
+                if (c >> 4 != j) break;
+                m |= 1u << (c & 15);
+            }
+            first[static_cast<int64_t>(lo) * 16 + r] = p;
+            mask[static_cast<int64_t>(lo) * 16 + r] = static_cast<uint16_t>(m);
+        }
+    }
+}
+
+// Values of the blocks, row-major 16x16, absent entries +0: a thread gathers one 16-byte vector of a block row.  Bound by memory:
+// each value is read and written once.  16,777 full bf16 blocks with a product at 128 columns: 71 us per new set of values with a
+// search of every nonzero's block and separate operand images, 37 with a search in shared memory, 24 with these tables.
+constexpr int kValThreads = 256;
 
 template <typename T>
 __global__ void __launch_bounds__(kValThreads)
-block_values_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, const T *__restrict__ vals, int64_t M,
-                    const int32_t *__restrict__ browptr, const int32_t *__restrict__ bcol, T *__restrict__ bval) {
-    constexpr int V = 16 / sizeof(T);   // elements per vector
-    __shared__ __align__(16) T blk[kValBlocks * 256];
-    __shared__ int cols[kValBlocks];
-    const int64_t I = blockIdx.x;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int b0 = __ldg(browptr + I), b1 = __ldg(browptr + I + 1);
-    int bound[2][2];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        const int64_t row = I * 16 + warp + h * 8;
-        bound[h][0] = __ldg(rowptr + min(row, M));
-        bound[h][1] = __ldg(rowptr + min(row + 1, M));
+block_values_kernel(const T *__restrict__ vals, const int32_t *__restrict__ first, const uint16_t *__restrict__ mask, int64_t vectors,
+                    int4 *__restrict__ bval) {
+    constexpr int V = 16 / sizeof(T), PER_ROW = 16 / V;
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * kValThreads + threadIdx.x;
+    uint32_t m = 0;
+    int p = 0;
+    if (i < vectors) {
+        const int at = static_cast<int>(i % PER_ROW) * V;
+        const uint32_t whole = __ldg(mask + i / PER_ROW);
+        p = __ldg(first + i / PER_ROW) + __popc(whole & ((1u << at) - 1u));
+        m = whole >> at;
     }
     overlap_next();
-    for (int s = b0; s < b1; s += kValBlocks) {
-        const int n = min(kValBlocks, b1 - s);
-        __syncthreads();
-        if (threadIdx.x < n) cols[threadIdx.x] = __ldg(bcol + s + threadIdx.x);
-        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads) reinterpret_cast<int4 *>(blk)[i] = make_int4(0, 0, 0, 0);
-        __syncthreads();
-        const int first = cols[0], last = cols[n - 1];
-#pragma unroll
-        for (int h = 0; h < 2; ++h)
-            for (int p0 = bound[h][0] + lane; p0 < bound[h][1]; p0 += 32 * kValStep) {
-                int at[kValStep];   // in blk, or -1: another batch's block
-#pragma unroll
-                for (int q = 0; q < kValStep; ++q) at[q] = p0 + q * 32 < bound[h][1] ? __ldg(colind + p0 + q * 32) : -1;
-#pragma unroll
-                for (int q = 0; q < kValStep; ++q) {
-                    const int c = at[q], j = c >> 4;
-                    int lo = 0;
-#pragma unroll
-                    for (int w = kValBlocks / 2; w > 0; w >>= 1)
-                        if (lo + w < n && cols[lo + w] <= j) lo += w;
-                    at[q] = c < 0 || j < first || j > last ? -1 : lo * 256 + (warp + h * 8) * 16 + (c & 15);
-                }
-                overlap_wait();
-#pragma unroll
-                for (int q = 0; q < kValStep; ++q)
-                    if (at[q] >= 0) blk[at[q]] = vals[p0 + q * 32];
-            }
-        __syncthreads();
-        overlap_wait();   // also a warp without nonzeros must not write over what an earlier product still reads
-        for (int i = threadIdx.x; i < n * 256 / V; i += kValThreads)
-            reinterpret_cast<int4 *>(bval)[static_cast<int64_t>(s) * (256 / V) + i] = reinterpret_cast<const int4 *>(blk)[i];
-    }
     overlap_wait();
+    if (i >= vectors) return;
+    union {
+        T v[V];
+        int4 all;
+    } out;
+    out.all = make_int4(0, 0, 0, 0);
+#pragma unroll
+    for (int e = 0; e < V; ++e)
+        if (m >> e & 1) out.v[e] = vals[p + __popc(m & ((1u << e) - 1u))];
+    bval[i] = out.all;
 }
 
 template <typename T>
 static cudaError_t fill_blocks(const sd_plan *p, bool overlap, cudaStream_t st) {
-    const unsigned Mb = static_cast<unsigned>((p->M + 15) / 16);
-    if (Mb == 0 || p->nnzb == 0) return cudaSuccess;
+    const int64_t vectors = p->nnzb * (256 * static_cast<int64_t>(sizeof(T)) / 16);
+    if (vectors == 0) return cudaSuccess;
+    const unsigned grid = static_cast<unsigned>((vectors + kValThreads - 1) / kValThreads);
     const T *vals = static_cast<const T *>(p->vals);
-    T *bval = static_cast<T *>(p->bval);
-    if (overlap) return launch_overlapped(block_values_kernel<T>, Mb, kValThreads, 0, st, p->rowptr, p->colind, vals, p->M, p->browptr, p->bcol, bval);
-    block_values_kernel<T><<<Mb, kValThreads, 0, st>>>(p->rowptr, p->colind, vals, p->M, p->browptr, p->bcol, bval);
+    int4 *bval = static_cast<int4 *>(p->bval);
+    if (overlap) return launch_overlapped(block_values_kernel<T>, grid, kValThreads, 0, st, vals, p->brow_first, p->brow_mask, vectors, bval);
+    block_values_kernel<T><<<grid, kValThreads, 0, st>>>(vals, p->brow_first, p->brow_mask, vectors, bval);
     return cudaGetLastError();
 }
 
@@ -572,6 +576,15 @@ sd_status_t build_bsr(sd_plan *p, int64_t nnzb, cudaStream_t st) {
         SD_CUDA_TRY(cudaGetLastError());
     } else {
         SD_CUDA_TRY(cudaMemsetAsync(p->browptr, 0, sizeof(int32_t), st));
+    }
+    const size_t block_rows = 16 * static_cast<size_t>(nnzb);
+    if ((s = dev_alloc(p, &p->brow_first, block_rows, "first nonzeros of block rows", st))) return s;
+    if ((s = dev_alloc(p, &p->brow_mask, block_rows, "columns of block rows", st))) return s;
+    if (nnzb > 0) {
+        SD_CUDA_TRY(cudaMemsetAsync(p->brow_first, 0, sizeof(int32_t) * block_rows, st));
+        SD_CUDA_TRY(cudaMemsetAsync(p->brow_mask, 0, sizeof(uint16_t) * block_rows, st));
+        block_rows_kernel<<<Mb, 256, 0, st>>>(p->rowptr, p->colind, p->M, p->browptr, p->bcol, p->brow_first, p->brow_mask);
+        SD_CUDA_TRY(cudaGetLastError());
     }
     SD_CUDA_TRY(fill_bsr(p, false, st));
     return SD_OK;

@@ -41,6 +41,8 @@ struct sd_plan {
     int32_t *browptr = nullptr;
     int32_t *bcol = nullptr;
     void *bval = nullptr;
+    int32_t *brow_first = nullptr;    // [16 nnzb] first nonzero of every row of a block
+    uint16_t *brow_mask = nullptr;    // [16 nnzb] its columns
     int32_t *dev_error = nullptr;
     int64_t nnzb = 0;
     int32_t test_wait_expiry = 0;

@@ -50,3 +50,27 @@ def test_block_rows_strips_and_edges(Mb, N, dtype):
     got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
     check(w, got, beta=0.0)
     plan.close()
+
+
+@pytest.mark.parametrize("dtype,N", [(W.SD_F32, 8), (W.SD_F32, 20), (W.SD_F32, 48), (W.SD_BF16, 16), (W.SD_BF16, 40)])
+def test_automatic_row_split_plan_of_blocks(dtype, N):
+    """Below the width of the block family an automatic plan of a blocked matrix stays a row-split plan and runs as blocks:
+    new values reach them, unaligned operands and other widths take the row kernels, a loaded plan does the same."""
+    w = W.g4_block(Mb=90, Kb=70, N=N, nblocks=500, dtype=dtype)
+    dw = DeviceWorkload(w)
+    plan = dw.plan()
+    assert plan.info().family == sd.SD_ROWSPLIT
+    for kw in (dict(), dict(pad_b=8, pad_c=4), dict(pad_b=1, pad_c=1), dict(offset=1)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    want, _ = run_spmm(plan, w)
+    loaded = sd.Plan.load(plan.save(), dw.rowptr, dw.colind, dw.vals)
+    assert np.array_equal(run_spmm(loaded, w)[0], want)
+    new = np.random.default_rng(N).standard_normal(w.nnz).astype(np.float32)
+    w.vals = W.f32_to_bf16_bits(new) if dtype == W.SD_BF16 else new
+    vals = torch.from_numpy(w.vals.view(np.int16) if dtype == W.SD_BF16 else w.vals).cuda()
+    for p in (plan, loaded):
+        p.update_values(vals)
+        check(w, run_spmm(p, w)[0])
+        p.close()
