@@ -460,6 +460,9 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
             cp.c1_val = plan->coo_c1_val;
             cp.c2_row = plan->coo_c2_row;
             cp.c2_val = plan->coo_c2_val;
+            cp.hot_colind = plan->coo_hot_colind;
+            cp.hot_cols = plan->coo_hot_cols;
+            cp.hot = plan->coo_hot;
             const bool bvec = aligned16(B) && (ldb * (plan->dtype == SD_F32 ? 4 : 2)) % 16 == 0;
             SD_CUDA_TRY(run_coo(cp, a, plan->dtype, bvec, plan->info.sm_count, st));
             return SD_OK;

@@ -415,6 +415,113 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
 // =====================================================================================
 // narrow dense operands
 // =====================================================================================
+// The columns that are worth a place in shared memory: the most frequent ones, as many as fit, in ascending order.
+constexpr int kDegreeBins = 1 << 16;
+
+__global__ void column_degrees_kernel(const int32_t *__restrict__ colind, int64_t nnz, int32_t *__restrict__ degree) {
+    for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < nnz; k += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        atomicAdd(degree + __ldg(colind + k), 1);
+}
+__global__ void degree_bins_kernel(const int32_t *__restrict__ degree, int64_t K, int32_t *__restrict__ bins) {
+    const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j < K) atomicAdd(bins + min(degree[j], kDegreeBins - 1), 1);
+}
+// The smallest degree that at most `most` columns reach; one CTA, the last bin first.
+__global__ void __launch_bounds__(1024)
+degree_threshold_kernel(const int32_t *__restrict__ bins, int64_t most, int32_t *__restrict__ threshold) {
+    constexpr int PER = kDegreeBins / 1024;
+    __shared__ long long above[1024];
+    const int t = threadIdx.x, top = kDegreeBins - 1 - t * PER;
+    long long sum = 0;
+    for (int i = 0; i < PER; ++i) sum += bins[top - i];
+    above[t] = sum;
+    __syncthreads();
+    if (t == 0) {
+        long long run = 0;
+        for (int i = 0; i < 1024; ++i) {
+            const long long v = above[i];
+            above[i] = run;
+            run += v;
+        }
+    }
+    __syncthreads();
+    long long run = above[t];
+    for (int i = 0; i < PER; ++i) {
+        const long long with = run + bins[top - i];
+        if (run <= most && with > most) *threshold = top - i + 1;
+        run = with;
+    }
+    if (t == 1023 && run <= most) *threshold = 0;
+}
+__global__ void hot_flags_kernel(const int32_t *__restrict__ degree, int64_t K, const int32_t *__restrict__ threshold, int32_t *__restrict__ flag,
+                                 unsigned long long *__restrict__ covered) {
+    const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const int deg = j < K ? degree[j] : 0;
+    const bool hot = j < K && deg > 0 && deg >= *threshold;
+    if (j <= K) flag[j] = hot;
+    const unsigned mine = hot ? static_cast<unsigned>(deg) : 0u, sum = __reduce_add_sync(0xffffffffu, mine);
+    if ((threadIdx.x & 31) == 0 && sum) atomicAdd(covered, static_cast<unsigned long long>(sum));
+}
+// degree becomes the new name of the column: its slot with bit 31 set, or itself
+__global__ void hot_names_kernel(int32_t *__restrict__ degree, int64_t K, const int32_t *__restrict__ slot, int32_t *__restrict__ hot_cols) {
+    const int64_t j = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (j >= K) return;
+    const int s = slot[j];
+    const bool hot = slot[j + 1] != s;
+    if (hot) hot_cols[s] = static_cast<int32_t>(j);
+    degree[j] = hot ? s | static_cast<int32_t>(0x80000000u) : static_cast<int32_t>(j);
+}
+__global__ void rename_columns_kernel(const int32_t *__restrict__ colind, int64_t nnz, const int32_t *__restrict__ name, int32_t *__restrict__ out) {
+    for (int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; k < nnz; k += static_cast<int64_t>(gridDim.x) * blockDim.x)
+        out[k] = __ldg(name + __ldg(colind + k));
+}
+
+// Taken from two columns on, where 4,096 columns pay for being fetched by every SM (a cycle each; at most nnz / 600 of them) and
+// if they cover a quarter of the nonzeros.  R-MAT with 32.4 M nonzeros: two fp32 columns 209 -> 173 us, two bf16 197 -> 163, four
+// 362 -> 270; with 3.4 M, two fp32 columns 30 -> 28.  One column gains nothing (the shuffles of the segmented scan take the same
+// unit as the gathers), four fp32 columns, one 16-byte gather, only on the largest (254 -> 242; with 3.4 M 33 -> 38).
+static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
+    const int64_t row_bytes = p->N * (p->dtype == SD_F32 ? 4 : 2);
+    const int64_t most = std::min<int64_t>({kCooHotBytes / row_bytes, p->nnz / 600, p->K});
+    if (p->N < 2 || most < 4096 || (row_bytes == 16 && p->nnz < 16000000)) return SD_OK;
+    sd_status_t s;
+    TempBuf degree(st), bins(st), flag(st), scratch(st), small(st);
+    const int64_t K = p->K;
+    if ((s = degree.get(sizeof(int32_t) * K, "column degrees"))) return s;
+    if ((s = bins.get(sizeof(int32_t) * kDegreeBins, "degree histogram"))) return s;
+    if ((s = flag.get(sizeof(int32_t) * (K + 1), "frequent columns"))) return s;
+    if ((s = small.get(16, "degree threshold"))) return s;
+    int32_t *threshold = small.as<int32_t>() + 2;
+    unsigned long long *covered = small.as<unsigned long long>();
+    SD_CUDA_TRY(cudaMemsetAsync(degree.p, 0, sizeof(int32_t) * K, st));
+    SD_CUDA_TRY(cudaMemsetAsync(bins.p, 0, sizeof(int32_t) * kDegreeBins, st));
+    SD_CUDA_TRY(cudaMemsetAsync(small.p, 0, 16, st));
+    const unsigned wide = static_cast<unsigned>(std::min<int64_t>((p->nnz + 255) / 256, p->info.sm_count * 32));
+    const unsigned cols = static_cast<unsigned>((K + 256) / 256);   // one thread more than columns at least
+    column_degrees_kernel<<<wide, 256, 0, st>>>(p->colind, p->nnz, degree.as<int32_t>());
+    degree_bins_kernel<<<cols, 256, 0, st>>>(degree.as<int32_t>(), K, bins.as<int32_t>());
+    degree_threshold_kernel<<<1, 1024, 0, st>>>(bins.as<int32_t>(), most, threshold);
+    hot_flags_kernel<<<cols, 256, 0, st>>>(degree.as<int32_t>(), K, threshold, flag.as<int32_t>(), covered);
+    SD_CUDA_TRY(cudaGetLastError());
+    size_t tb = 0;
+    SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(nullptr, tb, flag.as<int32_t>(), flag.as<int32_t>(), K + 1, st));
+    if ((s = scratch.get(tb, "scan scratch"))) return s;
+    SD_CUDA_TRY(cub::DeviceScan::ExclusiveSum(scratch.p, tb, flag.as<int32_t>(), flag.as<int32_t>(), K + 1, st));
+    int32_t hot = 0;
+    unsigned long long sum = 0;
+    SD_CUDA_TRY(cudaMemcpyAsync(&hot, flag.as<int32_t>() + K, sizeof hot, cudaMemcpyDeviceToHost, st));
+    SD_CUDA_TRY(cudaMemcpyAsync(&sum, covered, sizeof sum, cudaMemcpyDeviceToHost, st));
+    SD_CUDA_TRY(cudaStreamSynchronize(st));
+    if (hot < 1 || hot > most || 4 * static_cast<int64_t>(sum) < p->nnz) return SD_OK;
+    if ((s = dev_alloc(p, &p->coo_hot_cols, hot, "frequent columns", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_hot_colind, p->nnz, "renamed columns", st))) return s;
+    hot_names_kernel<<<cols, 256, 0, st>>>(degree.as<int32_t>(), K, flag.as<int32_t>(), p->coo_hot_cols);
+    rename_columns_kernel<<<wide, 256, 0, st>>>(p->colind, p->nnz, degree.as<int32_t>(), p->coo_hot_colind);
+    SD_CUDA_TRY(cudaGetLastError());
+    p->coo_hot = hot;
+    return SD_OK;
+}
+
 sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
     sd_status_t s;
     const int cchunk = coo_chunk(static_cast<int>(p->N));
@@ -427,7 +534,7 @@ sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
     if ((s = dev_alloc(p, &p->coo_c2_val, count3 * p->N, "carry sums (level 2)", st))) return s;
     SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, p->coo_row, st));
     p->info.launches = 2 + (count2 > kCooDirectFinal);
-    return SD_OK;
+    return coo_hot_columns(p, st);
 }
 
 // =====================================================================================

@@ -18,12 +18,19 @@
 // Rows without nonzeros are found from the row pointers by the first level and get beta * C.
 // Every row is written by exactly one thread and every sum has a fixed order: results are
 // reproducible bit for bit, no float atomics.
+//
+// What bounds it: the L1 data path, which the gathers (up to 32 tag cycles for 32 unrelated rows of B) and the shuffles of the
+// scan share: 85 % busy at one column (a scale-20 R-MAT matrix 120 us).  At two to four columns, where a few columns hold a large
+// part of the nonzeros, the HOT form keeps their rows of B in shared memory (one CTA per SM), where 32 unrelated words cost
+// about three cycles; the plan owns a copy of the columns with those renamed to slots (coo_hot_columns).
 #pragma once
 
 #include "sd_common.cuh"
 #include "sd_launch.cuh"
 
 namespace sd {
+
+constexpr int kCooHotThreads = 1024;
 
 struct CooArgs {
     const int32_t *row;      // [count] row of every item (ascending)
@@ -39,6 +46,8 @@ struct CooArgs {
     int64_t M;
     int32_t *carry_row;      // [2 * chunks] out
     float *carry_val;        // [2 * chunks][N] out
+    const int32_t *hot_cols; // HOT: ascending columns whose rows of B the kernel keeps; colind names slot i of them as i | bit 31
+    int32_t hot;
 };
 
 // N floats of row `col` of B, widened.  VEC: 16-byte loads are allowed (fp32, N = 4).
@@ -66,9 +75,21 @@ __device__ __forceinline__ void coo_gather(const void *B, int col, uint32_t ldb_
 }
 
 // LEVEL2: the items are carry entries (row, N partial sums); otherwise nonzeros of A.
-template <typename T, int N, bool VEC, bool LEVEL2>
-__global__ void __launch_bounds__(256)
+template <typename T, int N, bool VEC, bool LEVEL2, bool HOT = false>
+__global__ void __launch_bounds__(HOT ? kCooHotThreads : 256)
 coo_reduce_kernel(const CooArgs a) {
+    extern __shared__ __align__(16) char coo_hot_raw[];
+    overlap_next();
+    overlap_wait();
+    if constexpr (HOT) {
+        T *kept = reinterpret_cast<T *>(coo_hot_raw);
+        for (int i = threadIdx.x; i < a.hot; i += kCooHotThreads) {
+            const T *p = b_row(static_cast<const T *>(a.B), __ldg(a.hot_cols + i), a.ldb_bytes);
+#pragma unroll
+            for (int e = 0; e < N; ++e) kept[i * N + e] = p[e];
+        }
+        __syncthreads();
+    }
     constexpr unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
     const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -118,7 +139,17 @@ coo_reduce_kernel(const CooArgs a) {
                 av[u] = ok ? to_float(vals[k]) : 0.f;
             }
 #pragma unroll
-            for (int u = 0; u < kCooU; ++u) coo_gather<T, N, VEC>(a.B, col[u], a.ldb_bytes, p[u]);
+            for (int u = 0; u < kCooU; ++u) {
+                if constexpr (HOT) {   // every lane reads a slot (the others slot 0), those outside also their row of B
+                    const bool kept = col[u] < 0;
+                    const T *q = reinterpret_cast<const T *>(coo_hot_raw) + (kept ? col[u] & 0x7fffffff : 0) * N;
+#pragma unroll
+                    for (int e = 0; e < N; ++e) p[u][e] = to_float(q[e]);
+                    if (!kept) coo_gather<T, N, VEC>(a.B, col[u], a.ldb_bytes, p[u]);
+                    continue;
+                }
+                coo_gather<T, N, VEC>(a.B, col[u], a.ldb_bytes, p[u]);
+            }
 #pragma unroll
             for (int u = 0; u < kCooU; ++u)
 #pragma unroll
@@ -212,6 +243,8 @@ template <int N>
 __global__ void coo_final_kernel(const int32_t *__restrict__ row, const float *__restrict__ val, int64_t count, float *C,
                                  int64_t ldc, float alpha, float beta) {
     const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    overlap_next();
+    overlap_wait();
     if (i >= count) return;
     const int r = row[i];
     if (i > 0 && row[i - 1] == r) return;

@@ -65,7 +65,11 @@ struct CooPlan {
     float *c1_val;        // ... x N
     int32_t *c2_row;      // [2 * ceil(len(c1) / kCooCarryChunk)] second-level carries
     float *c2_val;
+    const int32_t *hot_colind;   // [nnz] columns, those of hot_cols renamed (hot == 0: none)
+    const int32_t *hot_cols;
+    int32_t hot;
 };
+constexpr int kCooHotBytes = 128 * 1024;   // the rest is L1 for the gathers outside: with 200 KB two fp32 columns took 281 us instead of 173
 cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, bool vec, int sm_count, cudaStream_t st);
 cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int32_t *row, cudaStream_t st);
 

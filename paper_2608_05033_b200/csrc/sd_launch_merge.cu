@@ -39,7 +39,7 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, bool vec, 
         const int64_t cap = static_cast<int64_t>(sm_count) * occ;
         return static_cast<unsigned>(want < cap ? (want > 0 ? want : 1) : cap);
     };
-    CooArgs a;
+    CooArgs a{};
     a.row = cp.row;
     a.colind = s.colind;
     a.vals = s.vals;
@@ -54,9 +54,23 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, bool vec, 
     a.M = cp.M;
     a.carry_row = cp.c1_row;
     a.carry_val = cp.c1_val;
-    if (vec) coo_reduce_kernel<T, N, true, false><<<grid_for(chunks1), 256, 0, st>>>(a);
-    else coo_reduce_kernel<T, N, false, false><<<grid_for(chunks1), 256, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    cudaError_t e;
+    const int kept = cp.hot * N * static_cast<int>(sizeof(T));
+    if (cp.hot > 0 && kept <= kCooHotBytes) {
+        auto kernel = vec ? coo_reduce_kernel<T, N, true, false, true> : coo_reduce_kernel<T, N, false, false, true>;
+        static std::atomic<bool> opted[kMaxDevices][2];
+        const int dev = current_device();
+        if (dev >= kMaxDevices || !opted[dev][vec].load(std::memory_order_acquire)) {
+            if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCooHotBytes)) != cudaSuccess) return e;
+            if (dev < kMaxDevices) opted[dev][vec].store(true, std::memory_order_release);
+        }
+        a.colind = cp.hot_colind;
+        a.hot_cols = cp.hot_cols;
+        a.hot = cp.hot;
+        e = launch_overlapped(kernel, static_cast<unsigned>(sm_count), kCooHotThreads, kept, st, a);
+    } else {
+        e = launch_overlapped(vec ? coo_reduce_kernel<T, N, true, false> : coo_reduce_kernel<T, N, false, false>, grid_for(chunks1), 256, 0, st, a);
+    }
     if (e != cudaSuccess) return e;
     const int32_t *frow = cp.c1_row;
     const float *fval = cp.c1_val;
@@ -70,14 +84,13 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, bool vec, 
         b.count = count2;
         b.carry_row = cp.c2_row;
         b.carry_val = cp.c2_val;
-        coo_reduce_kernel<float, N, false, true><<<grid_for(chunks2), 256, 0, st>>>(b);
-        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = launch_overlapped(coo_reduce_kernel<float, N, false, true>, grid_for(chunks2), 256, 0, st, b)) != cudaSuccess) return e;
         frow = cp.c2_row;
         fval = cp.c2_val;
         fcount = count3;
     }
-    coo_final_kernel<N><<<static_cast<unsigned>((fcount + 255) / 256), 256, 0, st>>>(frow, fval, fcount, s.C, s.ldc, s.alpha, s.beta);
-    return cudaGetLastError();
+    return launch_overlapped(coo_final_kernel<N>, static_cast<unsigned>((fcount + 255) / 256), 256, 0, st, frow, fval, fcount, s.C, s.ldc, s.alpha,
+                             s.beta);
 }
 
 template <typename T>

@@ -36,6 +36,8 @@ struct sd_plan {
     int32_t *coo_row = nullptr;
     int32_t *coo_c1_row = nullptr, *coo_c2_row = nullptr;
     float *coo_c1_val = nullptr, *coo_c2_val = nullptr;
+    int32_t *coo_hot_colind = nullptr, *coo_hot_cols = nullptr;   // columns kept in shared memory
+    int32_t coo_hot = 0;
 
     // BSR
     int32_t *browptr = nullptr;

@@ -1,0 +1,44 @@
+"""Two and three columns on a matrix whose nonzeros crowd into few columns: the kernel that keeps those columns' rows of B in
+shared memory, with columns outside, empty rows, a row over many chunks."""
+import numpy as np
+import pytest
+
+import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+torch = pytest.importorskip("torch")
+if torch.cuda.is_available():
+    import paper_2608_05033_b200 as sd
+    from test_gpu_parity import check
+    from util import DeviceWorkload, run_spmm
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [2, 3])
+def test_frequent_columns_in_shared_memory(N, dtype):
+    rng = np.random.default_rng(N)
+    M, K = 5203, 70001
+    rows = []
+    for i in range(M):
+        n = 0 if i % 37 == 5 else 30000 if i == 11 else 700
+        rows.append(np.unique((K * rng.random(n) ** 5).astype(np.int32)))
+    rowptr = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int32)
+    cols = np.concatenate(rows).astype(np.int32)
+    assert cols.size > 4096 * 600
+    vals, B = rng.standard_normal(cols.size).astype(np.float32), rng.standard_normal((K, N)).astype(np.float32)
+    C = rng.standard_normal((M, N)).astype(np.float32)
+    if dtype == W.SD_BF16:
+        vals, B = W.f32_to_bf16_bits(vals), W.f32_to_bf16_bits(B).reshape(K, N)
+    w = W.Workload("frequent_columns", M, K, N, rowptr, cols, vals, B, C, -0.75, 0.5, dtype, {})
+    plan = DeviceWorkload(w).plan(family=sd.SD_MERGE)
+    assert plan.info().plan_bytes > 8 * cols.size      # a row index and a renamed column per nonzero
+    for kw in (dict(), dict(pad_b=3, pad_c=1), dict(offset=1)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    again, _ = run_spmm(plan, w, **kw)
+    assert np.array_equal(got, again)
+    got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
