@@ -238,6 +238,121 @@ coo_reduce_kernel(const CooArgs a) {
     }
 }
 
+// One column, level 1: a lane owns eight consecutive nonzeros and adds them up itself, so a warp scans once per 256 nonzeros
+// and not per 32: the scan's shuffles share the L1 data path with the gathers.  Rows, columns and values come as 16-byte loads (the
+// arrays must be aligned).  Same runs, same carry entries.  R-MAT scale 20, bf16: 32.4 M nonzeros 134 -> 103 us, 8.1 M 47 -> 40;
+// scale 18, 7.9 M, fp32 36.5 -> 32.1, bf16 34.6 -> 27.6.
+template <typename T>
+__global__ void __launch_bounds__(256)
+coo_serial_kernel(const CooArgs a) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int U = 8, CHUNK = 32 * U;
+    static_assert(CHUNK == coo_chunk(1), "the carry list has two entries per chunk");
+    overlap_next();
+    const int lane = threadIdx.x & 31;
+    const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5, chunks = (a.count + CHUNK - 1) / CHUNK;
+    const T *__restrict__ vals = static_cast<const T *>(a.vals);
+    const T *__restrict__ x = static_cast<const T *>(a.B);
+    overlap_wait();
+    for (int64_t c = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; c < chunks; c += warps) {
+        const int64_t rpc = (a.M + chunks - 1) / chunks;   // this chunk's share of the rows without nonzeros
+        for (int64_t rr = c * rpc + lane; rr < min(a.M, (c + 1) * rpc); rr += 32)
+            if (__ldg(a.rowptr + rr) == __ldg(a.rowptr + rr + 1)) {
+                float *pc = a.C + rr * a.ldc;
+                *pc = (a.beta != 0.f) ? a.beta * *pc : 0.f;
+            }
+        const int64_t k0 = c * CHUNK + lane * U;
+        int r[U], col[U];
+        float p[U];
+        if ((c + 1) * CHUNK <= a.count) {
+#pragma unroll
+            for (int q = 0; q < U / 4; ++q) {
+                const int4 rv = __ldg(reinterpret_cast<const int4 *>(a.row + k0) + q), cv = __ldg(reinterpret_cast<const int4 *>(a.colind + k0) + q);
+                r[4 * q] = rv.x, r[4 * q + 1] = rv.y, r[4 * q + 2] = rv.z, r[4 * q + 3] = rv.w;
+                col[4 * q] = cv.x, col[4 * q + 1] = cv.y, col[4 * q + 2] = cv.z, col[4 * q + 3] = cv.w;
+            }
+            if constexpr (sizeof(T) == 4) {
+#pragma unroll
+                for (int q = 0; q < U / 4; ++q) {
+                    float t[4];
+                    RowLoad<T, 4>::ld(vals + k0 + 4 * q, t);
+#pragma unroll
+                    for (int e = 0; e < 4; ++e) p[4 * q + e] = t[e];
+                }
+            } else {
+                RowLoad<T, 8>::ld(vals + k0, p);
+            }
+            float b[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) b[u] = to_float(__ldg(b_row(x, col[u], a.ldb_bytes)));
+#pragma unroll
+            for (int u = 0; u < U; ++u) p[u] *= b[u];
+        } else {   // items past the end continue the last row with zeros
+            const int pad_row = __ldg(a.row + a.count - 1);
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const bool ok = k0 + u < a.count;
+                r[u] = ok ? __ldg(a.row + k0 + u) : pad_row;
+                p[u] = ok ? to_float(vals[k0 + u]) * to_float(__ldg(b_row(x, __ldg(a.colind + k0 + u), a.ldb_bytes))) : 0.f;
+            }
+        }
+        const int first_row = __shfl_sync(FULL, r[0], 0);
+        auto emit = [&](int row, float v) {
+            float *pc = a.C + static_cast<int64_t>(row) * a.ldc;
+            *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v) : a.alpha * v;
+        };
+        // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
+        float sum = p[0], head = 0.f;
+        bool closed = false;
+#pragma unroll
+        for (int u = 1; u < U; ++u) {
+            if (r[u] != r[u - 1]) {
+                if (closed) emit(r[u - 1], sum);
+                else head = sum;
+                closed = true;
+                sum = 0.f;
+            }
+            sum += p[u];
+        }
+        const int before = __shfl_up_sync(FULL, r[U - 1], 1);
+        const bool begins = lane == 0 || before != r[0];
+        const unsigned edges = __ballot_sync(FULL, begins), starts = __ballot_sync(FULL, begins || closed);
+        const int dist = lane - (31 - __clz(starts & (FULL >> (31 - lane))));
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const float up = __shfl_up_sync(FULL, sum, d);
+            if (dist >= d) sum += up;
+        }
+        const float in = __shfl_up_sync(FULL, sum, 1);
+        if (closed) {
+            if (!begins) head += in;
+            if (r[0] == first_row) {
+                a.carry_row[2 * c] = first_row;
+                a.carry_val[2 * c] = head;
+            } else {
+                emit(r[0], head);
+            }
+        }
+        if (lane < 31 && (edges >> (lane + 1) & 1u)) {   // a run that ends with the lane
+            if (r[U - 1] == first_row) {
+                a.carry_row[2 * c] = first_row;
+                a.carry_val[2 * c] = sum;
+            } else {
+                emit(r[U - 1], sum);
+            }
+        }
+        if (lane == 31) {   // what is still open at the end of the chunk; one single run: (row, sum), (row, 0)
+            const bool single = r[U - 1] == first_row;
+            a.carry_row[2 * c + 1] = r[U - 1];
+            a.carry_val[2 * c + 1] = single ? 0.f : sum;
+            if (single) {
+                a.carry_row[2 * c] = first_row;
+                a.carry_val[2 * c] = sum;
+            }
+        }
+    }
+}
+
 // Level 3: one thread per run of equal rows in a short carry list.
 template <int N>
 __global__ void coo_final_kernel(const int32_t *__restrict__ row, const float *__restrict__ val, int64_t count, float *C,

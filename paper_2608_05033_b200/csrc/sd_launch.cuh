@@ -41,11 +41,8 @@ cudaError_t run_chunk_reduce_wide(const float *chunk_out, const int32_t *chunk_p
 // C = beta * C.
 cudaError_t run_scale_c(float *C, int64_t ldc, int64_t M, int32_t N, float beta, cudaStream_t st);
 
-// Family (b): tile kernel, then the carry-out fix-up for the listed tiles (short chains one per
-// warp, long chains one per CTA).
-cudaError_t run_merge(const MergeArgs &m, int dtype, bool vec, const int32_t *fix_short, int32_t nshort,
-                      const int32_t *fix_long, int32_t nlong, cudaStream_t st);
-constexpr int kMergeLongChain = 8;   // chains of at least this many tiles go to the per-CTA fix-up
+// Merge-path tile kernel, fp32; the caller adds the carries.
+cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st);
 
 // Family (b) for dense widths up to kCooMaxN (beyond it the shuffles per nonzero outweigh the
 // gain; measured cross-over between 4 and 8 columns): segmented reduction over the nonzeros with an

@@ -279,10 +279,7 @@ merge_tile_kernel(const MergeArgs m) {
 
 // Fix-up: tile `t` closed a segment that began in an earlier tile.  Its total is the sum of
 // the carry-outs of the tiles since the one holding its first nonzero, plus this tile's head,
-// added in a fixed order (no atomics, so repeated runs give identical bits).  Chains shorter
-// than kFixLongChain tiles are handled one per warp, longer ones one per CTA.
-constexpr int kFixChains = 8;
-constexpr int kFixLongChain = 8;
+// added in a fixed order (no atomics, so repeated runs give identical bits).
 
 struct FixTarget {
     int64_t row;
@@ -313,50 +310,6 @@ __device__ __forceinline__ void fix_store(const SpmmArgs &a, const FixTarget &f,
     if (f.accumulate) r += *p;
     else if (a.beta != 0.f) r += a.beta * *p;
     *p = r;
-}
-
-static __global__ void __launch_bounds__(256)
-merge_fixup_short_kernel(const MergeArgs m, const int32_t *__restrict__ fix_tiles, int32_t nfix, int32_t tile_items) {
-    const int f = blockIdx.x * 8 + (threadIdx.x >> 5);
-    if (f >= nfix) return;
-    const int lane = threadIdx.x & 31;
-    const int t = fix_tiles[f];
-    const FixTarget ft = fix_target(m, t, tile_items);
-    for (int c = lane; c < m.s.N; c += 32) {
-        float sum = 0.f;
-        for (int tt = ft.ta; tt < t; ++tt) sum += m.tile_tail[static_cast<int64_t>(tt) * m.s.N + c];
-        sum += m.tile_head[static_cast<int64_t>(t) * m.s.N + c];
-        fix_store(m.s, ft, c, sum);
-    }
-}
-
-static __global__ void __launch_bounds__(32 * kFixChains)
-merge_fixup_long_kernel(const MergeArgs m, const int32_t *__restrict__ fix_tiles, int32_t nfix, int32_t tile_items) {
-    __shared__ float part[kFixChains][33];
-    const SpmmArgs &a = m.s;
-    const int f = blockIdx.x;
-    if (f >= nfix) return;
-    const int t = fix_tiles[f];
-    const FixTarget ft = fix_target(m, t, tile_items);
-    const int x = threadIdx.x & 31, y = threadIdx.x >> 5;
-    for (int c0 = 0; c0 < a.N; c0 += 32) {
-        const int c = c0 + x;
-        float sum = 0.f;
-        if (c < a.N) {
-#pragma unroll 4
-            for (int tt = ft.ta + y; tt < t; tt += kFixChains) sum += m.tile_tail[static_cast<int64_t>(tt) * a.N + c];
-        }
-        part[y][x] = sum;
-        __syncthreads();
-        if (y == 0 && c < a.N) {
-            float tot = part[0][x];
-#pragma unroll
-            for (int q = 1; q < kFixChains; ++q) tot += part[q][x];
-            tot += m.tile_head[static_cast<int64_t>(t) * a.N + c];
-            fix_store(a, ft, c, tot);
-        }
-        __syncthreads();
-    }
 }
 
 template <typename T, int VW, int LPR, int NV>

@@ -171,7 +171,7 @@ sd_status_t sd_spmm_merge_static(const int32_t *rowptr, const int32_t *colind, c
     SD_CUDA_TRY(cudaGetLastError());
     const bool vec = ((reinterpret_cast<uintptr_t>(B) | reinterpret_cast<uintptr_t>(C)) & 15u) == 0 && N % 4 == 0 &&
                      ldb % 4 == 0 && ldc % 4 == 0;
-    SD_CUDA_TRY(run_merge(m, SD_F32, vec, nullptr, 0, nullptr, 0, st));   // tile kernel only: no lists
+    SD_CUDA_TRY(run_merge(m, vec, st));
     merge_fixup_scan_kernel<<<ceil_div(ntiles, 8), 256, 0, st>>>(m, kMergeTile);
     SD_CUDA_TRY(cudaGetLastError());
     return SD_OK;

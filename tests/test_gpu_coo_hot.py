@@ -1,4 +1,4 @@
-"""Two and three columns on a matrix whose nonzeros crowd into few columns: the kernel that keeps those columns' rows of B in
+"""One column with a lane per eight nonzeros or, where the arrays are not aligned, per 32; two and three columns on a matrix whose nonzeros crowd into few columns: the kernel that keeps those columns' rows of B in
 shared memory, with columns outside, empty rows, a row over many chunks."""
 import numpy as np
 import pytest
@@ -11,7 +11,7 @@ torch = pytest.importorskip("torch")
 if torch.cuda.is_available():
     import paper_2608_05033_b200 as sd
     from test_gpu_parity import check
-    from util import DeviceWorkload, run_spmm
+    from util import DeviceWorkload, dev, run_spmm
 
 
 @pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
@@ -40,5 +40,22 @@ def test_frequent_columns_in_shared_memory(N, dtype):
     again, _ = run_spmm(plan, w, **kw)
     assert np.array_equal(got, again)
     got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("offset", [0, 1])
+@pytest.mark.parametrize("edges", [[0, 1, 7, 8, 9, 0, 15], [255, 256, 257, 1, 0, 511], [1], [1000, 3, 0, 0, 2048, 5]])
+def test_one_column_runs_and_aligned_arrays(edges, offset, dtype):
+    lengths = np.resize(edges, 301)
+    w = W.random_csr(301, 2500, 1, lengths, seed=len(edges), dtype=dtype, alpha=1.5, beta=-0.5)
+    colind, vals = (dev(np.concatenate([np.zeros(offset, a.dtype), a]))[offset:] for a in (w.colind, w.vals))
+    plan = sd.Plan(dev(w.rowptr), colind, vals, w.M, w.K, 1, dtype=dtype, family=sd.SD_MERGE)
+    got, intact = run_spmm(plan, w)
+    assert intact
+    check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w)[0])
+    got, _ = run_spmm(plan, w, c_fill=np.full((w.M, 1), np.nan, np.float32), beta=0.0)
     check(w, got, beta=0.0)
     plan.close()
