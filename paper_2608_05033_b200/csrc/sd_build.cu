@@ -112,34 +112,38 @@ void host_blocks_release() {
 // =====================================================================================
 // Rows by length: a stable counting sort on the key 0 (heavy) or T - length, one pass over the row pointers to count and one
 // to place.  The row-length histogram of the scan gives every key's first position, so the only scan left is over the
-// tiles of one key.
-constexpr int kSortTile = 2048, kSortWarps = 8, kSortBins = kHybridHeavyMax + 1;
+// tiles of one key.  A tile is PER x 256 rows: large ones mean fewer counters, small ones more CTAs and shorter chains (65,536 rows: placing 13 us
+// with PER = 8, 6 with 2).  The kernels' launches overlap.
+constexpr int kSortWarps = 8, kSortBins = kHybridHeavyMax + 1;
 
 __device__ __forceinline__ int sort_key(int len, int T) { return len >= T ? 0 : T - len; }
 
-// Keys of a warp's 256 rows (8 per lane), counted into its bins.
-__device__ __forceinline__ void count_keys(const int32_t *__restrict__ rowptr, int64_t M, int64_t base, int T, int (&key)[8], int *bins) {
+// Keys of a warp's rows (PER per lane), counted into its bins.
+template <int PER>
+__device__ __forceinline__ void count_keys(const int32_t *__restrict__ rowptr, int64_t M, int64_t base, int T, int (&key)[PER], int *bins) {
     const int lane = threadIdx.x & 31;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < PER; ++i) {
         const int64_t r = base + i * 32 + lane;
         key[i] = r < M ? sort_key(__ldg(rowptr + r + 1) - __ldg(rowptr + r), T) : -1;
     }
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < PER; ++i) {
         const unsigned same = __match_any_sync(0xffffffffu, key[i]);
         if (key[i] >= 0 && lane == __ffs(same) - 1) bins[key[i]] += __popc(same);
         __syncwarp();
     }
 }
 
+template <int PER>
 __global__ void __launch_bounds__(32 * kSortWarps)
 sort_count_kernel(const int32_t *__restrict__ rowptr, int64_t M, int T, int32_t ntiles, int32_t *__restrict__ hist) {
     __shared__ int bins[kSortWarps][kSortBins];
+    overlap_next();
     for (int i = threadIdx.x; i < kSortWarps * kSortBins; i += blockDim.x) (&bins[0][0])[i] = 0;
     __syncthreads();
-    int key[8];
-    count_keys(rowptr, M, static_cast<int64_t>(blockIdx.x) * kSortTile + (threadIdx.x >> 5) * 256, T, key, bins[threadIdx.x >> 5]);
+    int key[PER];
+    count_keys<PER>(rowptr, M, static_cast<int64_t>(blockIdx.x) * PER * 256 + (threadIdx.x >> 5) * (PER * 32), T, key, bins[threadIdx.x >> 5]);
     __syncthreads();
     for (int k = threadIdx.x; k <= T; k += blockDim.x) {
         int n = 0;
@@ -157,6 +161,8 @@ struct SortBases {
 __global__ void __launch_bounds__(256)
 sort_prefix_kernel(const SortBases b, int T, int32_t ntiles, int32_t *__restrict__ hist) {
     const int k = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
+    overlap_next();
+    overlap_wait();
     if (k > T) return;
     int run = b.first[k];
     for (int t0 = 0; t0 < ntiles; t0 += 32) {
@@ -174,16 +180,19 @@ sort_prefix_kernel(const SortBases b, int T, int32_t ntiles, int32_t *__restrict
 }
 
 // Places the rows; a light row's descriptor holds everything its first gather needs, in one 16-byte load.
+template <int PER>
 __global__ void __launch_bounds__(32 * kSortWarps)
 sort_place_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, int64_t M, int T, int32_t ntiles,
                   const int32_t *__restrict__ hist, int32_t nl, int32_t *__restrict__ rows, int4 *__restrict__ desc) {
     __shared__ int bins[kSortWarps][kSortBins];
+    overlap_next();
     for (int i = threadIdx.x; i < kSortWarps * kSortBins; i += blockDim.x) (&bins[0][0])[i] = 0;
     __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t base = static_cast<int64_t>(blockIdx.x) * kSortTile + warp * 256;
-    int key[8];
-    count_keys(rowptr, M, base, T, key, bins[warp]);
+    const int64_t base = static_cast<int64_t>(blockIdx.x) * PER * 256 + warp * (PER * 32);
+    int key[PER];
+    count_keys<PER>(rowptr, M, base, T, key, bins[warp]);
+    overlap_wait();
     __syncthreads();
     for (int k = threadIdx.x; k <= T; k += blockDim.x) {   // counts of the warps become their first positions
         int at = hist[static_cast<int64_t>(k) * ntiles + blockIdx.x];
@@ -196,7 +205,7 @@ sort_place_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
+    for (int i = 0; i < PER; ++i) {
         const unsigned same = __match_any_sync(0xffffffffu, key[i]);
         int at = 0;
         if (key[i] >= 0) at = bins[warp][key[i]] + __popc(same & ((1u << lane) - 1u));
@@ -222,6 +231,8 @@ chunk_ptr_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__
                  int32_t *__restrict__ item_ptr, int32_t *__restrict__ giant, int32_t *__restrict__ ngiant) {
     using Scan = cub::BlockScan<int, 1024>;
     __shared__ typename Scan::TempStorage tmp;
+    overlap_next();
+    overlap_wait();
     int c = 0, m = 0, g = 0;   // chunks, items and listed rows before this step, the same in all threads
     for (int64_t i0 = 0; i0 < nl; i0 += 1024) {
         const int64_t i = i0 + threadIdx.x;
@@ -265,6 +276,7 @@ items_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ row
              const int32_t *__restrict__ item_ptr, int32_t F, int64_t nl, int4 *__restrict__ items) {
     const int lane = threadIdx.x & 31;
     const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    overlap_wait();
     for (int64_t i = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; i < nl; i += warps) {
         const int32_t r = rows[i], p0 = __ldg(rowptr + r), p1 = __ldg(rowptr + r + 1), c0 = chunk_ptr[i], m0 = item_ptr[i], m1 = item_ptr[i + 1];
         for (int32_t m = m0 + lane; m < m1; m += 32) {
@@ -362,18 +374,19 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
         if (l >= kHybridWide) p->h_nw = at - nl;
     }
     p->h_nl = nl;
-    const int32_t ntiles = static_cast<int32_t>((p->M + kSortTile - 1) / kSortTile);
+    const bool fine = p->M <= 131072;
+    const int32_t ntiles = static_cast<int32_t>((p->M + (fine ? 511 : 2047)) / (fine ? 512 : 2048));
     TempBuf hist(st), ngiant(st), start(st), counts(st), offs(st), tmp(st);
     if ((s = hist.get(sizeof(int32_t) * (T + 1) * static_cast<size_t>(ntiles), "length counts"))) return s;
     if ((s = dev_alloc(p, &p->h_rows, p->M, "rows by length", st))) return s;
     if ((s = dev_alloc(p, &p->h_desc, p->M - nl, "light row descriptors", st))) return s;
-    sort_count_kernel<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->M, T, ntiles, hist.as<int32_t>());
+    auto count = fine ? sort_count_kernel<2> : sort_count_kernel<8>;
+    auto place = fine ? sort_place_kernel<2> : sort_place_kernel<8>;
+    count<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->M, T, ntiles, hist.as<int32_t>());
     SD_CUDA_TRY(cudaGetLastError());
-    sort_prefix_kernel<<<(T + 8) / 8, 256, 0, st>>>(bases, T, ntiles, hist.as<int32_t>());
-    SD_CUDA_TRY(cudaGetLastError());
-    sort_place_kernel<<<ntiles, 32 * kSortWarps, 0, st>>>(p->rowptr, p->colind, p->M, T, ntiles, hist.as<int32_t>(),
-                                                         static_cast<int32_t>(nl), p->h_rows, p->h_desc);
-    SD_CUDA_TRY(cudaGetLastError());
+    SD_CUDA_TRY(launch_overlapped(sort_prefix_kernel, static_cast<unsigned>((T + 8) / 8), 256, 0, st, bases, T, ntiles, hist.as<int32_t>()));
+    SD_CUDA_TRY(launch_overlapped(place, static_cast<unsigned>(ntiles), 32 * kSortWarps, 0, st, p->rowptr, p->colind, p->M, T, ntiles,
+                                  hist.as<int32_t>(), static_cast<int32_t>(nl), p->h_rows, p->h_desc));
     p->h_nc = p->h_ni = p->h_ng = 0;
     p->info.launches = 1;
     if (nl > 0) {
@@ -383,8 +396,8 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
         if ((s = ngiant.get(sizeof(int32_t), "count"))) return s;
         if ((s = dev_alloc(p, &p->h_item_ptr, nl + 1, "item pointers", st))) return s;
         if (W == 1) {
-            chunk_ptr_kernel<<<1, 1024, 0, st>>>(p->rowptr, p->h_rows, nullptr, nullptr, 1, F, nl, p->h_chunk_ptr, p->h_item_ptr, p->h_giant, ngiant.as<int32_t>());
-            SD_CUDA_TRY(cudaGetLastError());
+            SD_CUDA_TRY(launch_overlapped(chunk_ptr_kernel, 1u, 1024, 0, st, p->rowptr, p->h_rows, nullptr, nullptr, 1, F, nl, p->h_chunk_ptr,
+                                          p->h_item_ptr, p->h_giant, ngiant.as<int32_t>()));
             if (F > 1 && ng > 0) {   // the scan counted the rows of many chunks, this one those of many items
                 int32_t got = 0;
                 SD_CUDA_TRY(cudaMemcpyAsync(&got, ngiant.p, sizeof got, cudaMemcpyDeviceToHost, st));
@@ -392,8 +405,8 @@ sd_status_t build_schedule(sd_plan *p, int W, int32_t T, const ScanAccum &h, cud
                 ng = got;
             }
             if ((s = dev_alloc(p, &p->h_items, ni, "chunk descriptors", st))) return s;
-            items_kernel<<<ceil_div(std::min<int64_t>(nl, 148 * 64), 8), 256, 0, st>>>(p->rowptr, p->h_rows, p->h_chunk_ptr, p->h_item_ptr, F, nl, p->h_items);
-            SD_CUDA_TRY(cudaGetLastError());
+            SD_CUDA_TRY(launch_overlapped(items_kernel, static_cast<unsigned>(ceil_div(std::min<int64_t>(nl, 148 * 64), 8)), 256, 0, st, p->rowptr,
+                                          p->h_rows, p->h_chunk_ptr, p->h_item_ptr, F, nl, p->h_items));
         } else {
             const int64_t cells = nl * W, n = cells + 1;
             if (n > INT32_MAX) {

@@ -131,7 +131,7 @@ struct ScanAccum {
     unsigned long long giants;            // rows of more than kGiantChunks chunks
     unsigned long long len_hist[256];     // rows of exactly 0 .. 255 nonzeros
     long long nnz;                        // rowptr[M]
-    unsigned int large, huge;             // block-rows left to the second and third scan kernels
+    unsigned int huge;                    // block-rows left to the last scan kernel
 };
 
 constexpr int kChunkNnz = 128;      // heavy rows are cut into pieces of at most this many nonzeros
