@@ -128,3 +128,31 @@ def test_fp32_error_does_not_grow_with_the_blocks_of_a_row(per_row, N):
     want = A @ B.astype(np.float64)
     assert np.linalg.norm(got - want) <= 6e-7 * np.linalg.norm(want)
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("holes", [0, 1])
+def test_block_values_from_any_offset(dtype, holes):
+    """Whole vectors of a block's row come as one load where they are aligned, entry by entry otherwise: arrays that start at
+    every element of a 16-byte piece, whole blocks and blocks with a few absent entries, bit-exact."""
+    import oracle
+    w = W.g4_block(Mb=20, Kb=15, N=64, nblocks=90, dtype=dtype)
+    rowptr, colind = w.rowptr, w.colind
+    if holes:
+        keep = np.random.default_rng(1).random(colind.size) > 0.02
+        rowptr = np.concatenate([[0], np.cumsum(keep)])[rowptr].astype(np.int32)
+        colind = colind[keep]
+    vals = np.random.default_rng(2).standard_normal(colind.size).astype(np.float32)
+    if dtype == W.SD_BF16:
+        vals = W.f32_to_bf16_bits(vals)
+    ref = oracle.bsr16(rowptr, colind, vals, w.M, w.K)[2].tobytes()
+    rowptr_d, colind_d = torch.from_numpy(rowptr).cuda(), torch.from_numpy(colind).cuda()
+    old = torch.zeros(colind.size, device="cuda", dtype=torch.float32 if dtype == W.SD_F32 else torch.int16)
+    plan = sd.Plan(rowptr_d, colind_d, old, w.M, w.K, w.N, dtype=dtype, family=sd.SD_BSR_TC)
+    bits = vals.view(np.int16) if dtype == W.SD_BF16 else vals
+    for off in range(8):
+        new = torch.from_numpy(np.concatenate([np.zeros(off, bits.dtype), bits])).cuda()
+        plan.update_values(new[off:])
+        assert sd.sd_plan_get_bsr(plan.handle)[2].tobytes() == ref
+        plan.update_values(old)
+    plan.close()
