@@ -424,6 +424,7 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
             a.vals = plan->vals;
             CooPlan cp;
             cp.row = plan->coo_row;
+            cp.starts = plan->coo_starts;
             cp.rowptr = plan->rowptr;
             cp.M = plan->info.empty_rows > 0 ? M : 0;   // no search for rows without nonzeros when the scan found none
             cp.nnz = plan->nnz;
@@ -434,8 +435,7 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
             cp.hot_colind = plan->coo_hot_colind;
             cp.hot_cols = plan->coo_hot_cols;
             cp.hot = plan->coo_hot;
-            const bool bvec = aligned16(B) && (ldb * (plan->dtype == SD_F32 ? 4 : 2)) % 16 == 0;
-            SD_CUDA_TRY(run_coo(cp, a, plan->dtype, bvec, plan->info.sm_count, st));
+            SD_CUDA_TRY(run_coo(cp, a, plan->dtype, plan->info.sm_count, st));
             return SD_OK;
         }
         [[fallthrough]];   // wider ones run the hybrid schedule

@@ -512,14 +512,16 @@ __global__ void rename_columns_kernel(const int32_t *__restrict__ colind, int64_
         out[k] = __ldg(name + __ldg(colind + k));
 }
 
-// Taken from two columns on, where 4,096 columns pay for being fetched by every SM (a cycle each; at most nnz / 600 of them) and
-// if they cover a quarter of the nonzeros.  R-MAT with 32.4 M nonzeros: two fp32 columns 209 -> 173 us, two bf16 197 -> 163, four
-// 362 -> 270; with 3.4 M, two fp32 columns 30 -> 28.  One column gains nothing (the shuffles of the segmented scan take the same
-// unit as the gathers), four fp32 columns, one 16-byte gather, only on the largest (254 -> 242; with 3.4 M 33 -> 38).
+// Taken where 4,096 columns pay for being fetched by every SM (at most nnz / 600 of them, nnz / 1000 at
+// one column) and if they cover a quarter of the nonzeros.  Without and with, us: R-MAT with 32.4 M nonzeros at one, two, three and four
+// fp32 columns 111 -> 86, 141 -> 122, 228 -> 177, 179 -> 162, one and two bf16 102 -> 87, 121 -> 119; with 7.9 M at one 26.5 -> 23.8;
+// with 3.9 M one fp32 16.6 and 16.2, two bf16 18.9 and 20.7, four 24.8 and 22.8; four fp32 columns, one 16-byte gather, only on the
+// largest (with 7.9 M 46.8 and 46.5).  More than kCooHotColumns gain nothing (one bf16 column 87 us with 32,768, 89 with 54,000).
+constexpr int64_t kCooHotColumns = 32768;
 static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
     const int64_t row_bytes = p->N * (p->dtype == SD_F32 ? 4 : 2);
-    const int64_t most = std::min<int64_t>({kCooHotBytes / row_bytes, p->nnz / 600, p->K});
-    if (p->N < 2 || most < 4096 || (row_bytes == 16 && p->nnz < 16000000)) return SD_OK;
+    const int64_t most = std::min<int64_t>({kCooHotBytes / row_bytes, kCooHotColumns, p->nnz / (p->N == 1 ? 1000 : 600), p->K});
+    if (most < 4096 || (row_bytes == 16 && p->nnz < 16000000)) return SD_OK;
     sd_status_t s;
     TempBuf degree(st), bins(st), flag(st), scratch(st), small(st);
     const int64_t K = p->K;
@@ -560,15 +562,17 @@ static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
 
 sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
     sd_status_t s;
-    const int cchunk = coo_chunk(static_cast<int>(p->N));
-    const int64_t chunks1 = (p->nnz + cchunk - 1) / cchunk, count2 = 2 * chunks1;
+    const int64_t steps = coo_steps(p->nnz, static_cast<int>(p->N));
+    const int64_t count2 = 2 * std::min<int64_t>(steps, static_cast<int64_t>(kCooMaxWarps) * p->info.sm_count);
     const int64_t chunks2 = (count2 + kCooCarryChunk - 1) / kCooCarryChunk, count3 = 2 * chunks2;
-    if ((s = dev_alloc(p, &p->coo_row, p->nnz, "row index per nonzero", st))) return s;
+    const bool bits = p->N == 1 && p->info.empty_rows == 0;
+    if ((s = dev_alloc(p, &p->coo_row, bits ? 32 * steps : p->nnz, "rows of nonzeros", st))) return s;
+    if (bits && (s = dev_alloc(p, &p->coo_starts, 32 * steps, "starts of rows", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c1_row, count2, "carry rows", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c1_val, count2 * p->N, "carry sums", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c2_row, count3, "carry rows (level 2)", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c2_val, count3 * p->N, "carry sums (level 2)", st))) return s;
-    SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, p->coo_row, st));
+    SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, steps, p->coo_row, p->coo_starts, st));
     p->info.launches = 2 + (count2 > kCooDirectFinal);
     return coo_hot_columns(p, st);
 }

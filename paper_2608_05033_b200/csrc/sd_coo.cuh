@@ -1,28 +1,32 @@
-// Narrow dense operands (N <= 4, SpMV included) of family (b): a segmented reduction over the
-// nonzeros in storage order with an explicit row index per nonzero (the COO form that the paper's
-// Sec. 3.1 lists for SpMV-like widths).
+// Narrow dense operands (N <= 4, SpMV included) of family (b): a segmented reduction over the nonzeros in storage order (the COO
+// form that the paper's Sec. 3.1 lists for SpMV-like widths).
 //
-// With one to eight columns a lane group per row has nothing to share: the generic merge kernel
-// spends its time on per-lane searches and block-wide phases.  Here a warp owns 128 consecutive
-// nonzeros (256 at one or two columns: four or eight coalesced loads of row, column and value per lane, as many
-// gathers of B in flight),
-// multiplies, and reduces equal-row runs with warp shuffles; no shared memory, no block barrier.
+// With one to four columns a lane group per row has nothing to share.  Here the nonzeros are dealt out evenly: a warp owns a
+// contiguous range of them and walks it 256 (three or four columns: 128) at a time; a lane adds up eight (four) consecutive
+// nonzeros by itself, and one segmented scan over the warp's lanes joins the rows that run across lanes.  A row that lies inside
+// the range is complete: its lane writes alpha * sum + beta * C.  The first and the last row of the range may continue in the
+// neighbours': their sums go to a carry list, two entries per warp in order, (first row, sum) and (last row, sum), or, where the
+// range is one single row, (row, sum) and (row, 0), so that entries of one row stay adjacent.  The list is a row-sorted list
+// of values itself: a second kernel reduces it the same way, and the few entries that leaves over are added one row per thread.
+// Rows without nonzeros are found from the row pointers and get beta * C.  Every row is written by one thread and every sum has
+// a fixed order: results repeat bit for bit, no float atomics.
 //
-// Rows are ascending in storage order, so a row is one run.  A run that lies strictly inside a
-// warp's 128 nonzeros is complete: its lane writes alpha * sum + beta * C.
-// The first and the last run of a chunk may continue in the neighbours: their sums go to a carry
-// list, two entries per chunk in chunk order, (first row, sum) and (last row, sum) -- a chunk
-// that is one single run writes (row, sum) and (row, 0), so that entries of one row stay
-// adjacent.  The carry list is itself a row-sorted list of values: the same kernel reduces it
-// (level 2), and the few entries that level leaves over are added one run per thread (level 3).
-// Rows without nonzeros are found from the row pointers by the first level and get beta * C.
-// Every row is written by exactly one thread and every sum has a fixed order: results are
-// reproducible bit for bit, no float atomics.
+// Where rows begin: a bit per nonzero and the row of every eighth (0.6 bytes per nonzero; one column, no rows without
+// nonzeros), else a row index per nonzero (4 bytes).
 //
-// What bounds it: the L1 data path, which the gathers (up to 32 tag cycles for 32 unrelated rows of B) and the shuffles of the
-// scan share (one column, a scale-18 R-MAT matrix: L1 83 % busy; a scale-20 one takes 120 us).  At two to four columns, where a few columns hold a large
-// part of the nonzeros, the HOT form keeps their rows of B in shared memory (one CTA per SM), where 32 unrelated words cost
-// about three cycles; the plan owns a copy of the columns with those renamed to slots (coo_hot_columns).
+// What bounds it: L1, a cycle per line of B that a gather touches, 32 for 32 unrelated rows.  Where a few columns hold much of the
+// matrix, the HOT form keeps their rows of B in shared memory (one CTA per SM), where 32 unrelated words cost about five
+// cycles; the plan owns a copy of the columns with those renamed to slots (coo_hot_columns).
+//
+// 32.4 M nonzeros, R-MAT scale 20, us, with a scan per 32 nonzeros and a carry per 256 before (one fp32 column and all with frequent
+// columns kept: as far as that paid then), and now:
+//     columns    1           2            3            4
+//     fp32       121 -> 86   169 -> 122   225 -> 177   239 -> 162
+//     bf16        95 -> 87   159 -> 119                267 -> 143
+// 60 M nonzeros in rank-size rows, uniform columns: one column 268 -> 272, two 392 -> 326, four 533 -> 424.  Small matrices are
+// level within 5 % (scale 12 to 16), at one bf16 column of scale 17 15.0 -> 16.4.  Tried: the next step's columns and values
+// requested ahead (registers: 86 -> 97), products formed in storage order and dealt out through shared memory (110), the next
+// launch let in before the carries are written (scale 16 11.5 -> 12.1).
 #pragma once
 
 #include "sd_common.cuh"
@@ -31,21 +35,23 @@
 namespace sd {
 
 constexpr int kCooHotThreads = 1024;
+constexpr int coo_threads(int N) { return N == 1 ? 128 : 256; }
 
 struct CooArgs {
-    const int32_t *row;      // [count] row of every item (ascending)
-    const int32_t *colind;   // level 1: [count] column of every nonzero
-    const void *vals;        // level 1: [count] values of A; level 2: [count][N] float partial sums
-    const void *B;           // level 1
+    const int32_t *row;      // [count] row of every item (ascending), or with `starts` of every eighth
+    const uint8_t *starts;   // one column without empty rows: bit u of byte g: nonzero 8g + u begins a row
+    const int32_t *colind;   // [count] column of every nonzero
+    const void *vals;        // [count] values of A; carry list: [count][N] float partial sums
+    const void *B;
     uint32_t ldb_bytes;
     int64_t count;           // items
     float *C;
     int64_t ldc;
     float alpha, beta;
-    const int32_t *rowptr;   // level 1: [M + 1], to find the rows without nonzeros (they get beta * C)
+    const int32_t *rowptr;   // [M + 1], to find the rows without nonzeros (they get beta * C)
     int64_t M;
-    int32_t *carry_row;      // [2 * chunks] out
-    float *carry_val;        // [2 * chunks][N] out
+    int32_t *carry_row;      // [2 * warps] out
+    float *carry_val;        // [2 * warps][N] out
     const int32_t *hot_cols; // HOT: ascending columns whose rows of B the kernel keeps; colind names slot i of them as i | bit 31
     int32_t hot;
 };
@@ -74,283 +80,327 @@ __device__ __forceinline__ void coo_gather(const void *B, int col, uint32_t ldb_
     }
 }
 
-// LEVEL2: the items are carry entries (row, N partial sums); otherwise nonzeros of A.
-template <typename T, int N, bool VEC, bool LEVEL2, bool HOT = false>
-__global__ void __launch_bounds__(HOT ? kCooHotThreads : 256)
-coo_reduce_kernel(const CooArgs a) {
-    extern __shared__ __align__(16) char coo_hot_raw[];
-    overlap_wait();
-    if constexpr (HOT) {
-        T *kept = reinterpret_cast<T *>(coo_hot_raw);
-        for (int i = threadIdx.x; i < a.hot; i += kCooHotThreads) {
-            const T *p = b_row(static_cast<const T *>(a.B), __ldg(a.hot_cols + i), a.ldb_bytes);
-#pragma unroll
-            for (int e = 0; e < N; ++e) kept[i * N + e] = p[e];
-        }
-        __syncthreads();
-    }
-    constexpr unsigned FULL = 0xffffffffu;
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
-    constexpr int kCooChunk = LEVEL2 ? kCooCarryChunk : coo_chunk(N);
-    constexpr int kCooU = kCooChunk / 32;   // items per lane and warp step
-    const int64_t chunks = (a.count + kCooChunk - 1) / kCooChunk;
-    const T *vals = static_cast<const T *>(a.vals);
-    const float *pvals = static_cast<const float *>(a.vals);
+template <typename T> __device__ __forceinline__ T from_float(float v);   // of a value that T holds
+template <> __device__ __forceinline__ float from_float<float>(float v) { return v; }
+template <> __device__ __forceinline__ __nv_bfloat16 from_float<__nv_bfloat16>(float v) {
+    return __ushort_as_bfloat16(static_cast<unsigned short>(__float_as_uint(v) >> 16));
+}
 
-    for (int64_t c = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; c < chunks; c += warps) {
-        if constexpr (!LEVEL2) {
-            // rows without nonzeros have no writer among the runs: this chunk looks after its share of them
-            const int64_t rpc = (a.M + chunks - 1) / chunks;
-            for (int64_t rr = c * rpc + lane; rr < min(a.M, (c + 1) * rpc); rr += 32) {
-                if (__ldg(a.rowptr + rr) == __ldg(a.rowptr + rr + 1)) {
+// N floats of row `col` of B with one load where VEC says that its alignment allows it.
+template <typename T, int N, bool VEC>
+__device__ __forceinline__ void coo_row_of_b(const T *p, float (&b)[N]) {
+    if constexpr (VEC && N == 4 && sizeof(T) == 4) {
+        RowLoad<T, 4>::ld(p, b);
+    } else if constexpr (VEC && N == 2 && sizeof(T) == 4) {
+        const float2 v = live_load(reinterpret_cast<const float2 *>(p));
+        b[0] = v.x, b[1] = v.y;
+    } else if constexpr (VEC && N == 4) {
+        const uint2 v = live_load(reinterpret_cast<const uint2 *>(p));
+        b[0] = __uint_as_float(v.x << 16), b[1] = __uint_as_float(v.x & 0xFFFF0000u);
+        b[2] = __uint_as_float(v.y << 16), b[3] = __uint_as_float(v.y & 0xFFFF0000u);
+    } else if constexpr (VEC && N == 2) {
+        const uint32_t v = live_load(reinterpret_cast<const uint32_t *>(p));
+        b[0] = __uint_as_float(v << 16), b[1] = __uint_as_float(v & 0xFFFF0000u);
+    } else {
 #pragma unroll
-                    for (int e = 0; e < N; ++e) {
-                        float *pc = a.C + rr * a.ldc + e;
-                        *pc = (a.beta != 0.f) ? a.beta * *pc : 0.f;
-                    }
-                }
-            }
-        }
-        const int64_t k0 = c * kCooChunk + lane;
-        const bool whole = (c + 1) * kCooChunk <= a.count;   // warp-uniform: no item of the chunk is past the end
-        // ---- four items per lane: loads first, all gathers in flight together ------------------
-        int r[kCooU];
-        float p[kCooU][N];
-        if constexpr (LEVEL2) {
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u) {
-                const int64_t k = k0 + u * 32;
-                const bool ok = whole || k < a.count;
-                r[u] = ok ? a.row[k] : -1;   // the carry list of the kernel before: no read-only loads
-#pragma unroll
-                for (int e = 0; e < N; ++e) p[u][e] = ok ? pvals[k * N + e] : 0.f;
-            }
-        } else {
-            int col[kCooU];
-            float av[kCooU];
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u) {
-                const int64_t k = k0 + u * 32;
-                const bool ok = whole || k < a.count;
-                r[u] = ok ? __ldg(a.row + k) : -1;
-                col[u] = ok ? __ldg(a.colind + k) : 0;
-                av[u] = ok ? to_float(vals[k]) : 0.f;
-            }
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u) {
-                if constexpr (HOT) {   // every lane reads a slot (the others slot 0), those outside also their row of B
-                    const bool kept = col[u] < 0;
-                    const T *q = reinterpret_cast<const T *>(coo_hot_raw) + (kept ? col[u] & 0x7fffffff : 0) * N;
-#pragma unroll
-                    for (int e = 0; e < N; ++e) p[u][e] = to_float(q[e]);
-                    if (!kept) coo_gather<T, N, VEC>(a.B, col[u], a.ldb_bytes, p[u]);
-                    continue;
-                }
-                coo_gather<T, N, VEC>(a.B, col[u], a.ldb_bytes, p[u]);
-            }
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u)
-#pragma unroll
-                for (int e = 0; e < N; ++e) p[u][e] = (r[u] >= 0) ? p[u][e] * av[u] : 0.f;   // items past the end gathered row 0: never let its contents (Inf, NaN) in
-        }
-        if (!whole) {   // items past the end of the list continue the last row with zeros
-            const int64_t last = a.count - 1;
-            const int last_u = static_cast<int>((last - c * kCooChunk) >> 5), last_l = static_cast<int>(last & 31);
-            int pad_row = 0;
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u) {
-                const int t = __shfl_sync(FULL, r[u], last_l);
-                if (u == last_u) pad_row = t;
-            }
-#pragma unroll
-            for (int u = 0; u < kCooU; ++u)
-                if (r[u] < 0) r[u] = pad_row;
-        }
-
-        // A run is written when it closes: the run of the chunk's first row goes to the carry
-        // list (it may have begun in an earlier chunk), every other one is a complete row.
-        const int first_row = __shfl_sync(FULL, r[0], 0);
-        auto emit = [&](int row, const float (&v)[N]) {
-            if (row == first_row) {
-                a.carry_row[2 * c] = row;
-#pragma unroll
-                for (int e = 0; e < N; ++e) a.carry_val[(2 * c) * N + e] = v[e];
-            } else {
-#pragma unroll
-                for (int e = 0; e < N; ++e) {
-                    float *pc = a.C + static_cast<int64_t>(row) * a.ldc + e;
-                    *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v[e]) : a.alpha * v[e];
-                }
-            }
-        };
-        int crow = first_row;   // the run that reached the end of the previous 32 items ...
-        float cval[N];          // ... and its sum so far (both warp-uniform)
-#pragma unroll
-        for (int e = 0; e < N; ++e) cval[e] = 0.f;
-
-#pragma unroll
-        for (int u = 0; u < kCooU; ++u) {
-            // where runs start among these 32 items: one ballot replaces a row exchange per scan step
-            const int rp = __shfl_up_sync(FULL, r[u], 1);
-            const unsigned starts = __ballot_sync(FULL, lane == 0 || rp != r[u]);
-            const int my_start = 31 - __clz(starts & (FULL >> (31 - lane)));   // first lane of this lane's run
-            const int dist = lane - my_start;
-            // inclusive segmented scan over equal rows
-#pragma unroll
-            for (int d = 1; d < 32; d <<= 1) {
-#pragma unroll
-                for (int e = 0; e < N; ++e) {
-                    const float vu = __shfl_up_sync(FULL, p[u][e], d);
-                    if (dist >= d) p[u][e] += vu;
-                }
-            }
-            const bool cont = __shfl_sync(FULL, r[u], 0) == crow;
-            if (cont) {                 // the open run continues in the lanes of lane 0's run
-                if (my_start == 0) {
-#pragma unroll
-                    for (int e = 0; e < N; ++e) p[u][e] += cval[e];
-                }
-            } else if (lane == 0) {     // it ended exactly at the 32-item boundary
-                emit(crow, cval);
-            }
-            if (lane < 31 && ((starts >> (lane + 1)) & 1u)) emit(r[u], p[u]);   // runs that end inside these 32 items
-            crow = __shfl_sync(FULL, r[u], 31);                                  // the run reaching lane 31 stays open
-#pragma unroll
-            for (int e = 0; e < N; ++e) cval[e] = __shfl_sync(FULL, p[u][e], 31);
-        }
-        // ---- what is still open at the end of the chunk --------------------------------------
-        if (lane == 0) {
-            a.carry_row[2 * c + 1] = crow;
-            if (crow == first_row) {   // the whole chunk is one run: (row, sum), (row, 0)
-                a.carry_row[2 * c] = crow;
-#pragma unroll
-                for (int e = 0; e < N; ++e) {
-                    a.carry_val[(2 * c) * N + e] = cval[e];
-                    a.carry_val[(2 * c + 1) * N + e] = 0.f;
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < N; ++e) a.carry_val[(2 * c + 1) * N + e] = cval[e];
-            }
+        for (int e = 0; e < N; ++e) {
+            float t[1];
+            RowLoad<T, 1>::ld(p + e, t);
+            b[e] = t[0];
         }
     }
 }
 
-// One column, level 1: a lane owns eight consecutive nonzeros and adds them up itself, so a warp scans once per 256 nonzeros
-// and not per 32: the scan's shuffles share the L1 data path with the gathers.  Rows, columns and values come as 16-byte loads (the
-// arrays must be aligned).  Same runs, same carry entries.  R-MAT scale 20, bf16: 32.4 M nonzeros 134 -> 103 us, 8.1 M 47 -> 40;
-// scale 18, 7.9 M, fp32 36.5 -> 32.1, bf16 34.6 -> 27.6.
-template <typename T>
-__global__ void __launch_bounds__(256)
-coo_serial_kernel(const CooArgs a) {
-    constexpr unsigned FULL = 0xffffffffu;
-    constexpr int U = 8, CHUNK = 32 * U;
-    static_assert(CHUNK == coo_chunk(1), "the carry list has two entries per chunk");
-    const int lane = threadIdx.x & 31;
-    const int64_t warps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5, chunks = (a.count + CHUNK - 1) / CHUNK;
-    const T *vals = static_cast<const T *>(a.vals);
-    auto gather = [&](int col) {
-        float b[1];
-        coo_gather<T, 1, false>(a.B, col, a.ldb_bytes, b);
-        return b[0];
-    };
-    overlap_wait();
-    for (int64_t c = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5; c < chunks; c += warps) {
-        const int64_t rpc = (a.M + chunks - 1) / chunks;   // this chunk's share of the rows without nonzeros
-        for (int64_t rr = c * rpc + lane; rr < min(a.M, (c + 1) * rpc); rr += 32)
-            if (__ldg(a.rowptr + rr) == __ldg(a.rowptr + rr + 1)) {
-                float *pc = a.C + rr * a.ldc;
+// U consecutive elements, widened, with one load if `align`, the address of the array, allows it.
+template <typename T, int U>
+__device__ __forceinline__ void load_run(const T *p, unsigned align, float (&o)[U]) {
+    if (align % (U * sizeof(T)) == 0) {
+        if constexpr (U * sizeof(T) == 32) {
+            const Words8 v = live_load(reinterpret_cast<const Words8 *>(p));
+#pragma unroll
+            for (int u = 0; u < U; ++u) o[u] = __uint_as_float(v.w[u]);
+        } else if constexpr (U * sizeof(T) == 16) {
+            RowLoad<T, U>::ld(p, o);
+        } else {   // four bf16 values
+            const uint2 v = live_load(reinterpret_cast<const uint2 *>(p));
+            o[0] = __uint_as_float(v.x << 16), o[1] = __uint_as_float(v.x & 0xFFFF0000u);
+            o[2] = __uint_as_float(v.y << 16), o[3] = __uint_as_float(v.y & 0xFFFF0000u);
+        }
+    } else {
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = to_float(p[u]);
+    }
+}
+template <int U>
+__device__ __forceinline__ void load_ints(const int32_t *p, unsigned align, int (&o)[U]) {
+    float t[U];
+    load_run<float, U>(reinterpret_cast<const float *>(p), align, t);
+#pragma unroll
+    for (int u = 0; u < U; ++u) o[u] = __float_as_int(t[u]);
+}
+
+// Rows without nonzeros have no writer among the runs: one share of them per warp.
+template <int N>
+__device__ __forceinline__ void coo_empty_rows(const CooArgs &a, int64_t share, int64_t shares) {
+    const int64_t rpc = (a.M + shares - 1) / shares;
+    for (int64_t rr = share * rpc + (threadIdx.x & 31); rr < min(a.M, (share + 1) * rpc); rr += 32)
+        if (__ldg(a.rowptr + rr) == __ldg(a.rowptr + rr + 1)) {
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                float *pc = a.C + rr * a.ldc + e;
                 *pc = (a.beta != 0.f) ? a.beta * *pc : 0.f;
             }
-        const int64_t k0 = c * CHUNK + lane * U;
-        int r[U], col[U];
-        float p[U];
-        if ((c + 1) * CHUNK <= a.count) {
+        }
+}
+
+template <typename T, int N, bool VEC, bool HOT, bool BITS>
+__global__ void __launch_bounds__(HOT ? kCooHotThreads : coo_threads(N), HOT ? 1 : (N == 1 ? 9 : 4))
+coo_kernel(const CooArgs a) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int U = coo_items(N), STEP = 32 * U;
+    extern __shared__ __align__(16) char coo_hot_raw[];
+    T *kept = reinterpret_cast<T *>(coo_hot_raw);
+    overlap_wait();
+    if constexpr (HOT) {
+        constexpr int AT = 16 / N;   // a thread fetches them in batches: one by one, 32,768 columns took 30 us
+        for (int i0 = threadIdx.x; i0 < a.hot; i0 += AT * kCooHotThreads) {
+            int c[AT];
+            float b[AT][N];
 #pragma unroll
-            for (int q = 0; q < U / 4; ++q) {
-                const int4 rv = __ldg(reinterpret_cast<const int4 *>(a.row + k0) + q), cv = __ldg(reinterpret_cast<const int4 *>(a.colind + k0) + q);
-                r[4 * q] = rv.x, r[4 * q + 1] = rv.y, r[4 * q + 2] = rv.z, r[4 * q + 3] = rv.w;
-                col[4 * q] = cv.x, col[4 * q + 1] = cv.y, col[4 * q + 2] = cv.z, col[4 * q + 3] = cv.w;
-            }
-            if constexpr (sizeof(T) == 4) {
+            for (int j = 0; j < AT; ++j) c[j] = i0 + j * kCooHotThreads < a.hot ? __ldg(a.hot_cols + i0 + j * kCooHotThreads) : -1;
 #pragma unroll
-                for (int q = 0; q < U / 4; ++q) {
-                    float t[4];
-                    RowLoad<T, 4>::ld(vals + k0 + 4 * q, t);
+            for (int j = 0; j < AT; ++j)
+                if (c[j] >= 0) coo_row_of_b<T, N, VEC>(b_row(static_cast<const T *>(a.B), c[j], a.ldb_bytes), b[j]);
 #pragma unroll
-                    for (int e = 0; e < 4; ++e) p[4 * q + e] = t[e];
-                }
-            } else {
-                RowLoad<T, 8>::ld(vals + k0, p);
-            }
-            float b[U];
+            for (int j = 0; j < AT; ++j)
+                if (c[j] >= 0)
 #pragma unroll
-            for (int u = 0; u < U; ++u) b[u] = gather(col[u]);
+                    for (int e = 0; e < N; ++e) kept[(i0 + j * kCooHotThreads) * N + e] = from_float<T>(b[j][e]);
+        }
+        __syncthreads();
+    }
+    const int lane = threadIdx.x & 31;
+    const int64_t steps = (a.count + STEP - 1) / STEP, all = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5, warps = min(all, steps);
+    // Many steps per warp: neighbouring ranges go to different CTAs, since what a range costs depends on its rows and columns (60 M
+    // nonzeros in rank-size rows 279 -> 271 us).  Few: to the same one, whose L1 they share (R-MAT scale 14 8.2 -> 7.7 us).
+    const int64_t w = HOT || steps >= 8 * all ? static_cast<int64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x
+                                              : (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    if (w >= warps) return;
+    const int64_t s0 = steps * w / warps, s1 = steps * (w + 1) / warps;
+    coo_empty_rows<N>(a, w, warps);
+    const T *vals = static_cast<const T *>(a.vals), *B = static_cast<const T *>(a.B);
+    const unsigned va = static_cast<unsigned>(reinterpret_cast<uintptr_t>(vals)), ca = static_cast<unsigned>(reinterpret_cast<uintptr_t>(a.colind));
+
+    auto emit = [&](int row, const float (&v)[N]) {
 #pragma unroll
-            for (int u = 0; u < U; ++u) p[u] *= b[u];
-        } else {   // items past the end continue the last row with zeros
-            const int pad_row = __ldg(a.row + a.count - 1);
+        for (int e = 0; e < N; ++e) {
+            float *pc = a.C + static_cast<int64_t>(row) * a.ldc + e;
+            *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v[e]) : a.alpha * v[e];
+        }
+    };
+    auto carry = [&](int which, int row, const float (&v)[N]) {
+        a.carry_row[2 * w + which] = row;
+#pragma unroll
+        for (int e = 0; e < N; ++e) a.carry_val[(2 * w + which) * N + e] = v[e];
+    };
+    const int first_row = BITS ? __ldg(a.row + s0 * 32) : __ldg(a.row + s0 * STEP);
+    int open_row = first_row;   // the row that reached the end of the step before ...
+    float open[N] = {};         // ... and its sum so far (both the same in all lanes)
+    for (int64_t s = s0; s < s1; ++s) {
+        const int64_t k0 = s * STEP + lane * U;
+        int col[U], r[U];
+        float av[U];
+        unsigned starts = 0;    // items that begin a row
+        int row_in = 0;         // the row that is open where the lane begins ...
+        int row_out = 0;        // ... and where it ends
+        const bool whole = (s + 1) * STEP <= a.count;   // the same in all lanes: no item is past the end
+        if (whole) {
+            load_ints<U>(a.colind + k0, ca, col);
+            if constexpr (!BITS) load_ints<U>(a.row + k0, 0, r);
+            load_run<T, U>(vals + k0, va, av);
+        } else {                // items past the end continue the last row with zeros
+            const int pad = BITS ? 0 : __ldg(a.row + a.count - 1);
 #pragma unroll
             for (int u = 0; u < U; ++u) {
                 const bool ok = k0 + u < a.count;
-                r[u] = ok ? __ldg(a.row + k0 + u) : pad_row;
-                p[u] = ok ? to_float(vals[k0 + u]) * gather(__ldg(a.colind + k0 + u)) : 0.f;
+                col[u] = ok ? __ldg(a.colind + k0 + u) : 0;
+                av[u] = ok ? to_float(vals[k0 + u]) : 0.f;
+                r[u] = BITS ? 0 : (ok ? __ldg(a.row + k0 + u) : pad);
             }
         }
-        const int first_row = __shfl_sync(FULL, r[0], 0);
-        auto emit = [&](int row, float v) {
-            float *pc = a.C + static_cast<int64_t>(row) * a.ldc;
-            *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v) : a.alpha * v;
-        };
-        // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
-        float sum = p[0], head = 0.f;
-        bool closed = false;
+        if constexpr (BITS) {
+            starts = __ldg(a.starts + s * 32 + lane);
+            row_in = __ldg(a.row + s * 32 + lane);
+            row_out = row_in + __popc(starts >> 1);
+            row_in -= starts & 1u;
+            if (s == s0 && lane == 0) {
+                row_in = first_row;
+                starts &= ~1u;
+            }
+        }
+        float b[U][N];
 #pragma unroll
-        for (int u = 1; u < U; ++u) {
-            if (r[u] != r[u - 1]) {
-                if (closed) emit(r[u - 1], sum);
-                else head = sum;
-                closed = true;
-                sum = 0.f;
+        for (int u = 0; u < U; ++u) {
+            if constexpr (HOT) {   // every lane reads a slot (the others slot 0), those outside also their row of B
+                const bool in = col[u] < 0;
+                const T *q = kept + (in ? col[u] & 0x7fffffff : 0) * N;
+                if constexpr (VEC && N == 2 && sizeof(T) == 4) {
+                    const float2 v = *reinterpret_cast<const float2 *>(q);
+                    b[u][0] = v.x, b[u][1] = v.y;
+                } else {
+#pragma unroll
+                    for (int e = 0; e < N; ++e) b[u][e] = to_float(q[e]);
+                }
+                if (!in) coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
+            } else {
+                coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
             }
-            sum += p[u];
         }
-        const int before = __shfl_up_sync(FULL, r[U - 1], 1);
-        const bool begins = lane == 0 || before != r[0];
-        const unsigned edges = __ballot_sync(FULL, begins), starts = __ballot_sync(FULL, begins || closed);
-        const int dist = lane - (31 - __clz(starts & (FULL >> (31 - lane))));
+        if (!whole)   // they gathered row 0: never let its contents (Inf, NaN) in
+#pragma unroll
+            for (int u = 0; u < U; ++u)
+                if (k0 + u >= a.count)
+#pragma unroll
+                    for (int e = 0; e < N; ++e) b[u][e] = 0.f;
+        if constexpr (!BITS) {
+            const int before = __shfl_up_sync(FULL, r[U - 1], 1);
+            row_in = lane == 0 ? open_row : before;
+            row_out = r[U - 1];
+            starts = r[0] != row_in;
+#pragma unroll
+            for (int u = 1; u < U; ++u) starts |= static_cast<unsigned>(r[u] != r[u - 1]) << u;
+        }
+        // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
+        float sum[N] = {}, top[N] = {};
+        bool closed = false;
+        int now = row_in;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (starts >> u & 1u) {
+                if (closed) emit(now, sum);
+#pragma unroll
+                for (int e = 0; e < N; ++e) {
+                    if (!closed) top[e] = sum[e];
+                    sum[e] = 0.f;
+                }
+                closed = true;
+                now = BITS ? now + 1 : r[u];
+            }
+#pragma unroll
+            for (int e = 0; e < N; ++e) sum[e] = fmaf(av[u], b[u][e], sum[e]);
+        }
+        if (lane == 0) {
+#pragma unroll
+            for (int e = 0; e < N; ++e) (closed ? top[e] : sum[e]) += open[e];
+        }
+        const unsigned ends = __ballot_sync(FULL, closed) & (FULL >> (31 - lane));
+        const int dist = lane - (ends ? 31 - __clz(ends) : 0);
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1)
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                const float up = __shfl_up_sync(FULL, sum[e], d);
+                if (dist >= d) sum[e] += up;
+            }
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            const float in = __shfl_up_sync(FULL, sum[e], 1);
+            if (lane > 0) top[e] += in;
+            open[e] = __shfl_sync(FULL, sum[e], 31);
+        }
+        open_row = __shfl_sync(FULL, row_out, 31);
+        if (closed) {
+            if (row_in == first_row) carry(0, row_in, top);
+            else emit(row_in, top);
+        }
+    }
+    if (lane == 0) {   // what is still open at the end of the range; one single row: (row, sum), (row, 0)
+        const float none[N] = {};
+        if (open_row == first_row) {
+            carry(0, open_row, open);
+            carry(1, open_row, none);
+        } else {
+            carry(1, open_row, open);
+        }
+    }
+}
+
+// The carry list, reduced the same way: a warp per 128 entries, one row-segmented scan per 32.  The entries it leaves over are
+// two per warp again.
+template <int N>
+__global__ void __launch_bounds__(256)
+coo_carry_kernel(const CooArgs a) {
+    constexpr unsigned FULL = 0xffffffffu;
+    constexpr int PER = kCooCarryChunk / 32;
+    overlap_wait();
+    const int lane = threadIdx.x & 31;
+    const int64_t c = (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
+    if (c * kCooCarryChunk >= a.count) return;
+    const float *pvals = static_cast<const float *>(a.vals);
+    const int64_t k0 = c * kCooCarryChunk + lane, last = a.count - 1;
+    int r[PER];
+    float p[PER][N];
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {   // written by the kernel before: no read-only loads; entries past the end continue the last row with zeros
+        const int64_t k = k0 + u * 32;
+        r[u] = a.row[min(k, last)];
+#pragma unroll
+        for (int e = 0; e < N; ++e) p[u][e] = k <= last ? pvals[k * N + e] : 0.f;
+    }
+    // A run is written when it closes: the run of the first row goes to the carry list (it may have begun earlier), every other
+    // one is a complete row.
+    const int first_row = __shfl_sync(FULL, r[0], 0);
+    auto emit = [&](int row, const float (&v)[N]) {
+        if (row == first_row) {
+            a.carry_row[2 * c] = row;
+#pragma unroll
+            for (int e = 0; e < N; ++e) a.carry_val[(2 * c) * N + e] = v[e];
+        } else {
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                float *pc = a.C + static_cast<int64_t>(row) * a.ldc + e;
+                *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v[e]) : a.alpha * v[e];
+            }
+        }
+    };
+    int crow = first_row;   // the run that reached the end of the previous 32 entries ...
+    float cval[N] = {};     // ... and its sum so far (both warp-uniform)
+#pragma unroll
+    for (int u = 0; u < PER; ++u) {
+        const int rp = __shfl_up_sync(FULL, r[u], 1);
+        const unsigned starts = __ballot_sync(FULL, lane == 0 || rp != r[u]);
+        const int my_start = 31 - __clz(starts & (FULL >> (31 - lane)));   // first lane of this lane's run
+        const int dist = lane - my_start;
 #pragma unroll
         for (int d = 1; d < 32; d <<= 1) {
-            const float up = __shfl_up_sync(FULL, sum, d);
-            if (dist >= d) sum += up;
-        }
-        const float in = __shfl_up_sync(FULL, sum, 1);
-        if (closed) {
-            if (!begins) head += in;
-            if (r[0] == first_row) {
-                a.carry_row[2 * c] = first_row;
-                a.carry_val[2 * c] = head;
-            } else {
-                emit(r[0], head);
+#pragma unroll
+            for (int e = 0; e < N; ++e) {
+                const float vu = __shfl_up_sync(FULL, p[u][e], d);
+                if (dist >= d) p[u][e] += vu;
             }
         }
-        if (lane < 31 && (edges >> (lane + 1) & 1u)) {   // a run that ends with the lane
-            if (r[U - 1] == first_row) {
-                a.carry_row[2 * c] = first_row;
-                a.carry_val[2 * c] = sum;
-            } else {
-                emit(r[U - 1], sum);
+        const bool cont = __shfl_sync(FULL, r[u], 0) == crow;
+        if (cont) {                 // the open run continues in the lanes of lane 0's run
+            if (my_start == 0) {
+#pragma unroll
+                for (int e = 0; e < N; ++e) p[u][e] += cval[e];
             }
+        } else if (lane == 0) {     // it ended exactly at the 32-entry boundary
+            emit(crow, cval);
         }
-        if (lane == 31) {   // what is still open at the end of the chunk; one single run: (row, sum), (row, 0)
-            const bool single = r[U - 1] == first_row;
-            a.carry_row[2 * c + 1] = r[U - 1];
-            a.carry_val[2 * c + 1] = single ? 0.f : sum;
-            if (single) {
-                a.carry_row[2 * c] = first_row;
-                a.carry_val[2 * c] = sum;
-            }
+        if (lane < 31 && ((starts >> (lane + 1)) & 1u)) emit(r[u], p[u]);   // runs that end inside these 32 entries
+        crow = __shfl_sync(FULL, r[u], 31);                                  // the run reaching lane 31 stays open
+#pragma unroll
+        for (int e = 0; e < N; ++e) cval[e] = __shfl_sync(FULL, p[u][e], 31);
+    }
+    if (lane == 0) {   // what is still open; all one run: (row, sum), (row, 0)
+        a.carry_row[2 * c + 1] = crow;
+        const bool single = crow == first_row;
+        if (single) a.carry_row[2 * c] = crow;
+#pragma unroll
+        for (int e = 0; e < N; ++e) {
+            if (single) a.carry_val[(2 * c) * N + e] = cval[e];
+            a.carry_val[(2 * c + 1) * N + e] = single ? 0.f : cval[e];
         }
     }
 }
@@ -377,17 +427,24 @@ __global__ void coo_final_kernel(const int32_t *row, const float *val, int64_t c
     }
 }
 
-// Row index of every nonzero (plan time).
-static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64_t M, int64_t nnz, int32_t *__restrict__ row) {
-    const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (k >= nnz) return;
+// Plan time: the row of every nonzero, or of every eighth.
+static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64_t M, int64_t nnz, int64_t every, int64_t count, int32_t *__restrict__ row) {
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, k = min(i * every, nnz - 1);
+    if (i >= count) return;
     int64_t lo = 0, hi = M;   // last row with rowptr[row] <= k
     while (hi - lo > 1) {
         const int64_t mid = (lo + hi) >> 1;
         if (rowptr[mid] <= k) lo = mid;
         else hi = mid;
     }
-    row[k] = static_cast<int32_t>(lo);
+    row[i] = static_cast<int32_t>(lo);
+}
+// A bit per nonzero that begins a row; every row has one (`starts` is cleared before).
+static __global__ void coo_starts_kernel(const int32_t *__restrict__ rowptr, int64_t M, unsigned *__restrict__ starts) {
+    const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    if (r >= M) return;
+    const unsigned k = static_cast<unsigned>(__ldg(rowptr + r));
+    atomicOr(starts + (k >> 5), 1u << (k & 31));
 }
 
 }  // namespace sd

@@ -43,20 +43,20 @@ cudaError_t run_scale_c(float *C, int64_t ldc, int64_t M, int32_t N, float beta,
 cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st);
 
 // Family (b) for dense widths up to kCooMaxN (beyond it the shuffles per nonzero outweigh the
-// gain; measured cross-over between 4 and 8 columns): segmented reduction over the nonzeros with an
-// explicit row index per nonzero, carries reduced in two more levels.
+// gain; measured cross-over between 4 and 8 columns): segmented reduction over the nonzeros, carries reduced in two more levels.
 constexpr int kCooMaxN = 4;
-// nonzeros per warp step: 8 per lane at one or two columns (the gathers are 4 or 8 bytes: more of them
-// must be in flight; measured), 4 per lane at three or four; carry lists are always cut into 128-entry chunks
-constexpr int coo_chunk(int N) { return N <= 2 ? 256 : 128; }
+constexpr int coo_items(int N) { return N <= 2 ? 8 : 4; }   // nonzeros of a lane and step
+constexpr int64_t coo_steps(int64_t nnz, int N) { return (nnz + 32 * coo_items(N) - 1) / (32 * coo_items(N)); }
 constexpr int kCooCarryChunk = 128;
 constexpr int64_t kCooDirectFinal = 4096;  // carry lists up to this length skip the second level
+constexpr int kCooMaxWarps = 64;           // resident on one SM; each leaves two carry entries
 struct CooPlan {
-    const int32_t *row;   // [nnz] row of every nonzero
+    const int32_t *row;    // [nnz] row of every nonzero, or with `starts` [32 steps] of every eighth
+    const uint8_t *starts; // [32 steps] a bit per nonzero that begins a row
     const int32_t *rowptr; // [M + 1]
     int64_t M;             // rows to search for empty ones (0: the matrix has none)
     int64_t nnz;
-    int32_t *c1_row;      // [2 * ceil(nnz / coo_chunk(N))] first-level carries
+    int32_t *c1_row;      // [2 * min(steps, kCooMaxWarps * SMs)] first-level carries
     float *c1_val;        // ... x N
     int32_t *c2_row;      // [2 * ceil(len(c1) / kCooCarryChunk)] second-level carries
     float *c2_val;
@@ -65,8 +65,9 @@ struct CooPlan {
     int32_t hot;
 };
 constexpr int kCooHotBytes = 128 * 1024;   // the rest is L1 for the gathers outside: with 200 KB two fp32 columns took 281 us instead of 173
-cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, bool vec, int sm_count, cudaStream_t st);
-cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int32_t *row, cudaStream_t st);
+cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, int sm_count, cudaStream_t st);
+// starts != nullptr: a bit per nonzero and the row of every eighth; no row is empty.
+cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st);
 
 struct BsrArgs {
     const int32_t *browptr;  // [Mb + 1]

@@ -1,3 +1,5 @@
+#include <algorithm>
+
 #include "sd_launch.cuh"
 #include "sd_merge.cuh"
 #include "sd_coo.cuh"
@@ -12,23 +14,35 @@ cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st) {
 }
 
 // ---- narrow dense operands: COO segmented reduction --------------------------------------------
-template <typename T, int N>
-static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, bool vec, int sm_count, cudaStream_t st) {
-    const int64_t chunks1 = (cp.nnz + coo_chunk(N) - 1) / coo_chunk(N);
-    const int64_t count2 = 2 * chunks1;
-    const int64_t chunks2 = (count2 + kCooCarryChunk - 1) / kCooCarryChunk;
-    const int64_t count3 = 2 * chunks2;
-    // persistent grid: the CTAs that are resident together (the registers of the instance decide)
-    static std::atomic<int> occ_vec[kMaxDevices], occ_plain[kMaxDevices];
-    const int occ = vec ? occupancy_cached(occ_vec, coo_reduce_kernel<T, N, true, false>, 256)
-                        : occupancy_cached(occ_plain, coo_reduce_kernel<T, N, false, false>, 256);
-    auto grid_for = [&](int64_t chunks) {
-        const int64_t want = (chunks + 7) / 8;   // 8 warps per CTA, one chunk per warp step
-        const int64_t cap = static_cast<int64_t>(sm_count) * occ;
-        return static_cast<unsigned>(want < cap ? (want > 0 ? want : 1) : cap);
-    };
+// One instance: the grid is as many CTAs as are resident together, or as give every warp a step.  Returns the warps that work.
+template <typename T, int N, bool VEC, bool HOT, bool BITS>
+static cudaError_t launch_coo_kernel(const CooArgs &a, int sm_count, int kept, cudaStream_t st, int64_t &warps) {
+    auto kernel = coo_kernel<T, N, VEC, HOT, BITS>;
+    constexpr int threads = HOT ? kCooHotThreads : coo_threads(N);
+    int64_t ctas = sm_count;
+    if constexpr (HOT) {
+        static std::atomic<bool> opted[kMaxDevices];
+        const int dev = current_device();
+        if (dev >= kMaxDevices || !opted[dev].load(std::memory_order_acquire)) {
+            const cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCooHotBytes);
+            if (e != cudaSuccess) return e;
+            if (dev < kMaxDevices) opted[dev].store(true, std::memory_order_release);
+        }
+    } else {
+        static std::atomic<int> occ[kMaxDevices];
+        ctas *= std::min(occupancy_cached(occ, kernel, threads), kCooMaxWarps * 32 / threads);
+    }
+    const int64_t steps = coo_steps(a.count, N);
+    ctas = std::min(ctas, (steps + threads / 32 - 1) / (threads / 32));
+    warps = std::min(ctas * (threads / 32), steps);
+    return launch_overlapped(kernel, static_cast<unsigned>(ctas), threads, kept, st, a);
+}
+
+template <typename T, int N, bool VEC>
+static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, int sm_count, cudaStream_t st) {
     CooArgs a{};
     a.row = cp.row;
+    a.starts = cp.starts;
     a.colind = s.colind;
     a.vals = s.vals;
     a.B = s.B;
@@ -43,71 +57,74 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, bool vec, 
     a.carry_row = cp.c1_row;
     a.carry_val = cp.c1_val;
     cudaError_t e;
+    int64_t warps = 0;
     const int kept = cp.hot * N * static_cast<int>(sizeof(T));
-    if (cp.hot > 0 && kept <= kCooHotBytes) {
-        auto kernel = vec ? coo_reduce_kernel<T, N, true, false, true> : coo_reduce_kernel<T, N, false, false, true>;
-        static std::atomic<bool> opted[kMaxDevices][2];
-        const int dev = current_device();
-        if (dev >= kMaxDevices || !opted[dev][vec].load(std::memory_order_acquire)) {
-            if ((e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kCooHotBytes)) != cudaSuccess) return e;
-            if (dev < kMaxDevices) opted[dev][vec].store(true, std::memory_order_release);
-        }
+    const bool hot = cp.hot > 0 && kept <= kCooHotBytes;
+    if (hot) {
         a.colind = cp.hot_colind;
         a.hot_cols = cp.hot_cols;
         a.hot = cp.hot;
-        e = launch_overlapped(kernel, static_cast<unsigned>(sm_count), kCooHotThreads, kept, st, a);
-    } else if (N == 1 && (sizeof(T) == 2 || cp.nnz < 16000000) &&
-               ((reinterpret_cast<uintptr_t>(a.colind) | reinterpret_cast<uintptr_t>(a.vals) | reinterpret_cast<uintptr_t>(a.row)) & 15u) == 0) {
-        // fp32 on the largest matrices stays with the other kernel: there a warp's gathers of neighbouring nonzeros share more
-        // lines of B than those of every eighth (32.4 M nonzeros 121 against 126 us, 8.1 M 44 against 42).  The cause is B's size
-        // against L1 and the order of the columns; the line by nonzeros rests on these two R-MAT matrices.
-        static std::atomic<int> occ_serial[kMaxDevices];
-        const int64_t want = (chunks1 + 7) / 8, cap = static_cast<int64_t>(sm_count) * occupancy_cached(occ_serial, coo_serial_kernel<T>, 256);
-        e = launch_overlapped(coo_serial_kernel<T>, static_cast<unsigned>(want < cap ? want : cap), 256, 0, st, a);
+    }
+    if constexpr (N == 1) {
+        if (cp.starts)
+            e = hot ? launch_coo_kernel<T, N, VEC, true, true>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, true>(a, sm_count, 0, st, warps);
+        else
+            e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, warps);
     } else {
-        e = launch_overlapped(vec ? coo_reduce_kernel<T, N, true, false> : coo_reduce_kernel<T, N, false, false>, grid_for(chunks1), 256, 0, st, a);
+        e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, warps);
     }
     if (e != cudaSuccess) return e;
     const int32_t *frow = cp.c1_row;
     const float *fval = cp.c1_val;
-    int64_t fcount = count2;
-    if (count2 > kCooDirectFinal) {   // level 2: the carry list is reduced the same way
+    int64_t fcount = 2 * warps;
+    if (fcount > kCooDirectFinal) {   // level 2
+        const int64_t chunks = (fcount + kCooCarryChunk - 1) / kCooCarryChunk;
         CooArgs b = a;
         b.row = cp.c1_row;
-        b.colind = nullptr;
         b.vals = cp.c1_val;
-        b.B = nullptr;
-        b.count = count2;
+        b.count = fcount;
         b.carry_row = cp.c2_row;
         b.carry_val = cp.c2_val;
-        if ((e = launch_overlapped(coo_reduce_kernel<float, N, false, true>, grid_for(chunks2), 256, 0, st, b)) != cudaSuccess) return e;
+        if ((e = launch_overlapped(coo_carry_kernel<N>, static_cast<unsigned>((chunks + 7) / 8), 256, 0, st, b)) != cudaSuccess) return e;
         frow = cp.c2_row;
         fval = cp.c2_val;
-        fcount = count3;
+        fcount = 2 * chunks;
     }
     return launch_overlapped(coo_final_kernel<N>, static_cast<unsigned>((fcount + 255) / 256), 256, 0, st, frow, fval, fcount, s.C, s.ldc, s.alpha,
                              s.beta);
 }
 
+template <typename T, int N>
+static cudaError_t launch_coo_vec(const CooPlan &cp, const SpmmArgs &s, int sm_count, cudaStream_t st) {
+    constexpr uintptr_t bytes = N * sizeof(T);   // of a row of B: one load if all of them start at a multiple
+    if ((reinterpret_cast<uintptr_t>(s.B) | s.ldb_bytes) % bytes == 0) return launch_coo_n<T, N, true>(cp, s, sm_count, st);
+    return launch_coo_n<T, N, false>(cp, s, sm_count, st);
+}
+
 template <typename T>
-static cudaError_t launch_coo(const CooPlan &cp, const SpmmArgs &s, bool vec, int sm_count, cudaStream_t st) {
+static cudaError_t launch_coo(const CooPlan &cp, const SpmmArgs &s, int sm_count, cudaStream_t st) {
     switch (s.N) {
-    case 1: return launch_coo_n<T, 1>(cp, s, false, sm_count, st);
-    case 2: return launch_coo_n<T, 2>(cp, s, false, sm_count, st);
-    case 3: return launch_coo_n<T, 3>(cp, s, false, sm_count, st);
-    case 4: return launch_coo_n<T, 4>(cp, s, vec && sizeof(T) == 4, sm_count, st);
+    case 1: return launch_coo_n<T, 1, false>(cp, s, sm_count, st);
+    case 2: return launch_coo_vec<T, 2>(cp, s, sm_count, st);
+    case 3: return launch_coo_n<T, 3, false>(cp, s, sm_count, st);
+    case 4: return launch_coo_vec<T, 4>(cp, s, sm_count, st);
     default: return cudaErrorInvalidValue;
     }
 }
 
-// `vec`: B is 16-byte aligned and its row pitch a multiple of 16 bytes.
-cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, bool vec, int sm_count, cudaStream_t st) {
-    return dtype == SD_F32 ? launch_coo<float>(cp, s, vec, sm_count, st) : launch_coo<__nv_bfloat16>(cp, s, vec, sm_count, st);
+cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, int sm_count, cudaStream_t st) {
+    return dtype == SD_F32 ? launch_coo<float>(cp, s, sm_count, st) : launch_coo<__nv_bfloat16>(cp, s, sm_count, st);
 }
 
-cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int32_t *row, cudaStream_t st) {
+cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st) {
     if (nnz == 0) return cudaSuccess;
-    coo_rows_kernel<<<static_cast<unsigned>((nnz + 255) / 256), 256, 0, st>>>(rowptr, M, nnz, row);
+    const int64_t count = starts ? 32 * steps : nnz;
+    coo_rows_kernel<<<static_cast<unsigned>((count + 255) / 256), 256, 0, st>>>(rowptr, M, nnz, starts ? 8 : 1, count, row);
+    if (starts) {
+        const cudaError_t e = cudaMemsetAsync(starts, 0, 32 * steps, st);
+        if (e != cudaSuccess) return e;
+        coo_starts_kernel<<<static_cast<unsigned>((M + 255) / 256), 256, 0, st>>>(rowptr, M, reinterpret_cast<unsigned *>(starts));
+    }
     return cudaGetLastError();
 }
 

@@ -59,3 +59,26 @@ def test_one_column_runs_and_aligned_arrays(edges, offset, dtype):
     got, _ = run_spmm(plan, w, c_fill=np.full((w.M, 1), np.nan, np.float32), beta=0.0)
     check(w, got, beta=0.0)
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [1, 2, 3, 4])
+@pytest.mark.parametrize("M,length,empty", [(1, 3, 0), (1, 700000, 0), (40, 1, 0), (3, 256, 0), (5, 129, 1), (9000, 61, 0), (700000, 1, 0), (60000, 9, 7)])
+def test_ranges_of_warps(M, length, empty, N, dtype):
+    """One to thousands of warps with a step each or several: a single row over all of them, rows that end with a lane's items, a
+    step or a range, rows of one nonzero, empty rows (every seventh), the last step partly filled; operands at any offset."""
+    lengths = np.full(M, length)
+    lengths[::5] += 3 if length > 1 else 0
+    if empty:
+        lengths[1::7] = 0
+    K = 1500000 if M == 1 else 4000
+    w = W.random_csr(M, K, N, lengths, seed=M + N, dtype=dtype, alpha=1.25, beta=-0.5)
+    plan = DeviceWorkload(w).plan(family=sd.SD_MERGE)
+    for kw in (dict(), dict(pad_b=4 - N, pad_c=1), dict(offset=1)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
+    got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
