@@ -9,8 +9,9 @@
 
 namespace sd {
 
-// Per-lane view of B and C for one column slab.
-template <typename T, int VW, int LPR, int NV>
+// Per-lane view of B and C for one column slab.  EXACT: every lane has columns in every slab, so no gather is tested (a tested
+// one clears its registers first: five instructions more).
+template <typename T, int VW, int LPR, int NV, bool EXACT = false>
 struct LaneCols {
     const T *B;
     int cbase;
@@ -27,7 +28,7 @@ struct LaneCols {
         const T *row = b_row(B, col, ldb_bytes);
 #pragma unroll
         for (int v = 0; v < NV; ++v) {
-            if (use && ok[v]) b[v].ld(row + v * LPR * VW);
+            if (use && (EXACT || ok[v])) b[v].ld(row + v * LPR * VW);
             else b[v].zero();
         }
     }
@@ -38,7 +39,7 @@ struct LaneCols {
     __device__ __forceinline__ void store(float *crow, const float (&acc)[NV][VW], float alpha, float beta) const {
 #pragma unroll
         for (int v = 0; v < NV; ++v)
-            if (ok[v]) store_cols<VW>(crow + cbase + v * LPR * VW, acc[v], alpha, beta);
+            if (EXACT || ok[v]) store_cols<VW>(crow + cbase + v * LPR * VW, acc[v], alpha, beta);
     }
 };
 
@@ -62,20 +63,30 @@ __device__ __forceinline__ void sum_sets(float (&acc)[NV][VW], unsigned mask) {
 }
 
 // Nonzeros [p0, p1) by a group of LANES lanes.  A step loads NB x LANES (column, value) pairs, one coalesced load of each
-// per NB, and requests the next step's before this step's gathers; set k of the group takes pairs k, k + G, ... of a load,
-// handed round by shuffle.  Q gathers of a lane are in flight together.  Whole steps run without any test; only the
+// per NB, and requests the next step's before this step's gathers.  The pairs go round through shared memory: four columns or
+// four values per 16-byte load, which all lanes of a set read together, cost a quarter of the instructions and of the L1 cycles of
+// as many shuffles.  Q gathers of a lane are in flight together.  Whole steps run without any test; only the
 // last, partly filled one tests every pair: nothing may be gathered for a pair beyond the end (row 0 of B may hold
 // non-finite values, and 0 * Inf is NaN).
-template <typename T, int VW, int LPR, int NV, int LANES, typename Args>
-__device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, LPR, NV> &lc, int p0, int p1,
-                                          unsigned mask, float (&acc)[NV][VW]) {
+template <int LPR> constexpr int kGroupLoads = LPR >= 4 ? 1 : 4 / LPR;   // loads of pairs per step: at least four gathers per lane and step
+template <int THREADS, int LPR>
+struct GroupStage {   // of a CTA; nothing is handed round where every lane has its own nonzeros
+    static constexpr int N = LPR == 1 ? 1 : THREADS * kGroupLoads<LPR>;
+    alignas(16) int col[N];
+    alignas(16) float val[N];
+};
+template <typename T, int VW, int LPR, int NV, int LANES, bool EXACT, typename Args, int THREADS>
+__device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, LPR, NV, EXACT> &lc, GroupStage<THREADS, LPR> &stage, int p0,
+                                          int p1, unsigned mask, float (&acc)[NV][VW]) {
     constexpr int G = LANES / LPR;
-    constexpr int NB = LPR >= 4 ? 1 : 4 / LPR;          // loads of pairs per step: at least four gathers per lane and step
+    constexpr int NB = kGroupLoads<LPR>;
     constexpr int PER = NB * LPR;                       // gathers of a lane per step
     constexpr int QM = NV * VW * sizeof(T) > 16 ? 4 : 8;
     constexpr int Q = PER < QM ? PER : QM;
     const T *vals = static_cast<const T *>(a.vals);
     const int lg = threadIdx.x % LANES, k = lg / LPR;
+    int *const cols = LPR == 1 ? nullptr : stage.col + threadIdx.x / LANES * (LANES * NB);
+    float *const ws = LPR == 1 ? nullptr : stage.val + threadIdx.x / LANES * (LANES * NB);
     int c[NB];
     float w[NB];
     auto fetch = [&](int p) {
@@ -88,12 +99,17 @@ __device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, L
     };
     auto step = [&](int p, auto whole_tag) {
         constexpr bool WHOLE = decltype(whole_tag)::value;
-        int cc[NB];
-        float cw[NB];
+        // LPR == 1: every lane has its own four
+        const int4 own_col = make_int4(c[0], c[1 % NB], c[2 % NB], c[3 % NB]);
+        const float4 own_val = make_float4(w[0], w[1 % NB], w[2 % NB], w[3 % NB]);
+        if constexpr (LPR > 1) {
+            __syncwarp(mask);   // the step before has been read
 #pragma unroll
-        for (int n = 0; n < NB; ++n) {
-            cc[n] = c[n];
-            cw[n] = w[n];
+            for (int n = 0; n < NB; ++n) {
+                cols[n * LANES + lg] = c[n];
+                ws[n * LANES + lg] = w[n];
+            }
+            __syncwarp(mask);
         }
         constexpr int QS = WHOLE || Q < 4 ? Q : 4;
         if (WHOLE) fetch(p + NB * LANES);
@@ -102,15 +118,18 @@ __device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, L
             if (!WHOLE && p + i0 * G >= p1) break;
             Piece<T, VW> b[QS][NV];
 #pragma unroll
-            for (int u = 0; u < QS; ++u) {
-                const int n = NB == 1 ? 0 : u / LPR, src = NB == 1 ? (i0 + u) * G + k : u % LPR * G + k;
-                const int col = LPR == 1 ? cc[n] : __shfl_sync(mask, cc[n], src, LANES);
-                lc.gather(col, a.ldb_bytes, WHOLE || col >= 0, b[u]);
+            for (int u = 0; u < QS; u += 4) {   // set k takes pairs 4k .. 4k + 3 of every 4 G
+                const int4 x = LPR == 1 ? own_col : *reinterpret_cast<const int4 *>(cols + (i0 + u) * G + 4 * k);
+                const int col[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int v = 0; v < 4; ++v) lc.gather(col[v], a.ldb_bytes, WHOLE || col[v] >= 0, b[u + v]);
             }
 #pragma unroll
-            for (int u = 0; u < QS; ++u) {
-                const int n = NB == 1 ? 0 : u / LPR, src = NB == 1 ? (i0 + u) * G + k : u % LPR * G + k;
-                lc.fma(LPR == 1 ? cw[n] : __shfl_sync(mask, cw[n], src, LANES), b[u], acc);
+            for (int u = 0; u < QS; u += 4) {
+                const float4 x = LPR == 1 ? own_val : *reinterpret_cast<const float4 *>(ws + (i0 + u) * G + 4 * k);
+                const float wv[4] = {x.x, x.y, x.z, x.w};
+#pragma unroll
+                for (int v = 0; v < 4; ++v) lc.fma(wv[v], b[u + v], acc);
             }
         }
     };

@@ -8,7 +8,7 @@
 //   short    rows of fewer nonzeros, several per lane group (light_rows_body).
 //
 // What bounds it: on large matrices the rate at which L2 and L1 deliver gathered rows of B (64 bf16 columns, R-MAT scale
-// 20: 402 us = 10.3 TB/s, where one lane set per row and half as many gathers in flight took 481), on small ones the chain
+// 20: 402 us = 10.3 TB/s with pairs handed round by shuffle; scale 19 since then 207 -> 175), on small ones the chain
 // of dependent gathers of the longest item, which the lane sets cut (8 columns, 128 nonzeros: 64 steps of a pair of lanes
 // before, 2 steps of a warp now; R-MAT scale 14: 51 -> 9 us).
 #pragma once
@@ -41,18 +41,18 @@ struct HybridArgs {
     float alpha, beta;
 };
 
-template <typename T, int VW, int LPR, int NV, int LANES>
-__device__ __forceinline__ void items_body(const HybridArgs &a, unsigned bx) {
+template <typename T, int VW, int LPR, int NV, int LANES, bool EXACT>
+__device__ __forceinline__ void items_body(const HybridArgs &a, unsigned bx, GroupStage<kHybridThreads, LPR> &stage) {
     const int lane = threadIdx.x & 31, lg = threadIdx.x % LANES;
     const unsigned mask = LANES == 32 ? 0xffffffffu : ((1u << LANES % 32) - 1u) << (lane & ~(LANES - 1));
-    const LaneCols<T, VW, LPR, NV> lc(a.B, a.N, lg % LPR);
+    const LaneCols<T, VW, LPR, NV, EXACT> lc(a.B, a.N, lg % LPR);
     const int32_t stride = static_cast<int32_t>(a.gc) * (kHybridThreads / LANES), n = a.chunks + a.wide;
     for (int32_t s = (static_cast<int32_t>(bx) * kHybridThreads + static_cast<int32_t>(threadIdx.x)) / LANES; s < n; s += stride) {
         const bool chunk = s < a.chunks;
         const int4 d = __ldg(chunk ? a.items + s : a.desc + (s - a.chunks));
         float acc[NV][VW];
         clear_acc(acc);
-        group_sum<T, VW, LPR, NV, LANES>(a, lc, d.y, d.y + d.w, mask, acc);
+        group_sum<T, VW, LPR, NV, LANES, EXACT>(a, lc, stage, d.y, d.y + d.w, mask, acc);
         if (lg < LPR) {
             if (chunk && d.x >= 0) lc.store(a.scratch + static_cast<int64_t>(d.x) * a.N, acc, 1.f, 0.f);
             else lc.store(a.C + (d.x & 0x7FFFFFFF) * a.ldc, acc, a.alpha, a.beta);   // a light row, or a heavy row of one item
@@ -60,19 +60,19 @@ __device__ __forceinline__ void items_body(const HybridArgs &a, unsigned bx) {
     }
 }
 
-template <typename T, int VW, int LPR, int NV>
-__device__ __forceinline__ void medium_body(const HybridArgs &a, unsigned bx) {
+template <typename T, int VW, int LPR, int NV, bool EXACT>
+__device__ __forceinline__ void medium_body(const HybridArgs &a, unsigned bx, GroupStage<kHybridThreads, LPR> &stage) {
     constexpr int LANES = LPR < 8 ? 8 : LPR;
     const int lane = threadIdx.x & 31, lg = threadIdx.x % LANES;
     const unsigned mask = LANES == 32 ? 0xffffffffu : ((1u << LANES % 32) - 1u) << (lane & ~(LANES - 1));
-    const LaneCols<T, VW, LPR, NV> lc(a.B, a.N, lg % LPR);
+    const LaneCols<T, VW, LPR, NV, EXACT> lc(a.B, a.N, lg % LPR);
     const int4 *__restrict__ desc = a.desc + a.wide;
     const int32_t stride = static_cast<int32_t>(a.gm) * (kHybridThreads / LANES);
     for (int32_t s = (static_cast<int32_t>(bx) * kHybridThreads + static_cast<int32_t>(threadIdx.x)) / LANES; s < a.medium; s += stride) {
         const int4 cur = __ldg(desc + s);
         float acc[NV][VW];
         clear_acc(acc);
-        group_sum<T, VW, LPR, NV, LANES>(a, lc, cur.y, cur.y + cur.w, mask, acc);
+        group_sum<T, VW, LPR, NV, LANES, EXACT>(a, lc, stage, cur.y, cur.y + cur.w, mask, acc);
         if (lg < LPR) lc.store(a.C + cur.x * a.ldc, acc, a.alpha, a.beta);
     }
 }
@@ -83,9 +83,9 @@ __device__ __forceinline__ void medium_body(const HybridArgs &a, unsigned bx) {
 // nothing else (two dependent memory round trips per one-nonzero row: descriptor, row of B), and the (column, value)
 // pair of step j + 1 is requested before the gathers of step j.  The lanes of a group read the same pair with one
 // broadcast load.  Rows without nonzeros are written too (C = beta * C).
-template <typename T, int VW, int LPR, int NV, int R>
+template <typename T, int VW, int LPR, int NV, int R, bool EXACT>
 __device__ __forceinline__ void light_rows_body(const HybridArgs &a, unsigned bx) {
-    const LaneCols<T, VW, LPR, NV> lc(a.B, a.N, threadIdx.x % LPR);
+    const LaneCols<T, VW, LPR, NV, EXACT> lc(a.B, a.N, threadIdx.x % LPR);
     const int64_t r0 = (static_cast<int64_t>(bx) * kHybridThreads + threadIdx.x) / LPR * R;
     if (r0 >= a.light) return;
     const T *vals = static_cast<const T *>(a.vals);
@@ -130,20 +130,21 @@ __device__ __forceinline__ void light_rows_body(const HybridArgs &a, unsigned bx
 // short rows.  CTAs are placed in index order, so the item CTAs take the SMs first and the others fill in as they
 // retire: what side streams and a high stream priority would give, without depending on how streams map to the GPU's
 // hardware queues.
-template <typename T, int VW, int LPR, int NV, int IL, int R>
+template <typename T, int VW, int LPR, int NV, int IL, int R, bool EXACT>
 __global__ void __launch_bounds__(kHybridThreads, 4)
 hybrid_kernel(const HybridArgs a) {
+    __shared__ GroupStage<kHybridThreads, LPR> stage;
     overlap_wait();
-    if (blockIdx.x < a.gc) items_body<T, VW, LPR, NV, IL>(a, blockIdx.x);
-    else if (blockIdx.x < a.gc + a.gm) medium_body<T, VW, LPR, NV>(a, blockIdx.x - a.gc);
-    else light_rows_body<T, VW, LPR, NV, R>(a, blockIdx.x - a.gc - a.gm);
+    if (blockIdx.x < a.gc) items_body<T, VW, LPR, NV, IL, EXACT>(a, blockIdx.x, stage);
+    else if (blockIdx.x < a.gc + a.gm) medium_body<T, VW, LPR, NV, EXACT>(a, blockIdx.x - a.gc, stage);
+    else light_rows_body<T, VW, LPR, NV, R, EXACT>(a, blockIdx.x - a.gc - a.gm);
     overlap_next();
 }
 
-template <typename T, int VW, int LPR, int NV, int IL>
-cudaError_t launch_hybrid_il(HybridArgs a, cudaStream_t st) {
+template <typename T, int VW, int LPR, int NV, int IL, bool EXACT>
+cudaError_t launch_hybrid_exact(HybridArgs a, cudaStream_t st) {
     constexpr int R = NV * VW >= 8 ? 2 : 4;
-    auto kernel = hybrid_kernel<T, VW, LPR, NV, IL, R>;
+    auto kernel = hybrid_kernel<T, VW, LPR, NV, IL, R, EXACT>;
     static std::atomic<int> occ_cache[kMaxDevices];
     const int64_t cap = static_cast<int64_t>(sm_count_cached()) * occupancy_cached(occ_cache, kernel, kHybridThreads);
     constexpr int items_per_cta = kHybridThreads / IL, medium_per_cta = kHybridThreads / (LPR < 8 ? 8 : LPR);
@@ -158,6 +159,14 @@ cudaError_t launch_hybrid_il(HybridArgs a, cudaStream_t st) {
     constexpr int slab = LPR * NV * VW;
     return launch_overlapped(kernel, dim3(static_cast<unsigned>(total), static_cast<unsigned>((a.N + slab - 1) / slab)),
                              kHybridThreads, 0, st, a);
+}
+
+// Whole loads and every lane a column in every slab (8, 16, 32, ... columns): the lanes need no test.
+template <typename T, int VW, int LPR, int NV, int IL>
+cudaError_t launch_hybrid_il(const HybridArgs &a, cudaStream_t st) {
+    if constexpr (VW * sizeof(T) == 16)
+        if (a.N % (LPR * NV * VW) == 0) return launch_hybrid_exact<T, VW, LPR, NV, IL, true>(a, st);
+    return launch_hybrid_exact<T, VW, LPR, NV, IL, false>(a, st);
 }
 
 // Lanes per item.  A whole warp as long as half warps would not all get an item (the chain of dependent gathers is what

@@ -26,10 +26,8 @@ template <> struct Piece<float, 4> {
     __device__ __forceinline__ void ld(const float *p) { r = live_load(reinterpret_cast<const float4 *>(p)); }
     __device__ __forceinline__ void zero() { r = make_float4(0.f, 0.f, 0.f, 0.f); }
     __device__ __forceinline__ void fma(float a, float (&acc)[4]) const {
-        acc[0] = fmaf(a, r.x, acc[0]);
-        acc[1] = fmaf(a, r.y, acc[1]);
-        acc[2] = fmaf(a, r.z, acc[2]);
-        acc[3] = fmaf(a, r.w, acc[3]);
+        fma_pair(acc[0], acc[1], a, r.x, r.y);
+        fma_pair(acc[2], acc[3], a, r.z, r.w);
     }
 };
 template <> struct Piece<float, 2> {

@@ -11,7 +11,7 @@ namespace sd {
 constexpr int kRowGroupThreads = 256;
 constexpr int kRowGroupTerms = 512;
 
-template <typename T, int VW, int LPR, int NV, int LANES>
+template <typename T, int VW, int LPR, int NV, int LANES, bool EXACT>
 __global__ void __launch_bounds__(kRowGroupThreads, 5)
 rowgroup_kernel(const SpmmArgs a) {
     const int lane = threadIdx.x & 31, lg = threadIdx.x % LANES;
@@ -23,10 +23,11 @@ rowgroup_kernel(const SpmmArgs a) {
         p1 = __ldg(a.ptr + row + 1);
     }
     overlap_wait();
-    const LaneCols<T, VW, LPR, NV> lc(a.B, a.N, lg % LPR);
+    __shared__ GroupStage<kRowGroupThreads, LPR> stage;
+    const LaneCols<T, VW, LPR, NV, EXACT> lc(a.B, a.N, lg % LPR);
     float acc[NV][VW];
     clear_acc(acc);
-    group_sum<T, VW, LPR, NV, LANES>(a, lc, p0, p1, mask, acc);
+    group_sum<T, VW, LPR, NV, LANES, EXACT>(a, lc, stage, p0, p1, mask, acc);
     overlap_next();
     if (row < a.S && lg < LPR) lc.store(a.C + row * a.ldc, acc, a.alpha, a.beta);
 }
@@ -34,8 +35,10 @@ rowgroup_kernel(const SpmmArgs a) {
 template <typename T, int VW, int LPR, int NV, int LANES>
 cudaError_t launch_rowgroup_lanes(const SpmmArgs &a, cudaStream_t st) {
     constexpr int rows = kRowGroupThreads / LANES, slab = LPR * NV * VW;
-    return launch_overlapped(rowgroup_kernel<T, VW, LPR, NV, LANES>,
-                             dim3(static_cast<unsigned>((a.S + rows - 1) / rows), static_cast<unsigned>((a.N + slab - 1) / slab)),
+    auto kernel = rowgroup_kernel<T, VW, LPR, NV, LANES, false>;
+    if constexpr (VW * sizeof(T) == 16)
+        if (a.N % slab == 0) kernel = rowgroup_kernel<T, VW, LPR, NV, LANES, true>;
+    return launch_overlapped(kernel, dim3(static_cast<unsigned>((a.S + rows - 1) / rows), static_cast<unsigned>((a.N + slab - 1) / slab)),
                              kRowGroupThreads, 0, st, a);
 }
 
