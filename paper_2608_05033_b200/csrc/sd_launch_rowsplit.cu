@@ -6,31 +6,43 @@
 
 namespace sd {
 
-// Lane sets per row of the row-group kernel, or 0 where the kernels below are ahead.  Measured on uniform rows of 5 to 128
-// nonzeros, stencils and blocks, 5 to 128 columns, both value types:
+// Lane sets per row of the row-group kernel, or 0 where the kernels below are ahead.  Measured on Poisson rows of 3 to 44 nonzeros
+// (40,000 to 1 M of them), 5-point stencils and blocks (125 to 131 per row), 8 to 256 columns, both value types.  Some of it, us: the
+// kernels below / one set / four sets
 //   not whole 16-byte loads   always (41 columns: 1.8 to 3.9 times as fast as one scalar per lane)
 //   few rows                  four sets as soon as rows are 8 long: one set leaves the GPU idle (5,000 rows of 30 at 64 columns
 //                             17.9 -> 5.3 us, at 128 bf16 24.9 -> 6.7)
-//   narrow and short          up to eight loads per row of B and below 16 nonzeros, where a row is over before sets pay (800,000
-//                             rows of 12 at 64 bf16 columns 359 -> 227 us, at 32 fp32 columns 222 -> 192); stencil rows of fp32
-//                             values keep the plain kernel (7.9 against 9.2 us at 8 columns)
-//   8 columns                 four sets up to 64 nonzeros (rows of 30: fp32 19.7 -> 17.2, bf16 25.7 -> 15.9)
-//   long rows, wide           four sets from 64 nonzeros where the set kernel below does not reach (beyond 16 loads per row of
-//                             B, or not a power of two of them): blocks at 128 fp32 columns 180 -> 139 us.  Beyond 32 loads, where
-//                             the plain kernel has two loads per lane and half the warps, from 12 nonzeros (60,000 rows of 12, 24
-//                             and 48 at 256 fp32 columns 79 -> 75, 132 -> 121, 237 -> 199 us; rows of 8 at 192 columns 54 -> 55)
+//   short rows of one length  fp32 values, and wide rows of both: the plain kernel, whose loop has no last, tested step (stencil
+//                             at 8, 32, 64 fp32 columns 9.6, 38.9, 56.3 / 10.2, 49.1, 97.6 / -)
+//   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
+//   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four
+//                             (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below to 64 (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
+//                             rows of 40 at 32 bf16 columns 349 / 346 / 406), then four; others: one to 64 (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7, 26.3 / 37.7, 30.5), then four (32
+//                             columns, 125: 41.6 / 34.8 / 27.3)
+//   9 to 16 loads             one set from 8 (64 columns, 12, 24: 27.7, 47.2 / 24.9, 38.9 / 29.4, 42.7; 128 bf16 columns, 24: 63.7 / 47.3
+//                             / 54.6; 6: 56.3 / 58.2 / 86.0), and on shorter rows where the loads are no power of two (96 bf16 columns, 3: 83.7 /
+//                             76.0 / 121); four from 40
+//   17 to 32 loads            one set (128 columns, 6, 24: 89.9, 82.9 / 83.5, 72.3 / 109, 77.2), bf16 from 16 (200 columns, 12, 24: 66.1, 66.7 /
+//                             70.7, 57.8 / 72.1, 58.0); four from 40 (200 bf16 columns, 44: 77.5 / 64.4 / 58.8)
+//   beyond 32                 the plain kernel has two loads per lane and half the warps: one set to 12, then four (256 columns, 6, 12:
+//                             240, 109 / 179, 109 / 180, 113)
 static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     const int units = (a.N + vw - 1) / vw;
     const int64_t mean = a.mean_len;
     int lanes = 1;
     while (lanes < 32 && lanes < units) lanes <<= 1;
     const bool fills = a.S * lanes >= static_cast<int64_t>(sm_count_cached()) * 5 * kRowGroupThreads;
+    const bool pow2 = (units & (units - 1)) == 0, bf16 = dtype == SD_BF16;
+    const bool one_length = mean < 16 && a.max_len <= 2 * mean && (!bf16 || units > 8);
     int sets = 0;
     if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
     else if (!fills && mean >= 8) sets = 4;
-    else if (a.N <= 8 && mean >= 8 && mean < 64) sets = 4;
-    else if (units <= 8 && mean < 16 && (dtype == SD_BF16 || mean > 6)) sets = 1;
-    else if (mean >= (units > 32 ? 12 : 64) && (units > 16 || (units & (units - 1)) != 0)) sets = 4;
+    else if (one_length) sets = 0;
+    else if (a.N <= 8) sets = mean < 8 ? 1 : mean < 64 ? 4 : 0;
+    else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? 4 : units == 4 ? (mean < 64 ? 0 : 4) : mean < 64 ? 1 : 4;
+    else if (units <= 16) sets = mean >= 40 ? 4 : mean >= 8 || !pow2 ? 1 : 0;
+    else if (units <= 32) sets = mean >= 40 ? 4 : !bf16 || mean >= 16 ? 1 : 0;
+    else sets = mean >= 12 ? 4 : 1;
     return a.max_len > 0 && a.max_len <= static_cast<int64_t>(kRowGroupTerms) * sets ? sets : 0;
 }
 

@@ -33,3 +33,25 @@ def test_row_group_lengths_widths_and_alignment(edges, N, dtype):
     got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
     check(w, got, beta=0.0)
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [16, 32, 128, 192, 256])
+@pytest.mark.parametrize("edges", [[5], [0, 1, 2, 9], [15, 16, 17, 31], [39, 40, 47, 0], [63, 64, 65, 128]])
+def test_whole_widths_at_the_lines_of_the_rule(edges, N, dtype):
+    """Enough rows to fill the GPU, lengths on both sides of the lines between the row kernels, of one length and of several; every
+    lane has columns (16 to 256) or some have none (192).  A non-finite row of B reaches only the rows that name it."""
+    rng = np.random.default_rng(N + len(edges))
+    M, K = 12007, 700
+    w = W.random_csr(M, K, N, rng.permutation(np.resize(edges, M)), seed=N, dtype=dtype, alpha=-0.75, beta=0.5)
+    plan = DeviceWorkload(w).plan(family=sd.SD_ROWSPLIT)
+    got, intact = run_spmm(plan, w)
+    assert intact
+    check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w)[0])
+    w.B[0] = np.inf if dtype == W.SD_F32 else 0x7F80
+    named = np.zeros(M, bool)
+    named[np.repeat(np.arange(M), np.diff(w.rowptr))[w.colind == 0]] = True
+    got, _ = run_spmm(plan, w)
+    assert np.isfinite(got[~named]).all() and not np.isfinite(got[named]).any()
+    plan.close()
