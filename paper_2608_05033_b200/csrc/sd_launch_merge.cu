@@ -9,7 +9,7 @@ namespace sd {
 
 // The tile kernel alone, fp32 (the entry point without allocations adds the carries itself).
 cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st) {
-    const LaneGeom g = lane_geometry(m.s.N, vec, 4, false);
+    const LaneGeom g = lane_geometry(m.s.N, vec, 4, 0);
     return launch_merge<float>(m, vec, g.lpr, g.nv, st);
 }
 

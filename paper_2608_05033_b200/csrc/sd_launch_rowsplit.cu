@@ -12,8 +12,8 @@ namespace sd {
 //   not whole 16-byte loads   always (41 columns: 1.8 to 3.9 times as fast as one scalar per lane)
 //   few rows                  four sets as soon as rows are 8 long: one set leaves the GPU idle (5,000 rows of 30 at 64 columns
 //                             17.9 -> 5.3 us, at 128 bf16 24.9 -> 6.7)
-//   short rows of one length  fp32 values, and wide rows of both: the plain kernel, whose loop has no last, tested step (stencil
-//                             at 8, 32, 64 fp32 columns 9.6, 38.9, 56.3 / 10.2, 49.1, 97.6 / -)
+//   short rows of one length  the plain kernel, whose loop has no last, tested step (stencils of 360,000 rows at 8, 32, 64 fp32 columns 9.6, 38.9,
+//                             56.3 / 10.2, 49.1, 97.6 / -, of 1 M rows at 32, 64 bf16 columns 73.9, 137 / 85.8, 165 / -)
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
 //   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four
 //                             (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below to 64 (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
@@ -33,7 +33,7 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     while (lanes < 32 && lanes < units) lanes <<= 1;
     const bool fills = a.S * lanes >= static_cast<int64_t>(sm_count_cached()) * 5 * kRowGroupThreads;
     const bool pow2 = (units & (units - 1)) == 0, bf16 = dtype == SD_BF16;
-    const bool one_length = mean < 16 && a.max_len <= 2 * mean && (!bf16 || units > 8);
+    const bool one_length = mean < 16 && a.max_len <= 2 * mean;
     int sets = 0;
     if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
     else if (!fills && mean >= 8) sets = 4;

@@ -7,6 +7,7 @@
 #include <cstdlib>
 
 #include "sd_common.cuh"
+#include "sd_piece.cuh"
 
 namespace sd {
 
@@ -104,8 +105,12 @@ rowsplit_kernel(const SpmmArgs a) {
                     if (colok[v]) {
                         float b[VW];
                         RowLoad<T, VW>::ld(brow + (v * LPR + lg) * VW, b);
+                        if constexpr (VW == 1) {
+                            acc[v][0] = fmaf(av, b[0], acc[v][0]);
+                        } else {
 #pragma unroll
-                        for (int e = 0; e < VW; ++e) acc[v][e] = fmaf(av, b[e], acc[v][e]);
+                            for (int e = 0; e < VW; e += 2) fma_pair(acc[v][e], acc[v][e + 1], av, b[e], b[e + 1]);
+                        }
                     }
                 }
             }
@@ -151,17 +156,13 @@ cudaError_t launch_rowsplit_one(const SpmmArgs &a, cudaStream_t st) {
 
 // Lane geometry for a dense width: VW elements per 16-byte load when `vec`, LPR lanes per
 // row (a power of two), NV vectors per lane; wider rows are covered by grid.y slabs.
-// Two vectors per lane halve the per-nonzero instruction overhead (index broadcast, address
-// arithmetic) per byte gathered; they are used only when a group still covers a full 128-byte
-// line with one load instruction (at least 8 lanes), because a gather instruction costs one
-// L1 tag cycle per distinct line it touches.  The row-split kernel gains from them (short rows:
-// fewer instructions per byte); the merge-path and segment kernels measure faster with one
-// vector per lane and more lanes per row (`prefer_two` = false).
+// Two vectors per lane (from `two_from` vectors per row on; 0: never) halve the per-nonzero instruction overhead (index
+// broadcast, address arithmetic) per byte gathered; the merge-path kernel measures faster with one vector and more lanes per row.
 struct LaneGeom {
     int vw, lpr, nv;
 };
 inline int geom_nv_override() { return switches().geom_nv; }
-inline LaneGeom lane_geometry(int64_t N, bool vec, int vecw, bool prefer_two = true) {
+inline LaneGeom lane_geometry(int64_t N, bool vec, int vecw, int two_from) {
     LaneGeom g;
     g.vw = vec ? vecw : 1;
     const int64_t units = (N + g.vw - 1) / g.vw;
@@ -172,7 +173,7 @@ inline LaneGeom lane_geometry(int64_t N, bool vec, int vecw, bool prefer_two = t
         g.nv = units > 32 ? 4 : 1;
         return g;
     }
-    const bool two = prefer_two && units >= 16 && geom_nv_override() != 1;
+    const bool two = two_from > 0 && units >= two_from && geom_nv_override() != 1;
     const int64_t per = two ? (units + 1) / 2 : units;
     int lpr = 1;
     while (lpr < 32 && lpr < per) lpr <<= 1;
@@ -181,12 +182,25 @@ inline LaneGeom lane_geometry(int64_t N, bool vec, int vecw, bool prefer_two = t
     return g;
 }
 
+// Two vectors per lane where they leave no more lanes idle and a group still covers a 128-byte line with one load (a gather costs a
+// cycle of L1 per line it touches): from nine vectors on (1 M stencil rows at 48 fp32 columns 210 -> 143 us, at 64 also before).  fp32
+// also at five to seven (24 columns 107 -> 80, 160,000 rows 11.5 -> 10.9) and, where operands come from DRAM and the lines are the
+// smaller cost, at four and eight: C beyond 40 MB (32 columns: 1 M rows 111 -> 89, 360,000 rows 38.1 -> 31.6, 250,000 18.6 -> 19.0; 16
+// columns: 640,000 rows 36.6 -> 33.3, 360,000 14.4 -> 16.6).  bf16 lanes hold twice the sums: slower there (64 columns 137 -> 155).
+inline int rowsplit_two_from(const SpmmArgs &a, bool bf16) {
+    const int64_t units = (a.N + 3) / 4;
+    if (bf16) return 9;
+    return (units > 4 && units < 8) || (units >= 4 && a.S * a.N * 4 >= 40000000) ? 4 : 9;
+}
+
 template <typename T>
 cudaError_t launch_rowsplit(const SpmmArgs &a, bool vec, cudaStream_t st) {
     constexpr int VWV = vec_width<T>::value;
-    const LaneGeom g = lane_geometry(a.N, vec, VWV);
+    const LaneGeom g = lane_geometry(a.N, vec, VWV, rowsplit_two_from(a, sizeof(T) == 2));
     if (vec && g.nv == 2) {
         switch (g.lpr) {
+        case 2: return launch_rowsplit_one<T, VWV, 2, 2>(a, st);
+        case 4: return launch_rowsplit_one<T, VWV, 4, 2>(a, st);
         case 8: return launch_rowsplit_one<T, VWV, 8, 2>(a, st);
         case 16: return launch_rowsplit_one<T, VWV, 16, 2>(a, st);
         case 32: return launch_rowsplit_one<T, VWV, 32, 2>(a, st);

@@ -55,3 +55,21 @@ def test_whole_widths_at_the_lines_of_the_rule(edges, N, dtype):
     got, _ = run_spmm(plan, w)
     assert np.isfinite(got[~named]).all() and not np.isfinite(got[named]).any()
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [8, 16, 20, 24, 32, 36, 40, 48, 72, 128, 136, 264])
+@pytest.mark.parametrize("M,length", [(11, 5), (90001, 5), (90001, 1), (700000, 3)])
+def test_rows_of_one_length(M, length, N, dtype):
+    """Short rows of one length: one or two vectors per lane by width and size, idle lanes in the last vector."""
+    if M > 100000 and N > 24:
+        M = 13_000_000 // N   # either side of 40 MB of C
+    K = 1200
+    w = W.random_csr(M, K, N, np.full(M, length), seed=N, dtype=dtype, alpha=0.5, beta=-1.5)
+    plan = DeviceWorkload(w).plan(family=sd.SD_ROWSPLIT)
+    for kw in (dict(), dict(pad_b=8, pad_c=4)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
+    plan.close()
