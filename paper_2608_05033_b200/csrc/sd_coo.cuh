@@ -56,30 +56,6 @@ struct CooArgs {
     int32_t hot;
 };
 
-// N floats of row `col` of B, widened.  VEC: 16-byte loads are allowed (fp32, N = 4).
-template <typename T, int N, bool VEC>
-__device__ __forceinline__ void coo_gather(const void *B, int col, uint32_t ldb_bytes, float (&b)[N]) {
-    const T *p = b_row(static_cast<const T *>(B), col, ldb_bytes);
-    if constexpr (VEC && sizeof(T) == 4 && N % 4 == 0) {
-#pragma unroll
-        for (int q = 0; q < N / 4; ++q) {
-            float t[4];
-            RowLoad<T, 4>::ld(p + 4 * q, t);
-#pragma unroll
-            for (int e = 0; e < 4; ++e) b[4 * q + e] = t[e];
-        }
-    } else if constexpr (VEC && sizeof(T) == 2 && N == 8) {
-        RowLoad<T, 8>::ld(p, b);
-    } else {
-#pragma unroll
-        for (int e = 0; e < N; ++e) {
-            float t[1];
-            RowLoad<T, 1>::ld(p + e, t);
-            b[e] = t[0];
-        }
-    }
-}
-
 template <typename T> __device__ __forceinline__ T from_float(float v);   // of a value that T holds
 template <> __device__ __forceinline__ float from_float<float>(float v) { return v; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_float<__nv_bfloat16>(float v) {

@@ -50,8 +50,8 @@ cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t 
     const int vw = dtype == SD_F32 ? 4 : 8;
     const bool vec = vw_now == vw;
     if (a.N >= 1 && a.N <= 4 && !switches().no_narrow) {   // one to four columns: lanes share a row, not its columns
-        if (dtype == SD_F32) return launch_rowsplit_narrow<float>(a, vec, st);
-        return launch_rowsplit_narrow<__nv_bfloat16>(a, vec, st);
+        if (dtype == SD_F32) return launch_rowsplit_narrow<float>(a, st);
+        return launch_rowsplit_narrow<__nv_bfloat16>(a, st);
     }
     if (const int sets = rowgroup_sets(a, dtype, vw_now, vec))
         return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, sets, st) : run_rowgroup_bf16(a, vw_now, sets, st);

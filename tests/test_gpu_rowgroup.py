@@ -73,3 +73,18 @@ def test_rows_of_one_length(M, length, N, dtype):
         check(w, got)
     assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [2, 4])
+@pytest.mark.parametrize("mean", [1, 5, 20, 70])
+def test_two_and_four_columns_from_any_offset(mean, N, dtype):
+    """A row of B as one load where base and pitch allow it, with four columns also a row of C as one store."""
+    rng = np.random.default_rng(mean)
+    w = W.random_csr(901, 800, N, rng.poisson(mean, 901), seed=mean, dtype=dtype, alpha=1.5, beta=-0.5)
+    plan = DeviceWorkload(w).plan(family=sd.SD_ROWSPLIT)
+    for kw in (dict(), dict(offset=1), dict(offset=2), dict(pad_b=1), dict(pad_b=2, pad_c=1), dict(pad_b=4, pad_c=4), dict(offset=4)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    plan.close()
