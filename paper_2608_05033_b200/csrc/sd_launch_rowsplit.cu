@@ -15,13 +15,14 @@ namespace sd {
 //   short rows of one length  the plain kernel, whose loop has no last, tested step (stencils of 360,000 rows at 8, 32, 64 fp32 columns 9.6, 38.9,
 //                             56.3 / 10.2, 49.1, 97.6 / -, of 1 M rows at 32, 64 bf16 columns 73.9, 137 / 85.8, 165 / -)
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
-//   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four
-//                             (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below to 64 (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
-//                             rows of 40 at 32 bf16 columns 349 / 346 / 406), then four; others: one to 64 (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7, 26.3 / 37.7, 30.5), then four (32
-//                             columns, 125: 41.6 / 34.8 / 27.3)
+//   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four to
+//                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
+//                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64, of eight loads two, so that no row is one
+//                             longer chain of sums than in the set kernel (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7, 26.3 / 37.7, 30.5), then
+//                             four (32 columns, 125: 41.6 / 34.8 / 27.3)
 //   9 to 16 loads             one set from 8 (64 columns, 12, 24: 27.7, 47.2 / 24.9, 38.9 / 29.4, 42.7; 128 bf16 columns, 24: 63.7 / 47.3
 //                             / 54.6; 6: 56.3 / 58.2 / 86.0), and on shorter rows where the loads are no power of two (96 bf16 columns, 3: 83.7 /
-//                             76.0 / 121); four from 40
+//                             76.0 / 121); two of 16 loads from 32 and four from 40
 //   17 to 32 loads            one set (128 columns, 6, 24: 89.9, 82.9 / 83.5, 72.3 / 109, 77.2), bf16 from 16 (200 columns, 12, 24: 66.1, 66.7 /
 //                             70.7, 57.8 / 72.1, 58.0); four from 40 (200 bf16 columns, 44: 77.5 / 64.4 / 58.8)
 //   beyond 32                 the plain kernel has two loads per lane and half the warps: one set to 12, then four (256 columns, 6, 12:
@@ -39,8 +40,8 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     else if (!fills && mean >= 8) sets = 4;
     else if (one_length) sets = 0;
     else if (a.N <= 8) sets = mean < 8 ? 1 : mean < 64 ? 4 : 0;
-    else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? 4 : units == 4 ? (mean < 64 ? 0 : 4) : mean < 64 ? 1 : 4;
-    else if (units <= 16) sets = mean >= 40 ? 4 : mean >= 8 || !pow2 ? 1 : 0;
+    else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? (mean < 64 ? 4 : 0) : units == 4 ? 0 : mean < 64 ? (pow2 ? 2 : 1) : 4;
+    else if (units <= 16) sets = mean >= 40 ? 4 : pow2 && mean >= 32 ? 2 : mean >= 8 || !pow2 ? 1 : 0;
     else if (units <= 32) sets = mean >= 40 ? 4 : !bf16 || mean >= 16 ? 1 : 0;
     else sets = mean >= 12 ? 4 : 1;
     return a.max_len > 0 && a.max_len <= static_cast<int64_t>(kRowGroupTerms) * sets ? sets : 0;

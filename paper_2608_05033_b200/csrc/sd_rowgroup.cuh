@@ -42,10 +42,12 @@ cudaError_t launch_rowgroup_lanes(const SpmmArgs &a, cudaStream_t st) {
                              kRowGroupThreads, 0, st, a);
 }
 
-// Lane sets per row: 1 or 4 (as many as fit a warp).
+// Lane sets per row: 1, 4 (as many as fit a warp) or, with 8 or 16 lanes across the columns, 2.
 template <typename T, int VW, int LPR, int NV>
 cudaError_t launch_rowgroup_one(const SpmmArgs &a, int sets, cudaStream_t st) {
     constexpr int MANY = LPR * 4 > 32 ? 32 : LPR * 4;
+    if constexpr ((LPR == 8 || LPR == 16) && NV == 1 && VW * sizeof(T) == 16)
+        if (sets == 2) return launch_rowgroup_lanes<T, VW, LPR, NV, 2 * LPR>(a, st);
     if (sets > 1) return launch_rowgroup_lanes<T, VW, LPR, NV, MANY>(a, st);
     return launch_rowgroup_lanes<T, VW, LPR, NV, LPR>(a, st);
 }
