@@ -51,6 +51,14 @@ __device__ __forceinline__ void clear_acc(float (&acc)[NV][VW]) {
         for (int e = 0; e < VW; ++e) acc[v][e] = 0.f;
 }
 
+template <int NV, int VW>
+__device__ __forceinline__ void add_acc(float (&acc)[NV][VW], const float (&more)[NV][VW]) {
+#pragma unroll
+    for (int v = 0; v < NV; ++v)
+#pragma unroll
+        for (int e = 0; e < VW; ++e) acc[v][e] += more[v][e];
+}
+
 // Sum over the LANES / LPR lane sets of a group (a fixed order: results repeat bit for bit).
 template <int LANES, int LPR, int NV, int VW>
 __device__ __forceinline__ void sum_sets(float (&acc)[NV][VW], unsigned mask) {
@@ -68,6 +76,10 @@ __device__ __forceinline__ void sum_sets(float (&acc)[NV][VW], unsigned mask) {
 // as many shuffles.  Q gathers of a lane are in flight together.  Whole steps run without any test; only the
 // last, partly filled one tests every pair: nothing may be gathered for a pair beyond the end (row 0 of B may hold
 // non-finite values, and 0 * Inf is NaN).
+// FOLD: a set adds at most kGroupFold products in one accumulator before they go to a second one, so the longest chain of sums of a
+// row of L nonzeros is kGroupFold + L / (G * kGroupFold) long, not L / G.  The second accumulator is up to 16 registers, so rows
+// that are shorter do without it.
+constexpr int kGroupFold = 64;
 template <int LPR> constexpr int kGroupLoads = LPR >= 4 ? 1 : 4 / LPR;   // loads of pairs per step: at least four gathers per lane and step
 template <int THREADS, int LPR>
 struct GroupStage {   // of a CTA; with one lane across the columns every lane has its own nonzeros, with two shuffles are as good (5 % less at 8 columns)
@@ -75,7 +87,7 @@ struct GroupStage {   // of a CTA; with one lane across the columns every lane h
     alignas(16) int col[N];
     alignas(16) float val[N];
 };
-template <typename T, int VW, int LPR, int NV, int LANES, bool EXACT, typename Args, int THREADS>
+template <typename T, int VW, int LPR, int NV, int LANES, bool EXACT, bool FOLD, typename Args, int THREADS>
 __device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, LPR, NV, EXACT> &lc, GroupStage<THREADS, LPR> &stage, int p0,
                                           int p1, unsigned mask, float (&acc)[NV][VW]) {
     constexpr int G = LANES / LPR;
@@ -139,11 +151,24 @@ __device__ __forceinline__ void group_sum(const Args &a, const LaneCols<T, VW, L
             }
         }
     };
+    float tot[FOLD ? NV : 1][FOLD ? VW : 1];
+    if constexpr (FOLD) clear_acc(tot);
+    [[maybe_unused]] int steps = 0;
     int p = p0;
     fetch(p);
 #pragma unroll 1
-    for (; p + NB * LANES <= p1; p += NB * LANES) step(p, std::true_type{});
+    for (; p + NB * LANES <= p1; p += NB * LANES) {
+        step(p, std::true_type{});
+        if constexpr (FOLD) {
+            if (++steps == kGroupFold / PER) {
+                steps = 0;
+                add_acc(tot, acc);
+                clear_acc(acc);
+            }
+        }
+    }
     if (p < p1) step(p, std::false_type{});
+    if constexpr (FOLD) add_acc(acc, tot);
     sum_sets<LANES, LPR, NV, VW>(acc, mask);
 }
 

@@ -52,7 +52,7 @@ __device__ __forceinline__ void items_body(const HybridArgs &a, unsigned bx, Gro
         const int4 d = __ldg(chunk ? a.items + s : a.desc + (s - a.chunks));
         float acc[NV][VW];
         clear_acc(acc);
-        group_sum<T, VW, LPR, NV, LANES, EXACT>(a, lc, stage, d.y, d.y + d.w, mask, acc);
+        group_sum<T, VW, LPR, NV, LANES, EXACT, false>(a, lc, stage, d.y, d.y + d.w, mask, acc);
         if (lg < LPR) {
             if (chunk && d.x >= 0) lc.store(a.scratch + static_cast<int64_t>(d.x) * a.N, acc, 1.f, 0.f);
             else lc.store(a.C + (d.x & 0x7FFFFFFF) * a.ldc, acc, a.alpha, a.beta);   // a light row, or a heavy row of one item
@@ -72,7 +72,7 @@ __device__ __forceinline__ void medium_body(const HybridArgs &a, unsigned bx, Gr
         const int4 cur = __ldg(desc + s);
         float acc[NV][VW];
         clear_acc(acc);
-        group_sum<T, VW, LPR, NV, LANES, EXACT>(a, lc, stage, cur.y, cur.y + cur.w, mask, acc);
+        group_sum<T, VW, LPR, NV, LANES, EXACT, false>(a, lc, stage, cur.y, cur.y + cur.w, mask, acc);
         if (lg < LPR) lc.store(a.C + cur.x * a.ldc, acc, a.alpha, a.beta);
     }
 }

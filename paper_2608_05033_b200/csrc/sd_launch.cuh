@@ -20,8 +20,8 @@ struct MergeArgs {
 
 // Family (a).  `vw`: elements per load of B (piece_width).
 cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw, cudaStream_t st);
-cudaError_t run_rowgroup_f32(const SpmmArgs &a, int vw, int sets, cudaStream_t st);
-cudaError_t run_rowgroup_bf16(const SpmmArgs &a, int vw, int sets, cudaStream_t st);
+cudaError_t run_rowgroup_f32(const SpmmArgs &a, int vw, int sets, int terms, cudaStream_t st);
+cudaError_t run_rowgroup_bf16(const SpmmArgs &a, int vw, int sets, int terms, cudaStream_t st);
 
 // Hybrid family in one launch: items (chunks of the heavy rows, long light rows), medium rows, short rows.
 struct HybridArgs;

@@ -3,13 +3,13 @@
 
 namespace sd {
 
-// `vw`: elements per load of B (piece_width); `sets`: lane sets per row
-cudaError_t run_rowgroup_bf16(const SpmmArgs &a, int vw, int sets, cudaStream_t st) {
+// `vw`: elements per load of B (piece_width); `sets`: lane sets per row; `terms`: products of a set in one accumulator
+cudaError_t run_rowgroup_bf16(const SpmmArgs &a, int vw, int sets, int terms, cudaStream_t st) {
     switch (vw) {
-    case 8: return launch_rowgroup<__nv_bfloat16, 8>(a, sets, st);
-    case 4: return launch_rowgroup<__nv_bfloat16, 4>(a, sets, st);
-    case 2: return launch_rowgroup<__nv_bfloat16, 2>(a, sets, st);
-    default: return launch_rowgroup<__nv_bfloat16, 1>(a, sets, st);
+    case 8: return launch_rowgroup<__nv_bfloat16, 8>(a, sets, terms, st);
+    case 4: return launch_rowgroup<__nv_bfloat16, 4>(a, sets, terms, st);
+    case 2: return launch_rowgroup<__nv_bfloat16, 2>(a, sets, terms, st);
+    default: return launch_rowgroup<__nv_bfloat16, 1>(a, sets, terms, st);
     }
 }
 

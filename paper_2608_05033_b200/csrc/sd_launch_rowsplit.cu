@@ -17,9 +17,9 @@ namespace sd {
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
 //   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four to
 //                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
-//                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64, of eight loads two, so that no row is one
-//                             longer chain of sums than in the set kernel (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7, 26.3 / 37.7, 30.5), then
-//                             four (32 columns, 125: 41.6 / 34.8 / 27.3)
+//                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64 (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7,
+//                             26.3 / 37.7, 30.5), of eight loads two (32 columns, 44: one 25.4, two 23.6), then four (32 columns, 125: 41.6 /
+//                             34.8 / 27.3)
 //   9 to 16 loads             one set from 8 (64 columns, 12, 24: 27.7, 47.2 / 24.9, 38.9 / 29.4, 42.7; 128 bf16 columns, 24: 63.7 / 47.3
 //                             / 54.6; 6: 56.3 / 58.2 / 86.0), and on shorter rows where the loads are no power of two (96 bf16 columns, 3: 83.7 /
 //                             76.0 / 121); two of 16 loads from 32 and four from 40
@@ -47,6 +47,15 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     return a.max_len > 0 && a.max_len <= static_cast<int64_t>(kRowGroupTerms) * sets ? sets : 0;
 }
 
+// Products of a lane set in one accumulator: no more than in the kernels below, which would take the rows otherwise.  The set kernel and,
+// of two lanes, the plain kernel add 64 before they fold, the plain kernel of more lanes at least 128.  Rows beyond are folded every 64
+// (kGroupFold), in kernels with a second accumulator and four CTAs per SM for five (rows of 24, the longest 900, at 64 bf16 columns 42.9
+// -> 46.5 us, at 128 60.1 -> 62.4; with 64 everywhere also 400,000 rows of 35, the longest about 70, at 48 fp32 columns 275 -> 312).
+static int rowgroup_terms(const SpmmArgs &a, int vw) {
+    const int units = (a.N + vw - 1) / vw;
+    return units <= 2 || (units <= 16 && (units & (units - 1)) == 0 && a.mean_len >= 16) ? 64 : 128;
+}
+
 cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t st) {
     const int vw = dtype == SD_F32 ? 4 : 8;
     const bool vec = vw_now == vw;
@@ -54,8 +63,10 @@ cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t 
         if (dtype == SD_F32) return launch_rowsplit_narrow<float>(a, st);
         return launch_rowsplit_narrow<__nv_bfloat16>(a, st);
     }
-    if (const int sets = rowgroup_sets(a, dtype, vw_now, vec))
-        return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, sets, st) : run_rowgroup_bf16(a, vw_now, sets, st);
+    if (const int sets = rowgroup_sets(a, dtype, vw_now, vec)) {
+        const int terms = rowgroup_terms(a, vw_now);
+        return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, sets, terms, st) : run_rowgroup_bf16(a, vw_now, sets, terms, st);
+    }
     // 8 to 64 columns (fp32; 8 to 128 bf16) as whole 16-byte vectors and long rows: several lane sets per row
     if (vec && a.N % vw == 0 && a.N / vw <= 16 && ((a.N / vw) & (a.N / vw - 1)) == 0) {
         const int lpr = a.N / vw;
