@@ -563,7 +563,7 @@ static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
 sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
     sd_status_t s;
     const int64_t steps = coo_steps(p->nnz, static_cast<int>(p->N));
-    const int64_t count2 = 2 * std::min<int64_t>(steps, static_cast<int64_t>(kCooMaxWarps) * p->info.sm_count);
+    const int64_t count2 = 2 * coo_most_ranges(steps, static_cast<int64_t>(kCooMaxWarps) * p->info.sm_count);
     const int64_t chunks2 = (count2 + kCooCarryChunk - 1) / kCooCarryChunk, count3 = 2 * chunks2;
     const bool bits = p->N == 1 && p->info.empty_rows == 0;
     if ((s = dev_alloc(p, &p->coo_row, bits ? 32 * steps : p->nnz, "rows of nonzeros", st))) return s;

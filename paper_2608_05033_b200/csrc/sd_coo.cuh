@@ -50,8 +50,11 @@ struct CooArgs {
     float alpha, beta;
     const int32_t *rowptr;   // [M + 1], to find the rows without nonzeros (they get beta * C)
     int64_t M;
-    int32_t *carry_row;      // [2 * warps] out
-    float *carry_val;        // [2 * warps][N] out
+    int warps, per_warp;     // that work, ranges of each
+    int range, longer;       // steps of a range, and how many ranges (the first ones) have one more
+    int spread;              // neighbouring ranges go to different CTAs
+    int32_t *carry_row;      // [2 * warps * per_warp] out
+    float *carry_val;        // [2 * warps * per_warp][N] out
     const int32_t *hot_cols; // HOT: ascending columns whose rows of B the kernel keeps; colind names slot i of them as i | bit 31
     int32_t hot;
 };
@@ -156,14 +159,9 @@ coo_kernel(const CooArgs a) {
         __syncthreads();
     }
     const int lane = threadIdx.x & 31;
-    const int64_t steps = (a.count + STEP - 1) / STEP, all = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5, warps = min(all, steps);
-    // Many steps per warp: neighbouring ranges go to different CTAs, since what a range costs depends on its rows and columns (60 M
-    // nonzeros in rank-size rows 279 -> 271 us).  Few: to the same one, whose L1 they share (R-MAT scale 14 8.2 -> 7.7 us).
-    const int64_t w = HOT || steps >= 8 * all ? static_cast<int64_t>(threadIdx.x >> 5) * gridDim.x + blockIdx.x
-                                              : (static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5;
-    if (w >= warps) return;
-    const int64_t s0 = steps * w / warps, s1 = steps * (w + 1) / warps;
-    coo_empty_rows<N>(a, w, warps);
+    const int w = a.spread ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    if (w >= a.warps) return;
+    if (a.M > 0) coo_empty_rows<N>(a, w, a.warps);
     const T *vals = static_cast<const T *>(a.vals), *B = static_cast<const T *>(a.B);
     const unsigned va = static_cast<unsigned>(reinterpret_cast<uintptr_t>(vals)), ca = static_cast<unsigned>(reinterpret_cast<uintptr_t>(a.colind));
 
@@ -174,129 +172,135 @@ coo_kernel(const CooArgs a) {
             *pc = (a.beta != 0.f) ? fmaf(a.beta, *pc, a.alpha * v[e]) : a.alpha * v[e];
         }
     };
-    auto carry = [&](int which, int row, const float (&v)[N]) {
-        a.carry_row[2 * w + which] = row;
+    // One range for most matrices.  The open sum below takes one addition per step, so a range is at most kCooRange steps long: one billion
+    // nonzeros would make it 740, and the longest chain of sums with it.
+    for (int n = 0; n < a.per_warp; ++n) {
+        const int range = w + n * a.warps, s0 = range * a.range + min(range, a.longer), s1 = s0 + a.range + (range < a.longer);
+        auto carry = [&](int which, int row, const float (&v)[N]) {
+            const int64_t at = 2 * range + which;
+            a.carry_row[at] = row;
 #pragma unroll
-        for (int e = 0; e < N; ++e) a.carry_val[(2 * w + which) * N + e] = v[e];
-    };
-    const int first_row = BITS ? __ldg(a.row + s0 * 32) : __ldg(a.row + s0 * STEP);
-    int open_row = first_row;   // the row that reached the end of the step before ...
-    float open[N] = {};         // ... and its sum so far (both the same in all lanes)
-    for (int64_t s = s0; s < s1; ++s) {
-        const int64_t k0 = s * STEP + lane * U;
-        int col[U], r[U];
-        float av[U];
-        unsigned starts = 0;    // items that begin a row
-        int row_in = 0;         // the row that is open where the lane begins ...
-        int row_out = 0;        // ... and where it ends
-        const bool whole = (s + 1) * STEP <= a.count;   // the same in all lanes: no item is past the end
-        if (whole) {
-            load_ints<U>(a.colind + k0, ca, col);
-            if constexpr (!BITS) load_ints<U>(a.row + k0, 0, r);
-            load_run<T, U>(vals + k0, va, av);
-        } else {                // items past the end continue the last row with zeros
-            const int pad = BITS ? 0 : __ldg(a.row + a.count - 1);
+            for (int e = 0; e < N; ++e) a.carry_val[at * N + e] = v[e];
+        };
+        const int first_row = __ldg(a.row + static_cast<int64_t>(s0) * (BITS ? 32 : STEP));
+        int open_row = first_row;   // the row that reached the end of the step before ...
+        float open[N] = {};         // ... and its sum so far (both the same in all lanes)
+        for (int s = s0; s < s1; ++s) {
+            const unsigned k0 = static_cast<unsigned>(s) * STEP + lane * U, count = static_cast<unsigned>(a.count);   // below 2^31 + STEP
+            int col[U], r[U];
+            float av[U];
+            unsigned starts = 0;    // items that begin a row
+            int row_in = 0;         // the row that is open where the lane begins ...
+            int row_out = 0;        // ... and where it ends
+            const bool whole = k0 - lane * U + STEP <= count;   // the same in all lanes: no item is past the end
+            if (whole) {
+                load_ints<U>(a.colind + k0, ca, col);
+                if constexpr (!BITS) load_ints<U>(a.row + k0, 0, r);
+                load_run<T, U>(vals + k0, va, av);
+            } else {                // items past the end continue the last row with zeros
+                const int pad = BITS ? 0 : __ldg(a.row + a.count - 1);
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const bool ok = k0 + u < count;
+                    col[u] = ok ? __ldg(a.colind + k0 + u) : 0;
+                    av[u] = ok ? to_float(vals[k0 + u]) : 0.f;
+                    r[u] = BITS ? 0 : (ok ? __ldg(a.row + k0 + u) : pad);
+                }
+            }
+            if constexpr (BITS) {
+                starts = __ldg(a.starts + s * 32 + lane);
+                row_in = __ldg(a.row + s * 32 + lane);
+                row_out = row_in + __popc(starts >> 1);
+                row_in -= starts & 1u;
+                if (s == s0 && lane == 0) {
+                    row_in = first_row;
+                    starts &= ~1u;
+                }
+            }
+            float b[U][N];
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const bool ok = k0 + u < a.count;
-                col[u] = ok ? __ldg(a.colind + k0 + u) : 0;
-                av[u] = ok ? to_float(vals[k0 + u]) : 0.f;
-                r[u] = BITS ? 0 : (ok ? __ldg(a.row + k0 + u) : pad);
-            }
-        }
-        if constexpr (BITS) {
-            starts = __ldg(a.starts + s * 32 + lane);
-            row_in = __ldg(a.row + s * 32 + lane);
-            row_out = row_in + __popc(starts >> 1);
-            row_in -= starts & 1u;
-            if (s == s0 && lane == 0) {
-                row_in = first_row;
-                starts &= ~1u;
-            }
-        }
-        float b[U][N];
+                if constexpr (HOT) {   // every lane reads a slot (the others slot 0), those outside also their row of B
+                    const bool in = col[u] < 0;
+                    const T *q = kept + (in ? col[u] & 0x7fffffff : 0) * N;
+                    if constexpr (VEC && N == 2 && sizeof(T) == 4) {
+                        const float2 v = *reinterpret_cast<const float2 *>(q);
+                        b[u][0] = v.x, b[u][1] = v.y;
+                    } else {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if constexpr (HOT) {   // every lane reads a slot (the others slot 0), those outside also their row of B
-                const bool in = col[u] < 0;
-                const T *q = kept + (in ? col[u] & 0x7fffffff : 0) * N;
-                if constexpr (VEC && N == 2 && sizeof(T) == 4) {
-                    const float2 v = *reinterpret_cast<const float2 *>(q);
-                    b[u][0] = v.x, b[u][1] = v.y;
+                        for (int e = 0; e < N; ++e) b[u][e] = to_float(q[e]);
+                    }
+                    if (!in) coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
                 } else {
-#pragma unroll
-                    for (int e = 0; e < N; ++e) b[u][e] = to_float(q[e]);
+                    coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
                 }
-                if (!in) coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
-            } else {
-                coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
             }
-        }
-        if (!whole)   // they gathered row 0: never let its contents (Inf, NaN) in
+            if (!whole)   // they gathered row 0: never let its contents (Inf, NaN) in
 #pragma unroll
-            for (int u = 0; u < U; ++u)
-                if (k0 + u >= a.count)
+                for (int u = 0; u < U; ++u)
+                    if (k0 + u >= count)
 #pragma unroll
-                    for (int e = 0; e < N; ++e) b[u][e] = 0.f;
-        if constexpr (!BITS) {
-            const int before = __shfl_up_sync(FULL, r[U - 1], 1);
-            row_in = lane == 0 ? open_row : before;
-            row_out = r[U - 1];
-            starts = r[0] != row_in;
+                        for (int e = 0; e < N; ++e) b[u][e] = 0.f;
+            if constexpr (!BITS) {
+                const int before = __shfl_up_sync(FULL, r[U - 1], 1);
+                row_in = lane == 0 ? open_row : before;
+                row_out = r[U - 1];
+                starts = r[0] != row_in;
 #pragma unroll
-            for (int u = 1; u < U; ++u) starts |= static_cast<unsigned>(r[u] != r[u - 1]) << u;
-        }
-        // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
-        float sum[N] = {}, top[N] = {};
-        bool closed = false;
-        int now = row_in;
+                for (int u = 1; u < U; ++u) starts |= static_cast<unsigned>(r[u] != r[u - 1]) << u;
+            }
+            // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
+            float sum[N] = {}, top[N] = {};
+            bool closed = false;
+            int now = row_in;
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-            if (starts >> u & 1u) {
-                if (closed) emit(now, sum);
+            for (int u = 0; u < U; ++u) {
+                if (starts >> u & 1u) {
+                    if (closed) emit(now, sum);
+#pragma unroll
+                    for (int e = 0; e < N; ++e) {
+                        if (!closed) top[e] = sum[e];
+                        sum[e] = 0.f;
+                    }
+                    closed = true;
+                    now = BITS ? now + 1 : r[u];
+                }
+#pragma unroll
+                for (int e = 0; e < N; ++e) sum[e] = fmaf(av[u], b[u][e], sum[e]);
+            }
+            if (lane == 0) {
+#pragma unroll
+                for (int e = 0; e < N; ++e) (closed ? top[e] : sum[e]) += open[e];
+            }
+            const unsigned ends = __ballot_sync(FULL, closed) & (FULL >> (31 - lane));
+            const int dist = lane - (ends ? 31 - __clz(ends) : 0);
+#pragma unroll
+            for (int d = 1; d < 32; d <<= 1)
 #pragma unroll
                 for (int e = 0; e < N; ++e) {
-                    if (!closed) top[e] = sum[e];
-                    sum[e] = 0.f;
+                    const float up = __shfl_up_sync(FULL, sum[e], d);
+                    if (dist >= d) sum[e] += up;
                 }
-                closed = true;
-                now = BITS ? now + 1 : r[u];
-            }
-#pragma unroll
-            for (int e = 0; e < N; ++e) sum[e] = fmaf(av[u], b[u][e], sum[e]);
-        }
-        if (lane == 0) {
-#pragma unroll
-            for (int e = 0; e < N; ++e) (closed ? top[e] : sum[e]) += open[e];
-        }
-        const unsigned ends = __ballot_sync(FULL, closed) & (FULL >> (31 - lane));
-        const int dist = lane - (ends ? 31 - __clz(ends) : 0);
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1)
 #pragma unroll
             for (int e = 0; e < N; ++e) {
-                const float up = __shfl_up_sync(FULL, sum[e], d);
-                if (dist >= d) sum[e] += up;
+                const float in = __shfl_up_sync(FULL, sum[e], 1);
+                if (lane > 0) top[e] += in;
+                open[e] = __shfl_sync(FULL, sum[e], 31);
             }
-#pragma unroll
-        for (int e = 0; e < N; ++e) {
-            const float in = __shfl_up_sync(FULL, sum[e], 1);
-            if (lane > 0) top[e] += in;
-            open[e] = __shfl_sync(FULL, sum[e], 31);
+            open_row = __shfl_sync(FULL, row_out, 31);
+            if (closed) {
+                if (row_in == first_row) carry(0, row_in, top);
+                else emit(row_in, top);
+            }
         }
-        open_row = __shfl_sync(FULL, row_out, 31);
-        if (closed) {
-            if (row_in == first_row) carry(0, row_in, top);
-            else emit(row_in, top);
-        }
-    }
-    if (lane == 0) {   // what is still open at the end of the range; one single row: (row, sum), (row, 0)
-        const float none[N] = {};
-        if (open_row == first_row) {
-            carry(0, open_row, open);
-            carry(1, open_row, none);
-        } else {
-            carry(1, open_row, open);
+        if (lane == 0) {   // what is still open at the end of the range; one single row: (row, sum), (row, 0)
+            const float none[N] = {};
+            if (open_row == first_row) {
+                carry(0, open_row, open);
+                carry(1, open_row, none);
+            } else {
+                carry(1, open_row, open);
+            }
         }
     }
 }

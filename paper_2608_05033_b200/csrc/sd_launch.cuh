@@ -49,14 +49,16 @@ constexpr int coo_items(int N) { return N <= 2 ? 8 : 4; }   // nonzeros of a lan
 constexpr int64_t coo_steps(int64_t nnz, int N) { return (nnz + 32 * coo_items(N) - 1) / (32 * coo_items(N)); }
 constexpr int kCooCarryChunk = 128;
 constexpr int64_t kCooDirectFinal = 4096;  // carry lists up to this length skip the second level
-constexpr int kCooMaxWarps = 64;           // resident on one SM; each leaves two carry entries
+constexpr int kCooMaxWarps = 64;           // resident on one SM; each leaves two carry entries per range
+constexpr int kCooRange = 64;              // steps: longer shares of a warp are cut into several ranges
+constexpr int64_t coo_most_ranges(int64_t steps, int64_t warps) { return steps < warps ? steps : warps + steps / kCooRange; }
 struct CooPlan {
     const int32_t *row;    // [nnz] row of every nonzero, or with `starts` [32 steps] of every eighth
     const uint8_t *starts; // [32 steps] a bit per nonzero that begins a row
     const int32_t *rowptr; // [M + 1]
     int64_t M;             // rows to search for empty ones (0: the matrix has none)
     int64_t nnz;
-    int32_t *c1_row;      // [2 * min(steps, kCooMaxWarps * SMs)] first-level carries
+    int32_t *c1_row;      // [2 * coo_most_ranges(steps, kCooMaxWarps * SMs)] first-level carries
     float *c1_val;        // ... x N
     int32_t *c2_row;      // [2 * ceil(len(c1) / kCooCarryChunk)] second-level carries
     float *c2_val;

@@ -14,9 +14,9 @@ cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st) {
 }
 
 // ---- narrow dense operands: COO segmented reduction --------------------------------------------
-// One instance: the grid is as many CTAs as are resident together, or as give every warp a step.  Returns the warps that work.
+// One instance: the grid is as many CTAs as are resident together, or as give every warp a step.  Returns the ranges.
 template <typename T, int N, bool VEC, bool HOT, bool BITS>
-static cudaError_t launch_coo_kernel(const CooArgs &a, int sm_count, int kept, cudaStream_t st, int64_t &warps) {
+static cudaError_t launch_coo_kernel(CooArgs a, int sm_count, int kept, cudaStream_t st, int64_t &ranges) {
     auto kernel = coo_kernel<T, N, VEC, HOT, BITS>;
     constexpr int threads = HOT ? kCooHotThreads : coo_threads(N);
     int64_t ctas = sm_count;
@@ -34,7 +34,15 @@ static cudaError_t launch_coo_kernel(const CooArgs &a, int sm_count, int kept, c
     }
     const int64_t steps = coo_steps(a.count, N);
     ctas = std::min(ctas, (steps + threads / 32 - 1) / (threads / 32));
-    warps = std::min(ctas * (threads / 32), steps);
+    const int64_t all = ctas * (threads / 32);
+    a.warps = static_cast<int>(std::min(all, steps));
+    a.per_warp = static_cast<int>((steps + static_cast<int64_t>(a.warps) * kCooRange - 1) / (static_cast<int64_t>(a.warps) * kCooRange));
+    ranges = static_cast<int64_t>(a.warps) * a.per_warp;
+    a.range = static_cast<int>(steps / ranges);
+    a.longer = static_cast<int>(steps % ranges);
+    // Many steps per warp: neighbouring ranges go to different CTAs, since what a range costs depends on its rows and columns (60 M
+    // nonzeros in rank-size rows 279 -> 271 us).  Few: to the same one, whose L1 they share (R-MAT scale 14 8.2 -> 7.7 us).
+    a.spread = HOT || steps >= 8 * all;
     return launch_overlapped(kernel, static_cast<unsigned>(ctas), threads, kept, st, a);
 }
 
@@ -57,7 +65,7 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, int sm_cou
     a.carry_row = cp.c1_row;
     a.carry_val = cp.c1_val;
     cudaError_t e;
-    int64_t warps = 0;
+    int64_t ranges = 0;
     const int kept = cp.hot * N * static_cast<int>(sizeof(T));
     const bool hot = cp.hot > 0 && kept <= kCooHotBytes;
     if (hot) {
@@ -67,16 +75,16 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, int sm_cou
     }
     if constexpr (N == 1) {
         if (cp.starts)
-            e = hot ? launch_coo_kernel<T, N, VEC, true, true>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, true>(a, sm_count, 0, st, warps);
+            e = hot ? launch_coo_kernel<T, N, VEC, true, true>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, true>(a, sm_count, 0, st, ranges);
         else
-            e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, warps);
+            e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, ranges);
     } else {
-        e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, warps) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, warps);
+        e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, ranges);
     }
     if (e != cudaSuccess) return e;
     const int32_t *frow = cp.c1_row;
     const float *fval = cp.c1_val;
-    int64_t fcount = 2 * warps;
+    int64_t fcount = 2 * ranges;
     if (fcount > kCooDirectFinal) {   // level 2
         const int64_t chunks = (fcount + kCooCarryChunk - 1) / kCooCarryChunk;
         CooArgs b = a;

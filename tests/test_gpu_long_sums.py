@@ -50,3 +50,29 @@ def test_row_group_chains(loads, usual, longest, dtype):
     worst = (off / (additions * 2.0 ** -24)).max().item()
     plan.close()
     assert worst <= 1.0
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N,empty", [(1, False), (1, True), (3, False)])
+def test_ranges_of_many_steps(N, empty, dtype):
+    """One to four columns: a warp has 660 steps and more of 256 nonzeros (128 at three columns), rows are 700 steps long.  A lane adds
+    eight, the scan over the lanes five, the open sum one per step of a range, at most 64; a row lies in up to 13 ranges, whose sums
+    meet one by one in the end, and a dozen for the scans of the carries and scaling."""
+    step = 256 if N <= 2 else 128
+    length = 700 * step + 5
+    lengths = torch.full((900_000_000 // length,), length, dtype=torch.int64, device="cuda")
+    if step == 128:
+        lengths = lengths[: lengths.numel() // 2]
+    M = lengths.numel()
+    rowptr, colind, vals = absorbing_rows(lengths, 2.0 ** -25 / step, 1000, dtype)
+    if empty:
+        rowptr, M = torch.cat([rowptr, rowptr[-1:]]), M + 1
+    B = torch.ones(1000, N, dtype=vals.dtype, device="cuda")
+    C = torch.full((M, N), float("nan"), device="cuda")
+    plan = sd.Plan(rowptr, colind, vals, M, 1000, N, family=sd.SD_MERGE)
+    plan.spmm(B, C)
+    plan.close()
+    exact = 1.0 + (length - 1) * 2.0 ** -25 / step
+    additions = 8 + 5 + 64 + 13 + 12
+    assert ((C[: lengths.numel()].double() - exact).abs() / exact).max().item() <= additions * 2.0 ** -24
+    assert not empty or (C[-1] == 0).all()
