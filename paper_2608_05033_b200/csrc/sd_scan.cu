@@ -235,15 +235,19 @@ __device__ __forceinline__ int run_of(int j, bool in) {
 // The table belongs to one warp, so a slot is taken without an atomic operation, which in shared memory costs a cycle or two per
 // lane: lanes write their block columns and read back which one stayed.
 struct alignas(16) WarpTable {
-    unsigned word[kSmallSlots];   // block column and count; all ones: free
+    unsigned word[kSmallSlots];   // block column and count; all ones: free.  WIDE: block columns in the first half, counts in the second
     Rows rows;
 };
 
 // Adds k entries to block column j (every lane of the warp calls it, k == 0: none).
+// WIDE: block columns that leave no room for a count in their word.  The table then has half the slots and takes half the nonzeros
+// (creating row-split plans, 2^27 columns: 4 M rows of 3 1,756 -> 319 us, 1 M rows of 8 560 -> 140 with all of them in CTAs before).
+template <bool WIDE>
 __device__ __forceinline__ void warp_table_add(unsigned *word, unsigned mask, int j, int k, ScanShared &s, Counts &n) {
     constexpr unsigned FULL = 0xffffffffu;
     volatile unsigned *const slots = word;
-    const unsigned key = static_cast<unsigned>(j) << kCountBits;
+    constexpr int KEY_AT = WIDE ? 0 : kCountBits;
+    const unsigned key = static_cast<unsigned>(j) << KEY_AT;
     unsigned h = (static_cast<unsigned>(j) * 2654435761u) >> 7 & mask;
     bool looking = k > 0;
     while (__any_sync(FULL, looking)) {
@@ -252,12 +256,13 @@ __device__ __forceinline__ void warp_table_add(unsigned *word, unsigned mask, in
         if (is_free) slots[h] = key;
         __syncwarp();
         if (looking) {
-            if ((slots[h] ^ key) >> kCountBits == 0) looking = false;
+            if ((slots[h] ^ key) >> KEY_AT == 0) looking = false;
             else h = (h + 1) & mask;
         }
     }
     if (k > 0) {
-        const unsigned old = atomicAdd(word + h, static_cast<unsigned>(k)) & ((1u << kCountBits) - 1u);
+        const unsigned old = WIDE ? atomicAdd(word + kSmallSlots / 2 + h, static_cast<unsigned>(k))
+                                  : atomicAdd(word + h, static_cast<unsigned>(k)) & ((1u << kCountBits) - 1u);
         count_block(s, n, old, old + k);
     }
     __syncwarp();
@@ -265,6 +270,7 @@ __device__ __forceinline__ void warp_table_add(unsigned *word, unsigned mask, in
 
 static_assert(sizeof(ScanShared) % 16 == 0 && sizeof(WarpTable) % 16 == 0, "tables are cleared with 16-byte stores");
 
+template <bool WIDE>
 __global__ void __launch_bounds__(32 * kScanWarps)
 scan_small_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict__ colind, int64_t M, int64_t most, ScanAccum *__restrict__ out) {
     extern __shared__ __align__(16) unsigned char smem[];
@@ -294,9 +300,12 @@ scan_small_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
         unsigned slots = 128;
         while (static_cast<int>(slots) < 2 * len) slots <<= 1;
         row_ends(colind, w, lane);
-        for (unsigned i = lane * 4; i < slots; i += 128) *reinterpret_cast<int4 *>(table.word + i) = make_int4(-1, -1, -1, -1);
+        for (unsigned i = lane * 4; i < slots; i += 128) {
+            *reinterpret_cast<int4 *>(table.word + i) = make_int4(-1, -1, -1, -1);
+            if (WIDE) *reinterpret_cast<int4 *>(table.word + kSmallSlots / 2 + i) = make_int4(0, 0, 0, 0);
+        }
         __syncwarp();
-        walk_block_row<32, true>(colind, w, I, lane, n.sum[S_DIAG], [&](int j, int k) { warp_table_add(table.word, slots - 1, j, k, s, n); });
+        walk_block_row<32, true>(colind, w, I, lane, n.sum[S_DIAG], [&](int j, int k) { warp_table_add<WIDE>(table.word, slots - 1, j, k, s, n); });
         __syncwarp();
         if (w.excess) {
             unordered_rows<32>(colind, w, lane);
@@ -485,10 +494,13 @@ cudaError_t scan_structure(const int32_t *rowptr, const int32_t *colind, int64_t
     const int medium_smem = static_cast<int>(sizeof(ScanShared) + sizeof(CtaTable<kMediumThreads, kMediumSlots>));
     auto medium = scan_cta_kernel<kMediumThreads, kMediumSlots>;
     auto large = scan_cta_kernel<kLargeThreads, kLargeSlots>;
+    const bool wide = Kb >= (int64_t{1} << (32 - kCountBits)) - 1;   // block columns do not fit a word beside a count
+    auto warps = wide ? scan_small_kernel<true> : scan_small_kernel<false>;
     static std::atomic<int> attr_set[kMaxDevices];
     const int dev = current_device();
     if (dev >= kMaxDevices || !attr_set[dev].load(std::memory_order_acquire)) {
-        if ((e = cudaFuncSetAttribute(scan_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem)) != cudaSuccess ||
+        if ((e = cudaFuncSetAttribute(scan_small_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem)) != cudaSuccess ||
+            (e = cudaFuncSetAttribute(scan_small_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, small_smem)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(medium, cudaFuncAttributeMaxDynamicSharedMemorySize, medium_smem)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(large, cudaFuncAttributeMaxDynamicSharedMemorySize, large_smem)) != cudaSuccess ||
             (e = cudaFuncSetAttribute(scan_huge_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, large_smem)) != cudaSuccess) {
@@ -498,8 +510,7 @@ cudaError_t scan_structure(const int32_t *rowptr, const int32_t *colind, int64_t
         if (dev < kMaxDevices) attr_set[dev].store(1, std::memory_order_release);
     }
     const int sms = sm_count_cached();
-    // block columns of a wider matrix do not fit a word of the warp tables: all its block-rows take a CTA
-    const int64_t small = Kb < (int64_t{1} << (32 - kCountBits)) - 1 ? kSmallNnz : 0;
+    const int64_t small = wide ? kSmallNnz / 2 : kSmallNnz;
     // the longest chains first; the others fill in beside them.  With a block-row per SM at most the large CTAs take the medium ones too
     // (one launch less: 2,048 rows 45 -> 42 us for the whole plan).
     const bool few = Mb <= sms;
@@ -510,7 +521,7 @@ cudaError_t scan_structure(const int32_t *rowptr, const int32_t *colind, int64_t
         e = launch_overlapped(medium, static_cast<unsigned>(std::min<int64_t>(Mb, 3 * sms)), kMediumThreads, static_cast<size_t>(medium_smem), st, rowptr,
                               colind, M, Kb, small, kMediumNnz, nullptr, out);
     if (e == cudaSuccess)
-        e = launch_overlapped(scan_small_kernel, static_cast<unsigned>(std::min<int64_t>((Mb + kScanWarps - 1) / kScanWarps, 3 * sms)),
+        e = launch_overlapped(warps, static_cast<unsigned>(std::min<int64_t>((Mb + kScanWarps - 1) / kScanWarps, 3 * sms)),
                               32 * kScanWarps, static_cast<size_t>(small_smem), st, rowptr, colind, M, small, out);
     if (e == cudaSuccess && Kb > kLargeSlots) {
         scan_huge_kernel<<<static_cast<unsigned>(sms), kLargeThreads, large_smem, st>>>(rowptr, colind, M, Kb, huge, out);

@@ -47,3 +47,26 @@ def test_counts_at_the_edges_of_the_tables(K, order):
         mine = plan.info().as_dict()
         plan.close()
         assert {k: mine[k] for k in ref} == ref
+
+
+@pytest.mark.parametrize("K", [67108832, 67108833, 2 ** 27 + 5])
+@pytest.mark.parametrize("where", ["last", "any"])
+def test_highest_block_columns_of_the_warp_tables(where, K):
+    """The last matrix whose block columns share a word with a count (2^22 - 2 of them), the first that is wider and a much wider one:
+    block-rows of half as many, as many and more nonzeros as a warp takes, in the last block columns or anywhere."""
+    rng = np.random.default_rng(K % 1000)
+    lengths, cols = [], []
+    for n in rng.permutation(np.resize([1, 5, 499, 500, 501, 999, 1000, 1001, 4097], 200)):
+        r = rng.multinomial(n, np.full(16, 1 / 16))
+        lengths.append(r)
+        for k in r:
+            low = K - 5000 if where == "last" else 0
+            cols.append(np.sort(low + rng.choice(K - low, size=k, replace=False) if K - low < 10000 else np.unique(rng.integers(low, K, 2 * k))[:k]))
+            assert cols[-1].size == k
+    lengths, colind = np.concatenate(lengths), np.concatenate(cols).astype(np.int32)
+    rowptr = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    ref = oracle.summary(rowptr, colind, lengths.size, K, 1).as_dict()
+    plan = sd.Plan(dev(rowptr), dev(colind), torch.zeros(colind.size, device="cuda"), lengths.size, K, 1, family=sd.SD_ROWSPLIT)
+    mine = plan.info().as_dict()
+    plan.close()
+    assert {k: mine[k] for k in ref} == ref
