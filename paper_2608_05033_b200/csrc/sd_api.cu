@@ -428,6 +428,7 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
             cp.rowptr = plan->rowptr;
             cp.M = plan->info.empty_rows > 0 ? M : 0;   // no search for rows without nonzeros when the scan found none
             cp.nnz = plan->nnz;
+            cp.shift = plan->coo_shift;
             cp.c1_row = plan->coo_c1_row;
             cp.c1_val = plan->coo_c1_val;
             cp.c2_row = plan->coo_c2_row;

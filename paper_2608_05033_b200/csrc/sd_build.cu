@@ -552,9 +552,10 @@ static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
     SD_CUDA_TRY(cudaStreamSynchronize(st));
     if (hot < 1 || hot > most || 4 * static_cast<int64_t>(sum) < p->nnz) return SD_OK;
     if ((s = dev_alloc(p, &p->coo_hot_cols, hot, "frequent columns", st))) return s;
-    if ((s = dev_alloc(p, &p->coo_hot_colind, p->nnz, "renamed columns", st))) return s;
+    p->coo_shift = coo_shift(p->vals, p->dtype == SD_F32 ? 4 : 2, static_cast<int>(p->N));   // the renamed columns can begin anywhere
+    if ((s = dev_alloc(p, &p->coo_hot_colind, p->nnz + p->coo_shift, "renamed columns", st))) return s;
     hot_names_kernel<<<cols, 256, 0, st>>>(degree.as<int32_t>(), K, flag.as<int32_t>(), p->coo_hot_cols);
-    rename_columns_kernel<<<wide, 256, 0, st>>>(p->colind, p->nnz, degree.as<int32_t>(), p->coo_hot_colind);
+    rename_columns_kernel<<<wide, 256, 0, st>>>(p->colind, p->nnz, degree.as<int32_t>(), p->coo_hot_colind + p->coo_shift);
     SD_CUDA_TRY(cudaGetLastError());
     p->coo_hot = hot;
     return SD_OK;
@@ -562,19 +563,21 @@ static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
 
 sd_status_t build_coo(sd_plan *p, cudaStream_t st) {
     sd_status_t s;
-    const int64_t steps = coo_steps(p->nnz, static_cast<int>(p->N));
+    p->coo_shift = coo_shift(p->colind, sizeof(int32_t), static_cast<int>(p->N));   // values of the same slice then are one load too, or two
+    if ((s = coo_hot_columns(p, st))) return s;
+    const int64_t items = p->nnz + p->coo_shift, steps = coo_steps(items, static_cast<int>(p->N));
     const int64_t count2 = 2 * coo_most_ranges(steps, static_cast<int64_t>(kCooMaxWarps) * p->info.sm_count);
     const int64_t chunks2 = (count2 + kCooCarryChunk - 1) / kCooCarryChunk, count3 = 2 * chunks2;
     const bool bits = p->N == 1 && p->info.empty_rows == 0;
-    if ((s = dev_alloc(p, &p->coo_row, bits ? 32 * steps : p->nnz, "rows of nonzeros", st))) return s;
+    if ((s = dev_alloc(p, &p->coo_row, bits ? 32 * steps : items, "rows of nonzeros", st))) return s;
     if (bits && (s = dev_alloc(p, &p->coo_starts, 32 * steps, "starts of rows", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c1_row, count2, "carry rows", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c1_val, count2 * p->N, "carry sums", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c2_row, count3, "carry rows (level 2)", st))) return s;
     if ((s = dev_alloc(p, &p->coo_c2_val, count3 * p->N, "carry sums (level 2)", st))) return s;
-    SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, steps, p->coo_row, p->coo_starts, st));
+    SD_CUDA_TRY(build_coo_rows(p->rowptr, p->M, p->nnz, p->coo_shift, steps, p->coo_row, p->coo_starts, st));
     p->info.launches = 2 + (count2 > kCooDirectFinal);
-    return coo_hot_columns(p, st);
+    return SD_OK;
 }
 
 // =====================================================================================

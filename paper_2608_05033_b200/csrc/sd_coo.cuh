@@ -38,10 +38,13 @@ constexpr int kCooHotThreads = 1024;
 constexpr int coo_threads(int N) { return N == 1 ? 128 : 256; }
 
 struct CooArgs {
+    // Items are the nonzeros after `shift` others that are nothing: so many that item 0 of the columns lies on a multiple of what a lane
+    // loads at once.  The arrays start at item 0; those of the caller begin at item `shift`.
     const int32_t *row;      // [count] row of every item (ascending), or with `starts` of every eighth
-    const uint8_t *starts;   // one column without empty rows: bit u of byte g: nonzero 8g + u begins a row
+    const uint8_t *starts;   // one column without empty rows: bit u of byte g: item 8g + u begins a row
     const int32_t *colind;   // [count] column of every nonzero
     const void *vals;        // [count] values of A; carry list: [count][N] float partial sums
+    unsigned shift;
     const void *B;
     uint32_t ldb_bytes;
     int64_t count;           // items
@@ -90,30 +93,39 @@ __device__ __forceinline__ void coo_row_of_b(const T *p, float (&b)[N]) {
     }
 }
 
-// U consecutive elements, widened, with one load if `align`, the address of the array, allows it.
+// U consecutive elements, widened: one load, from a multiple of its size.
+template <typename T, int U>
+__device__ __forceinline__ void load_wide(const T *p, float (&o)[U]) {
+    if constexpr (U * sizeof(T) == 32) {
+        const Words8 v = live_load(reinterpret_cast<const Words8 *>(p));
+#pragma unroll
+        for (int u = 0; u < U; ++u) o[u] = __uint_as_float(v.w[u]);
+    } else if constexpr (U * sizeof(T) == 16) {
+        RowLoad<T, U>::ld(p, o);
+    } else {
+        coo_row_of_b<T, U, true>(p, o);
+    }
+}
+// ... or two, or one per element, as `align`, the address of the array, allows.
 template <typename T, int U>
 __device__ __forceinline__ void load_run(const T *p, unsigned align, float (&o)[U]) {
     if (align % (U * sizeof(T)) == 0) {
-        if constexpr (U * sizeof(T) == 32) {
-            const Words8 v = live_load(reinterpret_cast<const Words8 *>(p));
+        load_wide<T, U>(p, o);
+    } else if (align % (U / 2 * sizeof(T)) == 0) {
+        float low[U / 2], high[U / 2];
+        load_wide<T, U / 2>(p, low);
+        load_wide<T, U / 2>(p + U / 2, high);
 #pragma unroll
-            for (int u = 0; u < U; ++u) o[u] = __uint_as_float(v.w[u]);
-        } else if constexpr (U * sizeof(T) == 16) {
-            RowLoad<T, U>::ld(p, o);
-        } else {   // four bf16 values
-            const uint2 v = live_load(reinterpret_cast<const uint2 *>(p));
-            o[0] = __uint_as_float(v.x << 16), o[1] = __uint_as_float(v.x & 0xFFFF0000u);
-            o[2] = __uint_as_float(v.y << 16), o[3] = __uint_as_float(v.y & 0xFFFF0000u);
-        }
+        for (int u = 0; u < U / 2; ++u) o[u] = low[u], o[U / 2 + u] = high[u];
     } else {
 #pragma unroll
         for (int u = 0; u < U; ++u) o[u] = to_float(p[u]);
     }
 }
 template <int U>
-__device__ __forceinline__ void load_ints(const int32_t *p, unsigned align, int (&o)[U]) {
+__device__ __forceinline__ void load_ints(const int32_t *p, int (&o)[U]) {
     float t[U];
-    load_run<float, U>(reinterpret_cast<const float *>(p), align, t);
+    load_wide<float, U>(reinterpret_cast<const float *>(p), t);
 #pragma unroll
     for (int u = 0; u < U; ++u) o[u] = __float_as_int(t[u]);
 }
@@ -163,7 +175,7 @@ coo_kernel(const CooArgs a) {
     if (w >= a.warps) return;
     if (a.M > 0) coo_empty_rows<N>(a, w, a.warps);
     const T *vals = static_cast<const T *>(a.vals), *B = static_cast<const T *>(a.B);
-    const unsigned va = static_cast<unsigned>(reinterpret_cast<uintptr_t>(vals)), ca = static_cast<unsigned>(reinterpret_cast<uintptr_t>(a.colind));
+    const unsigned va = static_cast<unsigned>(reinterpret_cast<uintptr_t>(vals));
 
     auto emit = [&](int row, const float (&v)[N]) {
 #pragma unroll
@@ -192,19 +204,19 @@ coo_kernel(const CooArgs a) {
             unsigned starts = 0;    // items that begin a row
             int row_in = 0;         // the row that is open where the lane begins ...
             int row_out = 0;        // ... and where it ends
-            const bool whole = k0 - lane * U + STEP <= count;   // the same in all lanes: no item is past the end
+            const bool whole = k0 - lane * U >= a.shift && k0 - lane * U + STEP <= count;   // the same in all lanes: every item is a nonzero
             if (whole) {
-                load_ints<U>(a.colind + k0, ca, col);
-                if constexpr (!BITS) load_ints<U>(a.row + k0, 0, r);
+                load_ints<U>(a.colind + k0, col);
+                if constexpr (!BITS) load_ints<U>(a.row + k0, r);
                 load_run<T, U>(vals + k0, va, av);
-            } else {                // items past the end continue the last row with zeros
+            } else {                // items before the first nonzero are zeros of its row, those past the end of the last one's
                 const int pad = BITS ? 0 : __ldg(a.row + a.count - 1);
 #pragma unroll
                 for (int u = 0; u < U; ++u) {
-                    const bool ok = k0 + u < count;
+                    const bool ok = k0 + u >= a.shift && k0 + u < count;
                     col[u] = ok ? __ldg(a.colind + k0 + u) : 0;
                     av[u] = ok ? to_float(vals[k0 + u]) : 0.f;
-                    r[u] = BITS ? 0 : (ok ? __ldg(a.row + k0 + u) : pad);
+                    r[u] = BITS ? 0 : (k0 + u < count ? __ldg(a.row + k0 + u) : pad);
                 }
             }
             if constexpr (BITS) {
@@ -238,7 +250,7 @@ coo_kernel(const CooArgs a) {
             if (!whole)   // they gathered row 0: never let its contents (Inf, NaN) in
 #pragma unroll
                 for (int u = 0; u < U; ++u)
-                    if (k0 + u >= count)
+                    if (k0 + u < a.shift || k0 + u >= count)
 #pragma unroll
                         for (int e = 0; e < N; ++e) b[u][e] = 0.f;
             if constexpr (!BITS) {
@@ -407,9 +419,10 @@ __global__ void coo_final_kernel(const int32_t *row, const float *val, int64_t c
     }
 }
 
-// Plan time: the row of every nonzero, or of every eighth.
-static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64_t M, int64_t nnz, int64_t every, int64_t count, int32_t *__restrict__ row) {
-    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, k = min(i * every, nnz - 1);
+// Plan time: the row of every item, or of every eighth.
+static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64_t M, int64_t nnz, int64_t shift, int64_t every, int64_t count,
+                                       int32_t *__restrict__ row) {
+    const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x, k = min(max(i * every - shift, int64_t{0}), nnz - 1);
     if (i >= count) return;
     int64_t lo = 0, hi = M;   // last row with rowptr[row] <= k
     while (hi - lo > 1) {
@@ -419,11 +432,11 @@ static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64
     }
     row[i] = static_cast<int32_t>(lo);
 }
-// A bit per nonzero that begins a row; every row has one (`starts` is cleared before).
-static __global__ void coo_starts_kernel(const int32_t *__restrict__ rowptr, int64_t M, unsigned *__restrict__ starts) {
+// A bit per item that begins a row after the first; every row has one (`starts` is cleared before).
+static __global__ void coo_starts_kernel(const int32_t *__restrict__ rowptr, int64_t M, unsigned shift, unsigned *__restrict__ starts) {
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (r >= M) return;
-    const unsigned k = static_cast<unsigned>(__ldg(rowptr + r));
+    if (r < 1 || r >= M) return;
+    const unsigned k = static_cast<unsigned>(__ldg(rowptr + r)) + shift;
     atomicOr(starts + (k >> 5), 1u << (k & 31));
 }
 

@@ -46,30 +46,33 @@ cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st);
 // gain; measured cross-over between 4 and 8 columns): segmented reduction over the nonzeros, carries reduced in two more levels.
 constexpr int kCooMaxN = 4;
 constexpr int coo_items(int N) { return N <= 2 ? 8 : 4; }   // nonzeros of a lane and step
-constexpr int64_t coo_steps(int64_t nnz, int N) { return (nnz + 32 * coo_items(N) - 1) / (32 * coo_items(N)); }
+// items before the first nonzero: what a lane takes of `array` is then one load, wherever it begins
+inline int coo_shift(const void *array, int element, int N) { return static_cast<int>(reinterpret_cast<uintptr_t>(array) / element % coo_items(N)); }
+constexpr int64_t coo_steps(int64_t items, int N) { return (items + 32 * coo_items(N) - 1) / (32 * coo_items(N)); }
 constexpr int kCooCarryChunk = 128;
 constexpr int64_t kCooDirectFinal = 4096;  // carry lists up to this length skip the second level
 constexpr int kCooMaxWarps = 64;           // resident on one SM; each leaves two carry entries per range
 constexpr int kCooRange = 64;              // steps: longer shares of a warp are cut into several ranges
 constexpr int64_t coo_most_ranges(int64_t steps, int64_t warps) { return steps < warps ? steps : warps + steps / kCooRange; }
 struct CooPlan {
-    const int32_t *row;    // [nnz] row of every nonzero, or with `starts` [32 steps] of every eighth
-    const uint8_t *starts; // [32 steps] a bit per nonzero that begins a row
+    const int32_t *row;    // [shift + nnz] row of every item, or with `starts` [32 steps] of every eighth
+    const uint8_t *starts; // [32 steps] a bit per item that begins a row
     const int32_t *rowptr; // [M + 1]
     int64_t M;             // rows to search for empty ones (0: the matrix has none)
     int64_t nnz;
+    int shift;             // items before the first nonzero
     int32_t *c1_row;      // [2 * coo_most_ranges(steps, kCooMaxWarps * SMs)] first-level carries
     float *c1_val;        // ... x N
     int32_t *c2_row;      // [2 * ceil(len(c1) / kCooCarryChunk)] second-level carries
     float *c2_val;
-    const int32_t *hot_colind;   // [nnz] columns, those of hot_cols renamed (hot == 0: none)
+    const int32_t *hot_colind;   // [shift + nnz] columns, those of hot_cols renamed (hot == 0: none)
     const int32_t *hot_cols;
     int32_t hot;
 };
 constexpr int kCooHotBytes = 128 * 1024;   // the rest is L1 for the gathers outside: with 200 KB two fp32 columns took 281 us instead of 173
 cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, int sm_count, cudaStream_t st);
-// starts != nullptr: a bit per nonzero and the row of every eighth; no row is empty.
-cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st);
+// starts != nullptr: a bit per item and the row of every eighth; no row is empty.
+cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int shift, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st);
 
 struct BsrArgs {
     const int32_t *browptr;  // [Mb + 1]

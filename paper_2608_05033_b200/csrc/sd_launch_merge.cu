@@ -51,11 +51,12 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, int sm_cou
     CooArgs a{};
     a.row = cp.row;
     a.starts = cp.starts;
-    a.colind = s.colind;
-    a.vals = s.vals;
+    a.colind = s.colind - cp.shift;
+    a.vals = static_cast<const T *>(s.vals) - cp.shift;
+    a.shift = cp.shift;
     a.B = s.B;
     a.ldb_bytes = s.ldb_bytes;
-    a.count = cp.nnz;
+    a.count = cp.nnz + cp.shift;
     a.C = s.C;
     a.ldc = s.ldc;
     a.alpha = s.alpha;
@@ -124,14 +125,14 @@ cudaError_t run_coo(const CooPlan &cp, const SpmmArgs &s, int dtype, int sm_coun
     return dtype == SD_F32 ? launch_coo<float>(cp, s, sm_count, st) : launch_coo<__nv_bfloat16>(cp, s, sm_count, st);
 }
 
-cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st) {
+cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int shift, int64_t steps, int32_t *row, uint8_t *starts, cudaStream_t st) {
     if (nnz == 0) return cudaSuccess;
-    const int64_t count = starts ? 32 * steps : nnz;
-    coo_rows_kernel<<<static_cast<unsigned>((count + 255) / 256), 256, 0, st>>>(rowptr, M, nnz, starts ? 8 : 1, count, row);
+    const int64_t count = starts ? 32 * steps : nnz + shift;
+    coo_rows_kernel<<<static_cast<unsigned>((count + 255) / 256), 256, 0, st>>>(rowptr, M, nnz, shift, starts ? 8 : 1, count, row);
     if (starts) {
         const cudaError_t e = cudaMemsetAsync(starts, 0, 32 * steps, st);
         if (e != cudaSuccess) return e;
-        coo_starts_kernel<<<static_cast<unsigned>((M + 255) / 256), 256, 0, st>>>(rowptr, M, reinterpret_cast<unsigned *>(starts));
+        coo_starts_kernel<<<static_cast<unsigned>((M + 255) / 256), 256, 0, st>>>(rowptr, M, shift, reinterpret_cast<unsigned *>(starts));
     }
     return cudaGetLastError();
 }

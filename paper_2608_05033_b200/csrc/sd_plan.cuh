@@ -48,8 +48,9 @@ struct sd_plan {
     int32_t h_T = 0;                 // 0: no schedule (nothing to multiply, or another executor)
 
     // narrow dense operands (N <= kCooMaxN) of the merge family
-    int32_t *coo_row = nullptr;      // row of every nonzero, or with coo_starts of every eighth
-    uint8_t *coo_starts = nullptr;   // a bit per nonzero that begins a row (one column, no empty rows)
+    int coo_shift = 0;               // items before the first nonzero
+    int32_t *coo_row = nullptr;      // row of every item, or with coo_starts of every eighth
+    uint8_t *coo_starts = nullptr;   // a bit per item that begins a row (one column, no empty rows)
     int32_t *coo_c1_row = nullptr, *coo_c2_row = nullptr;
     float *coo_c1_val = nullptr, *coo_c2_val = nullptr;
     int32_t *coo_hot_colind = nullptr, *coo_hot_cols = nullptr;   // columns kept in shared memory

@@ -1,5 +1,6 @@
-"""One column with a lane per eight nonzeros or, where the arrays are not aligned, per 32; two and three columns on a matrix whose nonzeros crowd into few columns: the kernel that keeps those columns' rows of B in
-shared memory, with columns outside, empty rows, a row over many chunks."""
+"""One to four columns: a warp owns a range of nonzeros, a lane adds up eight or four consecutive ones, carries join the ranges.  On
+matrices whose nonzeros crowd into few columns the kernel keeps those columns' rows of B in shared memory, with columns outside, empty
+rows, a row over many ranges."""
 import numpy as np
 import pytest
 
@@ -75,6 +76,67 @@ def test_ranges_of_warps(M, length, empty, N, dtype):
     w = W.random_csr(M, K, N, lengths, seed=M + N, dtype=dtype, alpha=1.25, beta=-0.5)
     plan = DeviceWorkload(w).plan(family=sd.SD_MERGE)
     for kw in (dict(), dict(pad_b=4 - N, pad_c=1), dict(offset=1)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
+    got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
+    check(w, got, beta=0.0)
+    plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N", [1, 2, 3, 4])
+@pytest.mark.parametrize("empty", [False, True])
+def test_columns_and_values_from_any_offset(empty, N, dtype):
+    """Slices of a longer CSR: columns that begin at every entry of a 32-byte piece, values at the same, at another and, as new values
+    of the same plan, at a third; the first row shorter and longer than what is missing of the piece; rows without nonzeros."""
+    for first in (1, 2400):
+        lengths = np.random.default_rng(first).integers(1, 60, 701)
+        lengths[[0, 350]] = first, 2400
+        if empty:
+            lengths[::7] = 0
+        w = W.random_csr(701, 2500, N, lengths, seed=N + first, dtype=dtype, alpha=1.5, beta=-0.5)
+        w.B[0] = np.inf if dtype == W.SD_F32 else 0x7F80   # no row names column 0: items that are no nonzeros must not bring it in
+        w.colind[w.colind == 0] = 1
+        rowptr, column, value = dev(w.rowptr), {}, {}
+        for off in range(9):
+            column[off], value[off] = (dev(np.concatenate([np.zeros(off, a.dtype), a, np.zeros(8, a.dtype)]))[off:] for a in (w.colind, w.vals))
+        for co, vo in [(off, off) for off in range(8)] + [(0, 1), (1, 0), (4, 0), (0, 4), (3, 8), (2, 6)]:
+            plan = sd.Plan(rowptr, column[co], value[vo], w.M, w.K, N, dtype=dtype, family=sd.SD_MERGE)
+            got, intact = run_spmm(plan, w)
+            assert intact
+            check(w, got)
+            plan.update_values(value[(vo + 3) % 8])
+            assert np.array_equal(got, run_spmm(plan, w)[0])
+            plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("N,empty,offset", [(1, False, 0), (1, False, 3), (1, True, 0), (1, True, 5), (4, True, 1)])
+def test_frequent_columns_of_one_and_four_columns(N, empty, offset, dtype):
+    """One column from 4,096,000 nonzeros on, rows told by a bit per nonzero or, with empty rows among them, by a row index; four bf16
+    columns from 2,457,600 on, four fp32 columns without frequent ones; slices of a longer CSR."""
+    rng = np.random.default_rng(N + offset)
+    M, K = 9203, 70001
+    rows = []
+    for i in range(M):
+        n = 0 if empty and i % 37 == 5 else 30000 if i == 11 else 700
+        rows.append(np.unique((K * rng.random(n) ** 5).astype(np.int32)))
+    rowptr = np.concatenate([[0], np.cumsum([r.size for r in rows])]).astype(np.int32)
+    cols = np.concatenate(rows).astype(np.int32)
+    assert cols.size > 4096 * 1000
+    vals, B = rng.standard_normal(cols.size).astype(np.float32), rng.standard_normal((K, N)).astype(np.float32)
+    C = rng.standard_normal((M, N)).astype(np.float32)
+    if dtype == W.SD_BF16:
+        vals, B = W.f32_to_bf16_bits(vals), W.f32_to_bf16_bits(B).reshape(K, N)
+    w = W.Workload("frequent_columns", M, K, N, rowptr, cols, vals, B, C, -0.75, 0.5, dtype, {})
+    colind, values = (dev(np.concatenate([np.zeros(offset, a.dtype), a]))[offset:] for a in (cols, vals))
+    plan = sd.Plan(dev(rowptr), colind, values, M, K, N, dtype=dtype, family=sd.SD_MERGE)
+    renamed = 0 if N == 4 and dtype == W.SD_F32 else 4
+    rows_told = 0.625 if N == 1 and not empty else 4
+    assert (rows_told + renamed) * cols.size < plan.info().plan_bytes < (rows_told + renamed + 1) * cols.size
+    for kw in (dict(), dict(pad_b=3, pad_c=1), dict(offset=1)):
         got, intact = run_spmm(plan, w, **kw)
         assert intact
         check(w, got)
