@@ -17,12 +17,17 @@ namespace sd {
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
 //   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four to
 //                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
-//                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64 (64 bf16 columns, 24, 44: 31.3, 30.6 / 26.7,
-//                             26.3 / 37.7, 30.5), of eight loads two (32 columns, 44: one 25.4, two 23.6), then four (32 columns, 125: 41.6 /
-//                             34.8 / 27.3)
+//                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64 (24 columns, 24, 44: 18.7, 29.8 / 15.6,
+//                             25.0 / -), then four (32 columns, 125: 41.6 / 34.8 / 27.3).  8: two, as many as in the set kernel, which has
+//                             2,048 threads on an SM for 1,280: that is ahead where B is far from the SMs, beyond 16 MB with fp32 values and
+//                             with bf16 on rows below 32, unless some row is much longer and walked faster here
+//                             (32 columns, set kernel / two sets, 60,000 rows of 24, 44: 16.2, 25.3 / 15.3, 23.4, 200,000 47.1, 77.6 /
+//                             49.9, 79.0, 400,000 104, 158 / 120, 174; 64 bf16 columns 20.5, 30.4 / 19.1, 26.8, 61.4, 92.3 / 62.3, 86.4,
+//                             133, 195 / 141, 195)
 //   9 to 16 loads             one set from 8 (64 columns, 12, 24: 27.7, 47.2 / 24.9, 38.9 / 29.4, 42.7; 128 bf16 columns, 24: 63.7 / 47.3
 //                             / 54.6; 6: 56.3 / 58.2 / 86.0), and on shorter rows where the loads are no power of two (96 bf16 columns, 3: 83.7 /
-//                             76.0 / 121); two of 16 loads from 32 and four from 40
+//                             76.0 / 121); bf16 two of 16 loads from 32 and four from 40, of even length fp32 the set
+//                             kernel to 64 (64 columns, 35, set kernel / two sets: 60,000 rows 32.7 / 32.8, 200,000 109 / 127, 400,000 302 / 345)
 //   17 to 32 loads            one set (128 columns, 6, 24: 89.9, 82.9 / 83.5, 72.3 / 109, 77.2), bf16 from 16 (200 columns, 12, 24: 66.1, 66.7 /
 //                             70.7, 57.8 / 72.1, 58.0); four from 40 (200 bf16 columns, 44: 77.5 / 64.4 / 58.8)
 //   beyond 32                 the plain kernel has two loads per lane and half the warps: one set to 12, then four (256 columns, 6, 12:
@@ -34,13 +39,16 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     while (lanes < 32 && lanes < units) lanes <<= 1;
     const bool fills = a.S * lanes >= static_cast<int64_t>(sm_count_cached()) * 5 * kRowGroupThreads;
     const bool pow2 = (units & (units - 1)) == 0, bf16 = dtype == SD_BF16;
+    const bool even = a.max_len <= 4 * mean, far = a.b_bytes > 16000000 && even;
     const bool one_length = mean < 16 && a.max_len <= 2 * mean;
     int sets = 0;
     if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
     else if (!fills && mean >= 8) sets = 4;
     else if (one_length) sets = 0;
     else if (a.N <= 8) sets = mean < 8 ? 1 : mean < 64 ? 4 : 0;
-    else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? (mean < 64 ? 4 : 0) : units == 4 ? 0 : mean < 64 ? (pow2 ? 2 : 1) : 4;
+    else if (units == 8 && mean >= 16 && mean < 64) sets = far && (!bf16 || mean < 32) ? 0 : 2;
+    else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? (mean < 64 ? 4 : 0) : units == 4 ? 0 : mean < 64 ? 1 : 4;
+    else if (units == 16 && !bf16 && mean >= 32 && mean < 64 && even) sets = 0;
     else if (units <= 16) sets = mean >= 40 ? 4 : pow2 && mean >= 32 ? 2 : mean >= 8 || !pow2 ? 1 : 0;
     else if (units <= 32) sets = mean >= 40 ? 4 : !bf16 || mean >= 16 ? 1 : 0;
     else sets = mean >= 12 ? 4 : 1;
