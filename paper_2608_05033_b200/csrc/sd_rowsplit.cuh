@@ -184,13 +184,16 @@ inline LaneGeom lane_geometry(int64_t N, bool vec, int vecw, int two_from) {
 
 // Two vectors per lane where they leave no more lanes idle and a group still covers a 128-byte line with one load (a gather costs a
 // cycle of L1 per line it touches): from nine vectors on (1 M stencil rows at 48 fp32 columns 210 -> 143 us, at 64 also before).  fp32
-// also at five to seven (24 columns 107 -> 80, 160,000 rows 11.5 -> 10.9) and, where operands come from DRAM and the lines are the
-// smaller cost, at four and eight: C beyond 40 MB (32 columns: 1 M rows 111 -> 89, 360,000 rows 38.1 -> 31.6, 250,000 18.6 -> 19.0; 16
-// columns: 640,000 rows 36.6 -> 33.3, 360,000 14.4 -> 16.6).  bf16 lanes hold twice the sums: slower there (64 columns 137 -> 155).
+// also at five to seven with C beyond 10 MB (24 columns: 1 M rows 107 -> 80, 160,000 rows 11.5 -> 10.9, 62,500 5.2 -> 5.6) and, where
+// operands come from DRAM and the lines are the smaller cost, at four and eight: C beyond 40 MB (32 columns: 1 M rows 111 -> 89, 360,000
+// rows 38.1 -> 31.6, 250,000 18.6 -> 19.0; 16 columns: 640,000 rows 36.6 -> 33.3, 360,000 14.4 -> 16.6).  bf16 lanes hold twice the sums:
+// slower there (64 columns 137 -> 155).  Rows of more than 64 nonzeros, from 16 vectors on: fewer lanes request fewer pairs of a row at a
+// time, and one long row is what such a matrix waits for (the longest 900: 24 fp32 columns 123 -> 255 us, 96 bf16 columns 187 -> 280).
 inline int rowsplit_two_from(const SpmmArgs &a, bool bf16) {
-    const int64_t units = (a.N + 3) / 4;
+    if (a.max_len <= 0 || a.max_len > 64) return 16;
     if (bf16) return 9;
-    return (units > 4 && units < 8) || (units >= 4 && a.S * a.N * 4 >= 40000000) ? 4 : 9;
+    const int64_t units = (a.N + 3) / 4, c_bytes = a.S * a.N * 4;
+    return units >= 4 && c_bytes >= (units > 4 && units < 8 ? 10000000 : 40000000) ? 4 : 9;
 }
 
 template <typename T>
