@@ -411,6 +411,7 @@ static sd_status_t run_product(const sd_plan_t *plan, int64_t N, const void *B, 
     a.max_len = plan->info.max_r;
     a.mean_len = M > 0 ? (plan->nnz + M - 1) / M : 0;
     a.b_bytes = plan->K * N * (plan->dtype == SD_F32 ? 4 : 2);
+    a.shared = plan->nnz >= 4 * plan->info.nnzb16;
     a.N = static_cast<int32_t>(N);
     a.alpha = alpha;
     a.beta = beta;

@@ -167,6 +167,7 @@ struct SpmmArgs {
     int64_t max_len;        // longest row if known (0: unknown); lets the row-split kernel drop its second accumulator
     int64_t mean_len;       // mean row length rounded up if known (0: unknown): lanes per row of the narrow row-split kernel
     int64_t b_bytes;        // of the rows and columns of B that the product reads
+    bool shared;            // neighbouring rows name the same rows of B: four nonzeros per occupied 16x16 block at least
 };
 
 // A/B measurement switches (none is needed in normal use).  The environment is read once, at the

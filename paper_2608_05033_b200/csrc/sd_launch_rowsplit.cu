@@ -12,8 +12,14 @@ namespace sd {
 //   not whole 16-byte loads   always (41 columns: 1.8 to 3.9 times as fast as one scalar per lane)
 //   few rows                  four sets as soon as rows are 8 long: one set leaves the GPU idle (5,000 rows of 30 at 64 columns
 //                             17.9 -> 5.3 us, at 128 bf16 24.9 -> 6.7)
-//   short rows of one length  the plain kernel, whose loop has no last, tested step (stencils of 360,000 rows at 8, 32, 64 fp32 columns 9.6, 38.9,
-//                             56.3 / 10.2, 49.1, 97.6 / -, of 1 M rows at 32, 64 bf16 columns 73.9, 137 / 85.8, 165 / -)
+//   short rows of one length  the plain kernel, whose loop has no last, tested step, where neighbouring rows share rows of B, so that
+//                             instructions are the bound, from five loads on (stencils, us plain / one set: 5 points, 360,000 rows at 32, 64
+//                             fp32 columns 29.5, 48.8 / 39.9, 77.1, 1 M rows at 64 bf16 columns 115 / 129).  Others wait for their gathers:
+//                             one set from 12 nonzeros (400,000 rows of 12, 15 at 64 fp32 columns 136, 163 / 131, 156), from 6 with up to
+//                             four loads (60,000 rows of 6, 12 at 16 fp32 columns 4.7, 6.5 / 4.3, 5.6, 7-point stencils 30.0 / 28.2) and, but
+//                             where the plain kernel takes two loads per lane, up to eight (60,000 rows of 6, 12 at 24 fp32 columns 6.6,
+//                             10.9 / 5.9, 7.8, 400,000 33.0, 52.1 / 41.1, 50.6) and beyond 16; bf16 with one load always (1 M rows of 4
+//                             26.3 / 24.8, of 15 105 / 81, 5-point stencils 14.8 / 13.7)
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
 //   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four to
 //                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
@@ -32,6 +38,13 @@ namespace sd {
 //                             70.7, 57.8 / 72.1, 58.0); four from 40 (200 bf16 columns, 44: 77.5 / 64.4 / 58.8)
 //   beyond 32                 the plain kernel has two loads per lane and half the warps: one set to 12, then four (256 columns, 6, 12:
 //                             240, 109 / 179, 109 / 180, 113)
+static int one_length_from(const SpmmArgs &a, int units, bool bf16) {
+    if (bf16 && units == 1) return 1;
+    if (units <= 4) return 6;
+    if (a.shared || units > (bf16 ? 16 : 32)) return 16;
+    const bool two = !bf16 && units >= rowsplit_two_from(a, bf16);
+    return units > 16 || (units <= 8 && !two) ? 6 : 12;
+}
 static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     const int units = (a.N + vw - 1) / vw;
     const int64_t mean = a.mean_len;
@@ -44,7 +57,7 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     int sets = 0;
     if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
     else if (!fills && mean >= 8) sets = 4;
-    else if (one_length) sets = 0;
+    else if (one_length) sets = mean >= one_length_from(a, units, bf16) ? 1 : 0;
     else if (a.N <= 8) sets = mean < 8 ? 1 : mean < 64 ? 4 : 0;
     else if (units == 8 && mean >= 16 && mean < 64) sets = far && (!bf16 || mean < 32) ? 0 : 2;
     else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? (mean < 64 ? 4 : 0) : units == 4 ? 0 : mean < 64 ? 1 : 4;

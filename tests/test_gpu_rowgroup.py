@@ -110,3 +110,24 @@ def test_lane_sets_on_matrices_that_fill_the_gpu(loads, K, usual, longest, dtype
     check(w, got)
     assert np.array_equal(got, run_spmm(plan, w)[0])
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("loads", [1, 2, 4, 6, 8, 12, 20, 33])
+@pytest.mark.parametrize("length", [4, 6, 12, 15])
+@pytest.mark.parametrize("near", [False, True])
+def test_rows_of_one_length_that_share_rows_of_b(near, length, loads, dtype):
+    """Neighbouring rows name neighbouring columns, four nonzeros and more per occupied 16x16 block, or any: either side of the lines
+    between the plain and the row-group kernel, with more lanes than the GPU holds."""
+    N = loads * (4 if dtype == W.SD_F32 else 8)
+    M, K = 200_000 // min(32, loads) + 3, 5000
+    w = W.random_csr(M, K, N, np.full(M, length), seed=loads, dtype=dtype, alpha=0.5, beta=-1.5)
+    if near:
+        w.colind[:] = (np.arange(M)[:, None] // 4 % (K - length) + np.arange(length)).reshape(-1)
+    plan = DeviceWorkload(w).plan(family=sd.SD_ROWSPLIT)
+    assert (w.colind.size >= 4 * plan.info().nnzb16) == near
+    got, intact = run_spmm(plan, w)
+    assert intact
+    check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w)[0])
+    plan.close()
