@@ -432,11 +432,13 @@ static __global__ void coo_rows_kernel(const int32_t *__restrict__ rowptr, int64
     }
     row[i] = static_cast<int32_t>(lo);
 }
-// A bit per item that begins a row after the first; every row has one (`starts` is cleared before).
-static __global__ void coo_starts_kernel(const int32_t *__restrict__ rowptr, int64_t M, unsigned shift, unsigned *__restrict__ starts) {
+// A bit per item that begins a row after the first; every row has one (`starts` is cleared before).  Row pointers beyond the nonzeros, which
+// nobody has checked unless the caller asked for it, set none: the bits end with the nonzeros.
+static __global__ void coo_starts_kernel(const int32_t *__restrict__ rowptr, int64_t M, int64_t nnz, unsigned shift, unsigned *__restrict__ starts) {
     const int64_t r = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-    if (r < 1 || r >= M) return;
-    const unsigned k = static_cast<unsigned>(__ldg(rowptr + r)) + shift;
+    const int first = r < M ? __ldg(rowptr + r) : 0;
+    if (first <= 0 || first >= nnz) return;
+    const unsigned k = static_cast<unsigned>(first) + shift;
     atomicOr(starts + (k >> 5), 1u << (k & 31));
 }
 

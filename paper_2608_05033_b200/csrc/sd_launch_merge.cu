@@ -132,7 +132,7 @@ cudaError_t build_coo_rows(const int32_t *rowptr, int64_t M, int64_t nnz, int sh
     if (starts) {
         const cudaError_t e = cudaMemsetAsync(starts, 0, 32 * steps, st);
         if (e != cudaSuccess) return e;
-        coo_starts_kernel<<<static_cast<unsigned>((M + 255) / 256), 256, 0, st>>>(rowptr, M, shift, reinterpret_cast<unsigned *>(starts));
+        coo_starts_kernel<<<static_cast<unsigned>((M + 255) / 256), 256, 0, st>>>(rowptr, M, nnz, shift, reinterpret_cast<unsigned *>(starts));
     }
     return cudaGetLastError();
 }

@@ -124,3 +124,24 @@ def test_memory_kept_between_plans_is_given_back_on_request():
     assert torch.cuda.mem_get_info()[0] >= free0 - (64 << 20)   # the pool works in pieces of 32 MiB
     assert np.array_equal(run_spmm(kept, w)[0], before)
     kept.close()
+
+
+def test_row_starts_end_with_the_nonzeros():
+    """A blob whose summary no longer counts the empty rows, for a pattern with some at the end whose nonzeros fill a step of one column: the
+    bits of row starts end with the nonzeros, and the rows before the empty ones are right."""
+    lengths = np.concatenate([np.full(64, 4), np.zeros(40, np.int64)])
+    w = W.random_csr(104, 300, 1, lengths, seed=5)
+    dw = DeviceWorkload(w)
+    plan = dw.plan(family=sd.SD_MERGE)
+    info = plan.info()
+    blob = plan.save()
+    want, _ = run_spmm(plan, w)
+    plan.close()
+    at = blob.index(bytes(info))
+    assert info.empty_rows == 40
+    info.empty_rows = 0
+    plan = sd.Plan.load(blob[:at] + bytes(info) + blob[at + len(bytes(info)):], dw.rowptr, dw.colind, dw.vals)
+    got, intact = run_spmm(plan, w)
+    plan.close()
+    assert intact
+    np.testing.assert_allclose(got[:64], want[:64], rtol=1e-5, atol=1e-6)   # four products of one sign or the other per row
