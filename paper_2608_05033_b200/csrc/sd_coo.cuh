@@ -29,6 +29,8 @@
 // launch let in before the carries are written (scale 16 11.5 -> 12.1).
 #pragma once
 
+#include <type_traits>
+
 #include "sd_common.cuh"
 #include "sd_launch.cuh"
 
@@ -261,25 +263,53 @@ coo_kernel(const CooArgs a) {
 #pragma unroll
                 for (int u = 1; u < U; ++u) starts |= static_cast<unsigned>(r[u] != r[u - 1]) << u;
             }
-            // the lane's runs: the first may have begun before, the last may go on; those between are complete rows
+            // The lane's runs: the first may have begun before, the last may go on; those between are complete rows.  UPDATE: one column with
+            // beta, where a lane has up to seven of them: they wait for one round trip for the old values of C and not for one each (R-MAT
+            // scale 20, 32.4 M nonzeros fp32 130 -> 102 us, bf16 127 -> 98, scale 17 22.5 -> 18.0).
             float sum[N] = {}, top[N] = {};
+            [[maybe_unused]] float old_top = 0.f;
             bool closed = false;
-            int now = row_in;
+            auto runs = [&](auto update_tag) {
+                constexpr bool UPDATE = decltype(update_tag)::value;
+                unsigned held = 0;
+                int now = row_in;
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (starts >> u & 1u) {
-                    if (closed) emit(now, sum);
+                for (int u = 0; u < U; ++u) {
+                    const bool begins = starts >> u & 1u;
+                    float done[N];
+                    if (begins) {
+                        if (closed && !UPDATE) emit(now, sum);
+                        if (closed) held |= 1u << u;
+#pragma unroll
+                        for (int e = 0; e < N; ++e) {
+                            done[e] = sum[e];
+                            if (!closed) top[e] = sum[e];
+                            sum[e] = 0.f;
+                        }
+                        closed = true;
+                        now = BITS ? now + 1 : r[u];
+                    }
 #pragma unroll
                     for (int e = 0; e < N; ++e) {
-                        if (!closed) top[e] = sum[e];
-                        sum[e] = 0.f;
+                        sum[e] = fmaf(av[u], b[u][e], sum[e]);
+                        if (UPDATE && begins) b[u][e] = done[e];
                     }
-                    closed = true;
-                    now = BITS ? now + 1 : r[u];
                 }
+                if constexpr (UPDATE) {   // all old values are requested before the first is needed
+                    auto c_of = [&](int u) {
+                        return a.C + static_cast<int64_t>(BITS ? row_in + __popc(starts & ((1u << u) - 1u)) : r[u - 1]) * a.ldc;
+                    };
+                    float old[U];
 #pragma unroll
-                for (int e = 0; e < N; ++e) sum[e] = fmaf(av[u], b[u][e], sum[e]);
-            }
+                    for (int u = 1; u < U; ++u) old[u] = held >> u & 1u ? *c_of(u) : 0.f;
+                    if (closed && row_in != first_row) old_top = a.C[static_cast<int64_t>(row_in) * a.ldc];
+#pragma unroll
+                    for (int u = 1; u < U; ++u)
+                        if (held >> u & 1u) *c_of(u) = fmaf(a.beta, old[u], a.alpha * b[u][0]);
+                }
+            };
+            if (N == 1 && a.beta != 0.f) runs(std::bool_constant<N == 1>{});
+            else runs(std::false_type{});
             if (lane == 0) {
 #pragma unroll
                 for (int e = 0; e < N; ++e) (closed ? top[e] : sum[e]) += open[e];
@@ -302,6 +332,7 @@ coo_kernel(const CooArgs a) {
             open_row = __shfl_sync(FULL, row_out, 31);
             if (closed) {
                 if (row_in == first_row) carry(0, row_in, top);
+                else if (N == 1 && a.beta != 0.f) a.C[static_cast<int64_t>(row_in) * a.ldc] = fmaf(a.beta, old_top, a.alpha * top[0]);
                 else emit(row_in, top);
             }
         }

@@ -144,3 +144,22 @@ def test_frequent_columns_of_one_and_four_columns(N, empty, offset, dtype):
     got, _ = run_spmm(plan, w, c_fill=np.full((M, N), np.nan, np.float32), beta=0.0)
     check(w, got, beta=0.0)
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("lengths", [[1], [1, 2, 3], [7, 8, 9, 1, 1], [2, 300, 1, 5]])
+@pytest.mark.parametrize("empty", [False, True])
+def test_one_column_updates_c(empty, lengths, dtype):
+    """beta != 0 at one column: a lane has up to seven complete rows, whose old values it reads together, and the end of one that began
+    before; C with a pitch."""
+    rows = np.resize(lengths, 3001)
+    if empty:
+        rows[2::5] = 0
+    w = W.random_csr(3001, 700, 1, rows, seed=len(lengths), dtype=dtype, alpha=-0.5, beta=0.75)
+    plan = DeviceWorkload(w).plan(family=sd.SD_MERGE)
+    for kw in (dict(), dict(pad_c=2), dict(pad_b=1, offset=1)):
+        got, intact = run_spmm(plan, w, **kw)
+        assert intact
+        check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
+    plan.close()
