@@ -45,7 +45,15 @@ static int one_length_from(const SpmmArgs &a, int units, bool bf16) {
     const bool two = !bf16 && units >= rowsplit_two_from(a, bf16);
     return units > 16 || (units <= 8 && !two) ? 6 : 12;
 }
-static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
+// Products of a lane set in one accumulator: no more than in the kernels below where those would take the rows.  The set kernel and, of
+// two lanes, the plain kernel add 64 before they fold, the plain kernel of four 128, of more at least 256.  Rows beyond are folded every 64
+// (kGroupFold), in kernels with a second accumulator and four CTAs per SM for five (rows of 24, the longest 900, at 64 bf16 columns 42.9
+// -> 46.5 us, at 128 60.1 -> 62.4; with 64 everywhere also 400,000 rows of 35, the longest about 70, at 48 fp32 columns 275 -> 312, and
+// 6,000 rows of 150, the longest 300, at 64 and 200 bf16 columns 10.6 -> 11.7 and 45.3 -> 51.6).
+struct RowGroupForm {
+    int sets, terms;
+};
+static RowGroupForm rowgroup_form(const SpmmArgs &a, int dtype, int vw, bool vec) {
     const int units = (a.N + vw - 1) / vw;
     const int64_t mean = a.mean_len;
     int lanes = 1;
@@ -65,16 +73,10 @@ static int rowgroup_sets(const SpmmArgs &a, int dtype, int vw, bool vec) {
     else if (units <= 16) sets = mean >= 40 ? 4 : pow2 && mean >= 32 ? 2 : mean >= 8 || !pow2 ? 1 : 0;
     else if (units <= 32) sets = mean >= 40 ? 4 : !bf16 || mean >= 16 ? 1 : 0;
     else sets = mean >= 12 ? 4 : 1;
-    return a.max_len > 0 && a.max_len <= static_cast<int64_t>(kRowGroupTerms) * sets ? sets : 0;
-}
-
-// Products of a lane set in one accumulator: no more than in the kernels below, which would take the rows otherwise.  The set kernel and,
-// of two lanes, the plain kernel add 64 before they fold, the plain kernel of more lanes at least 128.  Rows beyond are folded every 64
-// (kGroupFold), in kernels with a second accumulator and four CTAs per SM for five (rows of 24, the longest 900, at 64 bf16 columns 42.9
-// -> 46.5 us, at 128 60.1 -> 62.4; with 64 everywhere also 400,000 rows of 35, the longest about 70, at 48 fp32 columns 275 -> 312).
-static int rowgroup_terms(const SpmmArgs &a, int vw) {
-    const int units = (a.N + vw - 1) / vw;
-    return units <= 2 || (units <= 16 && (units & (units - 1)) == 0 && a.mean_len >= 16) ? 64 : 128;
+    if (a.max_len <= 0 || a.max_len > static_cast<int64_t>(kRowGroupTerms) * sets) sets = 0;
+    const bool alone = !vec || (!fills && mean >= 8);
+    const bool set_kernel = units <= 16 && pow2 && mean >= 16;
+    return {sets, alone || units > 16 ? 256 : units <= 2 || set_kernel ? 64 : units <= 4 ? 128 : 256};
 }
 
 cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t st) {
@@ -84,10 +86,9 @@ cudaError_t run_rowsplit(const SpmmArgs &a, int dtype, int vw_now, cudaStream_t 
         if (dtype == SD_F32) return launch_rowsplit_narrow<float>(a, st);
         return launch_rowsplit_narrow<__nv_bfloat16>(a, st);
     }
-    if (const int sets = rowgroup_sets(a, dtype, vw_now, vec)) {
-        const int terms = rowgroup_terms(a, vw_now);
-        return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, sets, terms, st) : run_rowgroup_bf16(a, vw_now, sets, terms, st);
-    }
+    const RowGroupForm form = rowgroup_form(a, dtype, vw_now, vec);
+    if (form.sets > 0)
+        return dtype == SD_F32 ? run_rowgroup_f32(a, vw_now, form.sets, form.terms, st) : run_rowgroup_bf16(a, vw_now, form.sets, form.terms, st);
     // 8 to 64 columns (fp32; 8 to 128 bf16) as whole 16-byte vectors and long rows: several lane sets per row
     if (vec && a.N % vw == 0 && a.N / vw <= 16 && ((a.N / vw) & (a.N / vw - 1)) == 0) {
         const int lpr = a.N / vw;
