@@ -22,7 +22,9 @@ namespace sd {
 //                             26.3 / 24.8, of 15 105 / 81, 5-point stencils 14.8 / 13.7)
 //   8 columns                 four sets from 8 to 63 nonzeros (24: fp32 - / 18.6 / 15.3, bf16 - / 17.4 / 13.2), one below (3: 10.9 / 8.9 / 17.7)
 //   up to 8 loads             one set below 16 (32 columns, 3, 12: 24.0, 14.5 / 23.5, 14.5 / 71, 24); from there by the loads: 2: four to
-//                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
+//                             64 (16 bf16 columns, 24: 17.0 / 20.3 / 16.8), the set kernel with as many where B is beyond 8 MB, with fp32
+//                             values below 40 nonzeros (16 bf16 columns, set kernel / four sets here, 400,000 rows of 16, 24, 44: 41.6, 56.2, 91.7 /
+//                             46.0, 61.7, 95.0, 8 fp32 columns 37.9, 54.6, 88.1 / 40.6, 58.2, 89.0); 4: the set kernel below (16 columns, 24: 17.7 / 18.6 / 19.0; 1 M
 //                             rows of 40 at 32 bf16 columns 349 / 346 / 406); others: one to 64 (24 columns, 24, 44: 18.7, 29.8 / 15.6,
 //                             25.0 / -), then four (32 columns, 125: 41.6 / 34.8 / 27.3).  8: two, as many as in the set kernel, which has
 //                             2,048 threads on an SM for 1,280: that is ahead where B is far from the SMs, beyond 16 MB with fp32 values and
@@ -66,6 +68,7 @@ static RowGroupForm rowgroup_form(const SpmmArgs &a, int dtype, int vw, bool vec
     if (!vec) sets = mean >= 48 || (!fills && mean >= 8) ? 4 : 1;
     else if (!fills && mean >= 8) sets = 4;
     else if (one_length) sets = mean >= one_length_from(a, units, bf16) ? 1 : 0;
+    else if (units == 2 && mean >= 16 && mean < (bf16 ? 64 : 40) && a.b_bytes > 8000000 && even) sets = 0;
     else if (a.N <= 8) sets = mean < 8 ? 1 : mean < 64 ? 4 : 0;
     else if (units == 8 && mean >= 16 && mean < 64) sets = far && (!bf16 || mean < 32) ? 0 : 2;
     else if (units <= 8) sets = mean < 16 ? 1 : units == 2 ? (mean < 64 ? 4 : 0) : units == 4 ? 0 : mean < 64 ? 1 : 4;

@@ -208,6 +208,7 @@ inline int ksplit_group(int64_t mean_len, int lpr) {
     const int64_t per_set = lpr >= 16 ? 16 : 8;
     if (const int o = ksplit_override()) g = o;
     else while (2 * g * lpr <= lanes && 2 * g <= mean_len / per_set) g <<= 1;
+    if (lpr == 2 && mean_len >= 16 && g == 2 && !ksplit_override()) g = 4;   // as the row-group kernel has: these rows are its own but for the size of B
     while (g > 1 && g * lpr > 32) g >>= 1;
     return g;
 }

@@ -92,12 +92,12 @@ def test_two_and_four_columns_from_any_offset(mean, N, dtype):
 
 # 16-byte loads per row of B, columns of A, usual and longest row
 @pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
-@pytest.mark.parametrize("loads,K,usual,longest", [(2, 9000, 24, 30), (4, 9000, 24, 30), (8, 9000, 16, 64), (8, 9000, 33, 40), (8, 130000, 24, 30),
+@pytest.mark.parametrize("loads,K,usual,longest", [(2, 9000, 24, 30), (2, 260000, 24, 30), (2, 260000, 36, 40), (4, 9000, 24, 30), (8, 9000, 16, 64), (8, 9000, 33, 40), (8, 130000, 24, 30),
                                                    (8, 130000, 36, 40), (8, 130000, 24, 120), (16, 9000, 24, 30), (16, 9000, 36, 40),
                                                    (16, 9000, 36, 300), (16, 9000, 70, 80), (32, 9000, 20, 30)])
 def test_lane_sets_on_matrices_that_fill_the_gpu(loads, K, usual, longest, dtype):
     """More lanes than the GPU holds at five CTAs per SM (189,440), so that the rule goes by loads, mean length, longest row and size of B:
-    130,000 columns at eight loads are 16.6 MB."""
+    130,000 columns at eight loads are 16.6 MB, 260,000 at two 8.3."""
     N = loads * (4 if dtype == W.SD_F32 else 8)
     M = 200_000 // min(32, loads)
     rng = np.random.default_rng(loads + usual)
