@@ -56,7 +56,7 @@ struct CooArgs {
     const int32_t *rowptr;   // [M + 1], to find the rows without nonzeros (they get beta * C)
     int64_t M;
     int warps, per_warp;     // that work, ranges of each
-    int range, longer;       // steps of a range, and how many ranges (the first ones) have one more
+    uint64_t range;          // steps of a range, 32 bits of them behind the point: range r begins with the whole steps of r times this
     int spread;              // neighbouring ranges go to different CTAs
     int32_t *carry_row;      // [2 * warps * per_warp] out
     float *carry_val;        // [2 * warps * per_warp][N] out
@@ -189,7 +189,7 @@ coo_kernel(const CooArgs a) {
     // One range for most matrices.  The open sum below takes one addition per step, so a range is at most kCooRange steps long: one billion
     // nonzeros would make it 740, and the longest chain of sums with it.
     for (int n = 0; n < a.per_warp; ++n) {
-        const int range = w + n * a.warps, s0 = range * a.range + min(range, a.longer), s1 = s0 + a.range + (range < a.longer);
+        const int range = w + n * a.warps, s0 = static_cast<int>(range * a.range >> 32), s1 = static_cast<int>((range + 1) * a.range >> 32);
         auto carry = [&](int which, int row, const float (&v)[N]) {
             const int64_t at = 2 * range + which;
             a.carry_row[at] = row;
