@@ -146,11 +146,12 @@ __device__ __forceinline__ void coo_empty_rows(const CooArgs &a, int64_t share, 
         }
 }
 
-template <typename T, int N, bool VEC, bool HOT, bool BITS>
-__global__ void __launch_bounds__(HOT ? kCooHotThreads : coo_threads(N), HOT ? 1 : (N == 1 ? 9 : 4))
+template <typename T, int N, bool VEC, bool HOT, bool BITS, bool TURN = false>
+__global__ void __launch_bounds__(HOT ? kCooHotThreads : coo_threads(N), HOT ? 1 : (TURN ? 8 : N == 1 ? 9 : 4))
 coo_kernel(const CooArgs a) {
     constexpr unsigned FULL = 0xffffffffu;
     constexpr int U = coo_items(N), STEP = 32 * U;
+    static_assert(!TURN || (N == 1 && !HOT), "what a warp keeps to deal out its gathers");
     extern __shared__ __align__(16) char coo_hot_raw[];
     T *kept = reinterpret_cast<T *>(coo_hot_raw);
     overlap_wait();
@@ -172,6 +173,12 @@ coo_kernel(const CooArgs a) {
         }
         __syncthreads();
     }
+    // TURN: one column of a large matrix without frequent columns.  A gather takes 32 consecutive nonzeros there and not every eighth: those of a
+    // long row lie so close that some share a line of B (60 M nonzeros in rank-size rows, fp32 272 -> 262 us, 12 M in
+    // rows of 30,000 fp32 59 -> 54, bf16 52 -> 45; with few steps per warp the way through shared memory costs more than that, R-MAT scale
+    // 17 15.0 -> 16.5).
+    __shared__ __align__(16) float turns[TURN ? coo_threads(N) / 32 : 1][TURN ? STEP : 4];
+    [[maybe_unused]] float *const turn = turns[TURN ? threadIdx.x >> 5 : 0];
     const int lane = threadIdx.x & 31;
     const int w = a.spread ? (threadIdx.x >> 5) * gridDim.x + blockIdx.x : (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     if (w >= a.warps) return;
@@ -208,7 +215,12 @@ coo_kernel(const CooArgs a) {
             int row_out = 0;        // ... and where it ends
             const bool whole = k0 - lane * U >= a.shift && k0 - lane * U + STEP <= count;   // the same in all lanes: every item is a nonzero
             if (whole) {
-                load_ints<U>(a.colind + k0, col);
+                if constexpr (TURN) {
+#pragma unroll
+                    for (int u = 0; u < U; ++u) col[u] = __ldg(a.colind + (k0 - lane * U + u * 32 + lane));
+                } else {
+                    load_ints<U>(a.colind + k0, col);
+                }
                 if constexpr (!BITS) load_ints<U>(a.row + k0, r);
                 load_run<T, U>(vals + k0, va, av);
             } else {                // items before the first nonzero are zeros of its row, those past the end of the last one's
@@ -247,6 +259,19 @@ coo_kernel(const CooArgs a) {
                     if (!in) coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
                 } else {
                     coo_row_of_b<T, N, VEC>(b_row(B, col[u], a.ldb_bytes), b[u]);
+                }
+            }
+            if constexpr (TURN) {
+                if (whole) {   // dealt out in order
+                    __syncwarp();
+#pragma unroll
+                    for (int u = 0; u < U; ++u) turn[u * 32 + lane] = b[u][0];
+                    __syncwarp();
+#pragma unroll
+                    for (int u = 0; u < U; u += 4) {
+                        const float4 v = *reinterpret_cast<const float4 *>(turn + lane * U + u);
+                        b[u][0] = v.x, b[u + 1][0] = v.y, b[u + 2][0] = v.z, b[u + 3][0] = v.w;
+                    }
                 }
             }
             if (!whole)   // they gathered row 0: never let its contents (Inf, NaN) in

@@ -15,9 +15,9 @@ cudaError_t run_merge(const MergeArgs &m, bool vec, cudaStream_t st) {
 
 // ---- narrow dense operands: COO segmented reduction --------------------------------------------
 // One instance: the grid is as many CTAs as are resident together, or as give every warp a step.  Returns the ranges.
-template <typename T, int N, bool VEC, bool HOT, bool BITS>
+template <typename T, int N, bool VEC, bool HOT, bool BITS, bool TURN = false>
 static cudaError_t launch_coo_kernel(CooArgs a, int sm_count, int kept, cudaStream_t st, int64_t &ranges) {
-    auto kernel = coo_kernel<T, N, VEC, HOT, BITS>;
+    auto kernel = coo_kernel<T, N, VEC, HOT, BITS, TURN>;
     constexpr int threads = HOT ? kCooHotThreads : coo_threads(N);
     int64_t ctas = sm_count;
     if constexpr (HOT) {
@@ -77,10 +77,15 @@ static cudaError_t launch_coo_n(const CooPlan &cp, const SpmmArgs &s, int sm_cou
         a.hot = cp.hot;
     }
     if constexpr (N == 1) {
+        const bool turn = !hot && coo_steps(a.count, N) >= int64_t{8} * 32 * sm_count;   // eight steps and more for each of 32 warps per SM
         if (cp.starts)
-            e = hot ? launch_coo_kernel<T, N, VEC, true, true>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, true>(a, sm_count, 0, st, ranges);
+            e = hot    ? launch_coo_kernel<T, N, VEC, true, true>(a, sm_count, kept, st, ranges)
+                : turn ? launch_coo_kernel<T, N, VEC, false, true, true>(a, sm_count, 0, st, ranges)
+                       : launch_coo_kernel<T, N, VEC, false, true>(a, sm_count, 0, st, ranges);
         else
-            e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, ranges);
+            e = hot    ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, ranges)
+                : turn ? launch_coo_kernel<T, N, VEC, false, false, true>(a, sm_count, 0, st, ranges)
+                       : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, ranges);
     } else {
         e = hot ? launch_coo_kernel<T, N, VEC, true, false>(a, sm_count, kept, st, ranges) : launch_coo_kernel<T, N, VEC, false, false>(a, sm_count, 0, st, ranges);
     }

@@ -163,3 +163,30 @@ def test_one_column_updates_c(empty, lengths, dtype):
         check(w, got)
     assert np.array_equal(got, run_spmm(plan, w, **kw)[0])
     plan.close()
+
+
+@pytest.mark.parametrize("dtype", [W.SD_F32, W.SD_BF16])
+@pytest.mark.parametrize("M,length,empty", [(39, 300_000, False), (650_000, 18, True), (1, 11_000_000, False)])
+def test_one_column_of_many_steps(M, length, empty, dtype):
+    """More than eight steps of 256 nonzeros for each of 32 warps per SM (9.7 M nonzeros) without frequent columns: gathers of 32 consecutive
+    nonzeros, dealt out through shared memory; columns and values from an odd offset; a last step that is not whole."""
+    lengths = np.full(M, length)
+    if empty:
+        lengths[::9] = 0
+    K = 1_500_000
+    rng = np.random.default_rng(M)
+    rowptr = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int32)
+    colind = rng.integers(0, K, rowptr[-1]).astype(np.int32)   # repeated and in any order
+    vals, B = rng.standard_normal(colind.size).astype(np.float32), rng.standard_normal((K, 1)).astype(np.float32)
+    C = rng.standard_normal((M, 1)).astype(np.float32)
+    if dtype == W.SD_BF16:
+        vals, B = W.f32_to_bf16_bits(vals), W.f32_to_bf16_bits(B).reshape(K, 1)
+    w = W.Workload("many_steps", M, K, 1, rowptr, colind, vals, B, C, 1.5, -0.5, dtype, {})
+    colind, vals = (dev(np.concatenate([np.zeros(3, a.dtype), a]))[3:] for a in (colind, vals))
+    plan = sd.Plan(dev(rowptr), colind, vals, M, K, 1, dtype=dtype, family=sd.SD_MERGE)
+    assert plan.info().plan_bytes < 5 * colind.numel()   # no renamed columns
+    got, intact = run_spmm(plan, w)
+    assert intact
+    check(w, got)
+    assert np.array_equal(got, run_spmm(plan, w)[0])
+    plan.close()
