@@ -522,9 +522,10 @@ __global__ void rename_columns_kernel(const int32_t *__restrict__ colind, int64_
 
 // Taken where 4,096 columns pay for being fetched by every SM (at most nnz / 600 of them, nnz / 1000 at
 // one column) and if they cover a quarter of the nonzeros.  Without and with, us: R-MAT with 32.4 M nonzeros at one, two, three and four
-// fp32 columns 111 -> 86, 141 -> 122, 228 -> 177, 179 -> 162, one and two bf16 102 -> 87, 121 -> 119; with 7.9 M at one 26.5 -> 23.8;
-// with 3.9 M one fp32 16.6 and 16.2, two bf16 18.9 and 20.7, four 24.8 and 22.8; four fp32 columns, one 16-byte gather, only on the
-// largest (with 7.9 M 46.8 and 46.5).  More than kCooHotColumns gain nothing (one bf16 column 87 us with 32,768, 89 with 54,000).
+// fp32 columns 107 -> 83, 131 -> 110, 220 -> 169, 172 -> 155, bf16 96 -> 84, 117 -> 96, 215 -> 155, 159 -> 137; with 7.9 M at one 24.2 ->
+// 22.1, bf16 23.6 -> 22.7; with 4.6 M at one 18.2 and 18.5, bf16 17.0 and 17.3; with 3.9 M two bf16 16.1 and 16.4, four 23.1 and 21.5;
+// four fp32 columns, one 16-byte gather, only on the largest (with 16 M 86 -> 80).  More than kCooHotColumns gain nothing (one bf16 column
+// 87 us with 32,768, 89 with 54,000).  Plan creation takes longer for it: scale 18 at one column 437 us, 250 at 32 columns.
 constexpr int64_t kCooHotColumns = 32768;
 static sd_status_t coo_hot_columns(sd_plan *p, cudaStream_t st) {
     const int64_t row_bytes = p->N * (p->dtype == SD_F32 ? 4 : 2);
@@ -664,7 +665,8 @@ block_rows_kernel(const int32_t *__restrict__ rowptr, const int32_t *__restrict_
 // Values of the blocks, row-major 16x16, absent entries +0: a thread fetches one 16-byte vector of a block row, with one load if all
 // of it is there and aligned in the caller's array.  Bound by memory: each value is read and written once.  16,777 full bf16 blocks
 // with a product at 128 columns: 71 us per new set of values with a search of every nonzero's block and separate operand
-// images, 37 with a search in shared memory, 24 with these tables; 16,384 blocks 20.9 with a load per entry, 16.7 with vectors.
+// images, 37 with a search in shared memory, 24 with these tables; 16,384 blocks with values that the last calls have read too 20.9 with a
+// load per entry, 16.7 with vectors, with values that come from DRAM level.
 constexpr int kValThreads = 256;
 
 template <typename T>

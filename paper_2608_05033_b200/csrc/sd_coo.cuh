@@ -5,14 +5,14 @@
 // contiguous range of them and walks it 256 (three or four columns: 128) at a time; a lane adds up eight (four) consecutive
 // nonzeros by itself, and one segmented scan over the warp's lanes joins the rows that run across lanes.  A row that lies inside
 // the range is complete: its lane writes alpha * sum + beta * C.  The first and the last row of the range may continue in the
-// neighbours': their sums go to a carry list, two entries per warp in order, (first row, sum) and (last row, sum), or, where the
+// neighbours': their sums go to a carry list, two entries per range in order, (first row, sum) and (last row, sum), or, where the
 // range is one single row, (row, sum) and (row, 0), so that entries of one row stay adjacent.  The list is a row-sorted list
 // of values itself: a second kernel reduces it the same way, and the few entries that leaves over are added one row per thread.
 // Rows without nonzeros are found from the row pointers and get beta * C.  Every row is written by one thread and every sum has
 // a fixed order: results repeat bit for bit, no float atomics.
 //
-// Where rows begin: a bit per nonzero and the row of every eighth (0.6 bytes per nonzero; one column, no rows without
-// nonzeros), else a row index per nonzero (4 bytes).
+// Where rows begin: a bit per item and the row of every eighth (0.6 bytes per nonzero; one column, no rows without nonzeros), else
+// a row index per item (4 bytes).
 //
 // What bounds it: L1, a cycle per line of B that a gather touches, 32 for 32 unrelated rows.  Where a few columns hold much of the
 // matrix, the HOT form keeps their rows of B in shared memory (one CTA per SM), where 32 unrelated words cost about five
@@ -21,12 +21,13 @@
 // 32.4 M nonzeros, R-MAT scale 20, us, with a scan per 32 nonzeros and a carry per 256 before (one fp32 column and all with frequent
 // columns kept: as far as that paid then), and now:
 //     columns    1           2            3            4
-//     fp32       121 -> 86   169 -> 122   225 -> 177   239 -> 162
-//     bf16        95 -> 87   159 -> 119                267 -> 143
-// 60 M nonzeros in rank-size rows, uniform columns: one column 268 -> 272, two 392 -> 326, four 533 -> 424.  Small matrices are
-// level within 5 % (scale 12 to 16), at one bf16 column of scale 17 15.0 -> 16.4.  Tried: the next step's columns and values
-// requested ahead (registers: 86 -> 97), products formed in storage order and dealt out through shared memory (110), the next
-// launch let in before the carries are written (scale 16 11.5 -> 12.1).
+//     fp32       116 -> 83   170 -> 111   225 -> 170   238 -> 157
+//     bf16       102 -> 83   160 -> 98    237 -> 156   267 -> 137
+// 60 M nonzeros in rank-size rows, uniform columns: one column 251 -> 262, two 390 -> 303, four 512 -> 393.  Small matrices at one
+// column are level (scale 13 to 16 between 5.8 -> 6.2 and 11.2 -> 10.7), scale 17 16.4 -> 15.1, bf16 14.9 -> 14.7.  Tried: the next step's
+// columns and values requested ahead (registers: 86 -> 97), the frequent columns' products formed in storage order and dealt out through
+// shared memory (110), the next launch let in before the carries are written (scale 16 11.5 -> 12.1), the open sum folded in shared
+// memory every 32 steps (86 -> 88).
 #pragma once
 
 #include <type_traits>

@@ -8,7 +8,7 @@
 //   short    rows of fewer nonzeros, several per lane group (light_rows_body).
 //
 // What bounds it: on large matrices the rate at which L2 and L1 deliver gathered rows of B (64 bf16 columns, R-MAT scale
-// 20: 402 us = 10.3 TB/s with pairs handed round by shuffle; scale 19 since then 207 -> 175), on small ones the chain
+// 19, 16 M nonzeros: 181 us = 11.3 TB/s of rows of B; with pairs handed round by shuffle 207), on small ones the chain
 // of dependent gathers of the longest item, which the lane sets cut (8 columns, 128 nonzeros: 64 steps of a pair of lanes
 // before, 2 steps of a warp now; R-MAT scale 14: 51 -> 9 us).
 #pragma once
@@ -189,8 +189,9 @@ cudaError_t launch_hybrid_one(const HybridArgs &a, cudaStream_t st) {
 // Lanes across the columns for rows of `units` loads per row of B.  Full 16-byte loads: the next power of two up to 16, two
 // loads per lane beyond (128 fp32 columns on R-MAT scale 20 as 16 x 2: 1,212 us, as 32 x 1: 1,268).  Narrower loads (odd
 // widths, unaligned operands): two to four per lane, so that the work per nonzero on A is spread over more columns and few
-// lane slots are idle (R-MAT scale 17: 41 columns as 16 lanes x 3 61 us, as one warp x 4 101; 25 columns as 16 x 2 46 us,
-// as 32 x 1 56); wider rows run as slabs of about equal width.
+// lane slots are idle (compared on an earlier state of this kernel, R-MAT scale 17: 41 columns as 16 lanes x 3 61 us, as one warp
+// x 4 101; 25 columns as 16 x 2 46 us, as 32 x 1 56; 41 columns of 3.9 M nonzeros take 88 us now); wider rows run as slabs of
+// about equal width.
 template <typename T, int VW>
 cudaError_t launch_hybrid(const HybridArgs &a, cudaStream_t st) {
     constexpr bool FULL = VW * sizeof(T) == 16;

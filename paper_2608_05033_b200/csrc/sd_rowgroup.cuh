@@ -1,7 +1,7 @@
 // Family (a), one group of LANES lanes per row in natural order: LPR lanes stand across the columns, LANES / LPR lane sets share
 // the row's nonzeros (group_sum).  It serves every width that is not a whole number of 16-byte loads (odd widths, unaligned
 // operands: two to four loads of 8, 4 or 2 bytes per lane) and rows long enough to share at the others.  Rows of more than
-// kRowGroupTerms nonzeros per lane set that the rule asks for stay with the other kernels (not measured since long rows are folded).
+// kRowGroupTerms nonzeros per lane set that the rule asks for stay with the other kernels (a line from before long rows were folded).
 #pragma once
 
 #include "sd_group.cuh"
